@@ -7,18 +7,24 @@
 //   dense tiles   : original positions of one window (or of the sink region / the tail); seen
 //                   causally by the queries from the diagonal to the end of the last chunk that
 //                   still sees that window uncompressed
-// A CTA takes one tile and a segment of its (64-row query tile, query head of the group) list:
+// A CTA takes one tile and a segment of its (128-row query tile, query head of the group) list:
 //   S^T  = K_j Q_i^T     (smem x smem -> TMEM, keys on lanes)     P^T  = exp2(S^T*c - LSE_i*log2e)
 //   dP^T = V_j dO_i^T    (smem x smem -> TMEM)                    dS^T = P^T * (dP^T - D_i)
 //   dV  += P^T dO_i      (TMEM x smem -> TMEM)
 //   dK  += dS^T Q_i      (TMEM x smem -> TMEM)
-// P^T and dS^T are written back over S^T and dP^T as packed bf16; both are double-buffered so the
-// tensor core computes the next S^T/dP^T while the current pair is in the softmax, on which both
-// warpgroups work (32 query columns each).  Warps: 0 producer, 1-3 tensor-core issuers (S^T, dP^T,
-// dV/dK), 4-11 softmax and epilogue.  The softmax warps also sum P^T * dP^T over the keys (through
-// spare tensor-memory columns and a transposing load shape) and add it to a per-query-row accumulator:
-// D_i = sum_j P_ij dP_ij, the accurate replacement of rowsum(dO * O) that the dQ kernel (which runs
-// afterwards) needs.  The list of a tile runs from the last query tile backwards with the heads
+// P^T and dS^T are written back over S^T and dP^T as packed bf16.  One warp issues all products, in the order
+// dV(i), S^T(i+1), dK(i), dP^T(i+1): they run in that order, so single buffers for S^T and dP^T (all that tensor
+// memory has left beside the two D-wide accumulators) suffice, and the exponentials of step i+1 run while dK(i) and
+// dP^T(i+1) are computed, the rest of the softmax while dV and S^T are.  128 x 128 steps instead of 128 x 64 read
+// K_j and V_j half as often from shared memory (the tensor core's operands, 192 KB a step, are what bounds the
+// kernel together with the exponentials) and pay for half as many hand-offs: 5.23 -> 4.58 ms at 32K tokens, 28/4
+// heads, d = 128, one kept token in four.  Warps: 0 TMA producer, 1 issuer, 3 row statistics, 4-19 softmax and
+// epilogue.  A softmax warpgroup takes 32 query columns of every step: four warps per scheduler hide the latency
+// of one another's exponentials and tensor-memory accesses (two warps with 64 columns each: 4.71 ms), and P^T is
+// handed over in two halves so that dV starts on the first (in one piece: 4.90 ms).  The softmax warps also sum
+// P^T * dP^T over the keys (through their own dP^T columns and a transposing load shape) and add it to a
+// per-query-row accumulator: D_i = sum_j P_ij dP_ij, the accurate replacement of rowsum(dO * O) that the dQ kernel
+// (which runs afterwards) needs.  The list of a tile runs from the last query tile backwards with the heads
 // innermost, and compact tiles are launched segment by segment, so that the CTAs resident at one time
 // read the same Q_i / dO_i tiles (L2 hits instead of one DRAM pass per key tile).  At the end
 // the accumulators are added (fp32 atomics) to a zeroed workspace indexed by original position: a
@@ -31,8 +37,8 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kQRows = 64;    // query rows per inner tile
-constexpr int kSeg = 256;     // inner iterations per CTA at most
+constexpr int kQRows = 128;   // query rows per inner tile
+constexpr int kSeg = 128;     // inner iterations per CTA at most
 
 struct DkvPlan {
   int S, L, K, N, W, T, C, Wsel, ndp, Rc, G;
@@ -48,7 +54,7 @@ struct KvTile {
   int row0;      // first compact row / first key position
   int key_end;   // rows at or beyond this are not part of the tile
   int qb, qend;  // query positions [qb, qend) see (part of) the tile
-  int nq;        // 64-row query tiles per head
+  int nq;        // query tiles (kQRows rows) per head
 };
 
 inline DkvPlan make_dkv_plan(const Geom& g) {
@@ -167,14 +173,21 @@ __global__ void dkv_setup_kernel(const DkvPlan p, int* seg_cnt, int2* seg_map) {
 template <int D>
 struct DkvCfg {
   static constexpr int kSub = D / 64;
-  static constexpr int kKSubBytes = kTile * 128;            // 128 key rows x 128 bytes
-  static constexpr int kKTileBytes = kSub * kKSubBytes;     // K_j or V_j
-  static constexpr int kQSubBytes = kQRows * 128;           // 64 query rows x 128 bytes
-  static constexpr int kQTileBytes = kSub * kQSubBytes;     // Q_i or dO_i
-  static constexpr int kStageBytes = 2 * kQTileBytes;       // Q_i + dO_i
-  static constexpr int kStages = D == 128 ? 4 : 8;
-  static constexpr int kSmem = 2 * kKTileBytes + kStages * kStageBytes + 1024;
-  static constexpr int kThreads = 384;   // producer, three MMA issuers, eight softmax warps
+  static constexpr int kSubBytes = kTile * 128;             // 128 rows x 128 bytes (kQRows == kTile)
+  static constexpr int kTileBytes = kSub * kSubBytes;       // K_j, V_j, Q_i or dO_i
+  // Q_i is used by S^T(i) and, a whole step later, by dK(i); dO_i by dP^T(i) and dV(i), which follow each other:
+  // one slot more for Q_i keeps both prefetched by about a step.
+  static constexpr int kStQ = D == 128 ? 3 : 4;
+  static constexpr int kStO = D == 128 ? 2 : 3;
+  // K_j, V_j, the two rings, then per-row statistics (two slots of 128 x (-LSE*log2e, D)) and the barriers.
+  // At D = 128 this is all the shared memory a CTA can have, so nothing is static and nothing is padded.
+  static constexpr int kOffRingQ = 2 * kTileBytes;
+  static constexpr int kOffRingO = kOffRingQ + kStQ * kTileBytes;
+  static constexpr int kOffStats = kOffRingO + kStO * kTileBytes;
+  static constexpr int kOffCtl = kOffStats + 2 * 2 * kQRows * 4;
+  static constexpr int kSmem = kOffCtl + 512;
+  static constexpr int kSoftWarps = 16;  // four warpgroups, each 32 query columns of every step
+  static constexpr int kThreads = 128 + 32 * kSoftWarps;   // TMA producer, MMA issuer, (idle), statistics; softmax
   static constexpr uint32_t kColS = 0, kColP = 128, kColK = 256, kColV = 256 + D;
 };
 
@@ -193,11 +206,18 @@ struct DkvArgs {
   int* status;
 };
 
-struct DkvBars {
+// Barriers and per-step words, behind the statistics in shared memory.
+struct DkvCtl {
   uint64_t kv_full, acc_done;
-  uint64_t ring_full[8], ring_empty[8];
-  uint64_t s_full[2], p_full[2], buf_free[2], red_done[2];
+  uint64_t q_full[4], q_empty[4], o_full[3], o_empty[3];
+  uint64_t s_full, dp_full;      // S^T / dP^T of the step are in tensor memory
+  uint64_t p_full[2];            // halves of P^T: the first / last 16 query columns of every warpgroup
+  uint64_t st_full[2];           // statistics of the step (slot = step & 1) are staged
+  uint64_t ds_full[2];           // dS^T of the step is stored (slot = step & 1; also frees the statistics slot)
+  uint32_t tmem_base;
+  int abort;
 };
+static_assert(sizeof(DkvCtl) <= 512, "control block fits");
 
 __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
@@ -210,21 +230,16 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                     const __grid_constant__ CUtensorMap mapKg, const __grid_constant__ CUtensorMap mapVg,
                     const DkvArgs a) {
   using Cfg = DkvCfg<D>;
-  constexpr int NS = Cfg::kStages;
-  extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) DkvBars bars;
-  __shared__ __align__(16) float st_nl2[NS][kQRows];   // -LSE*log2(e) per query row of the stage (-inf: not seen)
-  __shared__ __align__(16) float st_D[NS][kQRows];
-  __shared__ int st_meta[NS][4];             // compact tiles: compact rows visible to the stage's first chunk,
-                                             // first column of its second chunk, rows visible to that chunk
-  __shared__ int st_q0[NS], st_hq[NS];       // first query position and query head of the stage (computed once,
-                                             // by the producer: an integer division per thread and tile is costly)
-  __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_s;
+  constexpr int NQ = Cfg::kStQ, NO = Cfg::kStO;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const uint32_t smem0 = smem_u32(smem_raw);
+  float* st_nl2 = reinterpret_cast<float*>(smem_raw + Cfg::kOffStats);   // [2][kQRows] -LSE*log2(e) (-inf: not seen)
+  float* st_D = st_nl2 + 2 * kQRows;                                     // [2][kQRows]
+  DkvCtl& ctl = *reinterpret_cast<DkvCtl*>(smem_raw + Cfg::kOffCtl);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t sK = smem0, sV = smem0 + Cfg::kKTileBytes, sRing = smem0 + 2 * Cfg::kKTileBytes;
+  const uint32_t sK = smem0, sV = smem0 + Cfg::kTileBytes;
+  const uint32_t sQ = smem0 + Cfg::kOffRingQ, sO = smem0 + Cfg::kOffRingO;
 
   // ---- which tile, which segment ----
   const DkvPlan& p = a.plan;
@@ -235,31 +250,39 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   const int n = min(kSeg, p.G * kt.nq - it_begin);
   const int hq0 = (bh_kv / a.Hkv) * a.Hq + (bh_kv % a.Hkv) * p.G;   // first query head of the group
 
+  if (smem0 & 1023u) {   // the swizzled tiles need it; dynamic shared memory starts there when nothing is static
+    if (tid == 0) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
+    return;
+  }
   if (tid == 0) {
-    abort_s = 0;
-    mbar_init(smem_u32(&bars.kv_full), 1);
-    mbar_init(smem_u32(&bars.acc_done), 1);
-    for (int i = 0; i < NS; ++i) { mbar_init(smem_u32(&bars.ring_full[i]), 1); mbar_init(smem_u32(&bars.ring_empty[i]), 1); }
+    ctl.abort = 0;
+    mbar_init(smem_u32(&ctl.kv_full), 1);
+    mbar_init(smem_u32(&ctl.acc_done), 1);
+    for (int i = 0; i < NQ; ++i) { mbar_init(smem_u32(&ctl.q_full[i]), 1); mbar_init(smem_u32(&ctl.q_empty[i]), 1); }
+    for (int i = 0; i < NO; ++i) { mbar_init(smem_u32(&ctl.o_full[i]), 1); mbar_init(smem_u32(&ctl.o_empty[i]), 1); }
+    mbar_init(smem_u32(&ctl.s_full), 1);
+    mbar_init(smem_u32(&ctl.dp_full), 1);
     for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_u32(&bars.s_full[b]), 2);      // the S^T issuer and the dP^T issuer
-      mbar_init(smem_u32(&bars.p_full[b]), 256);    // every softmax thread
-      mbar_init(smem_u32(&bars.buf_free[b]), 1);
-      mbar_init(smem_u32(&bars.red_done[b]), 256);  // every softmax thread has read its scratch columns back
+      mbar_init(smem_u32(&ctl.p_full[b]), Cfg::kSoftWarps);   // one arrival per softmax warp
+      mbar_init(smem_u32(&ctl.st_full[b]), 1);
+      mbar_init(smem_u32(&ctl.ds_full[b]), Cfg::kSoftWarps);
     }
     fence_barrier_init();
   }
-  if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), 512); tmem_relinquish(); }
+  if (warp == 1) { tmem_alloc(smem_u32(&ctl.tmem_base), 512); tmem_relinquish(); }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  const uint32_t tmem = tmem_base_s;
-  volatile int* abort = &abort_s;
+  const uint32_t tmem = ctl.tmem_base;
+  volatile int* abort = &ctl.abort;
+  // iteration gi of the tile: query tile nq-1 - gi/G (from the last query backwards) of head gi % G
+  const int qt0 = kt.nq - 1 - it_begin / p.G, hd0 = it_begin % p.G;
 
   if (warp == 0) {
-    // ---------------- producer (whole warp: lanes stage LSE and D, lane 0 drives TMA) ----------------
+    // ---------------- TMA producer ----------------
     if (lane == 0) {
       prefetch_tensormap(&mapQ); prefetch_tensormap(&mapdO);
-      mbar_expect_tx(smem_u32(&bars.kv_full), 2 * Cfg::kKTileBytes);
+      mbar_expect_tx(smem_u32(&ctl.kv_full), 2 * Cfg::kTileBytes);
     }
     __syncwarp();
     if (kt.kind == 0) {
@@ -270,21 +293,139 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
       for (int i = 0; i < 4; ++i)
         pos[i] = bh_kv * a.Nrow + compact_row_pos(kept, p.S, p.Rc, kt.row0 + 4 * lane + i, a.tok0);
       for (int h = 0; h < Cfg::kSub; ++h) {
-        tma_gather4_2d(sK + h * Cfg::kKSubBytes + lane * 512, &mapKg, h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&bars.kv_full));
-        tma_gather4_2d(sV + h * Cfg::kKSubBytes + lane * 512, &mapVg, h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&bars.kv_full));
+        tma_gather4_2d(sK + h * Cfg::kSubBytes + lane * 512, &mapKg, h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&ctl.kv_full));
+        tma_gather4_2d(sV + h * Cfg::kSubBytes + lane * 512, &mapVg, h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&ctl.kv_full));
       }
     } else if (lane == 0) {
       for (int h = 0; h < Cfg::kSub; ++h) {
-        tma_load_3d(sK + h * Cfg::kKSubBytes, &mapK, h * 64, kt.row0, bh_kv, smem_u32(&bars.kv_full));
-        tma_load_3d(sV + h * Cfg::kKSubBytes, &mapV, h * 64, kt.row0, bh_kv, smem_u32(&bars.kv_full));
+        tma_load_3d(sK + h * Cfg::kSubBytes, &mapK, h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
+        tma_load_3d(sV + h * Cfg::kSubBytes, &mapV, h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
       }
     }
-    bool ok = true;
-    int it = 0;
-    // per-row statistics of a stage are fetched one stage ahead, so that their latency overlaps the
-    // wait for a free slot instead of adding to it
-    // iteration gi: query tile nq-1 - gi/G (from the last query backwards) of head gi % G
-    int qt = kt.nq - 1 - it_begin / p.G, hd = it_begin % p.G;
+    if (lane == 0) {
+      int qt = qt0, hd = hd0, slq = 0, slo = 0, phq = 0, pho = 0;
+      int nq_issued = 0, no_issued = 0;
+      bool ok = true;
+      for (int it = 0; it < n; ++it) {
+        const int hq = hq0 + hd, q0 = kt.qb + qt * kQRows;
+        if (it >= NQ) ok = mbar_wait(smem_u32(&ctl.q_empty[slq]), phq ^ 1, abort);
+        if (!ok) break;
+        const uint32_t qf = smem_u32(&ctl.q_full[slq]);
+        mbar_expect_tx(qf, Cfg::kTileBytes);
+        for (int h = 0; h < Cfg::kSub; ++h)
+          tma_load_3d(sQ + slq * Cfg::kTileBytes + h * Cfg::kSubBytes, &mapQ, h * 64, q0, hq, qf);
+        ++nq_issued;
+        if (it >= NO) ok = mbar_wait(smem_u32(&ctl.o_empty[slo]), pho ^ 1, abort);
+        if (!ok) break;
+        const uint32_t of = smem_u32(&ctl.o_full[slo]);
+        mbar_expect_tx(of, Cfg::kTileBytes);
+        for (int h = 0; h < Cfg::kSub; ++h)
+          tma_load_3d(sO + slo * Cfg::kTileBytes + h * Cfg::kSubBytes, &mapdO, h * 64, q0, hq, of);
+        ++no_issued;
+        if (++slq == NQ) { slq = 0; phq ^= 1; }
+        if (++slo == NO) { slo = 0; pho ^= 1; }
+        if (++hd == p.G) { hd = 0; --qt; }
+      }
+      if (!ok) {
+        // give loads already in flight a bounded chance to land before the CTA's smem is released
+        auto drain = [](uint64_t* bars, int slots, int issued) {
+          for (int back = 1; back <= slots && back <= issued; ++back) {
+            const int i2 = issued - back;
+            const long long t0 = clock64();
+            while (!mbar_try_wait(smem_u32(&bars[i2 % slots]), (i2 / slots) & 1) && clock64() - t0 < 2000000) {}
+          }
+        };
+        drain(ctl.q_full, NQ, nq_issued);
+        drain(ctl.o_full, NO, no_issued);
+        drain(&ctl.kv_full, 1, 1);
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: dV(i), S^T(i+1), dK(i), dP^T(i+1), ... ----------------
+    // One warp issues everything, so the products run in this order on the tensor core: S^T(i+1) may overwrite
+    // P^T(i) and dP^T(i+1) may overwrite dS^T(i) without waiting for the products that read them.  The loop runs
+    // with all lanes (uniform control flow, descriptors computed once) and elects one lane per instruction.
+    constexpr uint32_t idesc_s = make_idesc_bf16(kTile, kQRows, 0, 0);  // 128 keys x 128 queries
+    constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);       // 128 keys x D
+    const uint64_t descK = make_smem_desc_sw128(sK, 16, 1024), descV = make_smem_desc_sw128(sV, 16, 1024);
+    const uint64_t descQ = make_smem_desc_sw128(sQ, 16, 1024), descO = make_smem_desc_sw128(sO, 16, 1024);   // K-major
+    const uint64_t descQm = make_smem_desc_sw128(sQ, Cfg::kSubBytes, 1024);                                   // MN-major
+    const uint64_t descOm = make_smem_desc_sw128(sO, Cfg::kSubBytes, 1024);
+    auto scores = [&](uint64_t dA, uint64_t dB, uint32_t d_tmem, uint64_t* bar) {
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk) {
+        const uint32_t off = (kk >> 2) * Cfg::kSubBytes + (kk & 3) * 32;
+        const uint64_t ad = desc_advance(dA, off), bd = desc_advance(dB, off);
+        if (elect_one()) umma_ss(d_tmem, ad, bd, idesc_s, kk > 0 ? 1u : 0u);
+      }
+      if (elect_one()) umma_commit(smem_u32(bar));
+      __syncwarp();
+    };
+    bool ok = mbar_wait_warp(smem_u32(&ctl.kv_full), 0, abort);
+    if (ok) ok = mbar_wait_warp(smem_u32(&ctl.q_full[0]), 0, abort);
+    if (ok) {
+      scores(descK, descQ, tmem + Cfg::kColS, &ctl.s_full);
+      ok = mbar_wait_warp(smem_u32(&ctl.o_full[0]), 0, abort);
+    }
+    if (ok) scores(descV, descO, tmem + Cfg::kColP, &ctl.dp_full);
+    int slq = 0, slo = 0, phq = 0, pho = 0;   // slots of step `it` and the phases of the slots of step it+1
+    for (int it = 0; it < n && ok; ++it) {
+      const int nslq = slq + 1 == NQ ? 0 : slq + 1, nslo = slo + 1 == NO ? 0 : slo + 1;
+      if (nslq == 0) phq ^= 1;
+      if (nslo == 0) pho ^= 1;
+      const uint32_t acc0 = it > 0 ? 1u : 0u;
+      // packed P^T / dS^T: the 32 query columns of warpgroup w in columns [32w, 32w+16) of the region
+      {
+        const uint64_t dB = desc_advance(descOm, slo * Cfg::kTileBytes);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          if (ok) ok = mbar_wait_warp(smem_u32(&ctl.p_full[half]), it & 1, abort);
+          if (!ok) break;
+          tc_fence_after_sync();
+#pragma unroll
+          for (int k4 = 0; k4 < 4; ++k4) {
+            const int kk = 2 * k4 + half;
+            const uint64_t bd = desc_advance(dB, kk * 2048);
+            if (elect_one())
+              umma_ts(tmem + Cfg::kColV, tmem + Cfg::kColS + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a,
+                      kk > 0 ? 1u : acc0);
+          }
+        }
+        if (!ok) break;
+        if (elect_one()) umma_commit(smem_u32(&ctl.o_empty[slo]));
+        __syncwarp();
+      }
+      if (it + 1 < n) {
+        ok = mbar_wait_warp(smem_u32(&ctl.q_full[nslq]), phq, abort);
+        if (!ok) break;
+        scores(descK, desc_advance(descQ, nslq * Cfg::kTileBytes), tmem + Cfg::kColS, &ctl.s_full);
+      }
+      ok = mbar_wait_warp(smem_u32(&ctl.ds_full[it & 1]), (it >> 1) & 1, abort);
+      if (!ok) break;
+      tc_fence_after_sync();
+      {
+        const uint64_t dB = desc_advance(descQm, slq * Cfg::kTileBytes);
+#pragma unroll
+        for (int kk = 0; kk < kQRows / 16; ++kk) {
+          const uint64_t bd = desc_advance(dB, kk * 2048);
+          if (elect_one())
+            umma_ts(tmem + Cfg::kColK, tmem + Cfg::kColP + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a, kk > 0 ? 1u : acc0);
+        }
+        if (elect_one()) umma_commit(smem_u32(&ctl.q_empty[slq]));
+        __syncwarp();
+      }
+      if (it + 1 < n) {
+        ok = mbar_wait_warp(smem_u32(&ctl.o_full[nslo]), pho, abort);
+        if (!ok) break;
+        scores(descV, desc_advance(descO, nslo * Cfg::kTileBytes), tmem + Cfg::kColP, &ctl.dp_full);
+      }
+      slq = nslq; slo = nslo;
+    }
+    if (ok && elect_one()) umma_commit(smem_u32(&ctl.acc_done));
+    __syncwarp();
+  } else if (warp == 3) {
+    // ---------------- per-row statistics of every step, fetched one step ahead ----------------
+    int qt = qt0, hd = hd0;
     auto fetch = [&](int qt_, int hd_, float2 (&v)[kQRows / 32]) {
       const int hq = hq0 + hd_, q0 = kt.qb + qt_ * kQRows;
 #pragma unroll
@@ -294,250 +435,160 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
       }
     };
     float2 cur[kQRows / 32], nxt[kQRows / 32];
-    if (n > 0) fetch(qt, hd, cur);
-    for (; it < n; ++it) {
-      const int slot = it % NS, use = it / NS;
+    bool ok = true;
+    fetch(qt, hd, cur);
+    for (int it = 0; it < n; ++it) {
+      const int b = it & 1;
       int qt_n = qt, hd_n = hd + 1;
       if (hd_n == p.G) { hd_n = 0; --qt_n; }
       if (it + 1 < n) fetch(qt_n, hd_n, nxt);
-      if (use > 0 && lane == 0) ok = mbar_wait(smem_u32(&bars.ring_empty[slot]), (use - 1) & 1, abort);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (it >= 2) ok = mbar_wait_warp(smem_u32(&ctl.ds_full[b]), ((it >> 1) - 1) & 1, abort);
       if (!ok) break;
-      const int hq = hq0 + hd, q0 = kt.qb + qt * kQRows;
 #pragma unroll
       for (int k = 0; k < kQRows / 32; ++k) {
-        st_nl2[slot][lane + 32 * k] = cur[k].x;
-        st_D[slot][lane + 32 * k] = cur[k].y;
+        st_nl2[b * kQRows + lane + 32 * k] = cur[k].x;
+        st_D[b * kQRows + lane + 32 * k] = cur[k].y;
         cur[k] = nxt[k];
       }
-      if (lane == 0) { st_q0[slot] = q0; st_hq[slot] = hq; }
-      if (lane == 0 && kt.kind == 0) {
-        const int cch = (q0 - p.S) / p.L;
-        st_meta[slot][0] = p.S + n_hist_windows(cch, p.ndp, p.Wsel) * p.K;
-        st_meta[slot][1] = min(kQRows, p.S + (cch + 1) * p.L - q0);
-        st_meta[slot][2] = p.S + n_hist_windows(cch + 1, p.ndp, p.Wsel) * p.K;
-      }
       __syncwarp();
-      if (lane == 0) {
-        const uint32_t full = smem_u32(&bars.ring_full[slot]);
-        mbar_expect_tx(full, Cfg::kStageBytes);
-        const uint32_t dst = sRing + slot * Cfg::kStageBytes;
-        for (int h = 0; h < Cfg::kSub; ++h) {
-          tma_load_3d(dst + h * Cfg::kQSubBytes, &mapQ, h * 64, q0, hq, full);
-          tma_load_3d(dst + Cfg::kQTileBytes + h * Cfg::kQSubBytes, &mapdO, h * 64, q0, hq, full);
-        }
-      }
+      if (lane == 0) mbar_arrive(smem_u32(&ctl.st_full[b]));
       qt = qt_n; hd = hd_n;
     }
-    if (!ok && lane == 0) {
-      for (int back = 1; back <= NS && back <= it; ++back) {
-        const int i2 = it - back;
-        const long long t0 = clock64();
-        while (!mbar_try_wait(smem_u32(&bars.ring_full[i2 % NS]), (i2 / NS) & 1) && clock64() - t0 < 2000000) {}
-      }
-    }
-  } else if (warp == 1 || warp == 2) {
-    // ---------------- S^T issuer (warp 1: K_j Q_i^T) and dP^T issuer (warp 2: V_j dO_i^T) ----------------
-    // Each issuing warp runs its loop with all lanes (uniform control flow, descriptors computed once)
-    // and elects one lane per instruction.
-    const int which = warp - 1;
-    constexpr uint32_t idesc_s = make_idesc_bf16(kTile, kQRows, 0, 0);  // 128 keys x 64 queries
-    const uint64_t descA = make_smem_desc_sw128(which == 0 ? sK : sV, 16, 1024);
-    const uint64_t descR = make_smem_desc_sw128(sRing + which * Cfg::kQTileBytes, 16, 1024);   // K-major Q_i / dO_i
-    bool ok = mbar_wait_warp(smem_u32(&bars.kv_full), 0, abort);
-    for (int it = 0; it < n && ok; ++it) {
-      const int slot = it % NS, b = it & 1;
-      ok = mbar_wait_warp(smem_u32(&bars.ring_full[slot]), (it / NS) & 1, abort);
-      if (ok && it >= 2) ok = mbar_wait_warp(smem_u32(&bars.buf_free[b]), ((it >> 1) - 1) & 1, abort);
-      if (ok && it >= 2) ok = mbar_wait_warp(smem_u32(&bars.red_done[b]), ((it >> 1) - 1) & 1, abort);
-      if (!ok) break;
-      tc_fence_after_sync();
-      const uint32_t d_tmem = tmem + (which == 0 ? Cfg::kColS : Cfg::kColP) + b * kQRows;
-      const uint64_t dB = desc_advance(descR, slot * Cfg::kStageBytes);
-#pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t koff = (kk >> 2) * Cfg::kKSubBytes + (kk & 3) * 32;
-        const uint32_t qoff = (kk >> 2) * Cfg::kQSubBytes + (kk & 3) * 32;
-        const uint64_t ad = desc_advance(descA, koff), bd = desc_advance(dB, qoff);
-        if (elect_one()) umma_ss(d_tmem, ad, bd, idesc_s, kk > 0 ? 1u : 0u);
-      }
-      if (elect_one()) umma_commit(smem_u32(&bars.s_full[b]));
-      __syncwarp();
-    }
-  } else if (warp == 3) {
-    // ---------------- dV / dK issuer ----------------
-    constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);       // 128 keys x D
-    const uint64_t descRmn = make_smem_desc_sw128(sRing, Cfg::kQSubBytes, 1024);     // MN-major Q_i / dO_i
-    bool ok = true;
-    for (int it = 0; it < n && ok; ++it) {
-      const int slot = it % NS, b = it & 1;
-      ok = mbar_wait_warp(smem_u32(&bars.p_full[b]), (it >> 1) & 1, abort);
-      if (!ok) break;
-      tc_fence_after_sync();
-      const uint64_t dQi = desc_advance(descRmn, slot * Cfg::kStageBytes);
-      const uint64_t ddOi = desc_advance(dQi, Cfg::kQTileBytes);
-      const uint32_t acc0 = it > 0 ? 1u : 0u;
-      // packed P^T / dS^T: queries [0,32) in columns [0,16) of the buffer, queries [32,64) in columns [32,48)
-#pragma unroll
-      for (int kk = 0; kk < kQRows / 16; ++kk) {
-        const uint64_t bd = desc_advance(ddOi, kk * 2048);
-        if (elect_one())
-          umma_ts(tmem + Cfg::kColV, tmem + Cfg::kColS + b * kQRows + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a,
-                  kk > 0 ? 1u : acc0);
-      }
-#pragma unroll
-      for (int kk = 0; kk < kQRows / 16; ++kk) {
-        const uint64_t bd = desc_advance(dQi, kk * 2048);
-        if (elect_one())
-          umma_ts(tmem + Cfg::kColK, tmem + Cfg::kColP + b * kQRows + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a,
-                  kk > 0 ? 1u : acc0);
-      }
-      if (elect_one()) {
-        umma_commit(smem_u32(&bars.ring_empty[slot]));
-        umma_commit(smem_u32(&bars.buf_free[b]));      // tile it+2 may overwrite the buffer
-      }
-      __syncwarp();
-    }
-    if (ok && elect_one()) umma_commit(smem_u32(&bars.acc_done));
-    __syncwarp();
-  } else {
-    // ---------------- P^T / dS^T: warpgroup `wg` takes query columns [32*wg, 32*wg+32) of every tile ----------------
+  } else if (warp >= 4) {
+    // ---------------- P^T / dS^T: warpgroup `wg` takes query columns [32*wg, 32*wg+32) of every step ----------------
     const int wg = (warp - 4) >> 2, quad = warp & 3;
     const int r = quad * 32 + lane;            // key row of this thread inside the tile
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    const uint32_t S_addr = tmem + lane_addr + Cfg::kColS + wg * 32;
+    const uint32_t P_addr = tmem + lane_addr + Cfg::kColP + wg * 32;
     const float c = a.scale_log2;
     const bool key_ok = kt.row0 + r < kt.key_end;
+    // First query position that sees this thread's key: its own (dense), or the start of the first chunk that sees
+    // its window compressed (list row; sinks: the first position after them).  Every later query sees it too.
+    int q_first = kt.row0 + r;
+    if (kt.kind == 0)
+      q_first = p.S + (q_first < p.S ? 0 : first_compressed_chunk((q_first - p.S) / p.K, p.ndp, p.Wsel, p.C) * p.L);
+    if (!key_ok) q_first = 0x40000000;
+    int q0 = kt.qb + qt0 * kQRows, hd = hd0;   // first query row and head (of the group) of the step
+    const int col = wg * 32 + 16 * ((lane >> 4) & 1) + 8 * ((lane >> 3) & 1) + 2 * (lane & 3) + ((lane >> 2) & 1);
     bool ok = true;
     for (int it = 0; it < n; ++it) {
-      const int slot = it % NS, b = it & 1;
-      ok = mbar_wait(smem_u32(&bars.s_full[b]), (it >> 1) & 1, abort);
-      if (ok) ok = mbar_wait(smem_u32(&bars.ring_full[slot]), (it / NS) & 1, abort);
+      const int b = it & 1;
+      const int lo = q_first - q0 - wg * 32;     // columns below it do not see the key
+      ok = mbar_wait_warp(smem_u32(&ctl.st_full[b]), (it >> 1) & 1, abort);
+      if (!ok) break;
+      const float4* nl2v = reinterpret_cast<const float4*>(st_nl2 + b * kQRows + wg * 32);
+      const float4* Dv = reinterpret_cast<const float4*>(st_D + b * kQRows + wg * 32);
+      ok = mbar_wait_warp(smem_u32(&ctl.s_full), it & 1, abort);
       if (!ok) break;
       tc_fence_after_sync();
-      const uint32_t S_addr = tmem + lane_addr + Cfg::kColS + b * kQRows + wg * 32;
-      const uint32_t P_addr = tmem + lane_addr + Cfg::kColP + b * kQRows + wg * 32;
-      uint32_t s[32], dp[32];
-      tmem_ld32(S_addr, s);
-      tmem_ld32(P_addr, dp);
-      tmem_wait_ld();
-      // first query column of this tile that sees this thread's key (64 = none)
-      const int q0 = st_q0[slot], hq = st_hq[slot];
-      int lo;
-      if (!key_ok) {
-        lo = kQRows;
-      } else if (kt.kind == 1) {
-        lo = kt.row0 + r - q0;                      // causal: query position >= key position
-      } else if (p.L >= kQRows) {                   // compact row, tile spans at most two chunks
-        const int cr = kt.row0 + r;
-        lo = cr < st_meta[slot][0] ? 0 : (cr < st_meta[slot][2] ? st_meta[slot][1] : kQRows);
-      } else {
-        const int cr = kt.row0 + r;                 // compact row: needs cr < S + n_hist(chunk)*K
-        lo = kQRows;
-        int col = 0;
-        while (col < kQRows) {
-          const int cch = (q0 + col - p.S) / p.L;
-          if (cr < p.S + n_hist_windows(cch, p.ndp, p.Wsel) * p.K) { lo = col; break; }
-          col = p.S + (cch + 1) * p.L - q0;         // first column of the next chunk
+      // P^T in halves of 16 columns: the tensor core starts dV on the first halves while the second are formed
+      float pr[32];
+      {
+        uint32_t s[32];
+        tmem_ld32(S_addr, s);
+        tmem_wait_ld();
+        if (lo > 0) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (i < lo) s[i] = 0xff800000u;
+        }
+        const uint64_t c2 = f2_pack(c, c);   // packed fp32 pairs: one issue slot for two elements
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t pp[8];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int e = 16 * h + 4 * v;
+            const float4 nl = nl2v[4 * h + v];
+            float a0, a1, a2, a3;
+            f2_unpack(f2_fma(f2_pack(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, f2_pack(nl.x, nl.y)), a0, a1);
+            f2_unpack(f2_fma(f2_pack(__uint_as_float(s[e + 2]), __uint_as_float(s[e + 3])), c2, f2_pack(nl.z, nl.w)), a2, a3);
+            pr[e] = ex2(a0); pr[e + 1] = ex2(a1); pr[e + 2] = ex2(a2); pr[e + 3] = ex2(a3);
+            pp[2 * v] = pack_bf16(pr[e], pr[e + 1]);
+            pp[2 * v + 1] = pack_bf16(pr[e + 2], pr[e + 3]);
+          }
+          tmem_st8(S_addr + 8 * h, pp);   // over the first half of this warpgroup's own columns, already loaded
+          tmem_wait_st();
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&ctl.p_full[h]));
         }
       }
-      lo -= wg * 32;
-      if (lo > 0) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (i < lo) s[i] = 0xff800000u;
-      }
-      const float4* nl2v = reinterpret_cast<const float4*>(st_nl2[slot] + wg * 32);
-      const float4* Dv = reinterpret_cast<const float4*>(st_D[slot] + wg * 32);
-      uint32_t pp[16], ds[16];
-      float x[32];   // P * dP, whose sum over the keys is the accurate D of the query column
+      ok = mbar_wait_warp(smem_u32(&ctl.dp_full), it & 1, abort);
+      if (!ok) break;
+      tc_fence_after_sync();
+      // dS^T = P dP - P D; x = P dP (whose sum over the keys is the accurate D of the query column) replaces P
+      uint32_t ds[16];
       {
-        // packed fp32 pairs: one issue slot for two elements of every multiply-add below
-        const uint64_t c2 = f2_pack(c, c);
+        uint32_t dp[32];
+        tmem_ld32(P_addr, dp);
+        tmem_wait_ld();
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
-          const float4 nl = nl2v[v], dd = Dv[v];
-          float a0, a1, a2, a3, d0, d1, d2, d3;
-          f2_unpack(f2_fma(f2_pack(__uint_as_float(s[4 * v + 0]), __uint_as_float(s[4 * v + 1])), c2, f2_pack(nl.x, nl.y)), a0, a1);
-          f2_unpack(f2_fma(f2_pack(__uint_as_float(s[4 * v + 2]), __uint_as_float(s[4 * v + 3])), c2, f2_pack(nl.z, nl.w)), a2, a3);
-          const float p0 = ex2(a0), p1 = ex2(a1), p2 = ex2(a2), p3 = ex2(a3);
-          pp[2 * v] = pack_bf16(p0, p1);
-          pp[2 * v + 1] = pack_bf16(p2, p3);
-          const uint64_t p01 = f2_pack(p0, p1), p23 = f2_pack(p2, p3);
+          const float4 dd = Dv[v];
+          float d0, d1, d2, d3;
+          const uint64_t p01 = f2_pack(pr[4 * v], pr[4 * v + 1]), p23 = f2_pack(pr[4 * v + 2], pr[4 * v + 3]);
           const uint64_t x01 = f2_mul(p01, f2_pack(__uint_as_float(dp[4 * v + 0]), __uint_as_float(dp[4 * v + 1])));
           const uint64_t x23 = f2_mul(p23, f2_pack(__uint_as_float(dp[4 * v + 2]), __uint_as_float(dp[4 * v + 3])));
-          f2_unpack(x01, x[4 * v + 0], x[4 * v + 1]);
-          f2_unpack(x23, x[4 * v + 2], x[4 * v + 3]);
-          f2_unpack(f2_fma(p01, f2_pack(-dd.x, -dd.y), x01), d0, d1);   // dS = P dP - P D
+          f2_unpack(f2_fma(p01, f2_pack(-dd.x, -dd.y), x01), d0, d1);
           f2_unpack(f2_fma(p23, f2_pack(-dd.z, -dd.w), x23), d2, d3);
+          f2_unpack(x01, pr[4 * v], pr[4 * v + 1]);
+          f2_unpack(x23, pr[4 * v + 2], pr[4 * v + 3]);
           ds[2 * v] = pack_bf16(d0, d1);
           ds[2 * v + 1] = pack_bf16(d2, d3);
         }
       }
-      tmem_st16(S_addr, pp);   // over the first half of this warpgroup's own columns
+      // Sum of x over the warp's 32 keys: the values go through this warpgroup's own dP^T columns (all loaded, and
+      // dS^T is not stored yet: the tensor core is busy with dV and the next S^T meanwhile) and come back with the
+      // 16-lane x 256-bit load shape, which hands every thread four key rows of eight query columns; the
+      // remaining three levels are register exchanges, after dS^T is on its way.
+      tmem_st32(P_addr, *reinterpret_cast<uint32_t(*)[32]>(&pr[0]));
+      tmem_wait_st();
+      uint32_t ra[16], rb[16];
+      tmem_ld_16x256b_x4(P_addr, ra);
+      tmem_ld_16x256b_x4(P_addr + (16u << 16), rb);
+      tmem_wait_ld();
       tmem_st16(P_addr, ds);
       tmem_wait_st();
       tc_fence_before_sync();
-      mbar_arrive(smem_u32(&bars.p_full[b]));
-      // Off the tensor core's critical path: sum x over the warp's 32 keys.  The values go through the
-      // upper halves of this warpgroup's own S^T and dP^T columns (free once P^T and dS^T are packed into
-      // the lower halves; the issuers wait for red_done before the buffer is written again) and come back
-      // with the 16-lane x 256-bit load shape, which hands every thread four key rows of eight query
-      // columns; the remaining three levels are register exchanges.  (A full five-level exchange in
-      // registers costs twice the instructions, and shuffles share the shared-memory pipe with the
-      // tensor core's operand reads.)
-      {
-        uint32_t xa[16], xb[16];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&ctl.ds_full[b]));
+      float c8[8];   // index 2j + e: column 8j + 2(lane%4) + e of the warpgroup's 32
 #pragma unroll
-        for (int i = 0; i < 16; ++i) { xa[i] = __float_as_uint(x[i]); xb[i] = __float_as_uint(x[16 + i]); }
-        tmem_st16(S_addr + 16, xa);
-        tmem_st16(P_addr + 16, xb);
-        tmem_wait_st();
-        uint32_t ra0[8], ra1[8], rb0[8], rb1[8];
-        tmem_ld_16x256b_x2(S_addr + 16, ra0);
-        tmem_ld_16x256b_x2(S_addr + 16 + (16u << 16), ra1);
-        tmem_ld_16x256b_x2(P_addr + 16, rb0);
-        tmem_ld_16x256b_x2(P_addr + 16 + (16u << 16), rb1);
-        tmem_wait_ld();
-        tc_fence_before_sync();
-        mbar_arrive(smem_u32(&bars.red_done[b]));
-        float c8[8];   // index 4B + 2j + e: column 16B + 8j + 2(lane%4) + e of the warpgroup's 32
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+        for (int e = 0; e < 2; ++e)
+          c8[2 * j + e] = (__uint_as_float(ra[4 * j + e]) + __uint_as_float(ra[4 * j + 2 + e])) +
+                          (__uint_as_float(rb[4 * j + e]) + __uint_as_float(rb[4 * j + 2 + e]));
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            c8[2 * j + e] = (__uint_as_float(ra0[4 * j + e]) + __uint_as_float(ra0[4 * j + 2 + e])) +
-                            (__uint_as_float(ra1[4 * j + e]) + __uint_as_float(ra1[4 * j + 2 + e]));
-            c8[4 + 2 * j + e] = (__uint_as_float(rb0[4 * j + e]) + __uint_as_float(rb0[4 * j + 2 + e])) +
-                                (__uint_as_float(rb1[4 * j + e]) + __uint_as_float(rb1[4 * j + 2 + e]));
-          }
+      for (int m = 4, bit = 16; m >= 1; m >>= 1, bit >>= 1) {
+        const bool up = (lane & bit) != 0;
 #pragma unroll
-        for (int m = 4, bit = 16; m >= 1; m >>= 1, bit >>= 1) {
-          const bool up = (lane & bit) != 0;
-#pragma unroll
-          for (int i = 0; i < m; ++i) {
-            const float send = up ? c8[i] : c8[i + m];
-            const float keep = up ? c8[i + m] : c8[i];
-            c8[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
-          }
+        for (int i = 0; i < m; ++i) {
+          const float send = up ? c8[i] : c8[i + m];
+          const float keep = up ? c8[i + m] : c8[i];
+          c8[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
         }
-        const int col = 16 * ((lane >> 4) & 1) + 8 * ((lane >> 3) & 1) + 2 * (lane & 3) + ((lane >> 2) & 1);
-        const int q = q0 + wg * 32 + col;
-        if (q < kt.qend) atomicAdd(a.Dacc + (size_t)hq * a.Nrow + q, c8[0]);
       }
+      if (q0 + col < kt.qend) atomicAdd(a.Dacc + (size_t)(hq0 + hd) * a.Nrow + q0 + col, c8[0]);
+      if (++hd == p.G) { hd = 0; q0 -= kQRows; }
     }
-    if (ok) ok = mbar_wait(smem_u32(&bars.acc_done), 0, abort);
+    if (ok) ok = mbar_wait_warp(smem_u32(&ctl.acc_done), 0, abort);
     if (ok) {
       tc_fence_after_sync();
-      // warpgroup 0 adds dK (scaled), warpgroup 1 adds dV
-      const uint32_t acc = tmem + lane_addr + (wg == 0 ? Cfg::kColK : Cfg::kColV);
-      const float mul = wg == 0 ? a.scale : 1.0f;
+      // warpgroups 0 and 1 add dK (scaled), 2 and 3 dV, half of the columns each
+      constexpr int CH = D / 2;
+      const bool is_k = wg < 2;
+      const uint32_t acc = tmem + lane_addr + (is_k ? Cfg::kColK : Cfg::kColV) + (wg & 1) * CH;
+      const float mul = is_k ? a.scale : 1.0f;
       // a row of a compact tile lands on the position it was gathered from
       const int out_row = kt.kind == 0
                               ? compact_row_pos(a.idx + (size_t)bh_kv * a.kept_stride, p.S, p.Rc, kt.row0 + r, a.tok0)
                               : kt.row0 + r;
-      float* dst = (wg == 0 ? a.dKf : a.dVf) + ((size_t)bh_kv * a.Nrow + out_row) * D;
+      float* dst = (is_k ? a.dKf : a.dVf) + ((size_t)bh_kv * a.Nrow + out_row) * D + (wg & 1) * CH;
 #pragma unroll
-      for (int q = 0; q < D / 32; ++q) {
+      for (int q = 0; q < CH / 32; ++q) {
         uint32_t o[32];
         tmem_ld32(acc + q * 32, o);
         tmem_wait_ld();
@@ -554,7 +605,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, 512);
-  if (tid == 0 && abort_s) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
+  if (tid == 0 && ctl.abort) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
 }
 
 // bf16 outputs from the fp32 accumulators [BHkv][N][d]; n4 = number of float4 groups
