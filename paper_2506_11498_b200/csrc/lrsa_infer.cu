@@ -11,9 +11,9 @@
 // with window c-1 as its reference) and its kept rows are appended to the list when the first token of
 // chunk c arrives: not earlier, because the queries of chunk c-1 still see it whole.
 //
-// Decode attention reads the list prefix and the ring once per KV head for all query heads of the group
-// (HBM-bound: 4*d bytes per key, a few FMAs per byte): the keys are split over CTAs, every warp keeps an
-// online softmax per query head, and a second small kernel merges the partial results.
+// Decode attention reads the list prefix and the ring once per KV head for (up to 16) query heads of the group
+// (HBM-bound: 4*d bytes per key, a few FMAs per byte): the keys are split over CTAs and warps, every warp keeps an
+// online softmax of its keys, and a second small kernel merges the partial results.
 #include "lrsa_internal.h"
 #include "sm100_ptx.h"
 
@@ -45,275 +45,314 @@ CacheLayout cache_layout(const Geom& g) {
   return c;
 }
 
-// New tokens [p0, p1) of every (batch, KV head) into the sink rows of the list or into the ring.
-// One warp per (head, token); src rows are [BH][n_new][d] with token p at row p - p_first.
-__global__ void cache_insert_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
-                                    __nv_bfloat16* k_list, __nv_bfloat16* v_list, __nv_bfloat16* k_ring,
-                                    __nv_bfloat16* v_ring, int BH, int n_new, int p_first, int p0, int p1, int S, int L,
-                                    int rows_list, int d) {
-  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int n = p1 - p0;
-  if (wid >= (long long)BH * n) return;
-  const int bh = (int)(wid / n), p = p0 + (int)(wid % n), lane = threadIdx.x & 31;
-  const size_t src = ((size_t)bh * n_new + (p - p_first)) * d;
-  __nv_bfloat16 *kd, *vd;
-  if (p < S) {
-    kd = k_list + ((size_t)bh * rows_list + p) * d; vd = v_list + ((size_t)bh * rows_list + p) * d;
+// ---- growing the cache ----
+struct CacheRows {
+  const __nv_bfloat16 *k_new, *v_new;               // [BH][n_new][d], token p at row p - p_first
+  __nv_bfloat16 *k_list, *v_list, *k_ring, *v_ring;
+  const int32_t* idx;                                // [BH][Wcap][K]
+  int* status;                                       // cleared when not null
+  int n_new, p_first, S, L, K, Wcap, rows_list, cpr; // cpr: 16-byte chunks per row (d / 8)
+  int n_sink;           // the new tokens of the call up to the last sink, when p0 lies beyond them
+  int p0, n_ins;        // tokens [p0, p0 + n_ins) go to the sink rows of the list or to the ring
+  int w0, n_keep;       // kept rows: n_keep = windows * K rows of windows w0 ...
+  int blocks;           // thread blocks per (batch, KV head)
+  int keep_from_ring;   // their source: the ring (a window that had entered the cache before) or the new tokens
+};
+
+// New tokens into the sink rows of the list or into the ring, and the kept rows of newly compressed windows into
+// the list (items: tokens first, then kept rows; a thread moves 16 bytes of K and of V).  Bound by the rows it moves
+// (one read and one write each); one launch for a whole prompt, whose tokens go to the ring only if they stay there.
+// A 32K prompt (windows of 1024 tokens, 4 KV heads, d = 128): window after window, three launches each, 1.25 ms;
+// scoring all windows in one launch and this kernel behind it 42 us.
+__global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
+  const int rpb = 256 / a.cpr;   // rows per block
+  const int bh = blockIdx.x / a.blocks, item = (blockIdx.x % a.blocks) * rpb + threadIdx.x / a.cpr, ch = threadIdx.x % a.cpr;
+  const int n_tok = a.n_sink + a.n_ins;
+  if (item >= n_tok + a.n_keep) return;
+  const size_t list0 = (size_t)bh * a.rows_list, ring0 = (size_t)bh * 2 * a.L;
+  size_t src, dst;
+  bool from_ring = false, to_list = true;
+  if (item < n_tok) {
+    const int p = item < a.n_sink ? a.p_first + item : a.p0 + (item - a.n_sink);
+    src = (size_t)bh * a.n_new + (p - a.p_first);
+    to_list = p < a.S;
+    dst = to_list ? list0 + p : ring0 + (p - a.S) % (2 * a.L);
   } else {
-    const size_t r = ((size_t)bh * 2 * L + (p - S) % (2 * L)) * d;
-    kd = k_ring + r; vd = v_ring + r;
+    const int r = item - n_tok;
+    const int pos = a.idx[((size_t)bh * a.Wcap + a.w0) * a.K + r];
+    from_ring = a.keep_from_ring != 0;
+    src = from_ring ? ring0 + (pos - a.S) % (2 * a.L) : (size_t)bh * a.n_new + (pos - a.p_first);
+    dst = list0 + a.S + (size_t)a.w0 * a.K + r;
   }
-  for (int c = lane * 2; c < d; c += 64) {
-    *reinterpret_cast<uint32_t*>(kd + c) = *reinterpret_cast<const uint32_t*>(k_new + src + c);
-    *reinterpret_cast<uint32_t*>(vd + c) = *reinterpret_cast<const uint32_t*>(v_new + src + c);
-  }
+  const uint4 k = reinterpret_cast<const uint4*>(from_ring ? a.k_ring : a.k_new)[src * a.cpr + ch];
+  const uint4 v = reinterpret_cast<const uint4*>(from_ring ? a.v_ring : a.v_new)[src * a.cpr + ch];
+  reinterpret_cast<uint4*>(to_list ? a.k_list : a.k_ring)[dst * a.cpr + ch] = k;
+  reinterpret_cast<uint4*>(to_list ? a.v_list : a.v_ring)[dst * a.cpr + ch] = v;
 }
 
-// The K kept rows of window w, from the ring to rows S + w*K ... of the list.  One warp per (head, kept row).
-__global__ void cache_keep_kernel(const int32_t* __restrict__ idx, const __nv_bfloat16* __restrict__ k_ring,
-                                  const __nv_bfloat16* __restrict__ v_ring, __nv_bfloat16* k_list, __nv_bfloat16* v_list,
-                                  int BH, int w, int Wcap, int K, int S, int L, int rows_list, int d) {
-  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (wid >= (long long)BH * K) return;
-  const int bh = (int)(wid / K), r = (int)(wid % K), lane = threadIdx.x & 31;
-  const int pos = idx[((size_t)bh * Wcap + w) * K + r];
-  const size_t src = ((size_t)bh * 2 * L + (pos - S) % (2 * L)) * d;
-  const size_t dst = ((size_t)bh * rows_list + S + (size_t)w * K + r) * d;
-  for (int c = lane * 2; c < d; c += 64) {
-    *reinterpret_cast<uint32_t*>(k_list + dst + c) = *reinterpret_cast<const uint32_t*>(k_ring + src + c);
-    *reinterpret_cast<uint32_t*>(v_list + dst + c) = *reinterpret_cast<const uint32_t*>(v_ring + src + c);
-  }
+// Launch that may start before the kernel in front of it has ended (the kernel waits for that itself).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+int launch_cache_rows(CacheRows a, int BH, cudaStream_t st) {
+  const int rows = a.n_sink + a.n_ins + a.n_keep, rpb = 256 / a.cpr;
+  a.blocks = (rows + rpb - 1) / rpb;
+  LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), st, a));
+  launch_counter().n++;
+  return LRSA_OK;
+}
 
 // ---- decode attention ----
-constexpr int kDecThreads = 128;
-constexpr int kDecHeads = 16;     // query heads of a group per pass over the keys (the M of the tensor-core product)
-constexpr int kDecKeys = 128;     // keys per CTA (32 per warp), staged in shared memory
+constexpr int kDecMaxWarps = 16;
+// Warps of the largest CTA: 128 registers hold the operands of one group of 8 heads; two groups take more.
+__host__ __device__ constexpr int dec_max_warps(int nh) { return nh == 1 ? kDecMaxWarps : kDecMaxWarps / 2; }
 
 struct DecodeArgs {
   const __nv_bfloat16 *q, *k_list, *v_list, *k_ring, *v_ring;
-  float* part;          // [BHkv][n_split][G][D + 2]: unnormalised output, running maximum (log2 domain), sum
+  float* part;          // [BHkv][n_split][G][D + 2]: unnormalised output, maximum (log2 domain), sum
   int* status;          // workspace status word
-  int BHkv, Hq, Hkv, G, rows_list, L, S;
-  int n_list, n_ring, ring0;   // keys: list rows [0, n_list), then n_ring ring rows starting at ring row ring0
-  int n_split;
+  int Hq, Hkv, G, rows_list, ring_rows;
+  int n_list, n_keys, ring0;   // keys: list rows [0, n_list), then ring rows from ring row ring0 on (wrapping)
+  int n_split, blocks;         // key blocks per (batch, KV head), dealt out evenly to the splits
   float scale_log2;
 };
 
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
 // D (16x8, fp32) += A (16x16, bf16, row) * B (16x8, bf16, col)
-__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                          uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// transpose of an 8x8 matrix of 16-bit elements held two per lane
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+__device__ __forceinline__ uint4 ld_stream(const void* p) {   // read once: no place in L1
+  uint4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
 }
 
-// Grid (n_split, BHkv).  One query token per (batch, head) and a few hundred to a few thousand keys per KV head:
-// the work is the transfer of K and V, so the CTA's (at most) 128 key rows are fetched at once (every thread
-// issues one bulk copy for its row of K and one for its row of V) and everything after that has to be short.
-// The query heads of the KV group form the rows of a small matrix product (GQA: 16 rows per pass, the unused
-// ones zero), so S = Q K^T and O = P V run on the warp-level tensor-core instructions (m16n8k16, bf16 operands,
-// fp32 accumulation; a 128-row tcgen05 product would be nine tenths padding here): a warp takes 32 keys, reads
-// Q, K and V fragments with ldmatrix from rows padded by 16 bytes (rows 128 or 256 bytes apart would put the
-// eight rows of a fragment on the same banks), forms the softmax of its 32 keys in registers and hands P over
-// as the A operand of the second product.  The four warps' partial results are merged through shared memory;
-// the splits by decode_merge_kernel.
-template <int D>
-__global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const DecodeArgs a) {
-  constexpr int CPR = D / 8;                 // 16-byte chunks per row
-  constexpr int KS = D / 16;                 // k-steps of Q K^T
-  constexpr int NT = D / 8;                  // 8-channel tiles of the output
-  constexpr int kRowBytes = D * 2, kStride = kRowBytes + 16;
-  extern __shared__ __align__(128) unsigned char dec_smem[];   // K rows [kDecKeys], V rows [kDecKeys], Q rows [16]
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ int s_fail;
+// Grid (n_split, BHkv), 4 to 16 warps.  One query token per (batch, head) over a few hundred to a few thousand keys
+// per KV head: the work is the transfer of K and V (two bytes per multiply-add of one head), so the kernel is built
+// around the loads.  A warp takes blocks of 2048 / D keys; it loads the block's K and V rows straight into the
+// registers in which the warp-level tensor-core products want them and has 8 KB in flight while the other warps of
+// the SM compute; nothing is staged in shared memory (with one bulk copy per row into it, a barrier and ldmatrix the
+// kernel took 90.6 us for 16 sequences of 9471 keys, 4 KV heads, d = 128; now 52.7 us = 5.9 TB/s, 90 % of a copy's rate;
+// one such sequence, where latency counts: 7.3 -> 7.1 us).  The query heads of the KV group are the n of the products
+// (8 at a time; a 128-row tcgen05 product would be nine tenths padding):
+//   S^T = K Q^T    A = K  (m = keys, k = channels): lane (g, t) = (lane / 4, lane % 4) loads 16-byte chunks t, t+4, ...
+//                  of rows g and g + 8; the order of the channels in the contraction is free, and Q is read alike
+//   O^T = V^T P^T  A = V^T (m = channels, k = keys): chunk g (+8) of rows 2t, 2t+1, 2t+8, 2t+9; a byte permute pairs
+//                  the keys.  P^T comes out of the first product with keys and heads the other way round: one
+//                  movmatrix per eight keys turns it.
+// The maximum is raised only when it grew by more than 2^8 (then O is rescaled); it is common to the warp, since the
+// second product sums over the keys of all its lanes.  The warps are merged through shared memory, the splits by
+// decode_merge_kernel.
+template <int D, int NH>
+__global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_partial_kernel(const DecodeArgs a) {
+  constexpr int U = 128 / D;                // 16-key groups per block
+  constexpr int KC = D / 32, VC = D / 64;   // 16-byte chunks per lane and row, of K and of V
+  constexpr int MT = D / 16;                // channel tiles of the output
+  constexpr int kSlots = dec_max_warps(NH) / 2;
+  __shared__ __align__(16) float sm_o[kSlots][8][D + 4];   // padded: lanes of a store differ in the head
+  __shared__ float sm_m[kSlots][8], sm_l[kSlots][8];
   const int bh = blockIdx.y, split = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_keys = a.n_list + a.n_ring;
-  const int k_lo = split * kDecKeys, k_hi = min(n_keys, k_lo + kDecKeys), nk = k_hi - k_lo;
+  const int nw = blockDim.x >> 5, g = lane >> 2, t = lane & 3;
   const int b = bh / a.Hkv, hkv = bh % a.Hkv;
-  const uint32_t sK = ptx::smem_u32(dec_smem), sV = sK + kDecKeys * kStride, sQ = sV + kDecKeys * kStride;
-  unsigned char* gQ = dec_smem + 2 * kDecKeys * kStride;
-  // The merge kernel is launched as a programmatic dependent of this one: its CTAs may be scheduled from here
-  // on and wait (griddepcontrol.wait) until this grid has completed and its stores are visible.
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the cache rows of the kernel in front of this one
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (tid == 0) {
-    s_fail = 0;
-    ptx::mbar_init(ptx::smem_u32(&bar), 1);
-    ptx::fence_barrier_init();
-    ptx::mbar_expect_tx(ptx::smem_u32(&bar), (uint32_t)nk * kRowBytes * 2);   // every row copy below reports here
-    // the only writer of the status word before a wait below can expire (seconds later)
-    if (split == 0 && bh == 0) *a.status = 0;
-  }
-  __syncthreads();
-  {
-    // this thread's row of K and of V
-    const int r = tid;
-    if (r < nk) {
-      const int k = k_lo + r;
-      const __nv_bfloat16 *ks, *vs;
-      if (k < a.n_list) {
-        const size_t off = ((size_t)bh * a.rows_list + k) * D;
-        ks = a.k_list + off; vs = a.v_list + off;
-      } else {
-        const size_t off = ((size_t)bh * 2 * a.L + (a.ring0 + (k - a.n_list)) % (2 * a.L)) * D;
-        ks = a.k_ring + off; vs = a.v_ring + off;
-      }
-      bulk_load(sK + r * kStride, ks, kRowBytes, ptx::smem_u32(&bar));
-      bulk_load(sV + r * kStride, vs, kRowBytes, ptx::smem_u32(&bar));
-    } else {
-      // rows beyond the split's keys: their probabilities are zero, their V must not be NaN
-#pragma unroll
-      for (int c = 0; c < CPR; ++c) {
-        *reinterpret_cast<uint4*>(dec_smem + r * kStride + c * 16) = make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4*>(dec_smem + (kDecKeys + r) * kStride + c * 16) = make_uint4(0, 0, 0, 0);
-      }
-    }
-  }
+  if (split == 0 && bh == 0 && tid == 0) *a.status = 0;
+  const unsigned char* kl = reinterpret_cast<const unsigned char*>(a.k_list) + (size_t)bh * a.rows_list * (D * 2);
+  const unsigned char* kr = reinterpret_cast<const unsigned char*>(a.k_ring) + (size_t)bh * a.ring_rows * (D * 2);
+  const ptrdiff_t v_of_list = reinterpret_cast<const unsigned char*>(a.v_list) - reinterpret_cast<const unsigned char*>(a.k_list);
+  const ptrdiff_t v_of_ring = reinterpret_cast<const unsigned char*>(a.v_ring) - reinterpret_cast<const unsigned char*>(a.k_ring);
+  // K row of key `key`, and what leads from there to its V row
+  auto row_of = [&](int key, ptrdiff_t& to_v) {
+    key = min(key, a.n_keys - 1);       // beyond the end: any row that is there (its probability is zero)
+    const bool in_list = key < a.n_list;
+    int r = key - a.n_list + a.ring0;
+    if (r >= a.ring_rows) r -= a.ring_rows;
+    to_v = in_list ? v_of_list : v_of_ring;
+    return in_list ? kl + (size_t)key * (D * 2) : kr + (size_t)r * (D * 2);
+  };
+  const int blk0 = (int)((long long)a.blocks * split / a.n_split), blk1 = (int)((long long)a.blocks * (split + 1) / a.n_split);
 
-  const int row = lane >> 2, cpair = (lane & 3) * 2;   // fragment coordinates of this lane
-  for (int g0 = 0; g0 < a.G; g0 += kDecHeads) {
-    const int ng = min(kDecHeads, a.G - g0);
-    // Q of this pass: 16 rows (heads g0 ..., zero beyond the group) into shared memory, 16 bytes per thread and step
-    for (int i = tid; i < kDecHeads * CPR; i += kDecThreads) {
-      const int g = i / CPR, cch = i % CPR;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (g < ng) v = *reinterpret_cast<const uint4*>(a.q + ((size_t)(b * a.Hq + hkv * a.G + g0 + g)) * D + cch * 8);
-      *reinterpret_cast<uint4*>(gQ + g * kStride + cch * 16) = v;
+  for (int g0 = 0; g0 < a.G; g0 += 8 * NH) {
+    // Q of head g0 + 8h + g as the B operand: the chunks this lane also takes of every key row
+    uint4 q[NH][KC];
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+#pragma unroll
+      for (int j = 0; j < KC; ++j) {
+        const int head = g0 + 8 * h + g;
+        q[h][j] = make_uint4(0, 0, 0, 0);
+        if (head < a.G)
+          q[h][j] = *reinterpret_cast<const uint4*>(a.q + ((size_t)(b * a.Hq + hkv * a.G + head)) * D + (t + 4 * j) * 8);
+      }
+    float o[NH][MT][4];        // tile 4j + f: channels 8(g + 8j) + 2f, + 1 of heads 2t, 2t + 1
+    float m[NH][2], l[NH][2];  // heads 2t, 2t + 1: maximum (the warp's), sum (this lane's keys)
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+      m[h][0] = m[h][1] = -INFINITY;
+      l[h][0] = l[h][1] = 0.f;
+#pragma unroll
+      for (int i = 0; i < MT; ++i) o[h][i][0] = o[h][i][1] = o[h][i][2] = o[h][i][3] = 0.f;
     }
-    if (g0 == 0) {
-      // bounded wait for the copies; a CTA that gives up records it, waits once more for its copies (they write
-      // this CTA's shared memory) and leaves its partial result empty
-      bool got = ptx::mbar_try_wait(ptx::smem_u32(&bar), 0);
-      const long long t0 = clock64();
-      while (!got) {
-        got = ptx::mbar_try_wait(ptx::smem_u32(&bar), 0);
-        if (!got && clock64() - t0 > 4000000000LL) { s_fail = 1; break; }
+    for (int blk = blk0 + warp; blk < blk1; blk += nw) {
+      const int key0 = blk * (16 * U);
+      uint4 kq[U][2][KC], vq[U][4][VC];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          ptrdiff_t to_v;
+          const unsigned char* r = row_of(key0 + 16 * u + g + 8 * i, to_v);
+#pragma unroll
+          for (int j = 0; j < KC; ++j) kq[u][i][j] = ld_stream(r + (t + 4 * j) * 16);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          ptrdiff_t to_v;
+          const unsigned char* r = row_of(key0 + 16 * u + 2 * t + (i & 1) + 8 * (i >> 1), to_v);
+#pragma unroll
+          for (int j = 0; j < VC; ++j) vq[u][i][j] = ld_stream(r + to_v + (g + 8 * j) * 16);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {
+        float s[U][4];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          s[u][0] = s[u][1] = s[u][2] = s[u][3] = 0.f;
+#pragma unroll
+          for (int j = 0; j < KC; ++j) {
+            mma_16816(s[u], kq[u][0][j].x, kq[u][1][j].x, kq[u][0][j].y, kq[u][1][j].y, q[h][j].x, q[h][j].y);
+            mma_16816(s[u], kq[u][0][j].z, kq[u][1][j].z, kq[u][0][j].w, kq[u][1][j].w, q[h][j].z, q[h][j].w);
+          }
+        }
+        // elements: e = 0, 1: key g, heads 2t, 2t + 1; e = 2, 3: key g + 8
+        float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            s[u][e] = key0 + 16 * u + g + 8 * (e >> 1) < a.n_keys ? s[u][e] * a.scale_log2 : -INFINITY;
+            mx[e & 1] = fmaxf(mx[e & 1], s[u][e]);
+          }
+        if (__any_sync(0xffffffffu, mx[0] > m[h][0] + 8.f || mx[1] > m[h][1] + 8.f)) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+#pragma unroll
+            for (int x = 4; x < 32; x <<= 1) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], x));
+            const float mn = fmaxf(m[h][e], mx[e]);   // finite: a block holds at least one key
+            const float f = m[h][e] == -INFINITY ? 0.f : exp2f(m[h][e] - mn);
+            m[h][e] = mn;
+            l[h][e] *= f;
+#pragma unroll
+            for (int i = 0; i < MT; ++i) { o[h][i][e] *= f; o[h][i][e + 2] *= f; }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float p[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            p[e] = exp2f(s[u][e] - m[h][e & 1]);
+            l[h][e & 1] += p[e];
+          }
+          const uint32_t b0 = transpose_8x8(ptx::pack_bf16(p[0], p[1])), b1 = transpose_8x8(ptx::pack_bf16(p[2], p[3]));
+#pragma unroll
+          for (int j = 0; j < VC; ++j)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+              auto w = [&](int i) { return f == 0 ? vq[u][i][j].x : f == 1 ? vq[u][i][j].y : f == 2 ? vq[u][i][j].z : vq[u][i][j].w; };
+              mma_16816(o[h][4 * j + f], __byte_perm(w(0), w(1), 0x5410), __byte_perm(w(0), w(1), 0x7632),
+                        __byte_perm(w(2), w(3), 0x5410), __byte_perm(w(2), w(3), 0x7632), b0, b1);
+            }
+        }
       }
     }
-    __syncthreads();
-    if (s_fail) {
-      if (tid == 0) {
-        atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
-        const long long t0 = clock64();
-        while (!ptx::mbar_try_wait(ptx::smem_u32(&bar), 0) && clock64() - t0 < 4000000000LL) {}
+    // Merge the warps: the upper half hands its state to the lower half, then all threads add what is left.
+    const int half = nw / 2;
+    const bool upper = warp >= half;
+    const int slot = upper ? warp - half : warp;   // nw is even and half <= kSlots
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+      float lh[2], mh[2];
+      auto put = [&]() {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float* dst = sm_o[slot][2 * t + e];
+#pragma unroll
+          for (int i = 0; i < MT; ++i)
+            *reinterpret_cast<float2*>(dst + 8 * (g + 8 * (i >> 2)) + 2 * (i & 3)) = make_float2(o[h][i][e], o[h][i][e + 2]);
+          if (g == 0) { sm_m[slot][2 * t + e] = mh[e]; sm_l[slot][2 * t + e] = lh[e]; }
+        }
+      };
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        mh[e] = m[h][e];
+        lh[e] = l[h][e];
+#pragma unroll
+        for (int y = 4; y < 32; y <<= 1) lh[e] += __shfl_xor_sync(0xffffffffu, lh[e], y);
+      }
+      __syncthreads();   // the buffer is free
+      if (upper) put();
+      __syncthreads();
+      if (!upper) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float mo = sm_m[slot][2 * t + e], mn = fmaxf(mh[e], mo);
+          const float f0 = mh[e] == -INFINITY ? 0.f : exp2f(mh[e] - mn), f1 = mo == -INFINITY ? 0.f : exp2f(mo - mn);
+          lh[e] = lh[e] * f0 + sm_l[slot][2 * t + e] * f1;
+          mh[e] = mn;
+          const float* srcp = sm_o[slot][2 * t + e];
+#pragma unroll
+          for (int i = 0; i < MT; ++i) {
+            const float2 v = *reinterpret_cast<const float2*>(srcp + 8 * (g + 8 * (i >> 2)) + 2 * (i & 3));
+            o[h][i][e] = o[h][i][e] * f0 + v.x * f1;
+            o[h][i][e + 2] = o[h][i][e + 2] * f0 + v.y * f1;
+          }
+        }
+        __syncwarp();   // every lane has read the slot before it is overwritten
+        put();
       }
       __syncthreads();
-      // empty partial results: maximum -inf, the merge kernel skips them
-      for (int i = tid; i < ng; i += kDecThreads) {
-        float* dst = a.part + (((size_t)bh * a.n_split + split) * a.G + g0 + i) * (D + 2);
-        dst[D] = -INFINITY; dst[D + 1] = 0.f;
-      }
-      continue;
-    }
-    // Q as A fragments: matrices (heads 0-7, channels k..k+7), (heads 8-15, same), then channels k+8..k+15
-    uint32_t qa[KS][4];
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
-      ldmatrix_x4(sQ + ((lane & 7) + 8 * ((lane >> 3) & 1)) * kStride + (2 * ks + (lane >> 4)) * 16, qa[ks]);
-    // S = Q K^T for this warp's 32 keys: four tiles of 8 keys
-    float s[4][4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
-      const int key = warp * 32 + 8 * j + (lane & 7);
-#pragma unroll
-      for (int q4 = 0; q4 < CPR / 4; ++q4) {
-        uint32_t kb[4];
-        ldmatrix_x4(sK + key * kStride + (4 * q4 + (lane >> 3)) * 16, kb);
-        mma_16816(s[j], qa[2 * q4], kb[0], kb[1]);
-        mma_16816(s[j], qa[2 * q4 + 1], kb[2], kb[3]);
+      const int ng = min(8, a.G - g0 - 8 * h);
+      for (int i = tid; i < ng * D; i += blockDim.x) {
+        const int hd = i / D, c = i % D;
+        float M = -INFINITY;
+        for (int w = 0; w < half; ++w) M = fmaxf(M, sm_m[w][hd]);
+        float ov = 0.f, ls = 0.f;
+        for (int w = 0; w < half; ++w) {
+          const float f = sm_m[w][hd] == -INFINITY ? 0.f : exp2f(sm_m[w][hd] - M);
+          ov = fmaf(sm_o[w][hd][c], f, ov);
+          ls = fmaf(sm_l[w][hd], f, ls);
+        }
+        float* dst = a.part + (((size_t)bh * a.n_split + split) * a.G + g0 + 8 * h + hd) * (D + 2);
+        dst[c] = ov;
+        if (c == 0) { dst[D] = M; dst[D + 1] = ls; }
       }
     }
-    // scale, mask the keys beyond the split, row maxima and sums (rows: head `row` -> index 0, `row + 8` -> 1)
-    float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int key = warp * 32 + 8 * j + cpair + (e & 1);
-        s[j][e] = key < nk ? s[j][e] * a.scale_log2 : -INFINITY;
-        mx[e >> 1] = fmaxf(mx[e >> 1], s[j][e]);
-      }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-    }
-    float sum[2] = {0.f, 0.f};
-    uint32_t pa[2][4];   // P as A fragments of the two 16-key steps
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float pr[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        pr[e] = mx[e >> 1] == -INFINITY ? 0.f : exp2f(s[j][e] - mx[e >> 1]);
-        sum[e >> 1] += pr[e];
-      }
-      pa[j >> 1][(j & 1) * 2 + 0] = ptx::pack_bf16(pr[0], pr[1]);
-      pa[j >> 1][(j & 1) * 2 + 1] = ptx::pack_bf16(pr[2], pr[3]);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      sum[h] += __shfl_xor_sync(0xffffffffu, sum[h], 1);
-      sum[h] += __shfl_xor_sync(0xffffffffu, sum[h], 2);
-    }
-    // O = P V: V fragments transposed on the way out of shared memory (keys are the contraction index)
-    float o[NT][4];
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
-      uint32_t vb[4];
-      ldmatrix_x4_trans(sV + (warp * 32 + lane) * kStride + nt * 16, vb);
-      mma_16816(o[nt], pa[0], vb[0], vb[1]);
-      mma_16816(o[nt], pa[1], vb[2], vb[3]);
-    }
-    // merge the four warps through shared memory (the K rows are no longer needed once every warp is here;
-    // with more than one pass over the heads they are needed again, so the merge buffer then follows V)
-    __syncthreads();
-    float* mrg = reinterpret_cast<float*>(dec_smem + (a.G > kDecHeads ? (2 * kDecKeys + kDecHeads) * kStride : 0));
-    float* mo = mrg;                                   // [4 warps][16 heads][D]
-    float* mm_ = mrg + 4 * kDecHeads * D;              // [4][16] maxima
-    float* ml = mm_ + 4 * kDecHeads;                   // [4][16] sums
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      *reinterpret_cast<float2*>(mo + ((warp * kDecHeads + row) * D + nt * 8 + cpair)) = make_float2(o[nt][0], o[nt][1]);
-      *reinterpret_cast<float2*>(mo + ((warp * kDecHeads + row + 8) * D + nt * 8 + cpair)) = make_float2(o[nt][2], o[nt][3]);
-    }
-    if ((lane & 3) == 0) {
-      mm_[warp * kDecHeads + row] = mx[0]; mm_[warp * kDecHeads + row + 8] = mx[1];
-      ml[warp * kDecHeads + row] = sum[0]; ml[warp * kDecHeads + row + 8] = sum[1];
-    }
-    __syncthreads();
-    for (int i = tid; i < ng * D; i += kDecThreads) {
-      const int g = i / D, c = i % D;
-      float M = -INFINITY;
-#pragma unroll
-      for (int w = 0; w < 4; ++w) M = fmaxf(M, mm_[w * kDecHeads + g]);
-      float ov = 0.f, lsum = 0.f;
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const float mw = mm_[w * kDecHeads + g];
-        const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
-        ov = fmaf(mo[(w * kDecHeads + g) * D + c], f, ov);
-        lsum = fmaf(ml[w * kDecHeads + g], f, lsum);
-      }
-      float* dst = a.part + (((size_t)bh * a.n_split + split) * a.G + g0 + g) * (D + 2);
-      dst[c] = ov;
-      if (c == 0) { dst[D] = M; dst[D + 1] = lsum; }
-    }
-    __syncthreads();   // the merge buffer is reused by the next pass
+    __syncthreads();   // the merge buffer is reused by the next heads
   }
 }
 
@@ -335,6 +374,7 @@ __global__ void __launch_bounds__(kMergeRows * D) decode_merge_kernel(const floa
   constexpr int kBatch = 4;
   // launched as a programmatic dependent of the partial kernel: wait for its grid to complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (int s0 = row; s0 < n_split; s0 += kMergeRows * kBatch) {
     float ms[kBatch], vs[kBatch], ls[kBatch];
 #pragma unroll
@@ -376,7 +416,39 @@ __global__ void __launch_bounds__(kMergeRows * D) decode_merge_kernel(const floa
   }
 }
 
-int decode_splits(int n_keys) { return n_keys > 0 ? (n_keys + kDecKeys - 1) / kDecKeys : 1; }
+// How the keys of the (batch, KV head) pairs are dealt out: `splits` CTAs of `warps` warps each.
+struct DecodePlan { int nh, warps, blocks, splits; };
+constexpr int kDecMaxSplits = 148;
+DecodePlan decode_plan(const Geom& g, int n_keys) {
+  DecodePlan p;
+  p.nh = g.G > 8 ? 2 : 1;
+  const int per_block = 2048 / g.d;
+  const long long BH = (long long)g.B * g.Hkv;
+  p.blocks = n_keys > 0 ? (n_keys + per_block - 1) / per_block : 1;
+  // 16 warps (8 with two groups of heads) are resident per SM, as one large CTA or several small ones.  Large ones
+  // leave fewer partial results to merge; small ones fill the SMs more evenly when every SM has several blocks per
+  // warp to do.  The number of splits is the one that ends first, counting a merge as two blocks.
+  const int max_warps = dec_max_warps(p.nh);
+  p.warps = BH * p.blocks > 2LL * 148 * max_warps ? 4 : max_warps;
+  const int slots = 148 * (max_warps / p.warps);
+  const long long useful = 4LL * slots / BH + 1;   // beyond four waves more splits only add merges
+  long long best = 0;
+  p.splits = 1;
+  for (int s = 1; s <= kDecMaxSplits && s <= useful && (s == 1 || (s - 1) * p.warps < p.blocks); ++s) {
+    const long long waves = (BH * s + slots - 1) / slots;
+    const int per_cta = (p.blocks + s - 1) / s;
+    const long long cost = waves * ((per_cta + p.warps - 1) / p.warps + 2);
+    if (s == 1 || cost < best) { best = cost; p.splits = s; }
+  }
+  return p;
+}
+
+template <int D, int NH>
+int launch_partial(const DecodeArgs& a, const DecodePlan& pl, int BHkv, cudaStream_t st) {
+  LRSA_CUDA_CHECK(launch_dependent(decode_partial_kernel<D, NH>, dim3(pl.splits, BHkv), dim3(pl.warps * 32), st, a));
+  launch_counter().n++;
+  return LRSA_OK;
+}
 
 }  // namespace
 }  // namespace lrsa
@@ -392,12 +464,15 @@ int lrsa_cache_bytes(const lrsa_params_t* params, size_t* cache_bytes, size_t* w
   if (params->n_seqs > 0 || g.ndp != 1) return LRSA_ERR_UNSUPPORTED;
   if (cache_bytes) *cache_bytes = cache_layout(g).total;
   if (workspace_bytes) {
-    // scoring scratch of a two-window problem, or the partial results of the decode kernel
-    Geom two = g;
-    two.N = two.Nrow = 2 * g.L; two.S = 0; two.W = 2; two.Wsel = 1; two.T = 0; two.C = 2;
-    const size_t a = score_select_ws_bytes(two);
-    // a sequence of N tokens never shows a query more than S + Wcap*K + 2L keys
-    const size_t b = 256 + (size_t)g.B * g.Hkv * decode_splits(cache_layout(g).rows_list + 2 * g.L) * g.G * (g.d + 2) * sizeof(float);
+    // scoring scratch of the windows of a whole prompt (lag windows beyond 4096 tokens), or the partial results of the
+    // decode kernel: no more splits than blocks of keys for four warps each
+    const CacheLayout lay = cache_layout(g);
+    Geom all = g;
+    all.W = lay.Wcap + 1 > 2 ? lay.Wcap + 1 : 2; all.Wsel = all.W - 1;
+    const size_t a = score_select_ws_bytes(all);
+    const int blocks = (int)(((long long)(lay.rows_list + 2 * g.L) * g.d + 2047) / 2048);
+    const int splits = blocks / 4 + 1 < kDecMaxSplits ? blocks / 4 + 1 : kDecMaxSplits;
+    const size_t b = 256 + (size_t)g.B * g.Hkv * splits * g.G * (g.d + 2) * sizeof(float);
     *workspace_bytes = a > b ? a : b;
   }
   return LRSA_OK;
@@ -428,46 +503,74 @@ int lrsa_cache_append(const lrsa_params_t* params, void* cache, size_t cache_byt
   auto* v_ring = reinterpret_cast<__nv_bfloat16*>(cb + lay.v_ring);
   auto* idx = reinterpret_cast<int32_t*>(cb + lay.idx);
   const int BH = g.B * g.Hkv;
-  LRSA_CUDA_CHECK(cudaMemsetAsync(workspace, 0, sizeof(WsHeader), st));
-  launch_counter().n++;
-  int pos = n_prev;
-  const int end = n_prev + n_new;
-  while (pos < end) {
-    int seg_end = end;
-    if (pos < g.S) {
-      seg_end = end < g.S ? end : g.S;
-    } else {
-      const int c = (pos - g.S) / g.L;
-      if (pos == g.S + c * g.L && c >= 2) {
-        // The first token of chunk c: window c-2 leaves the ring.  It is scored with window c-1 as its
-        // reference (the two halves of the ring, in either order) and its kept rows join the list.
-        const int w = c - 2;
-        Geom two = g;
-        two.N = 2 * g.L; two.Nrow = 2 * g.L; two.S = 0; two.W = 2; two.Wsel = 1; two.T = 0; two.C = 2;
-        two.tok0 = (w % 2) * g.L;
-        two.win_stride = (w % 2) ? -g.L : g.L;
-        two.emit_off = g.S + w * g.L;
-        two.Wtot = lay.Wcap; two.woff = w;
-        rc = launch_score_select(two, k_ring, v_ring, idx, nullptr, workspace, st);
-        if (rc != LRSA_OK) return rc;
-        const long long warps = (long long)BH * g.K;
-        cache_keep_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(idx, k_ring, v_ring, k_list, v_list, BH, w,
-                                                                     lay.Wcap, g.K, g.S, g.L, lay.rows_list, g.d);
-        LRSA_CUDA_CHECK(cudaGetLastError());
-        launch_counter().n++;
-      }
-      const int next = g.S + (c + 1) * g.L;
-      seg_end = end < next ? end : next;
+  CacheRows rows = {};
+  rows.k_new = static_cast<const __nv_bfloat16*>(k_new); rows.v_new = static_cast<const __nv_bfloat16*>(v_new);
+  rows.k_list = k_list; rows.v_list = v_list; rows.k_ring = k_ring; rows.v_ring = v_ring;
+  rows.idx = idx; rows.n_new = n_new; rows.p_first = n_prev;
+  rows.S = g.S; rows.L = g.L; rows.K = g.K; rows.Wcap = lay.Wcap; rows.rows_list = lay.rows_list; rows.cpr = g.d / 8;
+  // The status word is cleared by the first kernel of the call: a scoring kernel that can, else a memset in front of
+  // it, else the row copies.
+  int* status = &reinterpret_cast<WsHeader*>(workspace)->status;
+  bool cleared = false;
+  auto score = [&](const Geom& w, const __nv_bfloat16* k, const __nv_bfloat16* v) -> int {
+    const bool self = !cleared && score_select_clears_status(w);
+    if (!cleared && !self) {
+      LRSA_CUDA_CHECK(cudaMemsetAsync(workspace, 0, sizeof(WsHeader), st));
+      launch_counter().n++;
     }
-    const long long warps = (long long)BH * (seg_end - pos);
-    cache_insert_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), k_list, v_list, k_ring,
-        v_ring, BH, n_new, n_prev, pos, seg_end, g.S, g.L, lay.rows_list, g.d);
-    LRSA_CUDA_CHECK(cudaGetLastError());
-    launch_counter().n++;
-    pos = seg_end;
+    cleared = true;
+    return launch_score_select(w, k, v, idx, nullptr, workspace, st, self);
+  };
+  auto copy_rows = [&]() -> int {
+    if (rows.n_sink + rows.n_ins + rows.n_keep == 0) return LRSA_OK;
+    rows.status = cleared ? nullptr : status;
+    cleared = true;
+    return launch_cache_rows(rows, BH, st);
+  };
+  const int end = n_prev + n_new;
+  int pos = n_prev;                                     // tokens before it are in the list or the ring
+  int c = pos > g.S ? (pos - g.S + g.L - 1) / g.L : 0;  // next chunk whose first token has not arrived yet
+  if (c < 2) c = 2;
+  // Chunk start after chunk start while the window c-2 that leaves the ring holds tokens of earlier calls (at most
+  // two): the tokens up to it enter the ring, the window is scored with window c-1 as its reference (the two halves
+  // of the ring, in either order), and its kept rows join the list before its half is overwritten.
+  for (; g.S + c * g.L < end && g.S + (c - 2) * g.L < n_prev; ++c) {
+    const int w = c - 2;
+    rows.p0 = pos; rows.n_ins = g.S + c * g.L - pos; rows.n_keep = 0;
+    rc = copy_rows();
+    if (rc != LRSA_OK) return rc;
+    Geom two = g;
+    two.N = 2 * g.L; two.Nrow = 2 * g.L; two.S = 0; two.W = 2; two.Wsel = 1; two.T = 0; two.C = 2;
+    two.tok0 = (w % 2) * g.L;
+    two.win_stride = (w % 2) ? -g.L : g.L;
+    two.emit_off = g.S + w * g.L;
+    two.Wtot = lay.Wcap; two.woff = w;
+    rc = score(two, k_ring, v_ring);
+    if (rc != LRSA_OK) return rc;
+    rows.n_ins = 0; rows.w0 = w; rows.n_keep = g.K; rows.keep_from_ring = 1;
+    rc = copy_rows();
+    if (rc != LRSA_OK) return rc;
+    pos = g.S + c * g.L;
   }
-  return LRSA_OK;
+  rows.n_keep = 0;
+  rows.p0 = pos; rows.n_ins = end - pos;
+  if (g.S + c * g.L < end) {
+    // Windows c-2 .. c_last-2 lie in the new tokens as a whole: one scoring launch for all of them, then one for their
+    // kept rows, the sinks and the tokens that stay in the ring.
+    const int w0 = c - 2, nw = (end - 1 - g.S) / g.L - c + 1;
+    Geom many = g;
+    many.N = n_new; many.Nrow = n_new; many.S = 0; many.W = nw + 1; many.Wsel = nw; many.T = 0; many.C = nw + 1;
+    many.tok0 = g.S + w0 * g.L - n_prev;
+    many.emit_off = g.S + w0 * g.L;
+    many.Wtot = lay.Wcap; many.woff = w0;
+    rc = score(many, rows.k_new, rows.v_new);
+    if (rc != LRSA_OK) return rc;
+    rows.n_sink = pos < g.S ? g.S - pos : 0;
+    rows.p0 = end - 2 * g.L > pos ? end - 2 * g.L : pos;   // beyond the sinks: the call ends in chunk 2 or later
+    rows.n_ins = end - rows.p0;
+    rows.w0 = w0; rows.n_keep = nw * g.K; rows.keep_from_ring = 0;
+  }
+  return copy_rows();
 }
 
 int lrsa_cache_kept(const lrsa_params_t* params, const void* cache, const int32_t** idx, int32_t* w_cap) {
@@ -506,57 +609,33 @@ int lrsa_attn_decode(const lrsa_params_t* params, const void* cache, size_t cach
   a.k_ring = reinterpret_cast<const __nv_bfloat16*>(cb + lay.k_ring);
   a.v_ring = reinterpret_cast<const __nv_bfloat16*>(cb + lay.v_ring);
   a.part = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + 256);
-  a.BHkv = g.B * g.Hkv; a.Hq = g.Hq; a.Hkv = g.Hkv; a.G = g.G; a.rows_list = lay.rows_list > 0 ? lay.rows_list : 1;
-  a.L = g.L; a.S = g.S;
+  a.Hq = g.Hq; a.Hkv = g.Hkv; a.G = g.G; a.rows_list = lay.rows_list > 0 ? lay.rows_list : 1;
+  a.ring_rows = 2 * g.L;
   // the keys the query at position t = n_tokens - 1 sees (Attn-Fill 1/2): a sink query its causal prefix;
   // otherwise the sinks, the kept rows of windows 0..c-2, and positions [S + (c-1)L, t] from the ring
   const int t = n_tokens - 1;
   if (t < g.S) {
-    a.n_list = t + 1; a.n_ring = 0; a.ring0 = 0;
+    a.n_list = t + 1; a.n_keys = t + 1; a.ring0 = 0;
   } else {
     const int c = (t - g.S) / g.L, nc = c >= 1 ? c - 1 : 0;
     a.n_list = g.S + nc * g.K;
-    a.n_ring = t - (g.S + nc * g.L) + 1;
+    a.n_keys = a.n_list + t - (g.S + nc * g.L) + 1;
     a.ring0 = (nc * g.L) % (2 * g.L);
   }
-  a.n_split = decode_splits(a.n_list + a.n_ring);
+  const DecodePlan pl = decode_plan(g, a.n_keys);
+  a.n_split = pl.splits;
+  a.blocks = pl.blocks;
   a.scale_log2 = g.scale * 1.4426950408889634f;
   a.status = &reinterpret_cast<WsHeader*>(workspace)->status;
-  const dim3 grid(a.n_split, a.BHkv);
-  // K and V rows; the merge buffer (4 warps x 16 heads x (d + 2) floats) lies over them, or behind them when the
-  // group has more than 16 query heads and the rows are read again
-  const size_t rows_bytes = (size_t)(2 * kDecKeys + kDecHeads) * (g.d * sizeof(__nv_bfloat16) + 16);   // K, V and Q rows, padded
-  const size_t merge_bytes = (size_t)4 * kDecHeads * (g.d + 2) * sizeof(float);
-  const size_t smem = g.G > kDecHeads ? rows_bytes + merge_bytes : (rows_bytes > merge_bytes ? rows_bytes : merge_bytes);
-  if (g.d == 128) {
-    LRSA_CUDA_CHECK(cudaFuncSetAttribute(decode_partial_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    decode_partial_kernel<128><<<grid, kDecThreads, smem, st>>>(a);
-  } else {
-    LRSA_CUDA_CHECK(cudaFuncSetAttribute(decode_partial_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    decode_partial_kernel<64><<<grid, kDecThreads, smem, st>>>(a);
-  }
-  LRSA_CUDA_CHECK(cudaGetLastError());
-  launch_counter().n++;
-  {
-    // programmatic dependent launch: the merge kernel's launch latency overlaps the partial kernel
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.B * g.Hq);
-    cfg.blockDim = dim3(kMergeRows * g.d);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float* part = a.part;
-    __nv_bfloat16* op = static_cast<__nv_bfloat16*>(o);
-    if (g.d == 128)
-      LRSA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, decode_merge_kernel<128>, part, op, lse, g.Hq, g.Hkv, g.G, a.n_split));
-    else
-      LRSA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, decode_merge_kernel<64>, part, op, lse, g.Hq, g.Hkv, g.G, a.n_split));
-  }
-  LRSA_CUDA_CHECK(cudaGetLastError());
+  const int BHkv = g.B * g.Hkv;
+  const int pr = g.d == 128
+                     ? (pl.nh == 1 ? launch_partial<128, 1>(a, pl, BHkv, st) : launch_partial<128, 2>(a, pl, BHkv, st))
+                     : (pl.nh == 1 ? launch_partial<64, 1>(a, pl, BHkv, st) : launch_partial<64, 2>(a, pl, BHkv, st));
+  if (pr != LRSA_OK) return pr;
+  const float* part = a.part;
+  LRSA_CUDA_CHECK(launch_dependent(g.d == 128 ? decode_merge_kernel<128> : decode_merge_kernel<64>, dim3(g.B * g.Hq),
+                                   dim3(kMergeRows * g.d), st, part, static_cast<__nv_bfloat16*>(o), lse, g.Hq, g.Hkv,
+                                   g.G, a.n_split));
   launch_counter().n++;
   return LRSA_OK;
 }

@@ -64,6 +64,20 @@ class Params:
             cp._keepalive = arr          # the host array lives as long as the struct
         return cp
 
+    def ref(self, o_residual=None):
+        """The C struct by reference, for a call.  Without a residual it is built once per object, whose fields cannot
+        change (the library only reads it): building it on every call took a third of a decode step's host time."""
+        if o_residual is not None:
+            return ctypes.byref(self.c(o_residual))
+        r = self.__dict__.get("_ref")
+        if r is None:
+            r = ctypes.byref(self.c())
+            object.__setattr__(self, "_ref", r)
+        return r
+
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k != "_ref"}
+
     @staticmethod
     def from_workload(w, **kw) -> "Params":
         return Params(w.B, w.Hq, w.Hkv, w.N, w.d, w.L, w.K, w.S, **kw)
@@ -122,25 +136,22 @@ def _check(status: int, where: str):
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
 
 
 def lrsa_num_sel_windows(params: Params) -> int:
     out = ctypes.c_int32(0)
-    cp = params.c()
-    _check(lib().lrsa_num_sel_windows(ctypes.byref(cp), ctypes.byref(out)), "lrsa_num_sel_windows")
+    _check(lib().lrsa_num_sel_windows(params.ref(), ctypes.byref(out)), "lrsa_num_sel_windows")
     return out.value
 
 
 def lrsa_workspace_bytes(params: Params):
     a, b, c = ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_size_t(0)
-    cp = params.c()
-    _check(lib().lrsa_workspace_bytes(ctypes.byref(cp), ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)),
+    _check(lib().lrsa_workspace_bytes(params.ref(), ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)),
            "lrsa_workspace_bytes")
     return a.value, b.value, c.value
 
@@ -159,8 +170,7 @@ def lrsa_score_select(params: Params, K, V, idx=None, score=None, workspace=None
         score = torch.empty((params.batch, params.n_kv_heads, wsel, params.lag), dtype=torch.float32, device=K.device)
     if workspace is None:
         workspace = new_workspace(lrsa_workspace_bytes(params)[0], K.device)
-    cp = params.c()
-    _check(lib().lrsa_score_select(ctypes.byref(cp), _p(K), _p(V), _p(idx), _p(score), _p(workspace),
+    _check(lib().lrsa_score_select(params.ref(), _p(K), _p(V), _p(idx), _p(score), _p(workspace),
                                    workspace.numel(), _stream(stream)), "lrsa_score_select")
     return idx, score
 
@@ -173,8 +183,7 @@ def lrsa_score_select_static(params: Params, K, V, idx, score=None, stream=None)
     own fixed device array (STATIC_SCRATCH_BYTES) is used, so nothing is allocated here either -
     `idx` (and `score`, if wanted) must be passed in.  Problems that need more scratch raise
     LRSA_ERR_WORKSPACE_TOO_SMALL.  Calls that may overlap on the GPU must be serialised."""
-    cp = params.c()
-    _check(lib().lrsa_score_select_static(ctypes.byref(cp), _p(K), _p(V), _p(idx), _p(score), _stream(stream)),
+    _check(lib().lrsa_score_select_static(params.ref(), _p(K), _p(V), _p(idx), _p(score), _stream(stream)),
            "lrsa_score_select_static")
     return idx, score
 
@@ -194,8 +203,7 @@ def lrsa_attn_fwd(params: Params, Q, K, V, idx, O=None, LSE=None, workspace=None
         LSE = torch.empty(Q.shape[:3], dtype=torch.float32, device=Q.device)
     if workspace is None:
         workspace = new_workspace(lrsa_workspace_bytes(params)[1], Q.device)
-    cp = params.c(o_residual)
-    _check(lib().lrsa_attn_fwd(ctypes.byref(cp), _p(Q), _p(K), _p(V), _p(idx), _p(O), _p(LSE), _p(workspace),
+    _check(lib().lrsa_attn_fwd(params.ref(o_residual), _p(Q), _p(K), _p(V), _p(idx), _p(O), _p(LSE), _p(workspace),
                                workspace.numel(), _stream(stream)), "lrsa_attn_fwd")
     return O, LSE
 
@@ -211,8 +219,7 @@ def lrsa_attn_bwd(params: Params, Q, K, V, O, dO, LSE, idx, dQ=None, dK=None, dV
         dV = torch.empty_like(V)
     if workspace is None:
         workspace = new_workspace(lrsa_workspace_bytes(params)[2], Q.device)
-    cp = params.c(o_residual)
-    _check(lib().lrsa_attn_bwd(ctypes.byref(cp), _p(Q), _p(K), _p(V), _p(O), _p(dO), _p(LSE), _p(idx), _p(dQ),
+    _check(lib().lrsa_attn_bwd(params.ref(o_residual), _p(Q), _p(K), _p(V), _p(O), _p(dO), _p(LSE), _p(idx), _p(dQ),
                                _p(dK), _p(dV), _p(workspace), workspace.numel(), _stream(stream)), "lrsa_attn_bwd")
     return dQ, dK, dV
 
@@ -241,8 +248,7 @@ class KVCache:
     def __init__(self, params: Params, device="cuda"):
         self.params = params
         a, b = ctypes.c_size_t(0), ctypes.c_size_t(0)
-        cp = params.c()
-        _check(lib().lrsa_cache_bytes(ctypes.byref(cp), ctypes.byref(a), ctypes.byref(b)), "lrsa_cache_bytes")
+        _check(lib().lrsa_cache_bytes(params.ref(), ctypes.byref(a), ctypes.byref(b)), "lrsa_cache_bytes")
         self.buf = torch.zeros(a.value, dtype=torch.uint8, device=device)
         self.ws = new_workspace(b.value, device)
         self.n_tokens = 0
@@ -250,8 +256,7 @@ class KVCache:
     def append(self, k_new, v_new, stream=None):
         """k_new, v_new: bf16 [B, Hkv, n_new, d] (contiguous)."""
         n_new = k_new.shape[2]
-        cp = self.params.c()
-        _check(lib().lrsa_cache_append(ctypes.byref(cp), _p(self.buf), self.buf.numel(), _p(k_new), _p(v_new),
+        _check(lib().lrsa_cache_append(self.params.ref(), _p(self.buf), self.buf.numel(), _p(k_new), _p(v_new),
                                        self.n_tokens, n_new, _p(self.ws), self.ws.numel(), _stream(stream)),
                "lrsa_cache_append")
         self.n_tokens += n_new
@@ -262,16 +267,14 @@ class KVCache:
             o = torch.empty_like(q)
         if lse is None:
             lse = torch.empty(q.shape[:2], dtype=torch.float32, device=q.device)
-        cp = self.params.c()
-        _check(lib().lrsa_attn_decode(ctypes.byref(cp), _p(self.buf), self.buf.numel(), _p(q), self.n_tokens, _p(o),
+        _check(lib().lrsa_attn_decode(self.params.ref(), _p(self.buf), self.buf.numel(), _p(q), self.n_tokens, _p(o),
                                       _p(lse), _p(self.ws), self.ws.numel(), _stream(stream)), "lrsa_attn_decode")
         return o, lse
 
     def kept(self):
         """int32 [B, Hkv, w_cap, top_k] view of the kept positions (windows compressed so far are valid)."""
         ptr, wcap = ctypes.c_void_p(0), ctypes.c_int32(0)
-        cp = self.params.c()
-        _check(lib().lrsa_cache_kept(ctypes.byref(cp), _p(self.buf), ctypes.byref(ptr), ctypes.byref(wcap)),
+        _check(lib().lrsa_cache_kept(self.params.ref(), _p(self.buf), ctypes.byref(ptr), ctypes.byref(wcap)),
                "lrsa_cache_kept")
         off = ptr.value - self.buf.data_ptr()
         n = self.params.batch * self.params.n_kv_heads * wcap.value * self.params.top_k

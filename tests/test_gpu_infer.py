@@ -101,3 +101,58 @@ def test_cache_rejects_bad_arguments():
     with pytest.raises(lrsa.LrsaError) as e:
         lrsa.KVCache(lrsa.Params(1, 4, 2, 1000, 128, 128, 32, 4, n_dense_prev=0))
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("d,L,K,S,N,first", [
+    (128, 96, 24, 4, 4 + 9 * 96 + 17, 0),          # a prompt at once: every window lies in the new tokens
+    (64, 40, 11, 0, 10 * 40, 40 + 13),             # two windows hold earlier tokens, the others do not
+    (128, 33, 33, 7, 7 + 6 * 33 + 1, 7 + 33),      # starts and ends at a chunk start, every token kept
+    (64, 64, 16, 16, 16 + 2 * 64 + 1, 3),          # starts inside the sinks; one window, complete with the last token
+    (64, 4608, 100, 2, 2 + 3 * 4608 + 5, 4000),    # windows of the one-slice-per-CTA scoring kernel
+    (64, 4608, 100, 2, 2 + 4 * 4608 + 5, 0),       # several of them in one launch
+])
+def test_append_at_once_equals_token_ranges(d, L, K, S, N, first):
+    """The cache does not depend on how its tokens were cut into calls: one call for everything after `first` leaves
+    the bytes that calls of half a window leave (those never see a whole new window)."""
+    w = W("i_cuts", 2, 4, 2, N, d, L, K, S, seed=90, values="channel_offset")
+    dev = {k: v.cuda() for k, v in workloads.generate(w, ("K", "V")).items()}
+    p = lrsa.Params.from_workload(w)
+    cuts = {0, N, *(x for x in range(S, N, max(L // 2, 1)))}
+    bufs = []
+    for ends in (sorted(cuts), sorted({0, first, N})):
+        cache = lrsa.KVCache(p)
+        for lo, hi in zip(ends[:-1], ends[1:]):
+            cache.append(dev["K"][:, :, lo:hi].contiguous(), dev["V"][:, :, lo:hi].contiguous())
+            assert cache.status() == 0
+        assert cache.n_tokens == N
+        bufs.append(cache.buf)
+    assert torch.equal(bufs[0], bufs[1])
+
+
+@pytest.mark.parametrize("G", [1, 8, 9, 16])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,N", [(1, 1), (1, 17), (3, 700), (40, 2500)])
+def test_decode_against_fp64(G, d, B, N):
+    """Decode over caches of one key, a ragged block, a few splits and several blocks per warp (the small-CTA plan),
+    with one and two groups of eight heads, against fp64 attention over the visible keys.  P is rounded to bf16
+    (2^-9 relative, random signs) and so is the output: the contract's bound holds with room."""
+    w = W("i_dec", B, 2 * G, 2, N, d, 256, 64, min(4, N), seed=91)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    k = torch.randn((B, 2, N, d), generator=g, device="cuda").bfloat16()
+    v = torch.randn((B, 2, N, d), generator=g, device="cuda").bfloat16()
+    q = torch.randn((B, 2 * G, d), generator=g, device="cuda").bfloat16()
+    cache = lrsa.KVCache(lrsa.Params.from_workload(w))
+    cache.append(k, v)
+    o, lse = cache.decode(q)
+    assert cache.status() == 0
+    nc = max(max(N - 1 - w.S, 0) // w.L - 1, 0)
+    pos = torch.arange(w.S, device="cuda").expand(B, 2, -1)
+    if nc:
+        pos = torch.cat([pos, cache.kept()[:, :, :nc].reshape(B, 2, -1).long()], -1)
+    pos = torch.cat([pos, torch.arange(w.S + nc * w.L, N, device="cuda").expand(B, 2, -1)], -1)
+    ix = pos[..., None].expand(-1, -1, -1, d)
+    kk, vv = k.gather(2, ix).double(), v.gather(2, ix).double()
+    s = torch.einsum("bhgd,bhkd->bhgk", q.double().view(B, 2, G, d), kk) / d ** 0.5
+    want = torch.einsum("bhgk,bhkd->bhgd", s.softmax(-1), vv).reshape(B, 2 * G, d)
+    check_close("o", f64(o), want.cpu().numpy())
+    check_close("lse", f64(lse), s.logsumexp(-1).reshape(B, 2 * G).cpu().numpy(), max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
