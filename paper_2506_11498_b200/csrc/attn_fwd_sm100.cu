@@ -6,17 +6,23 @@
 // range of original positions up to the diagonal) in 128-key tiles; every K_j / V_j tile in shared memory
 // serves both query tiles.  Roles:
 //   warp 0      TMA producer: the Q tiles once, then K_j, V_j tiles through a ring of shared-memory slots
-//   warp 1      issues S_t = Q_t K_j^T (both operands in shared memory) into the tile's TMEM region; owns
-//               the TMEM allocation
-//   warp 2      issues O_t += P_t V_j with P_t read from tensor memory
+//   warp 1      issues all products, per key tile and query tile  O_t += P_t V_j (P_t from tensor memory), then
+//               S_t = Q_t K_{j+1}^T (both operands in shared memory); owns the TMEM allocation
 //   warps 4-7   softmax of query tile 0, warps 8-11 of query tile 1: one thread per row, S from TMEM, online
 //               softmax in fp32 with the maximum only raised when it grew by more than 2^8 (then O_t is
 //               rescaled in TMEM), P written back over S as packed bf16
 // The two tiles take turns on the tensor core: while one tile's scores are in its softmax warpgroup the
 // products of the other run.  A row belongs to one thread from its scores to its output, so the softmax
-// threads exchange nothing.  The issuing warps run their loops with all lanes and elect one lane per
-// instruction.  All mbarrier waits are bounded; on expiry the CTA records LRSA_ERR_TIMEOUT in the workspace
-// header and leaves.
+// threads exchange nothing, and its 128 scores are held in registers at once (setmaxnreg: 216 for these threads).
+// What bounds it: the chain of a tile from S_t over its exponentials (one MUFU result per two clocks and thread, 1024
+// cycles a tile) to O_t and the next S_t, and the 1000 W power limit, under which the clock settles near 1.65 GHz.
+// At 32K tokens, 28/4 heads, d = 128, one kept token in four: 2.75 -> 2.44 ms (of 1.50 at the measured bf16 rate); at
+// 64K 9.5 -> 8.5 ms, 15.1 -> 13.3 M cycles.  Before, two warps issued (S, and O += P V), with a barrier round trip
+// between a tile's products; scores were read twice; P was handed over in one piece.  Also measured: sixteen softmax
+// warps (16 rows x 128 columns each, 256-bit loads): 2.66 ms; exponentials started with the previous maximum, the tile
+// taken again when it was raised: 2.47 ms; a share of them on the FMA pipe: no gain at 1/8, 2.63 ms at 1/4.
+// The issuing warp runs its loop with all lanes and elects one lane per instruction.  All mbarrier waits are bounded;
+// on expiry the CTA records LRSA_ERR_TIMEOUT in the workspace header and leaves.
 #include "attn_common_sm100.h"
 
 namespace lrsa {
@@ -49,10 +55,13 @@ struct FwdArgs {
   int* status;
 };
 
+constexpr int kPParts = 2;   // P_t is handed to the tensor core in two halves (64 keys each)
+
 struct FwdBars {
   uint64_t q_full;
   uint64_t kv_full[12], kv_empty[12];
-  uint64_t s_full[2], p_full[2], buf_free[2], pv_done[2];   // per query tile
+  uint64_t s_full[2], pv_done[2];   // per query tile
+  uint64_t p_full[2][kPParts];      // per query tile: the parts of P_t (128 / kPParts keys each) are stored
 };
 
 template <int D>
@@ -86,8 +95,7 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     for (int i = 0; i < NS; ++i) { mbar_init(smem_u32(&bars.kv_full[i]), 1); mbar_init(smem_u32(&bars.kv_empty[i]), 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(smem_u32(&bars.s_full[t]), 1);
-      mbar_init(smem_u32(&bars.p_full[t]), 128);    // every softmax thread of the tile's warpgroup
-      mbar_init(smem_u32(&bars.buf_free[t]), 1);
+      for (int i = 0; i < kPParts; ++i) mbar_init(smem_u32(&bars.p_full[t][i]), 4);   // one arrival per softmax warp
       mbar_init(smem_u32(&bars.pv_done[t]), 1);
     }
     fence_barrier_init();
@@ -99,6 +107,10 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   const uint32_t tmem = tmem_base_s;
   volatile int* abort = &abort_s;
 
+  // The softmax threads hold a row of 128 scores: they take the registers the other warps do not need
+  // (128 x 72 + 256 x 216 = 384 x 168, what the CTA was launched with).
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
@@ -134,66 +146,80 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       }
     }
   } else if (warp == 1) {
-    // ---------------- S issuer: S_t = Q_t K_j^T for both query tiles ----------------
+    // ---------------- issuer: per key tile j and query tile t  O_t += P_t V_j, then S_t = Q_t K_{j+1}^T ----------------
+    // One warp issues everything, so the products run in this order on the tensor core: S_t of the next key tile may
+    // overwrite P_t without waiting for the product that reads it.
     constexpr uint32_t idesc_qk = make_idesc_bf16(kTile, kTile, 0, 0);
+    constexpr uint32_t idesc_pv = make_idesc_bf16(kTile, D, 0, 1);
     const uint64_t descK0 = make_smem_desc_sw128(sRing, 16, 1024);
+    const uint64_t descV0 = make_smem_desc_sw128(sRing, Cfg::kSubBytes, 1024);   // V_j MN-major
     const uint64_t descQ0 = make_smem_desc_sw128(sQ, 16, 1024);
     bool ok = mbar_wait_warp(smem_u32(&bars.q_full), 0, abort);
-    for (int j = 0; j < n && ok; ++j) {
-      const int it = 2 * j;   // ring order: K_j at 2j, V_j at 2j+1
-      ok = mbar_wait_warp(smem_u32(&bars.kv_full[it % NS]), (it / NS) & 1, abort);
-      const uint64_t dK = desc_advance(descK0, (it % NS) * Cfg::kTileBytes);
-      for (int t = 0; t < 2 && ok; ++t) {
-        if (j >= (t == 0 ? n0 : n1)) continue;
-        // S_t is also where P_t lives: the tile's previous O += P V must have read it
-        if (j >= 1) ok = mbar_wait_warp(smem_u32(&bars.buf_free[t]), (j - 1) & 1, abort);
+    int slot_v = 0, ph_v = 0, slot_k = 0, ph_k = 0;   // ring order: K_0, V_0, K_1, V_1, ...
+    auto next = [](int& slot, int& ph) { if (++slot == NS) { slot = 0; ph ^= 1; } };
+    for (int j = -1; j < n && ok; ++j) {
+      uint64_t dV = 0, dK = 0;
+      if (j >= 0) {
+        ok = mbar_wait_warp(smem_u32(&bars.kv_full[slot_v]), ph_v, abort);
         if (!ok) break;
-        tc_fence_after_sync();
-        const uint64_t dQ = desc_advance(descQ0, t * Cfg::kQRegion);
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * Cfg::kSubBytes + (kk & 3) * 32;
-          const uint64_t ad = desc_advance(dQ, off), bd = desc_advance(dK, off);
-          if (elect_one()) umma_ss(tmem + Cfg::kColS + t * kTile, ad, bd, idesc_qk, kk > 0 ? 1u : 0u);
-        }
-        if (elect_one()) umma_commit(smem_u32(&bars.s_full[t]));
-        __syncwarp();
+        dV = desc_advance(descV0, slot_v * Cfg::kTileBytes);
       }
-      if (ok && elect_one()) umma_commit(smem_u32(&bars.kv_empty[it % NS]));   // K_j is used by the S products only
-      __syncwarp();
-    }
-  } else if (warp == 2) {
-    // ---------------- O issuer: O_t += P_t V_j ----------------
-    constexpr uint32_t idesc_pv = make_idesc_bf16(kTile, D, 0, 1);
-    const uint64_t descV0 = make_smem_desc_sw128(sRing, Cfg::kSubBytes, 1024);   // V_j MN-major
-    bool ok = true;
-    for (int j = 0; j < n && ok; ++j) {
-      const int it = 2 * j + 1;
-      ok = mbar_wait_warp(smem_u32(&bars.kv_full[it % NS]), (it / NS) & 1, abort);
-      const uint64_t dV = desc_advance(descV0, (it % NS) * Cfg::kTileBytes);
+      bool k_here = false;
       for (int t = 0; t < 2 && ok; ++t) {
-        if (j >= (t == 0 ? n0 : n1)) continue;
-        ok = mbar_wait_warp(smem_u32(&bars.p_full[t]), j & 1, abort);
-        if (!ok) break;
-        tc_fence_after_sync();
-        // packed P_t: keys [16k, 16k+16) in columns [8k, 8k+8) of the tile's S region
+        const int nt = t == 0 ? n0 : n1;
+        if (j >= 0 && j < nt) {
+          // packed P_t: keys [16k, 16k+16) in columns [8k, 8k+8) of the tile's S region
 #pragma unroll
-        for (int kk = 0; kk < kTile / 16; ++kk) {
-          const uint64_t bd = desc_advance(dV, kk * 2048);
-          if (elect_one())
-            umma_ts(tmem + Cfg::kColO + t * kTile, tmem + Cfg::kColS + t * kTile + kk * 8, bd, idesc_pv,
-                    (kk > 0 || j > 0) ? 1u : 0u);
+          for (int part = 0; part < kPParts; ++part) {
+            if (ok) ok = mbar_wait_warp(smem_u32(&bars.p_full[t][part]), j & 1, abort);
+            if (!ok) break;
+            tc_fence_after_sync();
+#pragma unroll
+            for (int k8 = 0; k8 < kTile / 16 / kPParts; ++k8) {
+              const int kk = part * (kTile / 16 / kPParts) + k8;
+              const uint64_t bd = desc_advance(dV, kk * 2048);
+              if (elect_one())
+                umma_ts(tmem + Cfg::kColO + t * kTile, tmem + Cfg::kColS + t * kTile + kk * 8, bd, idesc_pv,
+                        (kk > 0 || j > 0) ? 1u : 0u);
+            }
+          }
+          if (!ok) break;
+          if (elect_one()) umma_commit(smem_u32(&bars.pv_done[t]));     // phase j: O_t holds key tiles 0..j
+          __syncwarp();
         }
-        if (elect_one()) {
-          umma_commit(smem_u32(&bars.buf_free[t]));    // S_t of the next key tile may overwrite P_t
-          umma_commit(smem_u32(&bars.pv_done[t]));     // phase j: O_t holds key tiles 0..j
+        if (j + 1 < nt) {
+          if (!k_here) {
+            ok = mbar_wait_warp(smem_u32(&bars.kv_full[slot_k]), ph_k, abort);
+            if (!ok) break;
+            dK = desc_advance(descK0, slot_k * Cfg::kTileBytes);
+            k_here = true;
+          }
+          tc_fence_after_sync();
+          const uint64_t dQ = desc_advance(descQ0, t * Cfg::kQRegion);
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk) {
+            const uint32_t off = (kk >> 2) * Cfg::kSubBytes + (kk & 3) * 32;
+            const uint64_t ad = desc_advance(dQ, off), bd = desc_advance(dK, off);
+            if (elect_one()) umma_ss(tmem + Cfg::kColS + t * kTile, ad, bd, idesc_qk, kk > 0 ? 1u : 0u);
+          }
+          if (elect_one()) umma_commit(smem_u32(&bars.s_full[t]));
+          __syncwarp();
         }
-        __syncwarp();
       }
-      if (ok && elect_one()) umma_commit(smem_u32(&bars.kv_empty[it % NS]));
+      if (!ok) break;
+      if (elect_one()) {
+        if (j >= 0) umma_commit(smem_u32(&bars.kv_empty[slot_v]));
+        if (j + 1 < n) umma_commit(smem_u32(&bars.kv_empty[slot_k]));
+      }
       __syncwarp();
+      next(slot_v, ph_v);
+      if (j >= 0) next(slot_v, ph_v);
+      next(slot_k, ph_k);
+      next(slot_k, ph_k);
     }
-  } else if (warp >= 4) {
+  }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
     // ---------------- softmax + epilogue: warpgroup t owns query tile t, one thread per row ----------------
     const int t = (warp - 4) >> 2, quad = warp & 3;
     const int row = quad * 32 + lane;
@@ -206,36 +232,32 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     float m = 0.f, l = 0.f;
     bool ok = true;
     for (int j = 0; j < nt && ok; ++j) {
-      ok = mbar_wait(smem_u32(&bars.s_full[t]), j & 1, abort);
+      ok = mbar_wait_warp(smem_u32(&bars.s_full[t]), j & 1, abort);
       if (!ok) break;
       tc_fence_after_sync();
       // keys of the tile this row may see: the first `limit`
       const int limit = j < n_ct ? rb.n_front - j * kTile : qpos - (rb.dense_start + (j - n_ct) * kTile) + 1;
-      // Row maximum over the 128 columns, 64 at a time; the second half stays in registers for its
-      // exponentials, the first half is read again afterwards (a second read of tensor memory is cheaper than
-      // 64 more live registers).
-      uint32_t s[64];
-      float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+      // the row's 128 scores and their maximum
+      uint32_t s[kTile];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        tmem_ld32(S_addr + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-        tmem_ld32(S_addr + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-        tmem_wait_ld();
-        if (limit < kTile) {
-          const int lim = limit - h * 64;
+      for (int h = 0; h < 4; ++h) tmem_ld32(S_addr + h * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[h * 32]));
+      tmem_wait_ld();
+      if (limit < kTile) {
 #pragma unroll
-          for (int i = 0; i < 64; ++i)
-            if (i >= lim) s[i] = 0xff800000u;  // -inf
-        }
-#pragma unroll
-        for (int i = 0; i < 64; i += 4) {
-          mx0 = fmaxf(mx0, __uint_as_float(s[i]));
-          mx1 = fmaxf(mx1, __uint_as_float(s[i + 1]));
-          mx2 = fmaxf(mx2, __uint_as_float(s[i + 2]));
-          mx3 = fmaxf(mx3, __uint_as_float(s[i + 3]));
-        }
+        for (int i = 0; i < kTile; ++i)
+          if (i >= limit) s[i] = 0xff800000u;  // -inf
       }
-      const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
+      float mx4[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mx4[e] = __uint_as_float(s[e]);
+#pragma unroll
+      for (int i = 4; i + 8 <= kTile; i += 8)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          mx4[e] = fmaxf(fmaxf(mx4[e], __uint_as_float(s[i + e])), __uint_as_float(s[i + 4 + e]));
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], __uint_as_float(s[kTile - 4 + e]));
+      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
       if (j == 0) {
         m = mx == -INFINITY ? 0.f : mx;
       } else {
@@ -244,7 +266,7 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         if (__any_sync(0xffffffffu, need)) {
           // O must hold every earlier tile before it is rescaled; the O issuer cannot start tile j before
           // this thread has arrived on p_full, so the rescale cannot race with it
-          ok = mbar_wait(smem_u32(&bars.pv_done[t]), (j - 1) & 1, abort);
+          ok = mbar_wait_warp(smem_u32(&bars.pv_done[t]), (j - 1) & 1, abort);
           if (!ok) break;
           tc_fence_after_sync();
           const float f = need ? ex2((m - mx) * c) : 1.f;
@@ -265,41 +287,45 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       const float nmc = -m * c;
       const uint64_t c2 = f2_pack(c, c), nmc2 = f2_pack(nmc, nmc);
       uint64_t sum2 = f2_pack(0.f, 0.f);
-      // exponentials of 64 columns held in s[]: scale and shift as packed pairs (one issue slot for two
-      // elements); one exponential in eight on the FMA pipe, the rest on the MUFU pipe
-      auto exps = [&](uint32_t (&pk)[32]) {
+      // exponentials: scale and shift as packed pairs (one issue slot for two elements).  P as packed bf16 over the
+      // first 64 columns of the tile's S (this thread's own lane: nobody else reads it), in two halves: the tensor core
+      // starts O_t += P_t V_j on the first while the second is formed (in four parts, with twice the waits for
+      // stores: 2.86 ms instead of 2.51 at the sizes of the file's head).  The steps are written a few elements ahead of
+      // the ones that take their results and kept in that order: one warp per scheduler is in this phase at a time, and
+      // nothing else hides the latencies (2.51 -> 2.44 ms).
+      constexpr int kPairs = kTile / 2 / kPParts, kLag = 4;
+      uint64_t sum2b = f2_pack(0.f, 0.f);
+      uint32_t pk[kPairs];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          float x0, x1;
-          f2_unpack(f2_fma(f2_pack(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), c2, nmc2), x0, x1);
-          const float p0 = ex2(x0);
-          const float p1 = (i & 3) == 3 ? ex2_fma(x1) : ex2(x1);
-          sum2 = f2_add(sum2, f2_pack(p0, p1));
-          pk[i] = pack_bf16(p0, p1);
+      for (int part = 0; part < kPParts; ++part) {
+#pragma unroll
+        for (int ii = 0; ii < kPairs + kLag; ++ii) {
+          if (ii < kPairs) {
+            const int i = part * kPairs + ii;
+            float x0, x1;
+            f2_unpack(f2_fma(f2_pack(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), c2, nmc2), x0, x1);
+            s[2 * i] = __float_as_uint(ex2_ordered(x0));
+            s[2 * i + 1] = __float_as_uint(ex2_ordered(x1));
+          }
+          if (ii >= kLag) {
+            const int i = part * kPairs + ii - kLag;
+            const float p0 = __uint_as_float(s[2 * i]), p1 = __uint_as_float(s[2 * i + 1]);
+            if (i & 1) sum2 = f2_add(sum2, f2_pack(p0, p1)); else sum2b = f2_add(sum2b, f2_pack(p0, p1));
+            pk[ii - kLag] = pack_bf16(p0, p1);
+          }
         }
-      };
-      uint32_t pk_hi[32], pk_lo[32];
-      exps(pk_hi);   // s[] holds columns 64..127 (masked)
-      tmem_ld32(S_addr, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-      tmem_ld32(S_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-      tmem_wait_ld();
-      if (limit < 64) {
-#pragma unroll
-        for (int i = 0; i < 64; ++i)
-          if (i >= limit) s[i] = 0xff800000u;
+        tmem_st32(S_addr + part * kPairs, pk);
+        tmem_wait_st();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.p_full[t][part]));
       }
-      exps(pk_lo);
+      sum2 = f2_add(sum2, sum2b);
       float sum0, sum1;
       f2_unpack(sum2, sum0, sum1);
       l += sum0 + sum1;
-      // P as packed bf16 over the first 64 columns of the tile's S (this thread's own lane: nobody else reads it)
-      tmem_st32(S_addr, pk_lo);
-      tmem_st32(S_addr + 32, pk_hi);
-      tmem_wait_st();
-      tc_fence_before_sync();
-      mbar_arrive(smem_u32(&bars.p_full[t]));
     }
-    if (ok && nt > 0) ok = mbar_wait(smem_u32(&bars.pv_done[t]), (nt - 1) & 1, abort);
+    if (ok && nt > 0) ok = mbar_wait_warp(smem_u32(&bars.pv_done[t]), (nt - 1) & 1, abort);
     // The output rows go through shared memory (the tile's Q region, idle once its last S product is done,
     // which pv_done implies) and leave as one bulk copy per row: per-thread 16-byte stores to rows 256 bytes
     // apart cost a transaction each.  Rows are padded by 16 bytes so that a warp's stores spread over the banks.
