@@ -13,7 +13,7 @@
 //
 // Decode attention reads the list prefix and the ring once per KV head for (up to 16) query heads of the group
 // (HBM-bound: 4*d bytes per key, a few FMAs per byte): the keys are split over CTAs and warps, every warp keeps an
-// online softmax of its keys, and a second small kernel merges the partial results.
+// online softmax of its keys, and the CTAs of a head form a cluster that merges the partial results.
 #include "lrsa_internal.h"
 #include "sm100_ptx.h"
 
@@ -93,25 +93,29 @@ __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
   reinterpret_cast<uint4*>(to_list ? a.v_list : a.v_ring)[dst * a.cpr + ch] = v;
 }
 
-// Launch that may start before the kernel in front of it has ended (the kernel waits for that itself).
+// Launch (in clusters of `cluster` CTAs) that may start before the kernel in front of it has ended (the kernel waits for
+// that itself).
 template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, int cluster, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 int launch_cache_rows(CacheRows a, int BH, cudaStream_t st) {
   const int rows = a.n_sink + a.n_ins + a.n_keep, rpb = 256 / a.cpr;
   a.blocks = (rows + rpb - 1) / rpb;
-  LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), st, a));
+  LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), st, 1, a));
   launch_counter().n++;
   return LRSA_OK;
 }
@@ -122,12 +126,15 @@ constexpr int kDecMaxWarps = 16;
 __host__ __device__ constexpr int dec_max_warps(int nh) { return nh == 1 ? kDecMaxWarps : kDecMaxWarps / 2; }
 
 struct DecodeArgs {
-  const __nv_bfloat16 *q, *k_list, *v_list, *k_ring, *v_ring;
-  float* part;          // [BHkv][n_split][G][D + 2]: unnormalised output, maximum (log2 domain), sum
+  const __nv_bfloat16 *q, *k_list, *k_ring;
+  long long v_of_list, v_of_ring;   // bytes from a K row to its V row
+  float* part;          // [BHkv][n_group][G][D + 2]: unnormalised output, maximum (log2 domain), sum
+  __nv_bfloat16* o;     // [B][Hq][D]
+  float* lse;           // [B][Hq], optional
   int* status;          // workspace status word
   int Hq, Hkv, G, rows_list, ring_rows;
   int n_list, n_keys, ring0;   // keys: list rows [0, n_list), then ring rows from ring row ring0 on (wrapping)
-  int n_split, blocks;         // key blocks per (batch, KV head), dealt out evenly to the splits
+  int n_split, n_group, blocks;   // key blocks per (batch, KV head), dealt out evenly to n_group clusters of n_split CTAs
   float scale_log2;
 };
 
@@ -144,13 +151,25 @@ __device__ __forceinline__ uint32_t transpose_8x8(uint32_t x) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
   return y;
 }
+// this CTA's variable at `p` as CTA `rank` of the cluster has it
+__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
+  float v;
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(ptx::smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint4 ld_stream(const void* p) {   // read once: no place in L1
   uint4 v;
   asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
 
-// Grid (n_split, BHkv), 4 to 16 warps.  One query token per (batch, head) over a few hundred to a few thousand keys
+// Grid (n_group * n_split, BHkv), clusters of n_split CTAs of 4 to 16 warps.  One query token per (batch, head) over a few hundred to a few thousand keys
 // per KV head: the work is the transfer of K and V (two bytes per multiply-add of one head), so the kernel is built
 // around the loads.  A warp takes blocks of 2048 / D keys; it loads the block's K and V rows straight into the
 // registers in which the warp-level tensor-core products want them and has 8 KB in flight while the other warps of
@@ -164,49 +183,52 @@ __device__ __forceinline__ uint4 ld_stream(const void* p) {   // read once: no p
 //                  the keys.  P^T comes out of the first product with keys and heads the other way round: one
 //                  movmatrix per eight keys turns it.
 // The maximum is raised only when it grew by more than 2^8 (then O is rescaled); it is common to the warp, since the
-// second product sums over the keys of all its lanes.  The warps are merged through shared memory, the splits by
-// decode_merge_kernel.
+// second product sums over the keys of all its lanes.  The warps are merged through shared memory, the CTAs through the
+// shared memory of their cluster (a second kernel for that, partial results in global memory, took 4.4 us beside 7.1 us of
+// this one for one sequence at 32K, and a launch on top: 26 us a token with it, 16 without).  Only where one cluster for
+// each head would leave most of the GPU idle for long (decode_plan), a head gets several and decode_merge_kernel
+// merges them.
 template <int D, int NH>
-__global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_partial_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const DecodeArgs a) {
   constexpr int U = 128 / D;                // 16-key groups per block
   constexpr int KC = D / 32, VC = D / 64;   // 16-byte chunks per lane and row, of K and of V
   constexpr int MT = D / 16;                // channel tiles of the output
   constexpr int kSlots = dec_max_warps(NH) / 2;
   __shared__ __align__(16) float sm_o[kSlots][8][D + 4];   // padded: lanes of a store differ in the head
   __shared__ float sm_m[kSlots][8], sm_l[kSlots][8];
-  const int bh = blockIdx.y, split = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ __align__(16) uint4 sm_q[NH][KC][32];
+  __shared__ float fin_o[8][D], fin_m[8], fin_l[8];   // the CTA's result, read by the cluster
+  const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nw = blockDim.x >> 5, g = lane >> 2, t = lane & 3;
   const int b = bh / a.Hkv, hkv = bh % a.Hkv;
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the cache rows of the kernel in front of this one
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (split == 0 && bh == 0 && tid == 0) *a.status = 0;
+  if (blockIdx.x == 0 && bh == 0 && tid == 0) *a.status = 0;
   const unsigned char* kl = reinterpret_cast<const unsigned char*>(a.k_list) + (size_t)bh * a.rows_list * (D * 2);
   const unsigned char* kr = reinterpret_cast<const unsigned char*>(a.k_ring) + (size_t)bh * a.ring_rows * (D * 2);
-  const ptrdiff_t v_of_list = reinterpret_cast<const unsigned char*>(a.v_list) - reinterpret_cast<const unsigned char*>(a.k_list);
-  const ptrdiff_t v_of_ring = reinterpret_cast<const unsigned char*>(a.v_ring) - reinterpret_cast<const unsigned char*>(a.k_ring);
   // K row of key `key`, and what leads from there to its V row
-  auto row_of = [&](int key, ptrdiff_t& to_v) {
+  auto row_of = [&](int key, long long& to_v) {
     key = min(key, a.n_keys - 1);       // beyond the end: any row that is there (its probability is zero)
     const bool in_list = key < a.n_list;
     int r = key - a.n_list + a.ring0;
     if (r >= a.ring_rows) r -= a.ring_rows;
-    to_v = in_list ? v_of_list : v_of_ring;
+    to_v = in_list ? a.v_of_list : a.v_of_ring;
     return in_list ? kl + (size_t)key * (D * 2) : kr + (size_t)r * (D * 2);
   };
-  const int blk0 = (int)((long long)a.blocks * split / a.n_split), blk1 = (int)((long long)a.blocks * (split + 1) / a.n_split);
+  const int nx = a.n_split * a.n_group;
+  const int blk0 = (int)((long long)a.blocks * blockIdx.x / nx), blk1 = (int)((long long)a.blocks * (blockIdx.x + 1) / nx);
 
   for (int g0 = 0; g0 < a.G; g0 += 8 * NH) {
-    // Q of head g0 + 8h + g as the B operand: the chunks this lane also takes of every key row
-    uint4 q[NH][KC];
-#pragma unroll
-    for (int h = 0; h < NH; ++h)
-#pragma unroll
-      for (int j = 0; j < KC; ++j) {
-        const int head = g0 + 8 * h + g;
-        q[h][j] = make_uint4(0, 0, 0, 0);
-        if (head < a.G)
-          q[h][j] = *reinterpret_cast<const uint4*>(a.q + ((size_t)(b * a.Hq + hkv * a.G + head)) * D + (t + 4 * j) * 8);
-      }
+    // Q of head g0 + 8h + g as the B operand: the chunks this lane also takes of every key row.  The same for every warp;
+    // in shared memory, because the registers are full of K, V and O.
+    for (int i = tid; i < NH * KC * 32; i += blockDim.x) {
+      const int h = i / (KC * 32), j = i / 32 % KC, head = g0 + 8 * h + (i & 31) / 4;
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (head < a.G)
+        v = *reinterpret_cast<const uint4*>(a.q + ((size_t)(b * a.Hq + hkv * a.G + head)) * D + ((i & 3) + 4 * j) * 8);
+      sm_q[h][j][i & 31] = v;
+    }
+    __syncthreads();
     float o[NH][MT][4];        // tile 4j + f: channels 8(g + 8j) + 2f, + 1 of heads 2t, 2t + 1
     float m[NH][2], l[NH][2];  // heads 2t, 2t + 1: maximum (the warp's), sum (this lane's keys)
 #pragma unroll
@@ -223,14 +245,14 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_partial_kern
       for (int u = 0; u < U; ++u) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-          ptrdiff_t to_v;
+          long long to_v;
           const unsigned char* r = row_of(key0 + 16 * u + g + 8 * i, to_v);
 #pragma unroll
           for (int j = 0; j < KC; ++j) kq[u][i][j] = ld_stream(r + (t + 4 * j) * 16);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          ptrdiff_t to_v;
+          long long to_v;
           const unsigned char* r = row_of(key0 + 16 * u + 2 * t + (i & 1) + 8 * (i >> 1), to_v);
 #pragma unroll
           for (int j = 0; j < VC; ++j) vq[u][i][j] = ld_stream(r + to_v + (g + 8 * j) * 16);
@@ -244,8 +266,11 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_partial_kern
           s[u][0] = s[u][1] = s[u][2] = s[u][3] = 0.f;
 #pragma unroll
           for (int j = 0; j < KC; ++j) {
-            mma_16816(s[u], kq[u][0][j].x, kq[u][1][j].x, kq[u][0][j].y, kq[u][1][j].y, q[h][j].x, q[h][j].y);
-            mma_16816(s[u], kq[u][0][j].z, kq[u][1][j].z, kq[u][0][j].w, kq[u][1][j].w, q[h][j].z, q[h][j].w);
+            uint4 q;
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
+                         : "r"(ptx::smem_u32(&sm_q[h][j][lane])));
+            mma_16816(s[u], kq[u][0][j].x, kq[u][1][j].x, kq[u][0][j].y, kq[u][1][j].y, q.x, q.y);
+            mma_16816(s[u], kq[u][0][j].z, kq[u][1][j].z, kq[u][0][j].w, kq[u][1][j].w, q.z, q.w);
           }
         }
         // elements: e = 0, 1: key g, heads 2t, 2t + 1; e = 2, 3: key g + 8
@@ -347,107 +372,108 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_partial_kern
           ov = fmaf(sm_o[w][hd][c], f, ov);
           ls = fmaf(sm_l[w][hd], f, ls);
         }
-        float* dst = a.part + (((size_t)bh * a.n_split + split) * a.G + g0 + 8 * h + hd) * (D + 2);
-        dst[c] = ov;
-        if (c == 0) { dst[D] = M; dst[D + 1] = ls; }
+        fin_o[hd][c] = ov;
+        if (c == 0) { fin_m[hd] = M; fin_l[hd] = ls; }
       }
+      cluster_sync();
+      // the CTAs of the cluster share the elements of the output
+      const int group = blockIdx.x / a.n_split, rank = blockIdx.x - group * a.n_split;
+      for (int i = rank * blockDim.x + tid; i < ng * D; i += a.n_split * blockDim.x) {
+        const int hd = i / D, c = i % D;
+        float M = -INFINITY;
+#pragma unroll 4
+        for (int r = 0; r < a.n_split; ++r) M = fmaxf(M, ld_cluster(&fin_m[hd], r));
+        float ov = 0.f, ls = 0.f;
+#pragma unroll 4
+        for (int r = 0; r < a.n_split; ++r) {
+          const float f = exp2f(ld_cluster(&fin_m[hd], r) - M);   // every split holds at least one key: finite
+          ov = fmaf(ld_cluster(&fin_o[hd][c], r), f, ov);
+          ls = fmaf(ld_cluster(&fin_l[hd], r), f, ls);
+        }
+        if (a.n_group > 1) {
+          float* dst = a.part + (((size_t)bh * a.n_group + group) * a.G + g0 + 8 * h + hd) * (D + 2);
+          dst[c] = ov;
+          if (c == 0) { dst[D] = M; dst[D + 1] = ls; }
+          continue;
+        }
+        const size_t head = (size_t)b * a.Hq + hkv * a.G + g0 + 8 * h + hd;
+        a.o[head * D + c] = __float2bfloat16(ov / ls);
+        if (c == 0 && a.lse) a.lse[head] = (M + log2f(ls)) * 0.6931471805599453f;
+      }
+      cluster_sync();   // the other CTAs have read this one's result: it may be overwritten, or the CTA may leave
     }
-    __syncthreads();   // the merge buffer is reused by the next heads
   }
 }
 
-// One CTA per (batch, query head): merges the partial results of the splits.  kMergeRows thread rows take
-// alternate splits, four at a time with all their loads issued before the arithmetic (the kernel is a chain of
-// L2 round trips otherwise), then the rows are merged through shared memory.
-constexpr int kMergeRows = 8;
+// Merges the clusters of one (batch, query head): one thread per channel.
 template <int D>
-__global__ void __launch_bounds__(kMergeRows * D) decode_merge_kernel(const float* __restrict__ part,
-                                                                       __nv_bfloat16* __restrict__ o,
-                                                                       float* __restrict__ lse, int Hq, int Hkv, int G,
-                                                                       int n_split) {
-  __shared__ float sm_m[kMergeRows], sm_l[kMergeRows], sm_o[kMergeRows][D];
-  const int bhq = blockIdx.x, b = bhq / Hq, hq = bhq % Hq, hkv = hq / G, g = hq % G;
-  const int c = threadIdx.x % D, row = threadIdx.x / D;
-  const float* base = part + (((size_t)(b * Hkv + hkv) * n_split) * G + g) * (D + 2);
+__global__ void __launch_bounds__(D) decode_merge_kernel(const float* part, __nv_bfloat16* o, float* lse, int Hq, int Hkv, int G,
+                                                         int n_group) {
+  const int bhq = blockIdx.x, b = bhq / Hq, hq = bhq % Hq, c = threadIdx.x;
+  const float* base = part + (((size_t)(b * Hkv + hq / G) * n_group) * G + hq % G) * (D + 2);
   const size_t stride = (size_t)G * (D + 2);
-  float M = -INFINITY, acc = 0.f, l = 0.f;
-  constexpr int kBatch = 4;
-  // launched as a programmatic dependent of the partial kernel: wait for its grid to complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int s0 = row; s0 < n_split; s0 += kMergeRows * kBatch) {
-    float ms[kBatch], vs[kBatch], ls[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int s = s0 + u * kMergeRows;
-      const bool in = s < n_split;
-      ms[u] = in ? __ldcg(base + s * stride + D) : -INFINITY;
-      vs[u] = in ? __ldcg(base + s * stride + c) : 0.f;
-      ls[u] = in ? __ldcg(base + s * stride + D + 1) : 0.f;
-    }
-    float mn = M;
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) mn = fmaxf(mn, ms[u]);
-    if (mn == -INFINITY) continue;
-    const float f0 = exp2f(M - mn);   // exp2f(-inf) = 0 while nothing has been merged
-    acc *= f0; l *= f0;
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const float f = exp2f(ms[u] - mn);
-      acc = fmaf(vs[u], f, acc);
-      l = fmaf(ls[u], f, l);
-    }
-    M = mn;
+  float M = -INFINITY;
+#pragma unroll 4
+  for (int r = 0; r < n_group; ++r) M = fmaxf(M, __ldcg(base + r * stride + D));
+  float ov = 0.f, ls = 0.f;
+#pragma unroll 4
+  for (int r = 0; r < n_group; ++r) {
+    const float f = exp2f(__ldcg(base + r * stride + D) - M);
+    ov = fmaf(__ldcg(base + r * stride + c), f, ov);
+    ls = fmaf(__ldcg(base + r * stride + D + 1), f, ls);
   }
-  sm_o[row][c] = acc;
-  if (c == 0) { sm_m[row] = M; sm_l[row] = l; }
-  __syncthreads();
-  if (row == 0) {
-    float Mt = -INFINITY;
-    for (int r = 0; r < kMergeRows; ++r) Mt = fmaxf(Mt, sm_m[r]);
-    float at = 0.f, lt = 0.f;
-    for (int r = 0; r < kMergeRows; ++r) {
-      const float f = sm_m[r] == -INFINITY ? 0.f : exp2f(sm_m[r] - Mt);
-      at = fmaf(sm_o[r][c], f, at);
-      lt = fmaf(sm_l[r], f, lt);
-    }
-    o[(size_t)bhq * D + c] = __float2bfloat16(at / lt);
-    if (c == 0 && lse) lse[bhq] = (Mt + log2f(lt)) * 0.6931471805599453f;
-  }
+  o[(size_t)bhq * D + c] = __float2bfloat16(ov / ls);
+  if (c == 0 && lse) lse[bhq] = (M + log2f(ls)) * 0.6931471805599453f;
 }
 
-// How the keys of the (batch, KV head) pairs are dealt out: `splits` CTAs of `warps` warps each.
-struct DecodePlan { int nh, warps, blocks, splits; };
-constexpr int kDecMaxSplits = 148;
-DecodePlan decode_plan(const Geom& g, int n_keys) {
+// How the keys of the (batch, KV head) pairs are dealt out: to `groups` clusters of `splits` CTAs of `warps` warps each.
+struct DecodePlan { int nh, warps, blocks, splits, groups; };
+constexpr int kDecMaxSplits = 16, kDecMaxGroups = 16;
+DecodePlan decode_plan(const Geom& g, int n_keys, int max_splits = kDecMaxSplits) {
   DecodePlan p;
   p.nh = g.G > 8 ? 2 : 1;
   const int per_block = 2048 / g.d;
   const long long BH = (long long)g.B * g.Hkv;
   p.blocks = n_keys > 0 ? (n_keys + per_block - 1) / per_block : 1;
   // 16 warps (8 with two groups of heads) are resident per SM, as one large CTA or several small ones.  Large ones
-  // leave fewer partial results to merge; small ones fill the SMs more evenly when every SM has several blocks per
-  // warp to do.  The number of splits is the one that ends first, counting a merge as two blocks.
+  // have fewer partial results to merge; small ones fill the SMs more evenly when every SM has several blocks per warp
+  // to do.  A round of blocks takes about 1.3 us, a CTA's start and merge as long as two, the second kernel as three; a
+  // cluster lies in one of the eight groups of 18 SMs.  (One sequence, 4 heads, d = 128: 9471 keys, one cluster for a
+  // head 17.7 us a token with 8 CTAs, 15.8 with 16; 66 000 keys 107 us with one cluster of 16, 34.5 with two.)
   const int max_warps = dec_max_warps(p.nh);
   p.warps = BH * p.blocks > 2LL * 148 * max_warps ? 4 : max_warps;
-  const int slots = 148 * (max_warps / p.warps);
-  const long long useful = 4LL * slots / BH + 1;   // beyond four waves more splits only add merges
-  long long best = 0;
-  p.splits = 1;
-  for (int s = 1; s <= kDecMaxSplits && s <= useful && (s == 1 || (s - 1) * p.warps < p.blocks); ++s) {
-    const long long waves = (BH * s + slots - 1) / slots;
-    const int per_cta = (p.blocks + s - 1) / s;
-    const long long cost = waves * ((per_cta + p.warps - 1) / p.warps + 2);
-    if (s == 1 || cost < best) { best = cost; p.splits = s; }
-  }
+  const int per_sm = max_warps / p.warps;
+  long long best = -1;
+  for (int s = 1; s <= max_splits; s *= 2)
+    for (int grp = 1; grp <= kDecMaxGroups; grp *= 2) {
+      const int n = s * grp;
+      if (n > 1 && ((n - 1) * p.warps >= p.blocks || BH * n > 148LL * per_sm * 4)) break;
+      const long long at_once = s == 1 ? 148 * per_sm : 8 * (18 * per_sm / s);
+      const long long waves = (BH * grp + at_once - 1) / at_once;
+      const int per_cta = (p.blocks + n - 1) / n;
+      const long long cost = waves * ((per_cta + p.warps - 1) / p.warps + 2) + (grp > 1 ? 3 : 0);
+      if (best < 0 || cost < best) { best = cost; p.splits = s; p.groups = grp; }
+    }
   return p;
 }
 
 template <int D, int NH>
-int launch_partial(const DecodeArgs& a, const DecodePlan& pl, int BHkv, cudaStream_t st) {
-  LRSA_CUDA_CHECK(launch_dependent(decode_partial_kernel<D, NH>, dim3(pl.splits, BHkv), dim3(pl.warps * 32), st, a));
-  launch_counter().n++;
-  return LRSA_OK;
+cudaError_t launch_decode_t(DecodeArgs& a, const DecodePlan& pl, int BHkv, cudaStream_t st) {
+  a.n_split = pl.splits; a.n_group = pl.groups; a.blocks = pl.blocks;
+  auto kern = decode_kernel<D, NH>;
+  if (pl.splits > 8) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_dependent(kern, dim3(pl.splits * pl.groups, BHkv), dim3(pl.warps * 32), st, pl.splits, a);
+}
+
+cudaError_t launch_decode(const Geom& g, DecodeArgs& a, const DecodePlan& pl, cudaStream_t st) {
+  const int BHkv = g.B * g.Hkv;
+  if (g.d == 128) return pl.nh == 1 ? launch_decode_t<128, 1>(a, pl, BHkv, st) : launch_decode_t<128, 2>(a, pl, BHkv, st);
+  return pl.nh == 1 ? launch_decode_t<64, 1>(a, pl, BHkv, st) : launch_decode_t<64, 2>(a, pl, BHkv, st);
 }
 
 }  // namespace
@@ -464,15 +490,15 @@ int lrsa_cache_bytes(const lrsa_params_t* params, size_t* cache_bytes, size_t* w
   if (params->n_seqs > 0 || g.ndp != 1) return LRSA_ERR_UNSUPPORTED;
   if (cache_bytes) *cache_bytes = cache_layout(g).total;
   if (workspace_bytes) {
-    // scoring scratch of the windows of a whole prompt (lag windows beyond 4096 tokens), or the partial results of the
-    // decode kernel: no more splits than blocks of keys for four warps each
-    const CacheLayout lay = cache_layout(g);
+    // scoring scratch of the windows of a whole prompt
     Geom all = g;
-    all.W = lay.Wcap + 1 > 2 ? lay.Wcap + 1 : 2; all.Wsel = all.W - 1;
+    const int wcap = cache_layout(g).Wcap;
+    all.W = wcap + 1 > 2 ? wcap + 1 : 2; all.Wsel = all.W - 1;
     const size_t a = score_select_ws_bytes(all);
-    const int blocks = (int)(((long long)(lay.rows_list + 2 * g.L) * g.d + 2047) / 2048);
-    const int splits = blocks / 4 + 1 < kDecMaxSplits ? blocks / 4 + 1 : kDecMaxSplits;
-    const size_t b = 256 + (size_t)g.B * g.Hkv * splits * g.G * (g.d + 2) * sizeof(float);
+    // or the partial results of decode (see decode_plan: several clusters for a head only below 592 CTAs of 16 warps)
+    const long long BH = (long long)g.B * g.Hkv;
+    const size_t b = sizeof(WsHeader) +
+                     (BH <= 4 * 592 ? (size_t)BH * kDecMaxGroups * g.G * (g.d + 2) * sizeof(float) : 0);
     *workspace_bytes = a > b ? a : b;
   }
   return LRSA_OK;
@@ -605,10 +631,12 @@ int lrsa_attn_decode(const lrsa_params_t* params, const void* cache, size_t cach
   DecodeArgs a;
   a.q = static_cast<const __nv_bfloat16*>(q);
   a.k_list = reinterpret_cast<const __nv_bfloat16*>(cb + lay.k_list);
-  a.v_list = reinterpret_cast<const __nv_bfloat16*>(cb + lay.v_list);
   a.k_ring = reinterpret_cast<const __nv_bfloat16*>(cb + lay.k_ring);
-  a.v_ring = reinterpret_cast<const __nv_bfloat16*>(cb + lay.v_ring);
-  a.part = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + 256);
+  a.v_of_list = (long long)(lay.v_list - lay.k_list);
+  a.v_of_ring = (long long)(lay.v_ring - lay.k_ring);
+  a.part = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + sizeof(WsHeader));
+  a.o = static_cast<__nv_bfloat16*>(o);
+  a.lse = lse;
   a.Hq = g.Hq; a.Hkv = g.Hkv; a.G = g.G; a.rows_list = lay.rows_list > 0 ? lay.rows_list : 1;
   a.ring_rows = 2 * g.L;
   // the keys the query at position t = n_tokens - 1 sees (Attn-Fill 1/2): a sink query its causal prefix;
@@ -622,21 +650,23 @@ int lrsa_attn_decode(const lrsa_params_t* params, const void* cache, size_t cach
     a.n_keys = a.n_list + t - (g.S + nc * g.L) + 1;
     a.ring0 = (nc * g.L) % (2 * g.L);
   }
-  const DecodePlan pl = decode_plan(g, a.n_keys);
-  a.n_split = pl.splits;
-  a.blocks = pl.blocks;
   a.scale_log2 = g.scale * 1.4426950408889634f;
   a.status = &reinterpret_cast<WsHeader*>(workspace)->status;
-  const int BHkv = g.B * g.Hkv;
-  const int pr = g.d == 128
-                     ? (pl.nh == 1 ? launch_partial<128, 1>(a, pl, BHkv, st) : launch_partial<128, 2>(a, pl, BHkv, st))
-                     : (pl.nh == 1 ? launch_partial<64, 1>(a, pl, BHkv, st) : launch_partial<64, 2>(a, pl, BHkv, st));
-  if (pr != LRSA_OK) return pr;
-  const float* part = a.part;
-  LRSA_CUDA_CHECK(launch_dependent(g.d == 128 ? decode_merge_kernel<128> : decode_merge_kernel<64>, dim3(g.B * g.Hq),
-                                   dim3(kMergeRows * g.d), st, part, static_cast<__nv_bfloat16*>(o), lse, g.Hq, g.Hkv,
-                                   g.G, a.n_split));
+  DecodePlan pl = decode_plan(g, a.n_keys);
+  cudaError_t e = launch_decode(g, a, pl, st);
+  if (e != cudaSuccess && pl.splits > 8) {   // clusters of 16 are not portable: a part of a GPU may not have room for them
+    (void)cudaGetLastError();
+    pl = decode_plan(g, a.n_keys, 8);
+    e = launch_decode(g, a, pl, st);
+  }
+  LRSA_CUDA_CHECK(e);
   launch_counter().n++;
+  if (pl.groups > 1) {
+    const float* part = a.part;
+    LRSA_CUDA_CHECK(launch_dependent(g.d == 128 ? decode_merge_kernel<128> : decode_merge_kernel<64>, dim3(g.B * g.Hq),
+                                     dim3(g.d), st, 1, part, a.o, lse, g.Hq, g.Hkv, g.G, pl.groups));
+    launch_counter().n++;
+  }
   return LRSA_OK;
 }
 

@@ -131,12 +131,12 @@ def test_append_at_once_equals_token_ranges(d, L, K, S, N, first):
 
 @pytest.mark.parametrize("G", [1, 8, 9, 16])
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("B,N", [(1, 1), (1, 17), (3, 700), (40, 2500)])
+@pytest.mark.parametrize("B,N", [(1, 1), (1, 17), (3, 700), (40, 2500), (1, 70000)])
 def test_decode_against_fp64(G, d, B, N):
-    """Decode over caches of one key, a ragged block, a few splits and several blocks per warp (the small-CTA plan),
-    with one and two groups of eight heads, against fp64 attention over the visible keys.  P is rounded to bf16
+    """Decode over caches of one key, a ragged block, a few splits, several blocks per warp (the small-CTA plan) and
+    several clusters for a head (long caches of few heads), with one and two groups of eight heads, against fp64 attention over the visible keys.  P is rounded to bf16
     (2^-9 relative, random signs) and so is the output: the contract's bound holds with room."""
-    w = W("i_dec", B, 2 * G, 2, N, d, 256, 64, min(4, N), seed=91)
+    w = W("i_dec", B, 2 * G, 2, N, d, 256, 256 if N > 2500 else 64, min(4, N), seed=91)
     g = torch.Generator(device="cuda").manual_seed(7)
     k = torch.randn((B, 2, N, d), generator=g, device="cuda").bfloat16()
     v = torch.randn((B, 2, N, d), generator=g, device="cuda").bfloat16()
