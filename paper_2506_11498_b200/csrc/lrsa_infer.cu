@@ -93,29 +93,10 @@ __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
   reinterpret_cast<uint4*>(to_list ? a.v_list : a.v_ring)[dst * a.cpr + ch] = v;
 }
 
-// Launch (in clusters of `cluster` CTAs) that may start before the kernel in front of it has ended (the kernel waits for
-// that itself).
-template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, int cluster, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = cluster;
-  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 int launch_cache_rows(CacheRows a, int BH, cudaStream_t st) {
   const int rows = a.n_sink + a.n_ins + a.n_keep, rpb = 256 / a.cpr;
   a.blocks = (rows + rpb - 1) / rpb;
-  LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), st, 1, a));
+  LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), 0, st, 1, a));
   launch_counter().n++;
   return LRSA_OK;
 }
@@ -467,7 +448,7 @@ cudaError_t launch_decode_t(DecodeArgs& a, const DecodePlan& pl, int BHkv, cudaS
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
-  return launch_dependent(kern, dim3(pl.splits * pl.groups, BHkv), dim3(pl.warps * 32), st, pl.splits, a);
+  return launch_dependent(kern, dim3(pl.splits * pl.groups, BHkv), dim3(pl.warps * 32), 0, st, pl.splits, a);
 }
 
 cudaError_t launch_decode(const Geom& g, DecodeArgs& a, const DecodePlan& pl, cudaStream_t st) {
@@ -664,7 +645,7 @@ int lrsa_attn_decode(const lrsa_params_t* params, const void* cache, size_t cach
   if (pl.groups > 1) {
     const float* part = a.part;
     LRSA_CUDA_CHECK(launch_dependent(g.d == 128 ? decode_merge_kernel<128> : decode_merge_kernel<64>, dim3(g.B * g.Hq),
-                                     dim3(g.d), st, 1, part, a.o, lse, g.Hq, g.Hkv, g.G, pl.groups));
+                                     dim3(g.d), 0, st, 1, part, a.o, lse, g.Hq, g.Hkv, g.G, pl.groups));
     launch_counter().n++;
   }
   return LRSA_OK;

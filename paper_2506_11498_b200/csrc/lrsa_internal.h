@@ -134,6 +134,26 @@ int launch_bwd_dkv_sm100(const Geom& whole, const Geom& g, const __nv_bfloat16* 
                          const int32_t* idx, void* ws_dkv, int* status, cudaStream_t st);
 int dkv_convert(const Geom& whole, void* ws_dkv, __nv_bfloat16* dK, __nv_bfloat16* dV, cudaStream_t st);
 
+// Launch (in clusters of `cluster` CTAs) that may start before the kernel in front of it has ended: the kernel itself waits
+// for that (griddepcontrol.wait) before it touches memory.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 #define LRSA_CUDA_CHECK(expr)                                 \
   do {                                                        \
     cudaError_t _e = (expr);                                  \

@@ -1,10 +1,9 @@
 // LagKV scoring and top-K selection (Section 3.2, Eq. 4-8 and the selection rule after Eq. 8).
 //
 // Two kernels, chosen by the lag window size:
-//   * score_select_chain_kernel (lag windows of up to 4096 tokens: the hot path).  A CTA owns a run of
-//     consecutive scored windows of one (batch, KV head), streams them downwards through a ring of bulk
-//     copies and keeps statistics and spreads in shared memory; no traffic between CTAs.  Described in
-//     front of the kernel below.
+//   * score_select_cluster_kernel (lag windows of up to 4096 tokens: the hot path).  A cluster of CTAs owns a run of
+//     consecutive scored windows of one (batch, KV head); statistics and spreads stay on the SMs.  Described in front
+//     of the kernel below.
 //   * score_select_kernel (longer windows).  The work unit is a slice of TOK tokens of one lag window; a
 //     CTA takes one unit from a ticket counter in DESCENDING window order and keeps its slice of K and V
 //     in registers for both phases:
@@ -48,10 +47,8 @@ struct ScoreArgs {
                           // Wtot windows per head of idx and score
   int emit_off;           // added to S + w*L + i when a position is written to idx
   int win_stride;         // tokens from window w to window w+1 in memory (L; -L or L for a two-window ring buffer)
-  long long elems;        // elements of K (and of V)
-  int clear_status;       // the chain kernel's first CTA clears the status word itself (saves a memset node)
+  int clear_status;       // the cluster kernel's first CTA clears the status word itself (saves a memset node)
   int unit_wait_limit;    // polls of the one-slice-per-CTA kernel's wait for the next window; negative: give up at once
-  int spin_limit;
 };
 
 // fp32 bits -> uint32 whose unsigned order is the float order (and back).
@@ -93,17 +90,16 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // Top-K of the window by the last CTA to finish it.  smem: sk[L], sv[L] floats, then scratch.
 // Bytes of the selection scratch: sk[L], sv[L], 256 histogram bins, 32 floats, 16 ints.
-// Rounded up to 16 bytes: the chain kernel puts a buffer of 16-byte vectors right behind this scratch
-// (an odd window length would leave it misaligned otherwise).
+// Rounded up to 16 bytes: the cluster kernel has two of them one behind the other.
 __host__ __device__ inline size_t select_scratch_bytes(int L) {
   return (((size_t)2 * L * 4 + 256 * 4 + 32 * 4 + 16 * 4) + 15) & ~(size_t)15;
 }
 
 // Barrier of the 256 scoring threads (named barrier 1): the whole block in the one-unit-per-CTA kernel,
-// all warps but the producer in the streaming kernel.
+// or of the cluster kernel.
 __device__ __forceinline__ void scoring_warps_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-// `in_smem`: the spreads are already in sk / sv (the chain kernel keeps them there) instead of in a.spread.
+// `in_smem`: the spreads are already in sk / sv (the cluster kernel keeps them there) instead of in a.spread.
 __device__ void select_window(const ScoreArgs& a, int bh, int w, unsigned char* smem, bool in_smem = false) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L;
   float* sk = reinterpret_cast<float*>(smem);
@@ -411,335 +407,213 @@ __global__ void __launch_bounds__(kThreads) score_select_kernel(const ScoreArgs 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Chain kernel (lag windows up to kChainMaxL tokens): no communication between CTAs at all.
+// Cluster kernel (lag windows up to kClusterMaxL tokens).
 //
-// A CTA owns a run of consecutive scored windows [w_a, w_b) of one (batch, KV head) and walks it
-// downwards.  It first streams window w_b only for its channel minima and maxima (Eq. 4-5); then for
-// w = w_b-1 ... w_a every 16 KB slice of K and of V is normalised with the statistics of window w+1,
-// already in shared memory (Eq. 6), reduced to per-token spreads (Eq. 7) that stay in shared memory,
-// and folded into the running statistics of window w itself for the next step; at the end of a
-// window the CTA soft-maxes, adds (Eq. 8) and selects.  A producer warp keeps a ring of slices in
-// flight with bulk asynchronous copies, so the loads never wait for the arithmetic; two groups of
-// eight scoring warps take alternate slices (the arithmetic of one slice is a chain of dependent
-// shuffles and reductions, and one group alone leaves the SM idle most of the time).  Each group has
-// its own ring of stages and waits for its slices in the order they were issued: a barrier is then
-// never waited on two phases ahead (a parity wait cannot tell "two phases ahead" from "done"), which
-// a shared ring allowed when one group ran ahead and bulk copies landed out of order.
-// With one window per CTA (the 32K benchmark: 120 windows on 148 SMs) every window is streamed
-// twice, by its own CTA and as the reference of the window before it; the second read comes a few
-// microseconds after the first and is served by L2 as long as K and V fit there (67 MB of 126 MB).
-// Longer runs per CTA (more windows than SMs) read 1 + 1/run of the data.
-constexpr int kChainMaxRing = 3;   // stages per scoring group (2 when the selection scratch is large)
-constexpr int kChainMaxL = 4096;
-constexpr int kChainGroups = 2;                           // scoring groups of kThreads threads, alternating slices
-constexpr int kChainThreads = kChainGroups * kThreads + 32;
+// A cluster of C CTAs owns a run of consecutive scored windows [w_a, w_b) of one (batch, KV head) and walks it
+// downwards; every CTA takes 1/C of the tokens of each window.  It first reads its part of window w_b only for the
+// channel minima and maxima (Eq. 4-5), which the CTAs exchange through shared memory; then for w = w_b-1 ... w_a its
+// tokens are normalised with the statistics of window w+1 (Eq. 6), reduced to per-token spreads (Eq. 7) that go to the
+// shared memory of the CTA that selects the window (the ranks take turns), and folded into the statistics of window w
+// for the next step.  The selecting CTA soft-maxes, adds (Eq. 8) and selects while the others go on.
+//
+// K and V are loaded straight into registers (nothing is staged): four lanes share a token's row (16-byte chunks t,
+// t + 4, ... of lane t), eight tokens a warp-wide load, T such groups in flight per warp; half of the warps take K, half
+// V.  The channels' scale and offset come from shared memory, one 16-byte broadcast per channel pair for T tokens, and
+// the sum over a token's channels ends with two shuffle levels.  A row per 16 lanes with scale and offset in registers,
+// the layout of the kernel this one replaces, spent twice the instructions (12 per channel pair, 6 here) on exchanges, and
+// one CTA per window left most of the GPU idle when there were few.  4 KV heads, d = 128: 32K tokens in windows of 1024
+// 35.9 -> 27.7 us a call (2.4 TB/s of algorithmic bytes; every window is read twice, the second time from L2), 64K of 2048
+// 61.6 -> 49, 1777 tokens of 512 20.5 -> 9.9; 8 KV heads, 128K of 4096 184 -> 161.  What is left is a chain: two streams
+// of at most 16 warps' loads an SM, the exchange, the selection (about 4 us).
+constexpr int kClusterMaxL = 4096;
+constexpr int kClusterMax = 8;
 
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {   // p as CTA `rank` of the cluster has it
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(ptx::smem_u32(p)), "r"(rank));
+  return addr;
+}
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void all_groups_sync() {
-  asm volatile("bar.sync 3, %0;" ::"n"(kChainGroups * kThreads) : "memory");
-}
-// Barriers that also OR a predicate over their threads: every thread leaves with the same verdict, so a
-// group (or the whole CTA) takes the give-up branch together even if the flag was raised while some of
-// its threads had already looked at it.
-__device__ __forceinline__ bool bar_or(int id, int nthreads, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %3, 0;\n\t"
-      "bar.red.or.pred p, %1, %2, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"(id), "r"(nthreads), "r"((uint32_t)pred)
-      : "memory");
-  return r != 0;
-}
-__device__ __forceinline__ bool group_sync_or(int grp, bool pred) { return bar_or(grp + 1, kThreads, pred); }
-__device__ __forceinline__ bool all_groups_sync_or(bool pred) { return bar_or(3, kChainGroups * kThreads, pred); }
-
-// Bounded wait on a shared-memory barrier phase; false when it gave up.
-__device__ __forceinline__ bool stage_wait(uint32_t bar, uint32_t parity, int limit) {
-  for (int it = 0; it < limit; ++it)
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-  return false;
-}
-
-template <int D>
-__global__ void __launch_bounds__(kChainThreads, 1) score_select_chain_kernel(const ScoreArgs a, int run, int runs_per_bh,
-                                                                              int ring) {
-  constexpr int LPR = D / 8;              // lanes per token row, 16 bytes each
-  constexpr int RPS = kThreads / LPR;     // rows per step
-  constexpr int TOK = kSteps * RPS;       // tokens per slice
-  constexpr int kSliceBytes = TOK * D * 2;
-  constexpr int kStageBytes = 2 * kSliceBytes;   // K slice, then V slice
+template <int D, bool FOLD>
+__global__ void __launch_bounds__(kThreads, 2) score_select_cluster_kernel(const ScoreArgs a, int run, int runs_per_bh, int C) {
+  constexpr int KC = D / 32;              // 16-byte chunks per lane and row
+  constexpr int T = FOLD ? 2 : 4;         // groups of eight tokens in flight
+  constexpr int kStatBytes = 4 * D * 2;   // [K, V][min, max][D] bf16
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ __align__(8) uint64_t full_bar[kChainGroups * kChainMaxRing], empty_bar[kChainGroups * kChainMaxRing];
-  __shared__ int s_abort;
-  // after the ring: scale/offset of the reference window [2 (K,V)][2 (sa,sb)][D], then the selection
-  // scratch (spreads sk[L], sv[L], histogram...), whose tail doubles as the min/max reduction buffer
-  float* sasb = reinterpret_cast<float*>(smem + kChainGroups * ring * kStageBytes);
-  unsigned char* sel = reinterpret_cast<unsigned char*>(sasb + 4 * D);
-  float* sk = reinterpret_cast<float*>(sel);
-  float* sv = sk + a.L;
-  __nv_bfloat16* red = reinterpret_cast<__nv_bfloat16*>(sel + select_scratch_bytes(a.L));   // [16 warps][4][D]
+  // [2 (K,V)][KC][4 pairs][4 lanes] (sa, sa, sb, sb); two buffers of statistics; per-warp partial statistics; two
+  // selection scratch areas (spreads sk[L], sv[L], histogram, ...)
+  float4* sasb = reinterpret_cast<float4*>(smem);
+  unsigned char* stat = smem + D * 16;
+  __nv_bfloat16* part = reinterpret_cast<__nv_bfloat16*>(stat + 2 * kStatBytes);   // [8 warps][min, max][D]
+  unsigned char* sel = stat + 2 * kStatBytes + 8 * 2 * D * 2;
+  const size_t sel_bytes = select_scratch_bytes(a.L);
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // A bounded wait needs seconds to expire, the first CTA of the grid starts with the launch: its clearing
-  // of the status word cannot overwrite another CTA's verdict.
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const int z = warp & 1, wz = warp >> 1;                 // tensor of this warp (0: K, 1: V), its place among four
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (a.clear_status && blockIdx.x == 0 && tid == 0) a.hdr->status = 0;
-  if (tid == 0) {
-    s_abort = 0;
-    for (int i = 0; i < kChainGroups * kChainMaxRing; ++i) {
-      ptx::mbar_init(ptx::smem_u32(&full_bar[i]), 1);
-      ptx::mbar_init(ptx::smem_u32(&empty_bar[i]), 1);
-    }
-    ptx::fence_barrier_init();
-  }
-  __syncthreads();
-  const int bh = blockIdx.x / runs_per_bh, seg = blockIdx.x % runs_per_bh;
+  const int item = blockIdx.x / C, rank = blockIdx.x % C;
+  const int bh = item / runs_per_bh, seg = item % runs_per_bh;
   const int w_a = seg * run, w_b = min(a.Wsel, w_a + run);   // scored windows [w_a, w_b); reference w_b <= W-1
-  const int n_win = w_b - w_a + 1;                            // windows streamed, the reference first
-  const int n_it = n_win * a.n_slices;
-  volatile int* abort = &s_abort;
-
-  if (warp == kChainGroups * kThreads / 32) {
-    // ---------------- producer ----------------
-    if (lane != 0) return;
-    // slice i goes to group i % 2; it is that group's k-th slice and uses slot k % ring of its ring in
-    // that slot's (k / ring)-th use.  All counters advance without divisions: one thread feeds the SM.
-    static_assert(kChainGroups == 2, "slot bookkeeping below");
-    int kr[2] = {0, 0}, use[2] = {0, 0};   // per group: k % ring and k / ring of its next slice
-    int w = w_b, slice = 0;
-    for (int i = 0; i < n_it; ++i) {
-      const int g = i & 1, slot = g * ring + kr[g];
-      if (use[g] > 0 && !stage_wait(ptx::smem_u32(&empty_bar[slot]), (use[g] - 1) & 1, a.spin_limit)) {
-        *abort = 1;
-        atomicExch(&a.hdr->status, (int)LRSA_ERR_TIMEOUT);
-        break;
-      }
-      if (*abort) break;
-      const int rows = min(TOK, a.L - slice * TOK);
-      const uint32_t bytes = (uint32_t)rows * D * 2;
-      const long long off = ((long long)bh * a.N + a.tok0 + a.S + (long long)w * a.win_stride + (long long)slice * TOK) * D;
-      const uint32_t bar = ptx::smem_u32(&full_bar[slot]);
-      const uint32_t dst = ptx::smem_u32(smem + slot * kStageBytes);
-      // self-check: the slice lies inside the tensor and the copy is 16-byte granular; otherwise give up
-      // (status word) instead of issuing it
-      if (w < 0 || w >= a.W || rows <= 0 || off < 0 || off + (long long)rows * D > a.elems || (bytes & 15u) ||
-          ((reinterpret_cast<uintptr_t>(a.K + off) | reinterpret_cast<uintptr_t>(a.V + off) | dst) & 15u)) {
-        *abort = 1;
-        atomicExch(&a.hdr->status, (int)LRSA_ERR_TIMEOUT);
-        break;
-      }
-      ptx::mbar_expect_tx(bar, 2 * bytes);
-      bulk_load(dst, a.K + off, bytes, bar);
-      bulk_load(dst + kSliceBytes, a.V + off, bytes, bar);
-      if (++kr[g] == ring) { kr[g] = 0; ++use[g]; }
-      if (++slice == a.n_slices) { slice = 0; --w; }
-    }
-    // No copy may be in flight when the CTA's shared memory is released, whether the run completed or a
-    // wait gave up: the producer leaves last, after the latest copy into every slot has landed (bounded).
-    for (int g = 0; g < kChainGroups; ++g)
-      for (int r = 0; r < ring; ++r) {
-        const int u = r < kr[g] ? use[g] : use[g] - 1;   // latest use of the slot that was issued
-        if (u >= 0) (void)stage_wait(ptx::smem_u32(&full_bar[g * ring + r]), u & 1, a.spin_limit);
-      }
-    return;
-  }
-
-  // ---------------- scoring warps ----------------
-  const int grp = tid / kThreads, gt = tid % kThreads;   // group and thread within the group
-  const int chunk = gt % LPR, row = gt / LPR;
+  const int per = (a.L + C - 1) / C;
+  const int i0 = min(a.L, rank * per), i1 = min(a.L, i0 + per);   // this CTA's tokens of every window
+  const __nv_bfloat16* base = (z == 0 ? a.K : a.V) + ((long long)bh * a.N + a.tok0 + a.S) * D;
   const float inv_dof = 1.0f / (float)(D - a.ddof);
-  const uint32_t PINF = 0x7F807F80u, NINF = 0xFF80FF80u;
-  uint32_t st[2][2][4];  // running [K,V][min,max][4 bf16 pairs] of this group's slices of the window
-  int it_all = 0, ckr = 0, cuse = 0;   // slices streamed so far by both groups; this group's ring position
-  for (int wi = 0; wi < n_win; ++wi) {
-   const int w = w_b - wi;
-   const bool scoring = wi > 0;          // the first window streamed is a reference only
-   const bool want_stats = w > w_a;      // its statistics serve the next window of the run
-   // scale and offset (Eq. 6) of this thread's eight channels, as packed pairs: [tensor][sa, sb][pair]
-   uint64_t sab2[2][2][4];
-   if (scoring) {
+
+  const int first = i0 + wz * 8 * T;   // this warp's first token
+  for (int w = w_b; w >= w_a; --w) {
+    const int it = w_b - w, buf = it & 1;
+    const bool scoring = it > 0, want_stats = w > w_a;
+    const __nv_bfloat16* win = base + (long long)w * a.win_stride * D;
+    const int sel_rank = it % C;
+    uint32_t mn[KC][4], mx[KC][4];
 #pragma unroll
-     for (int z = 0; z < 2; ++z)
+    for (int j = 0; j < KC; ++j)
 #pragma unroll
-       for (int m = 0; m < 2; ++m)
+      for (int p = 0; p < 4; ++p) { mn[j][p] = 0x7F807F80u; mx[j][p] = 0xFF80FF80u; }
+    for (int r0 = first; r0 < i1; r0 += 4 * 8 * T) {
+      uint4 x[T][KC];
 #pragma unroll
-         for (int h = 0; h < 2; ++h) {
-           const float4 v = *reinterpret_cast<const float4*>(sasb + (z * 2 + m) * D + chunk * 8 + h * 4);
-           sab2[z][m][2 * h] = ptx::f2_pack(v.x, v.y);
-           sab2[z][m][2 * h + 1] = ptx::f2_pack(v.z, v.w);
-         }
-   } else {
+      for (int s = 0; s < T; ++s) {
+        const int row = min(r0 + 8 * s + g, i1 - 1);    // beyond the part: its last token again (not written)
 #pragma unroll
-     for (int z = 0; z < 2; ++z)
+        for (int j = 0; j < KC; ++j)
+          x[s][j] = *reinterpret_cast<const uint4*>(win + (long long)row * D + (t + 4 * j) * 8);
+      }
+      if (want_stats && (FOLD || !scoring)) {
 #pragma unroll
-       for (int m = 0; m < 2; ++m)
+        for (int s = 0; s < T; ++s)
 #pragma unroll
-         for (int j = 0; j < 4; ++j) sab2[z][m][j] = 0ull;
-   }
+          for (int j = 0; j < KC; ++j) {
+            const uint32_t v[4] = {x[s][j].x, x[s][j].y, x[s][j].z, x[s][j].w};
 #pragma unroll
-   for (int j = 0; j < 4; ++j) { st[0][0][j] = st[1][0][j] = PINF; st[0][1][j] = st[1][1][j] = NINF; }
-   for (int slice = 0; slice < a.n_slices; ++slice, ++it_all) {
-    if ((it_all & 1) != grp) continue;
-    const int slot = grp * ring + ckr;   // this group's slice number k: ckr = k % ring, cuse = k / ring
-    // One barrier per slice: a warp whose wait ran out skips the arithmetic (warp-uniform, the
-    // arithmetic shuffles), raises the flag and still meets the group at the barrier below, after
-    // which every thread of the group reads the same verdict.
-    bool got = stage_wait(ptx::smem_u32(&full_bar[slot]), cuse & 1, a.spin_limit);
-    got = __all_sync(0xffffffffu, got);
-    if (!got) {
-      *abort = 1;
-      atomicExch(&a.hdr->status, (int)LRSA_ERR_TIMEOUT);
-    }
-    if (__all_sync(0xffffffffu, got && !*abort)) {
-    const unsigned char* stage = smem + slot * kStageBytes;
-    // this thread's rows of the slice: kSteps rows of K and of V, 16 bytes (8 channels) each
-    uint4 kq[kSteps], vq[kSteps];
-    bool valid[kSteps];
+            for (int p = 0; p < 4; ++p) { mn[j][p] = bmin2(mn[j][p], v[p]); mx[j][p] = bmax2(mx[j][p], v[p]); }
+          }
+      }
+      if (scoring) {
+        // Eq. 6 with the statistics of window w+1 (z' = x*sa + sb = zbar - 1/2), sums for the Std of Eq. 7
+        uint64_t sum2[T], sq2[T];
 #pragma unroll
-    for (int s = 0; s < kSteps; ++s) {
-      const int t = s * RPS + row;
-      valid[s] = slice * TOK + t < a.L;
-      if (valid[s]) {
-        kq[s] = *reinterpret_cast<const uint4*>(stage + (size_t)t * D * 2 + chunk * 16);
-        vq[s] = *reinterpret_cast<const uint4*>(stage + kSliceBytes + (size_t)t * D * 2 + chunk * 16);
-      } else {
-        kq[s] = make_uint4(0, 0, 0, 0);
-        vq[s] = make_uint4(0, 0, 0, 0);
+        for (int s = 0; s < T; ++s) sum2[s] = sq2[s] = 0ull;   // (+0, +0)
+#pragma unroll
+        for (int j = 0; j < KC; ++j)
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const float4 f = sasb[((z * KC + j) * 4 + p) * 4 + t];
+            const uint64_t sa = ptx::f2_pack(f.x, f.y), sb = ptx::f2_pack(f.z, f.w);
+#pragma unroll
+            for (int s = 0; s < T; ++s) {
+              const uint32_t v = p == 0 ? x[s][j].x : p == 1 ? x[s][j].y : p == 2 ? x[s][j].z : x[s][j].w;
+              const uint64_t z2 = ptx::f2_fma(ptx::f2_pack(bf_lo(v), bf_hi(v)), sa, sb);
+              sum2[s] = ptx::f2_add(sum2[s], z2);
+              sq2[s] = ptx::f2_fma(z2, z2, sq2[s]);
+            }
+          }
+        float v[T][2];
+#pragma unroll
+        for (int s = 0; s < T; ++s) {
+          float x0, x1;
+          ptx::f2_unpack(sum2[s], x0, x1); v[s][0] = x0 + x1;
+          ptx::f2_unpack(sq2[s], x0, x1); v[s][1] = x0 + x1;
+        }
+        // Sum over the four lanes of a row, halving: a lane hands half of its rows to its partner at each level
+        int mine = 0;   // row this lane ends up with
+        const bool up2 = (t & 2) != 0, up1 = (t & 1) != 0;
+        if constexpr (T == 4) {
+#pragma unroll
+          for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float send = up2 ? v[s][e] : v[s + 2][e], keep = up2 ? v[s + 2][e] : v[s][e];
+              v[s][e] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+            }
+          mine = up2 ? 2 : 0;
+        } else {
+#pragma unroll
+          for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) v[s][e] += __shfl_xor_sync(0xffffffffu, v[s][e], 2);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float send = up1 ? v[0][e] : v[1][e], keep = up1 ? v[1][e] : v[0][e];
+          v[0][e] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+        }
+        mine += up1 ? 1 : 0;
+        const int tok = r0 + 8 * mine + g;
+        if (tok < i1 && (T == 4 || !up2)) {
+          const float var = (v[0][1] - v[0][0] * v[0][0] * (1.0f / D)) * inv_dof;
+          const float spread = sqrtf(fmaxf(var, 0.f));
+          const uint32_t dst = cluster_addr(sel + buf * sel_bytes + ((size_t)z * a.L + tok) * 4, sel_rank);
+          asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(spread) : "memory");
+        }
       }
     }
     if (want_stats) {
-      // Eq. 4, Eq. 5, folded into the running statistics
+      // over the eight row groups of the warp, then over the four warps of the tensor
 #pragma unroll
-      for (int s = 0; s < kSteps; ++s) {
-        if (!valid[s]) continue;
-        const uint32_t kk[4] = {kq[s].x, kq[s].y, kq[s].z, kq[s].w}, vv[4] = {vq[s].x, vq[s].y, vq[s].z, vq[s].w};
+      for (int o = 16; o >= 4; o >>= 1)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          st[0][0][j] = bmin2(st[0][0][j], kk[j]); st[0][1][j] = bmax2(st[0][1][j], kk[j]);
-          st[1][0][j] = bmin2(st[1][0][j], vv[j]); st[1][1][j] = bmax2(st[1][1][j], vv[j]);
+        for (int j = 0; j < KC; ++j)
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            mn[j][p] = bmin2(mn[j][p], __shfl_xor_sync(0xffffffffu, mn[j][p], o));
+            mx[j][p] = bmax2(mx[j][p], __shfl_xor_sync(0xffffffffu, mx[j][p], o));
+          }
+      if (g == 0) {
+#pragma unroll
+        for (int j = 0; j < KC; ++j) {
+          *reinterpret_cast<uint4*>(part + (warp * 2 + 0) * D + (t + 4 * j) * 8) = make_uint4(mn[j][0], mn[j][1], mn[j][2], mn[j][3]);
+          *reinterpret_cast<uint4*>(part + (warp * 2 + 1) * D + (t + 4 * j) * 8) = make_uint4(mx[j][0], mx[j][1], mx[j][2], mx[j][3]);
         }
+      }
+      __syncthreads();
+      for (int v = tid; v < 2 * D; v += kThreads) {   // pairs of channels: [tensor][min, max][D / 2]
+        const int zz = v / D, m = v / (D / 2) & 1, ch = v % (D / 2);
+        uint32_t r = *reinterpret_cast<const uint32_t*>(part + (zz * 2 + m) * D + 2 * ch);
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+          const uint32_t y = *reinterpret_cast<const uint32_t*>(part + ((2 * k + zz) * 2 + m) * D + 2 * ch);
+          r = m ? bmax2(r, y) : bmin2(r, y);
+        }
+        *reinterpret_cast<uint32_t*>(stat + buf * kStatBytes + v * 4) = r;
       }
     }
-    if (scoring) {
-      // Eq. 6 with the statistics of window w+1 (z' = x*sa + sb = zbar - 1/2) and the per-token Std of
-      // Eq. 7.  Arithmetic on packed fp32 pairs; sa/sb of this thread's eight channels live in registers
-      // for the whole window (sab2, loaded below the window loop's head).
-      float part[2 * kSteps][2];   // [tensor * kSteps + step][sum, sum of squares] over this thread's 8 channels
-#pragma unroll
-      for (int z = 0; z < 2; ++z) {
-#pragma unroll
-        for (int s = 0; s < kSteps; ++s) {
-          const uint4 q = z == 0 ? kq[s] : vq[s];
-          const uint32_t pk[4] = {q.x, q.y, q.z, q.w};
-          uint64_t sum2 = 0ull, sq2 = 0ull;   // (+0, +0)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint64_t z2 = ptx::f2_fma(ptx::f2_pack(bf_lo(pk[j]), bf_hi(pk[j])), sab2[z][0][j], sab2[z][1][j]);
-            sum2 = ptx::f2_add(sum2, z2);
-            sq2 = ptx::f2_fma(z2, z2, sq2);
-          }
-          float s0, s1, q0, q1;
-          ptx::f2_unpack(sum2, s0, s1);
-          ptx::f2_unpack(sq2, q0, q1);
-          part[z * kSteps + s][0] = s0 + s1;
-          part[z * kSteps + s][1] = q0 + q1;
+    // Every CTA's spreads and statistics of this window are in place.  (A buffer is written again two windows later, behind
+    // the barrier of the window between, which a CTA only reaches when it has read the buffer.)
+    cluster_sync();
+    if (want_stats) {
+      for (int v = tid; v < D; v += kThreads) {   // pairs of channels: [tensor][D / 2]
+        const int zz = v / (D / 2), ch = v % (D / 2);   // channels 2ch, 2ch + 1
+        uint32_t lo = 0x7F807F80u, hi = 0xFF80FF80u;
+        for (int r = 0; r < C; ++r) {
+          uint32_t x, y;
+          const uint32_t src = cluster_addr(stat + buf * kStatBytes + zz * D * 4 + ch * 4, r);
+          asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(src) : "memory");
+          asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(y) : "r"(src + D * 2) : "memory");
+          lo = bmin2(lo, x);
+          hi = bmax2(hi, y);
         }
-      }
-      // Sum over the LPR lanes of a row.  Halving exchange: at every level a lane keeps half of its
-      // entries and hands the other half to its partner, so 2*kSteps entries cost 2*(2*kSteps - 1)
-      // shuffles instead of 2*kSteps*log2(LPR)*2; levels left over once one entry remains are plain
-      // butterflies.  The lane ends with entry e(chunk) complete.
-      int ent = 0;   // index of the entry this lane ends up with
-      {
-        int m = 2 * kSteps;   // entries still held
+        float f[4];
 #pragma unroll
-        for (int bit = LPR / 2; bit >= 1; bit >>= 1) {
-          if (m > 1) {
-            m >>= 1;
-            const bool up = (chunk & bit) != 0;
-#pragma unroll
-            for (int e = 0; e < kSteps; ++e) {   // kSteps >= m at every level
-              if (e < m) {
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                  const float send = up ? part[e][c] : part[e + m][c];
-                  const float keep = up ? part[e + m][c] : part[e][c];
-                  part[e][c] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
-                }
-              }
-            }
-            ent += up ? m : 0;
-          } else {
-            part[0][0] += __shfl_xor_sync(0xffffffffu, part[0][0], bit);
-            part[0][1] += __shfl_xor_sync(0xffffffffu, part[0][1], bit);
-          }
+        for (int e = 0; e < 2; ++e) {
+          // a channel with zero range has zbar = 0, i.e. z' = -1/2
+          const float a0 = e ? bf_hi(lo) : bf_lo(lo), a1 = e ? bf_hi(hi) : bf_lo(hi), range = a1 - a0;
+          const float inv = range > 0.f ? 1.0f / range : 0.f;
+          f[e] = inv;
+          f[2 + e] = range > 0.f ? -(0.5f * (a0 + a1)) * inv : -0.5f;
         }
-      }
-      {
-        const int z = ent / kSteps, st_ = ent % kSteps;
-        // lanes that differ only in the bits of the plain butterfly levels hold the same entry: one writes
-        constexpr int kDup = LPR / (2 * kSteps) > 1 ? LPR / (2 * kSteps) : 1;
-        const bool writer = (chunk & (kDup - 1)) == 0;
-        const int tkn = slice * TOK + st_ * RPS + row;
-        if (writer && tkn < a.L) {
-          const float var = (part[0][1] - part[0][0] * part[0][0] * (1.0f / D)) * inv_dof;
-          (z == 0 ? sk : sv)[tkn] = sqrtf(fmaxf(var, 0.f));
-        }
+        const int chunk = ch >> 2, p = ch & 3;   // chunk of eight channels: lane chunk % 4, its chunk / 4-th
+        sasb[((zz * KC + (chunk >> 2)) * 4 + p) * 4 + (chunk & 3)] = make_float4(f[0], f[1], f[2], f[3]);
       }
     }
-    }
-    // every read of the stage by this group is done; one verdict for the group
-    if (group_sync_or(grp, *abort != 0)) break;
-    if (gt == 0) ptx::mbar_arrive(ptx::smem_u32(&empty_bar[slot]));
-    if (++ckr == ring) { ckr = 0; ++cuse; }
-   }
-
-   // ---- end of window w: both groups have written their spreads and hold their part of the statistics ----
-   if (all_groups_sync_or(*abort != 0)) return;   // one verdict for the CTA
-   if (scoring && grp == 0) select_window(a, bh, w, sel, true);   // group 0 only (its own barrier inside)
-   if (want_stats) {
-      // reduce the running statistics over the rows of a warp, then over the warps, and turn them
-      // into the scale and offset the next window is normalised with
-#pragma unroll
-      for (int o = 16; o >= LPR; o >>= 1)
-#pragma unroll
-        for (int z = 0; z < 2; ++z)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            st[z][0][j] = bmin2(st[z][0][j], __shfl_xor_sync(0xffffffffu, st[z][0][j], o));
-            st[z][1][j] = bmax2(st[z][1][j], __shfl_xor_sync(0xffffffffu, st[z][1][j], o));
-          }
-      if (lane < LPR) {
-#pragma unroll
-        for (int z = 0; z < 2; ++z)
-#pragma unroll
-          for (int m = 0; m < 2; ++m)
-            *reinterpret_cast<uint4*>(red + ((warp * 4 + z * 2 + m) * D + lane * 8)) =
-                make_uint4(st[z][m][0], st[z][m][1], st[z][m][2], st[z][m][3]);
-      }
-      all_groups_sync();
-      for (int v = tid; v < 2 * D; v += kChainGroups * kThreads) {
-        const int z = v / D, ch = v % D;
-        float mn = __bfloat162float(red[(z * 2 + 0) * D + ch]), mx = __bfloat162float(red[(z * 2 + 1) * D + ch]);
-#pragma unroll
-        for (int ww = 1; ww < kChainGroups * kThreads / 32; ++ww) {
-          mn = fminf(mn, __bfloat162float(red[(ww * 4 + z * 2 + 0) * D + ch]));
-          mx = fmaxf(mx, __bfloat162float(red[(ww * 4 + z * 2 + 1) * D + ch]));
-        }
-        // a channel with zero range has zbar = 0, i.e. z' = -1/2
-        const float range = mx - mn;
-        const float inv = range > 0.f ? 1.0f / range : 0.f;
-        sasb[(z * 2 + 0) * D + ch] = inv;
-        sasb[(z * 2 + 1) * D + ch] = range > 0.f ? -(0.5f * (mn + mx)) * inv : -0.5f;
-      }
-   }
-   all_groups_sync();   // the next window's slices may overwrite the spreads and read the new statistics
+    if (scoring && rank == sel_rank) select_window(a, bh, w, sel + buf * sel_bytes, true);
+    __syncthreads();   // scale and offset are in place for the next window
   }
 }
 
@@ -754,7 +628,7 @@ size_t select_smem_bytes(int L, int d) {
 
 // Polls the one-slice-per-CTA kernel grants its wait for the following window's statistics.  Test hook:
 // a negative value makes that wait give up at once (the kernel holds its slice in registers and has no
-// copy in flight, so every thread returns after the verdict).  The chain kernel's limits are not touched.
+// copy in flight, so every thread returns after the verdict).
 int g_unit_wait_limit = 1 << 21;
 
 struct ScoreWs {
@@ -773,24 +647,45 @@ ScoreWs score_ws_layout(const Geom& g) {
   return w;
 }
 
+// Run length and cluster size by the measured cost of a CTA, in tokens streamed (21 ns each with two CTAs an SM): (run + 1)
+// windows' parts, 290 for launch, exchange and selection of the first scored window, 550 for every further one (a chain of
+// barriers, and half as many loads in flight beside the folded statistics).  At d = 128, 4 KV heads, run x C: 32K tokens in
+// windows of 1024: 1x1 30.4 us, 1x2 27.6, 1x4 33.3, 2x4 32.5, 4x8 45.7; 64K in windows of 2048: 1x2 49.1, 2x4 53.8;
+// 8 heads, 128K in windows of 4096: 1x1 171, 2x2 161, 4x4 175, 2x1 219.
+struct ClusterPlan { int run, C; };
+ClusterPlan cluster_plan(int BH, int Wsel, int L) {
+  ClusterPlan best = {1, 1};
+  double cost = -1;
+  for (int C = 1; C <= kClusterMax; C *= 2) {
+    const long long slots = C == 1 ? 2 * 148 : 8 * (2 * 18 / C);   // clusters at a time (eight groups of 18 SMs)
+    for (int r = 1; r <= Wsel; r = r < 8 ? r + 1 : r * 2) {
+      const long long clusters = (long long)BH * ((Wsel + r - 1) / r), waves = (clusters + slots - 1) / slots;
+      const double c = waves * ((r + 1.0) * ((L + C - 1) / C) + 290.0 + (r - 1) * 550.0);
+      if (cost < 0 || c < cost) { cost = c; best.run = r; best.C = C; }
+      if (waves == 1) break;
+    }
+  }
+  return best;
+}
+
 }  // namespace
 
-// The chain kernel uses nothing but the status header; the one-slice-per-CTA kernel needs its counters,
+// The cluster kernel uses nothing but the status header; the one-slice-per-CTA kernel needs its counters,
 // statistics and spreads.
-size_t score_select_ws_bytes(const Geom& g) { return g.L <= kChainMaxL ? sizeof(WsHeader) : score_ws_layout(g).total; }
+size_t score_select_ws_bytes(const Geom& g) { return g.L <= kClusterMaxL ? sizeof(WsHeader) : score_ws_layout(g).total; }
 
 void set_unit_wait_limit(int polls) { g_unit_wait_limit = polls; }
 
-bool score_select_clears_status(const Geom& g) { return g.Wsel > 0 && g.L <= kChainMaxL; }
+bool score_select_clears_status(const Geom& g) { return g.Wsel > 0 && g.L <= kClusterMaxL; }
 
 int launch_score_select(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx,
                         float* score, void* ws, cudaStream_t st, bool clear_status) {
   if (g.Wsel == 0) return LRSA_OK;  // nothing is scored
   const ScoreWs lay = score_ws_layout(g);
   unsigned char* base = static_cast<unsigned char*>(ws);
-  // The status word (the header) is cleared once per call by the caller.  The chain kernel keeps everything
+  // The status word (the header) is cleared once per call by the caller.  The cluster kernel keeps everything
   // else on chip; the one-slice-per-CTA kernel needs its ticket, counters and statistics at zero.
-  if (g.L > kChainMaxL) {
+  if (g.L > kClusterMaxL) {
     LRSA_CUDA_CHECK(cudaMemsetAsync(base + offsetof(WsHeader, ticket), 0, lay.zero_bytes - offsetof(WsHeader, ticket), st));
     launch_counter().n++;
   }
@@ -803,10 +698,8 @@ int launch_score_select(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat
   a.spread = reinterpret_cast<float*>(base + lay.spread);
   a.BH = g.B * g.Hkv; a.N = g.Nrow; a.L = g.L; a.Kk = g.K; a.S = g.S; a.W = g.W; a.Wsel = g.Wsel;
   a.tok0 = g.tok0; a.Wtot = g.Wtot; a.woff = g.woff; a.emit_off = g.emit_off; a.win_stride = g.win_stride;
-  a.elems = (long long)g.B * g.Hkv * g.Nrow * g.d;
   a.ddof = g.ddof;
   a.clear_status = clear_status && score_select_clears_status(g) ? 1 : 0;
-  a.spin_limit = 1 << 21;
   a.unit_wait_limit = g_unit_wait_limit;
   const int tok = g.d == 128 ? tok_per_unit<128>() : tok_per_unit<64>();
   a.n_slices = (g.L + tok - 1) / tok;
@@ -814,25 +707,17 @@ int launch_score_select(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat
   if (smem > 200 * 1024) return LRSA_ERR_UNSUPPORTED;
   const long long units = (long long)a.BH * g.W * a.n_slices;
   if (units > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  if (g.L <= kChainMaxL) {
-    // chain kernel: runs of consecutive windows per CTA, about one CTA per SM, no inter-CTA traffic
-    int dev = 0, sms = 0;
-    LRSA_CUDA_CHECK(cudaGetDevice(&dev));
-    LRSA_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int run = (a.BH * g.Wsel + sms - 1) / sms;
-    const int runs_per_bh = (g.Wsel + run - 1) / run;
-    const size_t stage = (size_t)2 * tok * g.d * sizeof(__nv_bfloat16);
-    const size_t rest = (size_t)4 * g.d * sizeof(float) + select_scratch_bytes(g.L) +
-                        (size_t)(kChainGroups * kThreads / 32) * 4 * g.d * sizeof(__nv_bfloat16);
-    const int ring = kChainGroups * kChainMaxRing * stage + rest <= 220 * 1024 ? kChainMaxRing : 2;
-    const size_t bytes = (size_t)kChainGroups * ring * stage                             // rings
-                         + (size_t)4 * g.d * sizeof(float)                               // scale / offset
-                         + select_scratch_bytes(g.L)
-                         + (size_t)(kChainGroups * kThreads / 32) * 4 * g.d * sizeof(__nv_bfloat16);   // min/max reduction
-    auto ckern = g.d == 128 ? score_select_chain_kernel<128> : score_select_chain_kernel<64>;
-    LRSA_CUDA_CHECK(cudaFuncSetAttribute(ckern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    ckern<<<(unsigned)(a.BH * runs_per_bh), kChainThreads, bytes, st>>>(a, run, runs_per_bh, ring);
-    LRSA_CUDA_CHECK(cudaGetLastError());
+  if (g.L <= kClusterMaxL) {
+    const ClusterPlan pl = cluster_plan(a.BH, g.Wsel, g.L);
+    const size_t bytes = (size_t)g.d * 16 + 2 * (4 * g.d * 2) + 8 * 2 * g.d * 2 + 2 * select_scratch_bytes(g.L);
+    auto kern = g.d == 128 ? (pl.run > 1 ? score_select_cluster_kernel<128, true> : score_select_cluster_kernel<128, false>)
+                           : (pl.run > 1 ? score_select_cluster_kernel<64, true> : score_select_cluster_kernel<64, false>);
+    if (bytes > 48 * 1024)
+      LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    const int runs_per_bh = (g.Wsel + pl.run - 1) / pl.run;
+    const long long grid = (long long)a.BH * runs_per_bh * pl.C;
+    if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
+    LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(kThreads), bytes, st, pl.C, a, pl.run, runs_per_bh, pl.C));
     launch_counter().n++;
     return LRSA_OK;
   }
