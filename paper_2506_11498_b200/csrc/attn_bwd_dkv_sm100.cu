@@ -30,145 +30,12 @@
 // the accumulators are added (fp32 atomics) to a zeroed workspace indexed by original position: a
 // row of a compact tile goes to the position it was gathered from, so a kept key's compressed and
 // uncompressed contributions meet in one row.  A small kernel then converts to bf16.
-#include "attn_common_sm100.h"
+#include "attn_bwd_sm100.h"
 
 namespace lrsa {
 namespace {
 
 using namespace ptx;
-
-constexpr int kQRows = 128;   // query rows per inner tile
-constexpr int kSeg = 128;     // inner iterations per CTA at most
-
-struct DkvPlan {
-  int S, L, K, N, W, T, C, Wsel, ndp, Rc, G;
-  int n_cmp;       // compact tiles
-  int n_sink;      // dense tiles of the sink region
-  int per_win;     // dense tiles per full window
-  int per_tail;    // dense tiles of the tail
-  int n_tiles;
-};
-
-struct KvTile {
-  int kind;      // 0 compact, 1 dense
-  int row0;      // first compact row / first key position
-  int key_end;   // rows at or beyond this are not part of the tile
-  int qb, qend;  // query positions [qb, qend) see (part of) the tile
-  int nq;        // query tiles (kQRows rows) per head
-};
-
-inline DkvPlan make_dkv_plan(const Geom& g) {
-  DkvPlan p;
-  p.S = g.S; p.L = g.L; p.K = g.K; p.N = g.N; p.W = g.W; p.T = g.T; p.C = g.C; p.Wsel = g.Wsel;
-  p.ndp = g.ndp; p.Rc = g.Rc; p.G = g.G;
-  p.n_cmp = (g.Rc + kTile - 1) / kTile;
-  p.n_sink = (g.S + kTile - 1) / kTile;
-  p.per_win = (g.L + kTile - 1) / kTile;
-  p.per_tail = (g.T + kTile - 1) / kTile;
-  p.n_tiles = p.n_cmp + p.n_sink + g.W * p.per_win + p.per_tail;
-  return p;
-}
-
-__host__ __device__ inline KvTile describe_tile(const DkvPlan& p, int tile) {
-  KvTile t;
-  if (tile < p.n_cmp) {
-    t.kind = 0;
-    t.row0 = tile * kTile;
-    t.key_end = p.Rc;
-    int cmin = 0;
-    if (t.row0 >= p.S) cmin = first_compressed_chunk((t.row0 - p.S) / p.K, p.ndp, p.Wsel, p.C);
-    t.qb = p.S + cmin * p.L;
-    t.qend = cmin >= p.C ? t.qb : p.N;
-  } else {
-    t.kind = 1;
-    int d = tile - p.n_cmp;
-    if (d < p.n_sink) {
-      t.row0 = d * kTile; t.key_end = p.S; t.qend = p.S;
-    } else {
-      d -= p.n_sink;
-      int w;
-      if (d < p.W * p.per_win) {
-        w = d / p.per_win;
-        t.row0 = p.S + w * p.L + (d % p.per_win) * kTile;
-        t.key_end = p.S + (w + 1) * p.L;
-      } else {
-        w = p.W;
-        t.row0 = p.S + p.W * p.L + (d - p.W * p.per_win) * kTile;
-        t.key_end = p.N;
-      }
-      const int cc = first_compressed_chunk(w, p.ndp, p.Wsel, p.C);
-      t.qend = cc >= p.C ? p.N : (p.S + cc * p.L < p.N ? p.S + cc * p.L : p.N);
-    }
-    t.qb = t.row0;
-  }
-  t.nq = t.qend > t.qb ? (t.qend - t.qb + kQRows - 1) / kQRows : 0;
-  return t;
-}
-
-__host__ __device__ inline int tile_segments(const DkvPlan& p, const KvTile& t) {
-  return (p.G * t.nq + kSeg - 1) / kSeg;
-}
-
-// Launch order of the (tile, segment) pairs (one block).  Iteration i of a tile is query tile
-// nq-1 - i/G (counted from the last query) of head i%G, so segment s of every compact tile covers the
-// same queries of the same heads.  Compact tiles are therefore issued segment-major: the CTAs that run at
-// the same time then stream the same Q_i / dO_i tiles and share them through L2 instead of fetching
-// them from DRAM once per key tile.  Dense tiles (short lists, neighbours already overlap) follow in
-// position order.  seg_cnt: scratch of n_tiles + 1 ints; seg_map[x] = (tile, segment of the tile).
-constexpr int kMaxSegsPerTile = 2048;
-__global__ void dkv_setup_kernel(const DkvPlan p, int* seg_cnt, int2* seg_map) {
-  __shared__ int off[kMaxSegsPerTile + 1];   // off[s] = pairs of compact tiles with a segment index below s
-  __shared__ int s_mode, s_cmp_total;
-  __shared__ int run_sum[256];   // blockDim.x = 256
-  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x) seg_cnt[i] = tile_segments(p, describe_tile(p, i));
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // segment-major order needs the compact tiles' segment counts to be non-increasing (later rows are
-    // seen by later chunks only) and few enough for the table; otherwise keep tile-major order
-    bool mono = p.n_cmp > 0 && seg_cnt[0] <= kMaxSegsPerTile;
-    for (int c = 1; c < p.n_cmp && mono; ++c) mono = seg_cnt[c] <= seg_cnt[c - 1];
-    int total = 0;
-    if (mono) {
-      int c = p.n_cmp;   // tiles [0, c) have more than s segments
-      const int maxs = seg_cnt[0];
-      for (int sgm = 0; sgm < maxs; ++sgm) {
-        while (c > 0 && seg_cnt[c - 1] <= sgm) --c;
-        off[sgm] = total;
-        total += c;
-      }
-    } else {
-      for (int c = 0; c < p.n_cmp; ++c) {
-        for (int sgm = 0; sgm < seg_cnt[c]; ++sgm) seg_map[total + sgm] = make_int2(c, sgm);
-        total += seg_cnt[c];
-      }
-    }
-    s_mode = mono ? 1 : 0;
-    s_cmp_total = total;
-  }
-  // dense tiles, position order: every thread takes a run of consecutive tiles
-  const int nd = p.n_tiles - p.n_cmp, per = (nd + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int d_lo = min(p.n_tiles, p.n_cmp + (int)threadIdx.x * per), d_hi = min(p.n_tiles, d_lo + per);
-  int mine = 0;
-  for (int t = d_lo; t < d_hi; ++t) mine += seg_cnt[t];
-  run_sum[threadIdx.x] = mine;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = s_cmp_total;
-    for (int i = 0; i < (int)blockDim.x; ++i) { const int v = run_sum[i]; run_sum[i] = acc; acc += v; }
-  }
-  __syncthreads();
-  {
-    int pos = run_sum[threadIdx.x];
-    for (int t = d_lo; t < d_hi; ++t) {
-      for (int sgm = 0; sgm < seg_cnt[t]; ++sgm) seg_map[pos + sgm] = make_int2(t, sgm);
-      pos += seg_cnt[t];
-    }
-  }
-  if (s_mode) {
-    for (int c = threadIdx.x; c < p.n_cmp; c += blockDim.x)
-      for (int sgm = 0; sgm < seg_cnt[c]; ++sgm) seg_map[off[sgm] + c] = make_int2(c, sgm);
-  }
-}
 
 template <int D>
 struct DkvCfg {
@@ -191,12 +58,23 @@ struct DkvCfg {
   static constexpr uint32_t kColS = 0, kColP = 128, kColK = 256, kColV = 256 + D;
 };
 
+template <int NSEQ>
+struct DkvMaps { CUtensorMap q[NSEQ], dO[NSEQ], k[NSEQ], v[NSEQ], kg[NSEQ], vg[NSEQ]; };   // kg, vg: row gathers
+
+template <int NSEQ>
 struct DkvArgs {
-  DkvPlan plan;
-  int BHkv, Hq, Hkv, total_segs;
-  const int32_t* idx;    // kept positions of this sequence's windows: head bh at idx + bh * kept_stride
+  DkvPlan plan[NSEQ];
+  int tok0[NSEQ];        // first token of the sequence
+  int kept_off[NSEQ];    // its first entry of idx, per (batch, KV head)
+  int map0[NSEQ];        // its part of seg_map
+  int seg0[NSEQ + 1];    // (tile, segment) pairs of the sequences before
+  int n_seqs;
+  int BHkv, Hq, Hkv;
+  const int32_t* idx;    // kept positions: head bh at idx + bh * kept_stride
   int kept_stride;       // Wtot * K entries per (batch, KV head)
-  int Nrow, tok0;        // tokens per (batch, head) row (the stride of every tensor); first token of the sequence
+  int Nrow;              // tokens per (batch, head) row (the stride of every tensor)
+  const float* kpart;    // when not null: partial sums of the mean key, to be finished
+  float* kbar;
   const float2* stats;   // per query row: (-LSE * log2(e), D~ = rowsum(dO * O) from the bf16 O)
   float* Dacc;           // [B*Hq][N], zeroed: receives sum_j P_tj dP_tj, the accurate D for the dQ kernel
   const int2* seg_map;   // launch order: (tile, segment of the tile)
@@ -223,12 +101,9 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-template <int D>
+template <int D, int NSEQ>
 __global__ void __launch_bounds__(DkvCfg<D>::kThreads, 1)
-lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapdO,
-                    const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
-                    const __grid_constant__ CUtensorMap mapKg, const __grid_constant__ CUtensorMap mapVg,
-                    const DkvArgs a) {
+lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_constant__ DkvArgs<NSEQ> a) {
   using Cfg = DkvCfg<D>;
   constexpr int NQ = Cfg::kStQ, NO = Cfg::kStO;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -242,12 +117,21 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   const uint32_t sQ = smem0 + Cfg::kOffRingQ, sO = smem0 + Cfg::kOffRingO;
 
   // ---- which tile, which segment ----
-  const DkvPlan& p = a.plan;
-  const int bh_kv = blockIdx.x % a.BHkv, seg = blockIdx.x / a.BHkv;
-  const int2 ts = a.seg_map[seg];
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int bh_kv = blockIdx.x % a.BHkv;
+  int seg = blockIdx.x / a.BHkv, sq = 0;
+  if constexpr (NSEQ > 1) {
+    while (sq + 1 < a.n_seqs && seg >= a.seg0[sq + 1]) ++sq;
+    seg -= a.seg0[sq];
+  }
+  const DkvPlan& p = a.plan[sq];
+  const int tok0 = a.tok0[sq];
+  const int32_t* kept = a.idx + (size_t)bh_kv * a.kept_stride + a.kept_off[sq];   // this head's, this sequence's windows
+  const int2 ts = a.seg_map[a.map0[sq] + seg];
   const KvTile kt = describe_tile(p, ts.x);
-  const int it_begin = ts.y * kSeg;
-  const int n = min(kSeg, p.G * kt.nq - it_begin);
+  const int it_begin = ts.y * p.seg;
+  const int n = min(p.seg, p.G * kt.nq - it_begin);
   const int hq0 = (bh_kv / a.Hkv) * a.Hq + (bh_kv % a.Hkv) * p.G;   // first query head of the group
 
   if (smem0 & 1023u) {   // the swizzled tiles need it; dynamic shared memory starts there when nothing is static
@@ -281,25 +165,24 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      prefetch_tensormap(&mapQ); prefetch_tensormap(&mapdO);
+      prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.dO[sq]);
       mbar_expect_tx(smem_u32(&ctl.kv_full), 2 * Cfg::kTileBytes);
     }
     __syncwarp();
     if (kt.kind == 0) {
       // every lane gathers four rows of the list tile from their positions in K and V
-      const int32_t* kept = a.idx + (size_t)bh_kv * a.kept_stride;
       int pos[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        pos[i] = bh_kv * a.Nrow + compact_row_pos(kept, p.S, p.Rc, kt.row0 + 4 * lane + i, a.tok0);
+        pos[i] = bh_kv * a.Nrow + compact_row_pos(kept, p.S, p.Rc, kt.row0 + 4 * lane + i, tok0);
       for (int h = 0; h < Cfg::kSub; ++h) {
-        tma_gather4_2d(sK + h * Cfg::kSubBytes + lane * 512, &mapKg, h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&ctl.kv_full));
-        tma_gather4_2d(sV + h * Cfg::kSubBytes + lane * 512, &mapVg, h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&ctl.kv_full));
+        tma_gather4_2d(sK + h * Cfg::kSubBytes + lane * 512, &maps.kg[sq], h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&ctl.kv_full));
+        tma_gather4_2d(sV + h * Cfg::kSubBytes + lane * 512, &maps.vg[sq], h * 64, pos[0], pos[1], pos[2], pos[3], smem_u32(&ctl.kv_full));
       }
     } else if (lane == 0) {
       for (int h = 0; h < Cfg::kSub; ++h) {
-        tma_load_3d(sK + h * Cfg::kSubBytes, &mapK, h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
-        tma_load_3d(sV + h * Cfg::kSubBytes, &mapV, h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
+        tma_load_3d(sK + h * Cfg::kSubBytes, &maps.k[sq], h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
+        tma_load_3d(sV + h * Cfg::kSubBytes, &maps.v[sq], h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
       }
     }
     if (lane == 0) {
@@ -313,14 +196,14 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const uint32_t qf = smem_u32(&ctl.q_full[slq]);
         mbar_expect_tx(qf, Cfg::kTileBytes);
         for (int h = 0; h < Cfg::kSub; ++h)
-          tma_load_3d(sQ + slq * Cfg::kTileBytes + h * Cfg::kSubBytes, &mapQ, h * 64, q0, hq, qf);
+          tma_load_3d(sQ + slq * Cfg::kTileBytes + h * Cfg::kSubBytes, &maps.q[sq], h * 64, q0, hq, qf);
         ++nq_issued;
         if (it >= NO) ok = mbar_wait(smem_u32(&ctl.o_empty[slo]), pho ^ 1, abort);
         if (!ok) break;
         const uint32_t of = smem_u32(&ctl.o_full[slo]);
         mbar_expect_tx(of, Cfg::kTileBytes);
         for (int h = 0; h < Cfg::kSub; ++h)
-          tma_load_3d(sO + slo * Cfg::kTileBytes + h * Cfg::kSubBytes, &mapdO, h * 64, q0, hq, of);
+          tma_load_3d(sO + slo * Cfg::kTileBytes + h * Cfg::kSubBytes, &maps.dO[sq], h * 64, q0, hq, of);
         ++no_issued;
         if (++slq == NQ) { slq = 0; phq ^= 1; }
         if (++slo == NO) { slo = 0; pho ^= 1; }
@@ -423,6 +306,19 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     }
     if (ok && elect_one()) umma_commit(smem_u32(&ctl.acc_done));
     __syncwarp();
+  } else if (warp == 2) {
+    // the mean key of head blockIdx.x from its partial sums, for the dQ kernel
+    if (a.kpart && blockIdx.x < a.BHkv) {
+      for (int ch = lane * 4; ch < D; ch += 128) {
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int i = 0; i < kMeanSplits; ++i) {
+          const float4 x = *reinterpret_cast<const float4*>(a.kpart + ((size_t)i * a.BHkv + blockIdx.x) * D + ch);
+          sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+        }
+        *reinterpret_cast<float4*>(a.kbar + (size_t)blockIdx.x * D + ch) = sum;
+      }
+    }
   } else if (warp == 3) {
     // ---------------- per-row statistics of every step, fetched one step ahead ----------------
     int qt = qt0, hd = hd0;
@@ -431,7 +327,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
 #pragma unroll
       for (int k = 0; k < kQRows / 32; ++k) {
         const int q = q0 + lane + 32 * k;
-        v[k] = q < kt.qend ? __ldg(a.stats + (size_t)hq * a.Nrow + q) : make_float2(-INFINITY, 0.f);
+        v[k] = q < kt.qend ? __ldg(a.stats + (size_t)hq * a.Nrow + tok0 + q) : make_float2(-INFINITY, 0.f);
       }
     };
     float2 cur[kQRows / 32], nxt[kQRows / 32];
@@ -571,7 +467,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
           c8[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
         }
       }
-      if (q0 + col < kt.qend) atomicAdd(a.Dacc + (size_t)(hq0 + hd) * a.Nrow + q0 + col, c8[0]);
+      if (q0 + col < kt.qend) atomicAdd(a.Dacc + (size_t)(hq0 + hd) * a.Nrow + tok0 + q0 + col, c8[0]);
       if (++hd == p.G) { hd = 0; q0 -= kQRows; }
     }
     if (ok) ok = mbar_wait_warp(smem_u32(&ctl.acc_done), 0, abort);
@@ -584,9 +480,9 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
       const float mul = is_k ? a.scale : 1.0f;
       // a row of a compact tile lands on the position it was gathered from
       const int out_row = kt.kind == 0
-                              ? compact_row_pos(a.idx + (size_t)bh_kv * a.kept_stride, p.S, p.Rc, kt.row0 + r, a.tok0)
+                              ? compact_row_pos(kept, p.S, p.Rc, kt.row0 + r, tok0)
                               : kt.row0 + r;
-      float* dst = (is_k ? a.dKf : a.dVf) + ((size_t)bh_kv * a.Nrow + out_row) * D + (wg & 1) * CH;
+      float* dst = (is_k ? a.dKf : a.dVf) + ((size_t)bh_kv * a.Nrow + tok0 + out_row) * D + (wg & 1) * CH;
 #pragma unroll
       for (int q = 0; q < CH / 32; ++q) {
         uint32_t o[32];
@@ -608,117 +504,50 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   if (tid == 0 && ctl.abort) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
 }
 
-// bf16 outputs from the fp32 accumulators [BHkv][N][d]; n4 = number of float4 groups
-__global__ void convert_dkv_kernel(const float* __restrict__ dKf, const float* __restrict__ dVf,
-                                   __nv_bfloat16* __restrict__ dK, __nv_bfloat16* __restrict__ dV, long long n4) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n4) return;
-  const long long e = i * 4;
-  const float4 k = *reinterpret_cast<const float4*>(dKf + e);
-  const float4 v = *reinterpret_cast<const float4*>(dVf + e);
-  uint2 ko, vo;
-  ko.x = pack_bf16(k.x, k.y); ko.y = pack_bf16(k.z, k.w);
-  vo.x = pack_bf16(v.x, v.y); vo.y = pack_bf16(v.z, v.w);
-  *reinterpret_cast<uint2*>(dK + e) = ko;
-  *reinterpret_cast<uint2*>(dV + e) = vo;
-}
-
 }  // namespace
 
-static int dkv_total_segs(const DkvPlan& p) {
-  int total = 0;
-  for (int i = 0; i < p.n_tiles; ++i) total += tile_segments(p, describe_tile(p, i));
-  return total;
-}
-
-// Layout: [segment counts: n_tiles + 1 ints][launch order: total_segs int2][dK fp32][dV fp32]
-size_t dkv_ws_bytes(const Geom& g, size_t* prefix_bytes) {
-  const DkvPlan p = make_dkv_plan(g);
-  const size_t cnt = align_up((size_t)(p.n_tiles + 1) * sizeof(int), 1024);
-  const size_t pre = cnt + align_up((size_t)(dkv_total_segs(p) + 1) * sizeof(int2), 1024);
-  if (prefix_bytes) *prefix_bytes = pre;
-  const size_t acc = align_up((size_t)g.B * g.Hkv * g.Nrow * g.d * sizeof(float), 1024);
-  return pre + 2 * acc;
-}
-
-template <int D>
-static int launch_dkv_t(const Geom& g, const DkvArgs& a, const CUtensorMap* m, cudaStream_t st) {
+template <int D, int NSEQ>
+static int launch_dkv_t(const Geom& whole, const SeqBatch& b, const DkvBatch& db, const BwdPtrs& p, bool mean, cudaStream_t st) {
   using Cfg = DkvCfg<D>;
-  auto kern = lrsa_bwd_dkv_kernel<D>;
+  DkvMaps<NSEQ> m;
+  DkvArgs<NSEQ> a;
+  const long long BHq = (long long)whole.B * whole.Hq, BHkv = (long long)whole.B * whole.Hkv;
+  a.seg0[0] = 0;
+  for (int s = 0; s < b.n; ++s) {
+    const Geom& g = b.g[s];
+    const size_t sh = (size_t)g.tok0 * D;
+    int r = make_tmap_bf16(&m.q[s], p.Q + sh, D, g.N, BHq, kQRows, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.dO[s], p.dO + sh, D, g.N, BHq, kQRows, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.k[s], p.K + sh, D, g.N, BHkv, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.v[s], p.V + sh, D, g.N, BHkv, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16_rows(&m.kg[s], p.K + sh, D, BHkv * g.Nrow - g.tok0);
+    if (r == LRSA_OK) r = make_tmap_bf16_rows(&m.vg[s], p.V + sh, D, BHkv * g.Nrow - g.tok0);
+    if (r != LRSA_OK) return r;
+    a.plan[s] = db.plan[s];
+    a.tok0[s] = g.tok0;
+    a.kept_off[s] = g.woff * g.K;
+    a.map0[s] = db.map0[s];
+    a.seg0[s + 1] = a.seg0[s] + db.segs[s];
+  }
+  a.n_seqs = b.n;
+  a.BHkv = (int)BHkv; a.Hq = whole.Hq; a.Hkv = whole.Hkv;
+  a.idx = p.idx; a.kept_stride = whole.Wtot * whole.K; a.Nrow = whole.Nrow;
+  a.kpart = mean ? p.kpart : nullptr; a.kbar = p.kbar;
+  a.stats = p.stats; a.Dacc = p.Dacc; a.seg_map = p.seg_map; a.dKf = p.dKf; a.dVf = p.dVf;
+  a.scale = whole.scale; a.scale_log2 = whole.scale * 1.4426950408889634f; a.status = p.status;
+  auto kern = lrsa_bwd_dkv_kernel<D, NSEQ>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
-  const long long grid = (long long)a.total_segs * a.BHkv;
+  const long long grid = (long long)a.seg0[b.n] * a.BHkv;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  if (grid == 0) return LRSA_OK;
-  kern<<<(unsigned)grid, Cfg::kThreads, Cfg::kSmem, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], a);
-  LRSA_CUDA_CHECK(cudaGetLastError());
+  LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));
   launch_counter().n++;
   return LRSA_OK;
 }
 
-// ws_dkv: region of dkv_ws_bytes(whole row) bytes.  Three steps: dkv_zero clears the fp32 accumulators of
-// the whole row, launch_bwd_dkv_sm100 runs the tile kernel of one sequence (its launch-order table is
-// rebuilt in the region's prefix, in stream order), dkv_convert writes bf16 dK, dV.
-static void dkv_regions(const Geom& whole, void* ws_dkv, int** seg_cnt, int2** seg_map, float** dKf, float** dVf,
-                        size_t* acc_bytes) {
-  size_t pre = 0;
-  const size_t total = dkv_ws_bytes(whole, &pre);
-  unsigned char* base = static_cast<unsigned char*>(ws_dkv);
-  const DkvPlan p = make_dkv_plan(whole);
-  *acc_bytes = (total - pre) / 2;
-  *seg_cnt = reinterpret_cast<int*>(base);
-  *seg_map = reinterpret_cast<int2*>(base + align_up((size_t)(p.n_tiles + 1) * sizeof(int), 1024));
-  *dKf = reinterpret_cast<float*>(base + pre);
-  *dVf = reinterpret_cast<float*>(base + pre + *acc_bytes);
-}
-
-int dkv_zero(const Geom& whole, void* ws_dkv, cudaStream_t st) {
-  int* seg_cnt; int2* seg_map; float *dKf, *dVf; size_t acc;
-  dkv_regions(whole, ws_dkv, &seg_cnt, &seg_map, &dKf, &dVf, &acc);
-  LRSA_CUDA_CHECK(cudaMemsetAsync(dKf, 0, 2 * acc, st));
-  launch_counter().n++;
-  return LRSA_OK;
-}
-
-int dkv_convert(const Geom& whole, void* ws_dkv, __nv_bfloat16* dK, __nv_bfloat16* dV, cudaStream_t st) {
-  int* seg_cnt; int2* seg_map; float *dKf, *dVf; size_t acc;
-  dkv_regions(whole, ws_dkv, &seg_cnt, &seg_map, &dKf, &dVf, &acc);
-  const long long n4 = (long long)whole.B * whole.Hkv * whole.Nrow * whole.d / 4;
-  convert_dkv_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(dKf, dVf, dK, dV, n4);
-  LRSA_CUDA_CHECK(cudaGetLastError());
-  launch_counter().n++;
-  return LRSA_OK;
-}
-
-// `whole`: the geometry of the whole row (workspace layout); `g`: the sequence to process.
-int launch_bwd_dkv_sm100(const Geom& whole, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* dO,
-                         const __nv_bfloat16* K, const __nv_bfloat16* V, const float2* stats, float* Dacc,
-                         const int32_t* idx, void* ws_dkv, int* status, cudaStream_t st) {
-  const DkvPlan p = make_dkv_plan(g);
-  int* seg_cnt; int2* seg_map; float *dKf, *dVf; size_t acc;
-  dkv_regions(whole, ws_dkv, &seg_cnt, &seg_map, &dKf, &dVf, &acc);
-  // a part of a row never needs more than the whole row; checked all the same
-  if (p.n_tiles > make_dkv_plan(whole).n_tiles || dkv_total_segs(p) > dkv_total_segs(make_dkv_plan(whole)))
-    return LRSA_ERR_WORKSPACE_TOO_SMALL;
-  dkv_setup_kernel<<<1, 256, 0, st>>>(p, seg_cnt, seg_map);
-  LRSA_CUDA_CHECK(cudaGetLastError());
-  launch_counter().n++;
-  const int total_segs = dkv_total_segs(p);
-
-  CUtensorMap m[6];
-  const size_t sh = (size_t)g.tok0 * g.d;
-  int r = make_tmap_bf16(&m[0], Q + sh, g.d, g.N, (long long)g.B * g.Hq, kQRows, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&m[1], dO + sh, g.d, g.N, (long long)g.B * g.Hq, kQRows, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&m[2], K + sh, g.d, g.N, (long long)g.B * g.Hkv, kTile, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&m[3], V + sh, g.d, g.N, (long long)g.B * g.Hkv, kTile, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16_rows(&m[4], K + sh, g.d, (long long)g.B * g.Hkv * g.Nrow - g.tok0);
-  if (r == LRSA_OK) r = make_tmap_bf16_rows(&m[5], V + sh, g.d, (long long)g.B * g.Hkv * g.Nrow - g.tok0);
-  if (r != LRSA_OK) return r;
-  DkvArgs a;
-  a.plan = p; a.BHkv = g.B * g.Hkv; a.Hq = g.Hq; a.Hkv = g.Hkv; a.total_segs = total_segs;
-  a.idx = idx + (size_t)g.woff * g.K; a.kept_stride = g.Wtot * g.K; a.Nrow = g.Nrow; a.tok0 = g.tok0;
-  a.stats = stats + g.tok0; a.Dacc = Dacc + g.tok0; a.seg_map = seg_map; a.dKf = dKf + sh; a.dVf = dVf + sh;
-  a.scale = g.scale; a.scale_log2 = g.scale * 1.4426950408889634f; a.status = status;
-  return g.d == 128 ? launch_dkv_t<128>(g, a, m, st) : launch_dkv_t<64>(g, a, m, st);
+int launch_bwd_dkv_sm100(const Geom& whole, const SeqBatch& b, const DkvBatch& db, const BwdPtrs& p, bool mean, cudaStream_t st) {
+  if (whole.d == 128)
+    return b.n == 1 ? launch_dkv_t<128, 1>(whole, b, db, p, mean, st) : launch_dkv_t<128, kMaxSeqs>(whole, b, db, p, mean, st);
+  return b.n == 1 ? launch_dkv_t<64, 1>(whole, b, db, p, mean, st) : launch_dkv_t<64, kMaxSeqs>(whole, b, db, p, mean, st);
 }
 
 }  // namespace lrsa

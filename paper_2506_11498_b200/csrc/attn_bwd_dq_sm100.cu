@@ -19,7 +19,7 @@
 // Rows of the exact dS sum to zero; after bf16 rounding they sum to r_t, which multiplies whatever
 // constant vector the keys of a head share (outlier channels).  The epilogue subtracts r_t * kbar,
 // kbar the mean key of the KV head; in exact arithmetic this subtracts zero.
-#include "attn_common_sm100.h"
+#include "attn_bwd_sm100.h"
 
 namespace lrsa {
 namespace {
@@ -43,8 +43,15 @@ struct DqCfg {
   static constexpr uint32_t kColQ = 0, kColdO = D / 2, kColA = D, kColBuf = 256, kColP = 64;
 };
 
+template <int NSEQ>
+struct DqMaps { CUtensorMap q[NSEQ], dO[NSEQ], k[NSEQ], v[NSEQ], kc[NSEQ], vc[NSEQ]; };
+
+template <int NSEQ>
 struct DqArgs {
-  BlockPlan plan;
+  BlockPlan plan[NSEQ];
+  int tok0[NSEQ];          // first token of the sequence
+  int block0[NSEQ + 1];    // blocks of the sequences before, per (batch, head)
+  int n_seqs;
   int BH, Hq, Hkv, G, N;   // N: tokens per (batch, head) row of stats, Dacc and dQ (the row stride)
   const float2* stats;   // per query row: (-LSE*log2e, D~); only the first component is used here
   const float* Dacc;     // per query row: D = sum_j P dP
@@ -60,12 +67,9 @@ struct DqBars {
   uint64_t s_full[2], p_full[2], buf_free[2];
 };
 
-template <int D>
+template <int D, int NSEQ>
 __global__ void __launch_bounds__(DqCfg<D>::kThreads, 1)
-lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapdO,
-                   const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
-                   const __grid_constant__ CUtensorMap mapKc, const __grid_constant__ CUtensorMap mapVc,
-                   const DqArgs a) {
+lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_constant__ DqArgs<NSEQ> a) {
   using Cfg = DqCfg<D>;
   constexpr int NS = Cfg::kStages;
   extern __shared__ unsigned char smem_raw[];
@@ -78,8 +82,14 @@ lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = smem0, sdO = smem0 + Cfg::kQTileBytes, sRing = smem0 + 2 * Cfg::kQTileBytes;
 
-  const int bh = blockIdx.x % a.BH, blk = blockIdx.x / a.BH;
-  const RowBlock rb = decode_block(a.plan, blk);
+  const int bh = blockIdx.x % a.BH;
+  int blk = blockIdx.x / a.BH, sq = 0;
+  if constexpr (NSEQ > 1) {
+    while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
+    blk -= a.block0[sq];
+  }
+  const RowBlock rb = decode_block(a.plan[sq], blk);
+  const size_t row0 = (size_t)bh * a.N + a.tok0[sq];   // the sequence's first row of stats, Dacc and dQ
   const int bh_kv = (bh / a.Hq) * a.Hkv + (bh % a.Hq) / a.G;
   const int n_ct = (rb.n_front + kKeys - 1) / kKeys;
   const int n = n_ct + (rb.q_end - 1 - rb.dense_start) / kKeys + 1;   // key tiles of this block (>= 1)
@@ -103,16 +113,18 @@ lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
   volatile int* abort = &abort_s;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      prefetch_tensormap(&mapQ); prefetch_tensormap(&mapdO); prefetch_tensormap(&mapK); prefetch_tensormap(&mapV);
-      prefetch_tensormap(&mapKc); prefetch_tensormap(&mapVc);
+      prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.dO[sq]); prefetch_tensormap(&maps.k[sq]);
+      prefetch_tensormap(&maps.v[sq]); prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
       mbar_expect_tx(smem_u32(&bars.q_full), 2 * Cfg::kQTileBytes);
       for (int h = 0; h < Cfg::kSub; ++h) {
-        tma_load_3d(sQ + h * Cfg::kQSubBytes, &mapQ, h * 64, rb.q0, bh, smem_u32(&bars.q_full));
-        tma_load_3d(sdO + h * Cfg::kQSubBytes, &mapdO, h * 64, rb.q0, bh, smem_u32(&bars.q_full));
+        tma_load_3d(sQ + h * Cfg::kQSubBytes, &maps.q[sq], h * 64, rb.q0, bh, smem_u32(&bars.q_full));
+        tma_load_3d(sdO + h * Cfg::kQSubBytes, &maps.dO[sq], h * 64, rb.q0, bh, smem_u32(&bars.q_full));
       }
       int it = 0;
       bool ok = true;
@@ -124,7 +136,7 @@ lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
           const uint32_t full = smem_u32(&bars.kv_full[slot]);
           mbar_expect_tx(full, Cfg::kKTileBytes);
           const bool compact = j < n_ct;
-          const CUtensorMap* map = compact ? (which ? &mapVc : &mapKc) : (which ? &mapV : &mapK);
+          const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
           const int row = compact ? j * kKeys : rb.dense_start + (j - n_ct) * kKeys;
           for (int h = 0; h < Cfg::kSub; ++h)
             tma_load_3d(sRing + slot * Cfg::kKTileBytes + h * Cfg::kKSubBytes, map, h * 64, row, bh_kv, full);
@@ -203,8 +215,8 @@ lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     const bool live = qpos < rb.q_end;
     const float c = a.scale_log2;
     // rows outside the block get lse = +inf so that P = 0
-    const float nl2 = live ? a.stats[(size_t)bh * a.N + qpos].x : -INFINITY;
-    const float Dt = live ? a.Dacc[(size_t)bh * a.N + qpos] : 0.f;
+    const float nl2 = live ? a.stats[row0 + qpos].x : -INFINITY;
+    const float Dt = live ? a.Dacc[row0 + qpos] : 0.f;
     float rsum = 0.f;
     // copy this thread's row of Q (warpgroup 0) or dO (warpgroup 1) from the swizzled shared-memory
     // tile into tensor memory: 16-byte chunk c of row r of a 64-column sub-tile sits at chunk c ^ (r & 7)
@@ -303,7 +315,7 @@ lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");   // both halves of every row are staged (or a wait gave up)
     if (half == 0 && live && !*abort) {
-      __nv_bfloat16* orow = a.dQ + ((size_t)bh * a.N + qpos) * D;
+      __nv_bfloat16* orow = a.dQ + (row0 + qpos) * D;
       asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(orow),
                    "r"(smem_u32(stage_out + row * kStageStride)), "r"((uint32_t)kRowBytes)
                    : "memory");
@@ -318,133 +330,48 @@ lrsa_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
   if (tid == 0 && abort_s) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
 }
 
-// Per query row: D~_t = sum_c dO[t,c] * O[t,c] and -LSE_t * log2(e).  d/8 lanes share a row (16 bytes
-// each) and a warp takes kPrepUnroll groups of 256/d rows with all loads issued before the arithmetic:
-// the kernel only streams O and dO once and should run at memory speed.  With the rounding remainder of O
-// (Olo, optional) the sum runs over O + Olo, which is O to fp32 accuracy.
-constexpr int kPrepUnroll = 4;
-__global__ void bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ Olo,
-                                const __nv_bfloat16* __restrict__ dO, const float* __restrict__ LSE,
-                                float2* __restrict__ stats, long long rows, int d) {
-  const int lane = threadIdx.x & 31;
-  const int lpr = d >> 3, rpw = 32 / lpr;   // lanes per row, rows per warp-wide load (d = 64: 8, 4; d = 128: 16, 2)
-  const long long warp_id = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const long long row0 = warp_id * (kPrepUnroll * rpw) + lane / lpr;
-  const int c = (lane % lpr) * 8;
-  uint4 o[kPrepUnroll], l[kPrepUnroll], g[kPrepUnroll];
-#pragma unroll
-  for (int u = 0; u < kPrepUnroll; ++u) {
-    const long long row = row0 + u * rpw;
-    o[u] = l[u] = g[u] = make_uint4(0, 0, 0, 0);
-    if (row < rows) {
-      o[u] = *reinterpret_cast<const uint4*>(O + row * d + c);
-      g[u] = *reinterpret_cast<const uint4*>(dO + row * d + c);
-      if (Olo) l[u] = *reinterpret_cast<const uint4*>(Olo + row * d + c);
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kPrepUnroll; ++u) {
-    const uint32_t ow[4] = {o[u].x, o[u].y, o[u].z, o[u].w}, gw[4] = {g[u].x, g[u].y, g[u].z, g[u].w};
-    const uint32_t lw[4] = {l[u].x, l[u].y, l[u].z, l[u].w};
-    float acc = 0.f, acc_lo = 0.f;   // the remainder's products are 2^-9 of the others: summed apart, added last
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      acc = fmaf(__uint_as_float(ow[j] << 16), __uint_as_float(gw[j] << 16), acc);
-      acc = fmaf(__uint_as_float(ow[j] & 0xffff0000u), __uint_as_float(gw[j] & 0xffff0000u), acc);
-      acc_lo = fmaf(__uint_as_float(lw[j] << 16), __uint_as_float(gw[j] << 16), acc_lo);
-      acc_lo = fmaf(__uint_as_float(lw[j] & 0xffff0000u), __uint_as_float(gw[j] & 0xffff0000u), acc_lo);
-    }
-    acc += acc_lo;
-    for (int off = lpr >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    const long long row = row0 + u * rpw;
-    if ((lane % lpr) == 0 && row < rows) stats[row] = make_float2(-LSE[row] * 1.4426950408889634f, acc);
-  }
-}
-
-// kbar[bh][c] += (1/N) * sum of K[bh][t][c] over this block's rows (kbar zeroed beforehand).
-__global__ void __launch_bounds__(256) kbar_kernel(const __nv_bfloat16* __restrict__ K, float* __restrict__ kbar,
-                                                   int N, int d, int rows_per_block) {
-  __shared__ float red[256 * 8];
-  const int bh = blockIdx.y, tid = threadIdx.x;
-  const int lpr = d / 8, rps = 256 / lpr;          // lanes per row (16 bytes each), rows per step
-  const int chunk = tid % lpr, r_in = tid / lpr;
-  const int r0 = blockIdx.x * rows_per_block, r1 = min(N, r0 + rows_per_block);
-  float acc[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-  for (int r = r0 + r_in; r < r1; r += rps) {
-    const uint4 q = *reinterpret_cast<const uint4*>(K + ((size_t)bh * N + r) * d + chunk * 8);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      acc[2 * e] += __uint_as_float(w[e] << 16);
-      acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
-    }
-  }
-#pragma unroll
-  for (int e = 0; e < 8; ++e) red[tid * 8 + e] = acc[e];
-  __syncthreads();
-  if (tid < d) {
-    const int ch = tid / 8, e = tid % 8;
-    float sum = 0.f;
-    for (int r = 0; r < rps; ++r) sum += red[(r * lpr + ch) * 8 + e];
-    atomicAdd(kbar + (size_t)bh * d + tid, sum / (float)N);
-  }
-}
-
 }  // namespace
 
-int launch_bwd_prep(const Geom& g, const __nv_bfloat16* O, const __nv_bfloat16* Olo, const __nv_bfloat16* dO,
-                    const float* LSE, const __nv_bfloat16* K, float2* stats, float* kbar, cudaStream_t st) {
-  const long long rows = (long long)g.B * g.Hq * g.N;
-  const long long rows_per_block = 8LL * kPrepUnroll * (32 / (g.d >> 3));
-  bwd_prep_kernel<<<(unsigned)((rows + rows_per_block - 1) / rows_per_block), 256, 0, st>>>(O, Olo, dO, LSE, stats, rows, g.d);
-  LRSA_CUDA_CHECK(cudaGetLastError());
-  launch_counter().n++;
-  const int nsplit = 64, rpb = (g.N + nsplit - 1) / nsplit;
-  kbar_kernel<<<dim3(nsplit, g.B * g.Hkv), 256, 0, st>>>(K, kbar, g.N, g.d, rpb);
-  LRSA_CUDA_CHECK(cudaGetLastError());
-  launch_counter().n++;
-  return LRSA_OK;
-}
-
-template <int D>
-static int launch_dq_t(const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* dO, const __nv_bfloat16* K,
-                       const __nv_bfloat16* V, const __nv_bfloat16* Kc, const __nv_bfloat16* Vc, const float2* stats,
-                       const float* Dacc, const float* kbar, __nv_bfloat16* dQ, int* status, cudaStream_t st) {
+template <int D, int NSEQ>
+static int launch_dq_t(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, cudaStream_t st) {
   using Cfg = DqCfg<D>;
-  CUtensorMap mQ, mdO, mK, mV, mKc, mVc;
-  const long long rc = g.Rc > 0 ? g.Rc : 1;
-  // the sequence starts at token tok0 of rows of Nrow tokens: shifted bases, rows beyond its end read as zero
-  const size_t sh = (size_t)g.tok0 * D;
-  int r = make_tmap_bf16(&mQ, Q + sh, D, g.N, (long long)g.B * g.Hq, kTile, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&mdO, dO + sh, D, g.N, (long long)g.B * g.Hq, kTile, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&mK, K + sh, D, g.N, (long long)g.B * g.Hkv, kKeys, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&mV, V + sh, D, g.N, (long long)g.B * g.Hkv, kKeys, g.Nrow);
-  if (r == LRSA_OK) r = make_tmap_bf16(&mKc, Kc, D, rc, (long long)g.B * g.Hkv, kKeys);
-  if (r == LRSA_OK) r = make_tmap_bf16(&mVc, Vc, D, rc, (long long)g.B * g.Hkv, kKeys);
-  if (r != LRSA_OK) return r;
-  DqArgs a;
-  a.plan = make_plan(g, kTile);
-  a.BH = g.B * g.Hq; a.Hq = g.Hq; a.Hkv = g.Hkv; a.G = g.G; a.N = g.Nrow;
-  a.stats = stats + g.tok0; a.Dacc = Dacc + g.tok0; a.kbar = kbar; a.dQ = dQ + sh;
-  a.scale = g.scale; a.scale_log2 = g.scale * 1.4426950408889634f;
-  a.status = status;
-  const long long grid = (long long)a.plan.total * a.BH;
+  DqMaps<NSEQ> m;
+  DqArgs<NSEQ> a;
+  const long long BHq = (long long)whole.B * whole.Hq, BHkv = (long long)whole.B * whole.Hkv;
+  a.block0[0] = 0;
+  for (int s = 0; s < b.n; ++s) {
+    const Geom& g = b.g[s];
+    const long long rc = g.Rc > 0 ? g.Rc : 1;
+    // the sequence starts at token tok0 of rows of Nrow tokens: shifted bases, rows beyond its end read as zero
+    const size_t sh = (size_t)g.tok0 * D, csh = g.Rc > 0 ? (size_t)b.row0[s] * D : 0;
+    int r = make_tmap_bf16(&m.q[s], p.Q + sh, D, g.N, BHq, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.dO[s], p.dO + sh, D, g.N, BHq, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.k[s], p.K + sh, D, g.N, BHkv, kKeys, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.v[s], p.V + sh, D, g.N, BHkv, kKeys, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.kc[s], p.Kc + csh, D, rc, BHkv, kKeys);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.vc[s], p.Vc + csh, D, rc, BHkv, kKeys);
+    if (r != LRSA_OK) return r;
+    a.plan[s] = make_plan(g, kTile);
+    a.tok0[s] = g.tok0;
+    a.block0[s + 1] = a.block0[s] + a.plan[s].total;
+  }
+  a.n_seqs = b.n;
+  a.BH = (int)BHq; a.Hq = whole.Hq; a.Hkv = whole.Hkv; a.G = whole.G; a.N = whole.Nrow;
+  a.stats = p.stats; a.Dacc = p.Dacc; a.kbar = p.kbar; a.dQ = p.dQ;
+  a.scale = whole.scale; a.scale_log2 = whole.scale * 1.4426950408889634f;
+  a.status = p.status;
+  const long long grid = (long long)a.block0[b.n] * a.BH;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  auto kern = lrsa_bwd_dq_kernel<D>;
+  auto kern = lrsa_bwd_dq_kernel<D, NSEQ>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
-  kern<<<(unsigned)grid, Cfg::kThreads, Cfg::kSmem, st>>>(mQ, mdO, mK, mV, mKc, mVc, a);
-  LRSA_CUDA_CHECK(cudaGetLastError());
+  LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));
   launch_counter().n++;
   return LRSA_OK;
 }
 
-int launch_bwd_dq_sm100(const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* dO, const __nv_bfloat16* K,
-                        const __nv_bfloat16* V, const __nv_bfloat16* Kc, const __nv_bfloat16* Vc, const float2* stats,
-                        const float* Dacc, const float* kbar, __nv_bfloat16* dQ, int* status, cudaStream_t st) {
-  return g.d == 128 ? launch_dq_t<128>(g, Q, dO, K, V, Kc, Vc, stats, Dacc, kbar, dQ, status, st)
-                    : launch_dq_t<64>(g, Q, dO, K, V, Kc, Vc, stats, Dacc, kbar, dQ, status, st);
+int launch_bwd_dq_sm100(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, cudaStream_t st) {
+  if (whole.d == 128) return b.n == 1 ? launch_dq_t<128, 1>(whole, b, p, st) : launch_dq_t<128, kMaxSeqs>(whole, b, p, st);
+  return b.n == 1 ? launch_dq_t<64, 1>(whole, b, p, st) : launch_dq_t<64, kMaxSeqs>(whole, b, p, st);
 }
 
 }  // namespace lrsa

@@ -1,0 +1,177 @@
+// What the kernels of the backward share: the tiles and launch order of the dK/dV kernel, the pointers of a call.
+#pragma once
+
+#include "attn_common_sm100.h"
+
+namespace lrsa {
+
+constexpr int kQRows = 128;   // query rows per inner tile
+// Inner iterations per CTA of the dK/dV kernel, from their number in the whole call: at most 128 (a CTA's start and its
+// additions to the accumulators are then lost in the rest), fewer in small problems, so that the longest list does not
+// outlast an even share by much.
+constexpr int kSegMax = 128;
+inline int dkv_segment(long long iters) {
+  const long long s = iters / (148 * 4);
+  return s < 16 ? 16 : s > kSegMax ? kSegMax : (int)s;
+}
+
+struct DkvPlan {
+  int S, L, K, N, W, T, C, Wsel, ndp, Rc, G;
+  int n_cmp;       // compact tiles
+  int n_sink;      // dense tiles of the sink region
+  int per_win;     // dense tiles per full window
+  int per_tail;    // dense tiles of the tail
+  int n_tiles;
+  int seg;         // inner iterations per CTA at most
+};
+
+struct KvTile {
+  int kind;      // 0 compact, 1 dense
+  int row0;      // first compact row / first key position
+  int key_end;   // rows at or beyond this are not part of the tile
+  int qb, qend;  // query positions [qb, qend) see (part of) the tile
+  int nq;        // query tiles (kQRows rows) per head
+};
+
+inline DkvPlan make_dkv_plan(const Geom& g, int seg) {
+  DkvPlan p;
+  p.S = g.S; p.L = g.L; p.K = g.K; p.N = g.N; p.W = g.W; p.T = g.T; p.C = g.C; p.Wsel = g.Wsel;
+  p.ndp = g.ndp; p.Rc = g.Rc; p.G = g.G;
+  p.n_cmp = (g.Rc + kTile - 1) / kTile;
+  p.n_sink = (g.S + kTile - 1) / kTile;
+  p.per_win = (g.L + kTile - 1) / kTile;
+  p.per_tail = (g.T + kTile - 1) / kTile;
+  p.n_tiles = p.n_cmp + p.n_sink + g.W * p.per_win + p.per_tail;
+  p.seg = seg;
+  return p;
+}
+
+__host__ __device__ inline KvTile describe_tile(const DkvPlan& p, int tile) {
+  KvTile t;
+  if (tile < p.n_cmp) {
+    t.kind = 0;
+    t.row0 = tile * kTile;
+    t.key_end = p.Rc;
+    int cmin = 0;
+    if (t.row0 >= p.S) cmin = first_compressed_chunk((t.row0 - p.S) / p.K, p.ndp, p.Wsel, p.C);
+    t.qb = p.S + cmin * p.L;
+    t.qend = cmin >= p.C ? t.qb : p.N;
+  } else {
+    t.kind = 1;
+    int d = tile - p.n_cmp;
+    if (d < p.n_sink) {
+      t.row0 = d * kTile; t.key_end = p.S; t.qend = p.S;
+    } else {
+      d -= p.n_sink;
+      int w;
+      if (d < p.W * p.per_win) {
+        w = d / p.per_win;
+        t.row0 = p.S + w * p.L + (d % p.per_win) * kTile;
+        t.key_end = p.S + (w + 1) * p.L;
+      } else {
+        w = p.W;
+        t.row0 = p.S + p.W * p.L + (d - p.W * p.per_win) * kTile;
+        t.key_end = p.N;
+      }
+      const int cc = first_compressed_chunk(w, p.ndp, p.Wsel, p.C);
+      t.qend = cc >= p.C ? p.N : (p.S + cc * p.L < p.N ? p.S + cc * p.L : p.N);
+    }
+    t.qb = t.row0;
+  }
+  t.nq = t.qend > t.qb ? (t.qend - t.qb + kQRows - 1) / kQRows : 0;
+  return t;
+}
+
+__host__ __device__ inline int tile_segments(const DkvPlan& p, const KvTile& t) {
+  return (p.G * t.nq + p.seg - 1) / p.seg;
+}
+
+// Launch order of the (tile, segment) pairs (one block of 256 threads).  Iteration i of a tile is query tile
+// nq-1 - i/G (counted from the last query) of head i%G, so segment s of every compact tile covers the
+// same queries of the same heads.  Compact tiles are therefore issued segment-major: the CTAs that run at
+// the same time then stream the same Q_i / dO_i tiles and share them through L2 instead of fetching
+// them from DRAM once per key tile.  Dense tiles (short lists, neighbours already overlap) follow in
+// position order.  seg_cnt: scratch of n_tiles + 1 ints; seg_map[x] = (tile, segment of the tile).
+constexpr int kMaxSegsPerTile = 2048;
+__device__ inline void dkv_setup(const DkvPlan& p, int* seg_cnt, int2* seg_map) {
+  __shared__ int off[kMaxSegsPerTile + 1];   // off[s] = pairs of compact tiles with a segment index below s
+  __shared__ int s_mode, s_cmp_total;
+  __shared__ int run_sum[256];   // blockDim.x = 256
+  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x) seg_cnt[i] = tile_segments(p, describe_tile(p, i));
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // segment-major order needs the compact tiles' segment counts to be non-increasing (later rows are
+    // seen by later chunks only) and few enough for the table; otherwise keep tile-major order
+    bool mono = p.n_cmp > 0 && seg_cnt[0] <= kMaxSegsPerTile;
+    for (int c = 1; c < p.n_cmp && mono; ++c) mono = seg_cnt[c] <= seg_cnt[c - 1];
+    int total = 0;
+    if (mono) {
+      int c = p.n_cmp;   // tiles [0, c) have more than s segments
+      const int maxs = seg_cnt[0];
+      for (int sgm = 0; sgm < maxs; ++sgm) {
+        while (c > 0 && seg_cnt[c - 1] <= sgm) --c;
+        off[sgm] = total;
+        total += c;
+      }
+    } else {
+      for (int c = 0; c < p.n_cmp; ++c) {
+        for (int sgm = 0; sgm < seg_cnt[c]; ++sgm) seg_map[total + sgm] = make_int2(c, sgm);
+        total += seg_cnt[c];
+      }
+    }
+    s_mode = mono ? 1 : 0;
+    s_cmp_total = total;
+  }
+  // dense tiles, position order: every thread takes a run of consecutive tiles
+  const int nd = p.n_tiles - p.n_cmp, per = (nd + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int d_lo = min(p.n_tiles, p.n_cmp + (int)threadIdx.x * per), d_hi = min(p.n_tiles, d_lo + per);
+  int mine = 0;
+  for (int t = d_lo; t < d_hi; ++t) mine += seg_cnt[t];
+  run_sum[threadIdx.x] = mine;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int acc = s_cmp_total;
+    for (int i = 0; i < (int)blockDim.x; ++i) { const int v = run_sum[i]; run_sum[i] = acc; acc += v; }
+  }
+  __syncthreads();
+  {
+    int pos = run_sum[threadIdx.x];
+    for (int t = d_lo; t < d_hi; ++t) {
+      for (int sgm = 0; sgm < seg_cnt[t]; ++sgm) seg_map[pos + sgm] = make_int2(t, sgm);
+      pos += seg_cnt[t];
+    }
+  }
+  if (s_mode) {
+    for (int c = threadIdx.x; c < p.n_cmp; c += blockDim.x)
+      for (int sgm = 0; sgm < seg_cnt[c]; ++sgm) seg_map[off[sgm] + c] = make_int2(c, sgm);
+  }
+}
+
+// Pointers of one backward call (whole rows; the workspace's parts among them).
+struct BwdPtrs {
+  const __nv_bfloat16 *Q, *K, *V, *O, *Olo, *dO;
+  const float* LSE;
+  const int32_t* idx;
+  __nv_bfloat16 *dQ, *dK, *dV;
+  __nv_bfloat16 *Kc, *Vc;   // compact buffers
+  float2* stats;            // per query row: (-LSE * log2(e), D~ = rowsum(dO * O))
+  float* Dacc;              // per query row: sum_j P dP, the accurate D (zeroed, then filled by the dK/dV kernel)
+  float *kbar, *kpart;      // mean key per (batch, KV head); its partial sums [kMeanSplits][B*Hkv][d]
+  int* seg_cnt;             // dK/dV launch order: scratch, and (tile, segment) pairs
+  int2* seg_map;
+  float *dKf, *dVf;         // fp32 accumulators [B*Hkv][N][d], zeroed
+  int* status;
+};
+constexpr int kMeanSplits = 64;
+
+// Per sequence of the batch: its plan, where its parts of seg_cnt and seg_map start, its number of (tile, segment) pairs.
+struct DkvBatch {
+  DkvPlan plan[kMaxSeqs];
+  int cnt0[kMaxSeqs], map0[kMaxSeqs], segs[kMaxSeqs];
+};
+
+int launch_bwd_dq_sm100(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, cudaStream_t st);
+// `mean`: also finish the mean key from its partial sums (once per call).
+int launch_bwd_dkv_sm100(const Geom& whole, const SeqBatch& b, const DkvBatch& db, const BwdPtrs& p, bool mean, cudaStream_t st);
+
+}  // namespace lrsa

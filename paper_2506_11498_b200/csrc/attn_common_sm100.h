@@ -97,12 +97,62 @@ __device__ __forceinline__ RowBlock decode_block(const BlockPlan& p, int blk) {
 int make_tmap_bf16(CUtensorMap* map, const void* base, int d, long long rows, long long outer, int box_rows,
                    long long row_stride = 0);
 
-// Gathers the sink rows and the kept rows of K and V into the compact buffers
-// Kc, Vc [B*Hkv][Rc][d] (the condensed KV cache of Section 3.2) for the query-outer kernels, which
-// stream the list once per query tile: a TMA row gather in their main loops was measured at about
-// 6 bytes per clock and SM, a fifth of what they consume.
-int launch_compact_kv(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, const int32_t* idx,
-                      __nv_bfloat16* Kc, __nv_bfloat16* Vc, cudaStream_t st);
+// The sequences of a packed batch are taken up to kMaxSeqs at a time by one launch of each kernel (their tensor maps travel
+// as kernel parameters), longest first.  An unpacked batch is one sequence.  row0: first row of the sequence's part of the
+// compact buffers.
+constexpr int kMaxSeqs = 16;
+struct SeqBatch {
+  int n;
+  Geom g[kMaxSeqs];
+  long long row0[kMaxSeqs];
+};
+struct SeqBatches {
+  const Geom& whole;
+  int s = 0, woff = 0;
+  long long row0 = 0;
+  explicit SeqBatches(const Geom& w) : whole(w) {}
+  bool next(SeqBatch* b);   // false: none left
+};
+
+// Gather of the sink rows and the kept rows of K and V into the compact buffers: per sequence Kc, Vc [B*Hkv][Rc][d] (the
+// condensed KV cache of Section 3.2) for the query-outer kernels, which stream the list once per query tile (a TMA row
+// gather in their main loops was measured at about 6 bytes per clock and SM, a fifth of what they consume).  256 threads
+// a block, 16 bytes of K and of V each.
+struct CompactArgs {
+  const __nv_bfloat16 *K, *V;
+  const int32_t* idx;
+  __nv_bfloat16 *Kc, *Vc;
+  int* status;                 // cleared when not null
+  int Nrow, cpr, kept_stride, n;   // cpr: 16-byte chunks per row
+  int item0[kMaxSeqs + 1];     // rows before the sequence's, over all (batch, KV head) pairs
+  int Rc[kMaxSeqs], S[kMaxSeqs], tok0[kMaxSeqs], kept_off[kMaxSeqs];
+  long long row0[kMaxSeqs];
+  int blocks() const { return (int)(((long long)item0[n] * cpr + 255) / 256); }
+};
+inline CompactArgs compact_args(const Geom& whole, const SeqBatch& b, const __nv_bfloat16* K, const __nv_bfloat16* V,
+                                const int32_t* idx, __nv_bfloat16* Kc, __nv_bfloat16* Vc, int* status) {
+  CompactArgs c;
+  c.K = K; c.V = V; c.idx = idx; c.Kc = Kc; c.Vc = Vc; c.status = status;
+  c.Nrow = whole.Nrow; c.cpr = whole.d / 8; c.kept_stride = whole.Wtot * whole.K; c.n = b.n;
+  c.item0[0] = 0;
+  for (int s = 0; s < b.n; ++s) {
+    const Geom& g = b.g[s];
+    c.item0[s + 1] = c.item0[s] + g.B * g.Hkv * g.Rc;
+    c.Rc[s] = g.Rc; c.S[s] = g.S; c.tok0[s] = g.tok0; c.kept_off[s] = g.woff * g.K; c.row0[s] = b.row0[s];
+  }
+  return c;
+}
+__device__ __forceinline__ void compact_rows(const CompactArgs& c, int block) {
+  const int item = block * (256 / c.cpr) + (int)threadIdx.x / c.cpr, ch = threadIdx.x % c.cpr;
+  if (item >= c.item0[c.n]) return;
+  int s = 0;
+  while (item >= c.item0[s + 1]) ++s;
+  const int i = item - c.item0[s], bh = i / c.Rc[s], r = i - bh * c.Rc[s];
+  const int pos = r < c.S[s] ? r + c.tok0[s] : __ldg(c.idx + (size_t)bh * c.kept_stride + c.kept_off[s] + (r - c.S[s]));
+  const size_t src = ((size_t)bh * c.Nrow + pos) * c.cpr + ch, dst = (size_t)(c.row0[s] + i) * c.cpr + ch;
+  reinterpret_cast<uint4*>(c.Kc)[dst] = __ldg(reinterpret_cast<const uint4*>(c.K) + src);
+  reinterpret_cast<uint4*>(c.Vc)[dst] = __ldg(reinterpret_cast<const uint4*>(c.V) + src);
+}
 
 // 2-D bf16 tensor map over [rows][d] with a (64 x 1) box and 128-byte swizzle, for row gathers
 // (tile::gather4).  The key-outer dK/dV kernel loads its one list tile per CTA this way, four rows per

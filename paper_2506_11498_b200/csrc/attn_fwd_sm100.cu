@@ -45,8 +45,15 @@ struct FwdCfg {
   static constexpr uint32_t kColO = 0, kColS = 256;
 };
 
+template <int NSEQ>
+struct FwdMaps { CUtensorMap q[NSEQ], k[NSEQ], v[NSEQ], kc[NSEQ], vc[NSEQ]; };
+
+template <int NSEQ>
 struct FwdArgs {
-  BlockPlan plan;          // blocks of up to 256 query rows (two tiles)
+  BlockPlan plan[NSEQ];    // blocks of up to 256 query rows (two tiles)
+  int tok0[NSEQ];          // first token of the sequence
+  int block0[NSEQ + 1];    // blocks of the sequences before, per (batch, head)
+  int n_seqs;
   int BH, Hq, Hkv, G, N;   // N: tokens per (batch, head) row of O and LSE (the row stride)
   __nv_bfloat16* O;
   __nv_bfloat16* Olo;        // optional: receives bf16(O_fp32 - O), the part of the output the bf16 O cannot hold
@@ -64,11 +71,9 @@ struct FwdBars {
   uint64_t p_full[2][kPParts];      // per query tile: the parts of P_t (128 / kPParts keys each) are stored
 };
 
-template <int D>
+template <int D, int NSEQ>
 __global__ void __launch_bounds__(FwdCfg<D>::kThreads, 1)
-lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapKc,
-                const __grid_constant__ CUtensorMap mapVc, const FwdArgs a) {
+lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constant__ FwdArgs<NSEQ> a) {
   using Cfg = FwdCfg<D>;
   constexpr int NS = Cfg::kStages;
   extern __shared__ unsigned char smem_raw[];
@@ -80,8 +85,14 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = smem0, sRing = smem0 + 2 * Cfg::kQRegion;
 
-  const int bh = blockIdx.x % a.BH, blk = blockIdx.x / a.BH;
-  const RowBlock rb = decode_block(a.plan, blk);
+  const int bh = blockIdx.x % a.BH;
+  int blk = blockIdx.x / a.BH, sq = 0;
+  if constexpr (NSEQ > 1) {
+    while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
+    blk -= a.block0[sq];
+  }
+  const RowBlock rb = decode_block(a.plan[sq], blk);
+  const size_t row0 = (size_t)bh * a.N + a.tok0[sq];   // the sequence's first row of O and LSE
   const int bh_kv = (bh / a.Hq) * a.Hkv + (bh % a.Hq) / a.G;
   const int n_ct = (rb.n_front + kTile - 1) / kTile;
   // key tiles of query tile t: the list, then the dense range up to the tile's last row (0: the tile is empty)
@@ -106,6 +117,8 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
   volatile int* abort = &abort_s;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // The softmax threads hold a row of 128 scores: they take the registers the other warps do not need
   // (128 x 72 + 256 x 216 = 384 x 168, what the CTA was launched with).
@@ -114,12 +127,12 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      prefetch_tensormap(&mapQ); prefetch_tensormap(&mapK); prefetch_tensormap(&mapV);
-      prefetch_tensormap(&mapKc); prefetch_tensormap(&mapVc);
+      prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.k[sq]); prefetch_tensormap(&maps.v[sq]);
+      prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
       mbar_expect_tx(smem_u32(&bars.q_full), (n1 > 0 ? 2 : 1) * Cfg::kTileBytes);
       for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)
         for (int h = 0; h < Cfg::kSub; ++h)
-          tma_load_3d(sQ + t * Cfg::kQRegion + h * Cfg::kSubBytes, &mapQ, h * 64, rb.q0 + t * kTile, bh, smem_u32(&bars.q_full));
+          tma_load_3d(sQ + t * Cfg::kQRegion + h * Cfg::kSubBytes, &maps.q[sq], h * 64, rb.q0 + t * kTile, bh, smem_u32(&bars.q_full));
       int it = 0;
       bool ok = true;
       for (int j = 0; j < n && ok; ++j) {
@@ -130,7 +143,7 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           const uint32_t full = smem_u32(&bars.kv_full[slot]);
           mbar_expect_tx(full, Cfg::kTileBytes);
           const bool compact = j < n_ct;
-          const CUtensorMap* map = compact ? (which ? &mapVc : &mapKc) : (which ? &mapV : &mapK);
+          const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
           const int row = compact ? j * kTile : rb.dense_start + (j - n_ct) * kTile;
           for (int h = 0; h < Cfg::kSub; ++h)
             tma_load_3d(sRing + slot * Cfg::kTileBytes + h * Cfg::kSubBytes, map, h * 64, row, bh_kv, full);
@@ -338,7 +351,7 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       const float inv = 1.0f / l;
       unsigned char* srow = stage_out + row * kStageStride;
       // the remainder goes straight to global memory (contiguous bytes per thread, written once)
-      __nv_bfloat16* lo_row = a.Olo && store ? a.Olo + ((size_t)bh * a.N + qpos) * D : nullptr;
+      __nv_bfloat16* lo_row = a.Olo && store ? a.Olo + (row0 + qpos) * D : nullptr;
 #pragma unroll
       for (int q = 0; q < D / 32; ++q) {
         uint32_t o[32];
@@ -363,10 +376,10 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           }
         }
       }
-      if (store) a.LSE[(size_t)bh * a.N + qpos] = m * a.scale + logf(l);
+      if (store) a.LSE[row0 + qpos] = m * a.scale + logf(l);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy reads this thread's stores
       if (store && !*abort) {
-        __nv_bfloat16* orow = a.O + ((size_t)bh * a.N + qpos) * D;
+        __nv_bfloat16* orow = a.O + (row0 + qpos) * D;
         asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(orow),
                      "r"(smem_u32(srow)), "r"((uint32_t)kRowBytes)
                      : "memory");
@@ -382,24 +395,11 @@ lrsa_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   if (tid == 0 && abort_s) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
 }
 
-// K, V point at the sequence's first token; `kept` entries are positions in the whole row (tok0 + local).
-__global__ void compact_kv_kernel(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
-                                  const int32_t* __restrict__ idx, __nv_bfloat16* __restrict__ Kc,
-                                  __nv_bfloat16* __restrict__ Vc, int BHkv, int Nrow, int d, int S, int Rc, int tok0,
-                                  int kept_stride, int kept_off) {
-  // one warp per compact row; a row is d*2 bytes = 8 (d=128) or 4 (d=64) bytes per lane
-  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (wid >= (long long)BHkv * Rc) return;
-  const int bh = (int)(wid / Rc), r = (int)(wid % Rc), lane = threadIdx.x & 31;
-  const int pos = r < S ? r : idx[(size_t)bh * kept_stride + kept_off + (r - S)] - tok0;
-  const size_t src = ((size_t)bh * Nrow + pos) * d, dst = ((size_t)bh * Rc + r) * d;
-  if (d == 128) {
-    reinterpret_cast<uint2*>(Kc + dst)[lane] = reinterpret_cast<const uint2*>(K + src)[lane];
-    reinterpret_cast<uint2*>(Vc + dst)[lane] = reinterpret_cast<const uint2*>(V + src)[lane];
-  } else {
-    reinterpret_cast<uint32_t*>(Kc + dst)[lane] = reinterpret_cast<const uint32_t*>(K + src)[lane];
-    reinterpret_cast<uint32_t*>(Vc + dst)[lane] = reinterpret_cast<const uint32_t*>(V + src)[lane];
-  }
+__global__ void __launch_bounds__(256) compact_kv_kernel(const __grid_constant__ CompactArgs c) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (c.status && blockIdx.x == 0 && threadIdx.x == 0) *c.status = 0;
+  compact_rows(c, blockIdx.x);
 }
 
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -421,7 +421,7 @@ struct FwdWs {
 };
 FwdWs fwd_ws_layout(const Geom& g) {
   FwdWs w;
-  const size_t rc = g.Rc > 0 ? g.Rc : 1;
+  const size_t rc = g.Rtot > 0 ? g.Rtot : 1;
   const size_t bytes = align_up((size_t)g.B * g.Hkv * rc * g.d * sizeof(__nv_bfloat16), 1024);
   w.kc = 1024;
   w.vc = w.kc + bytes;
@@ -459,47 +459,41 @@ int make_tmap_bf16_rows(CUtensorMap* map, const void* base, int d, long long row
   return r == CUDA_SUCCESS ? LRSA_OK : LRSA_ERR_CUDA;
 }
 
-int launch_compact_kv(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, const int32_t* idx,
-                      __nv_bfloat16* Kc, __nv_bfloat16* Vc, cudaStream_t st) {
-  if (g.Rc == 0) return LRSA_OK;
-  const long long warps = (long long)g.B * g.Hkv * g.Rc;
-  const unsigned blocks = (unsigned)((warps + 7) / 8);
-  const size_t sh = (size_t)g.tok0 * g.d;
-  compact_kv_kernel<<<blocks, 256, 0, st>>>(K + sh, V + sh, idx, Kc, Vc, g.B * g.Hkv, g.Nrow, g.d, g.S, g.Rc, g.tok0,
-                                            g.Wtot * g.K, g.woff * g.K);
-  LRSA_CUDA_CHECK(cudaGetLastError());
-  launch_counter().n++;
-  return LRSA_OK;
-}
-
 size_t attn_fwd_ws_bytes(const Geom& g) { return fwd_ws_layout(g).total; }
 
-template <int D>
-static int launch_fwd_t(const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K, const __nv_bfloat16* V,
-                        const __nv_bfloat16* Kc, const __nv_bfloat16* Vc, __nv_bfloat16* O, __nv_bfloat16* Olo, float* LSE,
-                        int* status, cudaStream_t st) {
+template <int D, int NSEQ>
+static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                        const __nv_bfloat16* V, const __nv_bfloat16* Kc, const __nv_bfloat16* Vc, __nv_bfloat16* O,
+                        __nv_bfloat16* Olo, float* LSE, int* status, cudaStream_t st) {
   using Cfg = FwdCfg<D>;
-  CUtensorMap mQ, mK, mV, mKc, mVc;
-  const long long rc = g.Rc > 0 ? g.Rc : 1;
-  // the sequence starts at token tok0 of rows of Nrow tokens: shifted bases, rows beyond its end read as zero
-  const size_t sh = (size_t)g.tok0 * D;
-  int rc_ = make_tmap_bf16(&mQ, Q + sh, D, g.N, (long long)g.B * g.Hq, kTile, g.Nrow);
-  if (rc_ == LRSA_OK) rc_ = make_tmap_bf16(&mK, K + sh, D, g.N, (long long)g.B * g.Hkv, kTile, g.Nrow);
-  if (rc_ == LRSA_OK) rc_ = make_tmap_bf16(&mV, V + sh, D, g.N, (long long)g.B * g.Hkv, kTile, g.Nrow);
-  if (rc_ == LRSA_OK) rc_ = make_tmap_bf16(&mKc, Kc, D, rc, (long long)g.B * g.Hkv, kTile);
-  if (rc_ == LRSA_OK) rc_ = make_tmap_bf16(&mVc, Vc, D, rc, (long long)g.B * g.Hkv, kTile);
-  if (rc_ != LRSA_OK) return rc_;
-  FwdArgs a;
-  a.plan = make_plan(g, 2 * kTile);
-  a.BH = g.B * g.Hq; a.Hq = g.Hq; a.Hkv = g.Hkv; a.G = g.G; a.N = g.Nrow;
-  a.O = O + sh; a.Olo = Olo ? Olo + sh : nullptr; a.LSE = LSE + g.tok0; a.scale = g.scale; a.scale_log2 = g.scale * 1.4426950408889634f;
+  FwdMaps<NSEQ> m;
+  FwdArgs<NSEQ> a;
+  const long long BHq = (long long)whole.B * whole.Hq, BHkv = (long long)whole.B * whole.Hkv;
+  a.block0[0] = 0;
+  for (int s = 0; s < b.n; ++s) {
+    const Geom& g = b.g[s];
+    const long long rc = g.Rc > 0 ? g.Rc : 1;
+    // the sequence starts at token tok0 of rows of Nrow tokens: shifted bases, rows beyond its end read as zero
+    const size_t sh = (size_t)g.tok0 * D, csh = g.Rc > 0 ? (size_t)b.row0[s] * D : 0;
+    int r = make_tmap_bf16(&m.q[s], Q + sh, D, g.N, BHq, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.k[s], K + sh, D, g.N, BHkv, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.v[s], V + sh, D, g.N, BHkv, kTile, g.Nrow);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.kc[s], Kc + csh, D, rc, BHkv, kTile);
+    if (r == LRSA_OK) r = make_tmap_bf16(&m.vc[s], Vc + csh, D, rc, BHkv, kTile);
+    if (r != LRSA_OK) return r;
+    a.plan[s] = make_plan(g, 2 * kTile);
+    a.tok0[s] = g.tok0;
+    a.block0[s + 1] = a.block0[s] + a.plan[s].total;
+  }
+  a.n_seqs = b.n;
+  a.BH = (int)BHq; a.Hq = whole.Hq; a.Hkv = whole.Hkv; a.G = whole.G; a.N = whole.Nrow;
+  a.O = O; a.Olo = Olo; a.LSE = LSE; a.scale = whole.scale; a.scale_log2 = whole.scale * 1.4426950408889634f;
   a.status = status;
-  const long long grid = (long long)a.plan.total * a.BH;
+  const long long grid = (long long)a.block0[b.n] * a.BH;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  auto kern = lrsa_fwd_kernel<D>;
+  auto kern = lrsa_fwd_kernel<D, NSEQ>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
-  kern<<<(unsigned)grid, Cfg::kThreads, Cfg::kSmem, st>>>(mQ, mK, mV, mKc, mVc, a);
-  LRSA_CUDA_CHECK(cudaGetLastError());
+  LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));
   launch_counter().n++;
   return LRSA_OK;
 }
@@ -509,23 +503,22 @@ int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
                           cudaStream_t st) {
   const FwdWs lay = fwd_ws_layout(g);
   unsigned char* base = static_cast<unsigned char*>(ws);
-  LRSA_CUDA_CHECK(cudaMemsetAsync(base, 0, sizeof(WsHeader), st));
-  launch_counter().n++;
   __nv_bfloat16* Kc = reinterpret_cast<__nv_bfloat16*>(base + lay.kc);
   __nv_bfloat16* Vc = reinterpret_cast<__nv_bfloat16*>(base + lay.vc);
   int* status = &reinterpret_cast<WsHeader*>(base)->status;
   __nv_bfloat16* Olo = static_cast<__nv_bfloat16*>(params->o_residual);
-  // sequence after sequence (one for an unpacked batch); the compact buffers are reused in stream order
-  const int n_seqs = geom_n_seqs(params);
-  int woff = 0;
-  for (int s = 0; s < n_seqs; ++s) {
-    Geom gs;
-    seq_geom(g, params->cu_seqlens, params->n_seqs, s, woff, &gs);
-    woff += gs.Wsel;
-    int rc = launch_compact_kv(gs, K, V, idx, Kc, Vc, st);
-    if (rc == LRSA_OK)
-      rc = gs.d == 128 ? launch_fwd_t<128>(gs, Q, K, V, Kc, Vc, O, Olo, LSE, status, st)
-                       : launch_fwd_t<64>(gs, Q, K, V, Kc, Vc, O, Olo, LSE, status, st);
+  SeqBatches batches(g);
+  SeqBatch b;
+  for (bool first = true; batches.next(&b); first = false) {
+    const CompactArgs c = compact_args(g, b, K, V, idx, Kc, Vc, first ? status : nullptr);
+    const int blocks = c.blocks();
+    if (blocks > 0 || first) {
+      LRSA_CUDA_CHECK(launch_dependent(compact_kv_kernel, dim3(blocks > 0 ? blocks : 1), dim3(256), 0, st, 1, c));
+      launch_counter().n++;
+    }
+    const auto fwd = g.d == 128 ? (b.n == 1 ? launch_fwd_t<128, 1> : launch_fwd_t<128, kMaxSeqs>)
+                                : (b.n == 1 ? launch_fwd_t<64, 1> : launch_fwd_t<64, kMaxSeqs>);
+    const int rc = fwd(g, b, Q, K, V, Kc, Vc, O, Olo, LSE, status, st);
     if (rc != LRSA_OK) return rc;
   }
   return LRSA_OK;

@@ -1,7 +1,7 @@
 // C ABI entry points: argument validation on the host, workspace layout, kernel dispatch.
 #include <math.h>
 
-#include "lrsa_internal.h"
+#include "attn_common_sm100.h"
 
 namespace lrsa {
 
@@ -42,21 +42,23 @@ int make_geom(const lrsa_params_t* p, Geom* g) {
   if (reinterpret_cast<uintptr_t>(p->o_residual) & 15u) return LRSA_ERR_INVALID_ARG;
   g->has_o_res = p->o_residual != nullptr;
   if (p->n_seqs < 0) return LRSA_ERR_INVALID_ARG;
+  g->cu = nullptr; g->n_seqs = 0; g->Rtot = g->Rc;
   if (p->n_seqs > 0) {
     if (!p->cu_seqlens || p->cu_seqlens[0] != 0 || p->cu_seqlens[p->n_seqs] != p->seq_len) return LRSA_ERR_INVALID_ARG;
-    int wtot = 0;
+    int wtot = 0, rtot = 0;
     for (int s = 0; s < p->n_seqs; ++s) {
       const int n = p->cu_seqlens[s + 1] - p->cu_seqlens[s];
       if (n < 1) return LRSA_ERR_INVALID_ARG;
       const int w = n > g->S ? (n - g->S) / g->L : 0;
       wtot += w > 1 ? w - 1 : 0;
+      rtot += (n < g->S ? n : g->S) + (w > 1 ? w - 1 : 0) * g->K;
     }
     g->Wtot = wtot;
+    g->Rtot = rtot;
+    g->cu = p->cu_seqlens; g->n_seqs = p->n_seqs;
   }
   return LRSA_OK;
 }
-
-int geom_n_seqs(const lrsa_params_t* p) { return p->n_seqs > 0 ? p->n_seqs : 1; }
 
 void seq_geom(const Geom& whole, const int32_t* cu, int n_seqs, int s, int woff, Geom* out) {
   *out = whole;
@@ -72,24 +74,42 @@ void seq_geom(const Geom& whole, const int32_t* cu, int n_seqs, int s, int woff,
   g.Wsel = g.W > 1 ? g.W - 1 : 0;
   g.Rc = g.S + g.Wsel * g.K;
   g.woff = woff;
+  g.cu = nullptr; g.n_seqs = 0; g.Rtot = g.Rc;
+}
+
+bool SeqBatches::next(SeqBatch* b) {
+  const int total = whole.n_seqs > 0 ? whole.n_seqs : 1;
+  b->n = 0;
+  for (; s < total && b->n < kMaxSeqs; ++s) {
+    Geom g;
+    seq_geom(whole, whole.cu, whole.n_seqs, s, woff, &g);
+    int at = b->n++;
+    for (; at > 0 && b->g[at - 1].N < g.N; --at) { b->g[at] = b->g[at - 1]; b->row0[at] = b->row0[at - 1]; }
+    b->g[at] = g;
+    b->row0[at] = row0;
+    woff += g.Wsel;
+    row0 += (long long)g.B * g.Hkv * g.Rc;
+  }
+  return b->n > 0;
 }
 
 int run_score_select(const lrsa_params_t* p, const Geom& whole, const __nv_bfloat16* K, const __nv_bfloat16* V,
                      int32_t* idx, float* score, void* ws, cudaStream_t st) {
-  const int n_seqs = geom_n_seqs(p);
-  // one sequence scored by the kernel that clears the status word itself: a single launch
-  const bool in_kernel = n_seqs == 1 && score_select_clears_status(whole);
+  // the first launch clears the status word when it can: a single launch then, but for very many sequences
+  const bool in_kernel = score_select_clears_status(whole);
   if (!in_kernel) {
     LRSA_CUDA_CHECK(cudaMemsetAsync(ws, 0, sizeof(WsHeader), st));
     launch_counter().n++;
   }
-  int woff = 0;
-  for (int s = 0; s < n_seqs; ++s) {
-    Geom g;
-    seq_geom(whole, p->cu_seqlens, p->n_seqs, s, woff, &g);
-    const int rc = launch_score_select(g, K, V, idx, score, ws, st, in_kernel);
+  SeqBatch b;
+  bool clear = in_kernel;
+  for (SeqBatches it(whole); it.next(&b);) {
+    int windows = 0;
+    for (int s = 0; s < b.n; ++s) windows += b.g[s].Wsel;
+    if (windows == 0) continue;
+    const int rc = launch_score_select(b.g, b.n, K, V, idx, score, ws, st, clear);
     if (rc != LRSA_OK) return rc;
-    woff += g.Wsel;
+    clear = false;
   }
   return LRSA_OK;
 }

@@ -526,7 +526,7 @@ int lrsa_cache_append(const lrsa_params_t* params, void* cache, size_t cache_byt
       launch_counter().n++;
     }
     cleared = true;
-    return launch_score_select(w, k, v, idx, nullptr, workspace, st, self);
+    return launch_score_select(&w, 1, k, v, idx, nullptr, workspace, st, self);
   };
   auto copy_rows = [&]() -> int {
     if (rows.n_sink + rows.n_ins + rows.n_keep == 0) return LRSA_OK;

@@ -30,13 +30,15 @@ struct Geom {
   // Scoring only: value added to the positions written to idx (tok0 unless the rows are a ring buffer)
   // and distance in tokens from window w to window w+1 (L unless the rows are a ring buffer).
   int emit_off, win_stride;
+  // Packed batches, host only: the boundaries (valid during the call) and number of sequences (0: one sequence).
+  const int32_t* cu;
+  int n_seqs;
+  int Rtot;        // rows of the compact buffers per KV head over all sequences (<= N)
   int has_o_res;   // the caller gave a buffer for the rounding remainder of O (lrsa_params_t::o_residual)
 };
 
 // Sequence s of a packed batch (cu = boundaries, n_seqs + 1 entries) as a Geom of its own.
 void seq_geom(const Geom& whole, const int32_t* cu, int n_seqs, int s, int woff, Geom* out);
-// Number of sequences and boundaries of `p` (a single sequence when it has no cu_seqlens).
-int geom_n_seqs(const lrsa_params_t* p);
 
 // Validates `p` and fills `g`. Returns an lrsa_status.
 int make_geom(const lrsa_params_t* p, Geom* g);
@@ -82,10 +84,11 @@ LaunchCounter& launch_counter();
 int run_score_select(const lrsa_params_t* p, const Geom& whole, const __nv_bfloat16* K, const __nv_bfloat16* V,
                      int32_t* idx, float* score, void* ws, cudaStream_t st);
 
-// score_select.cu (one sequence; the status header of `ws` is cleared by the caller)
+// score_select.cu : scores and selects the windows of n sequences of a packed row (or one sequence).  The status header of
+// `ws` is cleared by the caller, or (clear_status) by the kernel.
 size_t score_select_ws_bytes(const Geom& g);
-int launch_score_select(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx,
-                        float* score, void* ws, cudaStream_t st, bool clear_status = false);
+int launch_score_select(const Geom* gs, int n, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx,
+                        float* score, void* ws, cudaStream_t st, bool clear_status);
 // True when the kernel that scores `g` can clear the status word itself (clear_status above).
 bool score_select_clears_status(const Geom& g);
 void set_unit_wait_limit(int polls);
@@ -118,22 +121,6 @@ int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
                           const __nv_bfloat16* V, const __nv_bfloat16* O, const __nv_bfloat16* dO,
                           const float* LSE, const int32_t* idx, __nv_bfloat16* dQ, __nv_bfloat16* dK,
                           __nv_bfloat16* dV, void* ws, cudaStream_t st);
-// Backward helpers.  stats[row] = (-LSE * log2(e), rowsum(dO * O)) per query row; kbar[b*Hkv+h][c] is the
-// mean key (accumulated into a zeroed array).  The dK/dV kernel runs first and adds sum_j P dP, the
-// accurate D of every query row, into the zeroed Dacc; the dQ kernel reads it.
-int launch_bwd_prep(const Geom& g, const __nv_bfloat16* O, const __nv_bfloat16* Olo, const __nv_bfloat16* dO,
-                    const float* LSE, const __nv_bfloat16* K, float2* stats, float* kbar, cudaStream_t st);
-int launch_bwd_dq_sm100(const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* dO, const __nv_bfloat16* K,
-                        const __nv_bfloat16* V, const __nv_bfloat16* Kc, const __nv_bfloat16* Vc, const float2* stats,
-                        const float* Dacc, const float* kbar, __nv_bfloat16* dQ, int* status, cudaStream_t st);
-
-size_t dkv_ws_bytes(const Geom& g, size_t* prefix_bytes);
-int dkv_zero(const Geom& whole, void* ws_dkv, cudaStream_t st);
-int launch_bwd_dkv_sm100(const Geom& whole, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* dO,
-                         const __nv_bfloat16* K, const __nv_bfloat16* V, const float2* stats, float* Dacc,
-                         const int32_t* idx, void* ws_dkv, int* status, cudaStream_t st);
-int dkv_convert(const Geom& whole, void* ws_dkv, __nv_bfloat16* dK, __nv_bfloat16* dV, cudaStream_t st);
-
 // Launch (in clusters of `cluster` CTAs) that may start before the kernel in front of it has ended: the kernel itself waits
 // for that (griddepcontrol.wait) before it touches memory.
 template <typename... P, typename... A>

@@ -100,15 +100,17 @@ __host__ __device__ inline size_t select_scratch_bytes(int L) {
 __device__ __forceinline__ void scoring_warps_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // `in_smem`: the spreads are already in sk / sv (the cluster kernel keeps them there) instead of in a.spread.
-__device__ void select_window(const ScoreArgs& a, int bh, int w, unsigned char* smem, bool in_smem = false) {
+// `wi`: the window's place among all windows of idx and score; `pos0`: position of its first token; `gk`: its spreads in global
+// memory otherwise.
+__device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsigned char* smem, bool in_smem,
+                              const float* gk = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L;
   float* sk = reinterpret_cast<float*>(smem);
   float* sv = sk + L;
   uint32_t* hist = reinterpret_cast<uint32_t*>(sv + L);  // 256 bins
   float* red = reinterpret_cast<float*>(hist + 256);     // 32 floats
   int* ibuf = reinterpret_cast<int*>(red + 32);          // 16 ints
-  const float* gk = in_smem ? sk : a.spread + ((size_t)(bh * a.Wsel + w) * 2 + 0) * L;
-  const float* gv = in_smem ? sv : gk + L;
+  const float* gv = gk + L;
 
   // Eq. 7: softmax over the L tokens of the window, for K and for V
   float mk = -INFINITY, mv = -INFINITY;
@@ -137,7 +139,7 @@ __device__ void select_window(const ScoreArgs& a, int bh, int w, unsigned char* 
 #pragma unroll
   for (int i = 0; i < 8; ++i) { ek += red[i]; ev += red[8 + i]; }
   // Eq. 8
-  float* gs = a.score ? a.score + (size_t)(bh * a.Wtot + a.woff + w) * L : nullptr;
+  float* gs = a.score ? a.score + (size_t)(bh * a.Wtot + wi) * L : nullptr;
   uint32_t kmin = 0xffffffffu, kmax = 0u;   // range of the keys (scores are positive: bit order = value order)
   for (int i = tid; i < L; i += kThreads) {
     const float s = sk[i] / ek + sv[i] / ev;
@@ -212,8 +214,7 @@ __device__ void select_window(const ScoreArgs& a, int bh, int w, unsigned char* 
 
   // emit kept positions in ascending order: every thread takes a run of consecutive tokens, one block
   // scan gives the number of kept tokens before the run
-  int32_t* out = a.idx + (size_t)(bh * a.Wtot + a.woff + w) * a.Kk;
-  const int pos0 = a.emit_off + a.S + w * L;   // position of the window's first token
+  int32_t* out = a.idx + (size_t)(bh * a.Wtot + wi) * a.Kk;
   const int per = (L + kThreads - 1) / kThreads;
   const int i_lo = min(L, tid * per), i_hi = min(L, i_lo + per);
   int packed = 0;   // tokens above the K-th score | tokens equal to it << 16
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(kThreads) score_select_kernel(const ScoreArgs 
   __syncthreads();
   if (s_flag != 2) return;
   __threadfence();
-  select_window(a, bh, w, smem);
+  select_window(a, bh, a.woff + w, a.emit_off + a.S + w * a.L, smem, false, a.spread + (size_t)(bh * a.Wsel + w) * 2 * a.L);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -438,8 +439,18 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Where the sequences of a launch lie (up to kScoreSeqs of a packed row; the windows of all of them have the same length).
+constexpr int kScoreSeqs = 16;
+struct ScoreSeqs {
+  int n;
+  int item0[kScoreSeqs + 1];    // clusters of the sequences before
+  int runs[kScoreSeqs], Wsel[kScoreSeqs], first[kScoreSeqs];   // runs per (batch, KV head); scored windows; token of window 0
+  int woff[kScoreSeqs], emit0[kScoreSeqs];                     // first window in idx and score; position of window 0
+};
+
 template <int D, bool FOLD>
-__global__ void __launch_bounds__(kThreads, 2) score_select_cluster_kernel(const ScoreArgs a, int run, int runs_per_bh, int C) {
+__global__ void __launch_bounds__(kThreads, 2)
+score_select_cluster_kernel(const __grid_constant__ ScoreArgs a, const __grid_constant__ ScoreSeqs seqs, int run, int C) {
   constexpr int KC = D / 32;              // 16-byte chunks per lane and row
   constexpr int T = FOLD ? 2 : 4;         // groups of eight tokens in flight
   constexpr int kStatBytes = 4 * D * 2;   // [K, V][min, max][D] bf16
@@ -457,12 +468,15 @@ __global__ void __launch_bounds__(kThreads, 2) score_select_cluster_kernel(const
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (a.clear_status && blockIdx.x == 0 && tid == 0) a.hdr->status = 0;
-  const int item = blockIdx.x / C, rank = blockIdx.x % C;
-  const int bh = item / runs_per_bh, seg = item % runs_per_bh;
-  const int w_a = seg * run, w_b = min(a.Wsel, w_a + run);   // scored windows [w_a, w_b); reference w_b <= W-1
+  const int rank = blockIdx.x % C;
+  int item = blockIdx.x / C, sq = 0;
+  while (sq + 1 < seqs.n && item >= seqs.item0[sq + 1]) ++sq;
+  item -= seqs.item0[sq];
+  const int bh = item / seqs.runs[sq], seg = item % seqs.runs[sq];
+  const int w_a = seg * run, w_b = min(seqs.Wsel[sq], w_a + run);   // scored windows [w_a, w_b); reference w_b <= W-1
   const int per = (a.L + C - 1) / C;
   const int i0 = min(a.L, rank * per), i1 = min(a.L, i0 + per);   // this CTA's tokens of every window
-  const __nv_bfloat16* base = (z == 0 ? a.K : a.V) + ((long long)bh * a.N + a.tok0 + a.S) * D;
+  const __nv_bfloat16* base = (z == 0 ? a.K : a.V) + ((long long)bh * a.N + seqs.first[sq]) * D;
   const float inv_dof = 1.0f / (float)(D - a.ddof);
 
   const int first = i0 + wz * 8 * T;   // this warp's first token
@@ -612,7 +626,8 @@ __global__ void __launch_bounds__(kThreads, 2) score_select_cluster_kernel(const
         sasb[((zz * KC + (chunk >> 2)) * 4 + p) * 4 + (chunk & 3)] = make_float4(f[0], f[1], f[2], f[3]);
       }
     }
-    if (scoring && rank == sel_rank) select_window(a, bh, w, sel + buf * sel_bytes, true);
+    if (scoring && rank == sel_rank)
+      select_window(a, bh, seqs.woff[sq] + w, seqs.emit0[sq] + w * a.L, sel + buf * sel_bytes, true);
     __syncthreads();   // scale and offset are in place for the next window
   }
 }
@@ -676,30 +691,74 @@ size_t score_select_ws_bytes(const Geom& g) { return g.L <= kClusterMaxL ? sizeo
 
 void set_unit_wait_limit(int polls) { g_unit_wait_limit = polls; }
 
-bool score_select_clears_status(const Geom& g) { return g.Wsel > 0 && g.L <= kClusterMaxL; }
+bool score_select_clears_status(const Geom& g) { return (g.n_seqs > 0 ? g.Wtot : g.Wsel) > 0 && g.L <= kClusterMaxL; }
 
-int launch_score_select(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx,
-                        float* score, void* ws, cudaStream_t st, bool clear_status) {
+static ScoreArgs score_args(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx, float* score, void* ws) {
+  unsigned char* base = static_cast<unsigned char*>(ws);
+  ScoreArgs a = {};
+  a.K = K; a.V = V; a.idx = idx; a.score = score;
+  a.hdr = reinterpret_cast<WsHeader*>(base);
+  a.BH = g.B * g.Hkv; a.N = g.Nrow; a.L = g.L; a.Kk = g.K; a.S = g.S; a.W = g.W; a.Wsel = g.Wsel;
+  a.tok0 = g.tok0; a.Wtot = g.Wtot; a.woff = g.woff; a.emit_off = g.emit_off; a.win_stride = g.win_stride;
+  a.ddof = g.ddof;
+  return a;
+}
+
+static int launch_cluster(const Geom* gs, int n_seqs, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx, float* score,
+                          void* ws, cudaStream_t st, bool clear_status) {
+  for (int s0 = 0; s0 < n_seqs;) {
+    // the next sequences with anything to score
+    ScoreSeqs q;
+    q.n = 0;
+    int windows = 0, s1 = s0;
+    for (; s1 < n_seqs && q.n < kScoreSeqs; ++s1)
+      if (gs[s1].Wsel > 0) { ++q.n; windows += gs[s1].Wsel; }
+    if (q.n == 0) return LRSA_OK;
+    const Geom& g = gs[s0];
+    ScoreArgs a = score_args(g, K, V, idx, score, ws);
+    a.clear_status = clear_status ? 1 : 0;
+    const ClusterPlan pl = cluster_plan(a.BH, windows, g.L);
+    q.n = 0;
+    q.item0[0] = 0;
+    for (int s = s0; s < s1; ++s) {
+      const Geom& e = gs[s];
+      if (e.Wsel == 0) continue;
+      q.runs[q.n] = (e.Wsel + pl.run - 1) / pl.run;
+      q.Wsel[q.n] = e.Wsel;
+      q.first[q.n] = e.tok0 + e.S;
+      q.woff[q.n] = e.woff;
+      q.emit0[q.n] = e.emit_off + e.S;
+      q.item0[q.n + 1] = q.item0[q.n] + a.BH * q.runs[q.n];
+      ++q.n;
+    }
+    const long long grid = (long long)q.item0[q.n] * pl.C;
+    if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
+    const size_t bytes = (size_t)g.d * 16 + 2 * (4 * g.d * 2) + 8 * 2 * g.d * 2 + 2 * select_scratch_bytes(g.L);
+    auto kern = g.d == 128 ? (pl.run > 1 ? score_select_cluster_kernel<128, true> : score_select_cluster_kernel<128, false>)
+                           : (pl.run > 1 ? score_select_cluster_kernel<64, true> : score_select_cluster_kernel<64, false>);
+    if (bytes > 48 * 1024)
+      LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(kThreads), bytes, st, pl.C, a, q, pl.run, pl.C));
+    launch_counter().n++;
+    clear_status = false;
+    s0 = s1;
+  }
+  return LRSA_OK;
+}
+
+static int launch_unit(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx, float* score, void* ws,
+                       cudaStream_t st) {
   if (g.Wsel == 0) return LRSA_OK;  // nothing is scored
   const ScoreWs lay = score_ws_layout(g);
   unsigned char* base = static_cast<unsigned char*>(ws);
-  // The status word (the header) is cleared once per call by the caller.  The cluster kernel keeps everything
-  // else on chip; the one-slice-per-CTA kernel needs its ticket, counters and statistics at zero.
-  if (g.L > kClusterMaxL) {
-    LRSA_CUDA_CHECK(cudaMemsetAsync(base + offsetof(WsHeader, ticket), 0, lay.zero_bytes - offsetof(WsHeader, ticket), st));
-    launch_counter().n++;
-  }
-  ScoreArgs a;
-  a.K = K; a.V = V; a.idx = idx; a.score = score;
-  a.hdr = reinterpret_cast<WsHeader*>(base);
+  // The status word (the header) is cleared once per call by the caller; the ticket, the counters and the statistics here.
+  LRSA_CUDA_CHECK(cudaMemsetAsync(base + offsetof(WsHeader, ticket), 0, lay.zero_bytes - offsetof(WsHeader, ticket), st));
+  launch_counter().n++;
+  ScoreArgs a = score_args(g, K, V, idx, score, ws);
   a.ready = reinterpret_cast<int*>(base + lay.ready);
   a.done = reinterpret_cast<int*>(base + lay.done);
   a.mm = reinterpret_cast<uint32_t*>(base + lay.mm);
   a.spread = reinterpret_cast<float*>(base + lay.spread);
-  a.BH = g.B * g.Hkv; a.N = g.Nrow; a.L = g.L; a.Kk = g.K; a.S = g.S; a.W = g.W; a.Wsel = g.Wsel;
-  a.tok0 = g.tok0; a.Wtot = g.Wtot; a.woff = g.woff; a.emit_off = g.emit_off; a.win_stride = g.win_stride;
-  a.ddof = g.ddof;
-  a.clear_status = clear_status && score_select_clears_status(g) ? 1 : 0;
   a.unit_wait_limit = g_unit_wait_limit;
   const int tok = g.d == 128 ? tok_per_unit<128>() : tok_per_unit<64>();
   a.n_slices = (g.L + tok - 1) / tok;
@@ -707,25 +766,22 @@ int launch_score_select(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat
   if (smem > 200 * 1024) return LRSA_ERR_UNSUPPORTED;
   const long long units = (long long)a.BH * g.W * a.n_slices;
   if (units > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  if (g.L <= kClusterMaxL) {
-    const ClusterPlan pl = cluster_plan(a.BH, g.Wsel, g.L);
-    const size_t bytes = (size_t)g.d * 16 + 2 * (4 * g.d * 2) + 8 * 2 * g.d * 2 + 2 * select_scratch_bytes(g.L);
-    auto kern = g.d == 128 ? (pl.run > 1 ? score_select_cluster_kernel<128, true> : score_select_cluster_kernel<128, false>)
-                           : (pl.run > 1 ? score_select_cluster_kernel<64, true> : score_select_cluster_kernel<64, false>);
-    if (bytes > 48 * 1024)
-      LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    const int runs_per_bh = (g.Wsel + pl.run - 1) / pl.run;
-    const long long grid = (long long)a.BH * runs_per_bh * pl.C;
-    if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-    LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(kThreads), bytes, st, pl.C, a, pl.run, runs_per_bh, pl.C));
-    launch_counter().n++;
-    return LRSA_OK;
-  }
   auto kern = g.d == 128 ? score_select_kernel<128> : score_select_kernel<64>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<(unsigned)units, kThreads, smem, st>>>(a);
   LRSA_CUDA_CHECK(cudaGetLastError());
   launch_counter().n++;
+  return LRSA_OK;
+}
+
+int launch_score_select(const Geom* gs, int n_seqs, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx,
+                        float* score, void* ws, cudaStream_t st, bool clear_status) {
+  const Geom& g = gs[0];   // the shape is the same for all; windows and places differ
+  if (g.L <= kClusterMaxL) return launch_cluster(gs, n_seqs, K, V, idx, score, ws, st, clear_status);
+  for (int s = 0; s < n_seqs; ++s) {
+    const int rc = launch_unit(gs[s], K, V, idx, score, ws, st);
+    if (rc != LRSA_OK) return rc;
+  }
   return LRSA_OK;
 }
 

@@ -205,6 +205,9 @@ PACKED_CASES = [
     (W("p_three64", 2, 4, 4, 1200, 64, 64, 16, 16, seed=52), (0, 16 + 8 * 64, 16 + 8 * 64 + 10, 1200), 1),  # T = 0; shorter than S
     (W("p_gqa7", 1, 7, 1, 1000, 128, 100, 30, 3, seed=53, values="channel_offset"), (0, 333, 334, 1000), 1),  # one-token sequence
     (W("p_ndp0", 1, 2, 2, 900, 64, 128, 32, 4, seed=54), (0, 500, 900), 0),
+    # more sequences than one launch takes (16): two batches, the last of one sequence
+    (W("p_17", 1, 2, 1, 1700, 128, 32, 8, 4, seed=55), (0, 90, 93, *range(200, 1600, 100), 1700), 1),
+    (W("p_20", 2, 2, 2, 1300, 64, 24, 5, 2, seed=56), (0, *range(17, 1000, 53), 1300), 1),
 ]
 
 
