@@ -511,29 +511,38 @@ score_select_cluster_kernel(const __grid_constant__ ScoreArgs a, const __grid_co
       }
       if (scoring) {
         // Eq. 6 with the statistics of window w+1 (z' = x*sa + sb = zbar - 1/2), sums for the Std of Eq. 7
-        uint64_t sum2[T], sq2[T];
+        // The sums are formed chunk by chunk (eight channels) and the chunks added in a tree over the distances 8, 4, 2, 1,
+        // whatever the layout: a score that ties with the K-th one falls on the same side in every version of this kernel.
+        float v[T][2], first2[T][2];
 #pragma unroll
-        for (int s = 0; s < T; ++s) sum2[s] = sq2[s] = 0ull;   // (+0, +0)
+        for (int k = 0; k < KC; ++k) {
+          const int j = KC == 4 ? (k & 1) * 2 + (k >> 1) : k;   // 0, 2, 1, 3
+          uint64_t sum2[T], sq2[T];
 #pragma unroll
-        for (int j = 0; j < KC; ++j)
+          for (int s = 0; s < T; ++s) sum2[s] = sq2[s] = 0ull;   // (+0, +0)
 #pragma unroll
           for (int p = 0; p < 4; ++p) {
             const float4 f = sasb[((z * KC + j) * 4 + p) * 4 + t];
             const uint64_t sa = ptx::f2_pack(f.x, f.y), sb = ptx::f2_pack(f.z, f.w);
 #pragma unroll
             for (int s = 0; s < T; ++s) {
-              const uint32_t v = p == 0 ? x[s][j].x : p == 1 ? x[s][j].y : p == 2 ? x[s][j].z : x[s][j].w;
-              const uint64_t z2 = ptx::f2_fma(ptx::f2_pack(bf_lo(v), bf_hi(v)), sa, sb);
+              const uint32_t u = p == 0 ? x[s][j].x : p == 1 ? x[s][j].y : p == 2 ? x[s][j].z : x[s][j].w;
+              const uint64_t z2 = ptx::f2_fma(ptx::f2_pack(bf_lo(u), bf_hi(u)), sa, sb);
               sum2[s] = ptx::f2_add(sum2[s], z2);
               sq2[s] = ptx::f2_fma(z2, z2, sq2[s]);
             }
           }
-        float v[T][2];
 #pragma unroll
-        for (int s = 0; s < T; ++s) {
-          float x0, x1;
-          ptx::f2_unpack(sum2[s], x0, x1); v[s][0] = x0 + x1;
-          ptx::f2_unpack(sq2[s], x0, x1); v[s][1] = x0 + x1;
+          for (int s = 0; s < T; ++s) {
+            float x0, x1, y0, y1;
+            ptx::f2_unpack(sum2[s], x0, x1);
+            ptx::f2_unpack(sq2[s], y0, y1);
+            const float a0 = x0 + x1, a1 = y0 + y1;
+            if (k == 0) { v[s][0] = a0; v[s][1] = a1; }
+            else if (k == 1) { v[s][0] += a0; v[s][1] += a1; }
+            else if (k == 2) { first2[s][0] = a0; first2[s][1] = a1; }
+            else { v[s][0] += first2[s][0] + a0; v[s][1] += first2[s][1] + a1; }
+          }
         }
         // Sum over the four lanes of a row, halving: a lane hands half of its rows to its partner at each level
         int mine = 0;   // row this lane ends up with
