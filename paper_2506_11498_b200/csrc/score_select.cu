@@ -89,10 +89,10 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // Top-K of the window by the last CTA to finish it.  smem: sk[L], sv[L] floats, then scratch.
-// Bytes of the selection scratch: sk[L], sv[L], 256 histogram bins, 32 floats, 16 ints.
+// Bytes of the selection scratch: sk[L], sv[L] (rounded up to 16 bytes), two histograms of 256 bins, 32 floats, 16 + 8 words.
 // Rounded up to 16 bytes: the cluster kernel has two of them one behind the other.
 __host__ __device__ inline size_t select_scratch_bytes(int L) {
-  return (((size_t)2 * L * 4 + 256 * 4 + 32 * 4 + 16 * 4) + 15) & ~(size_t)15;
+  return (((size_t)2 * L * 4 + 15) & ~(size_t)15) + 2 * 256 * 4 + 32 * 4 + 16 * 4 + 8 * 4;
 }
 
 // Barrier of the 256 scoring threads (named barrier 1): the whole block in the one-unit-per-CTA kernel,
@@ -107,10 +107,12 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L;
   float* sk = reinterpret_cast<float*>(smem);
   float* sv = sk + L;
-  uint32_t* hist = reinterpret_cast<uint32_t*>(sv + L);  // 256 bins
-  float* red = reinterpret_cast<float*>(hist + 256);     // 32 floats
-  int* ibuf = reinterpret_cast<int*>(red + 32);          // 16 ints
+  uint32_t* hist = reinterpret_cast<uint32_t*>(smem + (((size_t)2 * L * 4 + 15) & ~(size_t)15));   // two of 256 bins
+  float* red = reinterpret_cast<float*>(hist + 512);            // [maxima of K, V][sums of K, V] of the eight warps
+  uint32_t* kred = reinterpret_cast<uint32_t*>(red + 32);       // [least, largest key] of the eight warps
+  int* wtot = reinterpret_cast<int*>(kred + 16);                // kept keys of the eight warps
   const float* gv = gk + L;
+  hist[tid] = hist[256 + tid] = 0;
 
   // Eq. 7: softmax over the L tokens of the window, for K and for V
   float mk = -INFINITY, mv = -INFINITY;
@@ -125,7 +127,6 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
   mk = red[0]; mv = red[8];
 #pragma unroll
   for (int i = 1; i < 8; ++i) { mk = fmaxf(mk, red[i]); mv = fmaxf(mv, red[8 + i]); }
-  scoring_warps_sync();
   float ek = 0.f, ev = 0.f;
   for (int i = tid; i < L; i += kThreads) {
     const float x = expf(sk[i] - mk), y = expf(sv[i] - mv);
@@ -133,11 +134,11 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
     ek += x; ev += y;
   }
   ek = warp_sum(ek); ev = warp_sum(ev);
-  if (lane == 0) { red[warp] = ek; red[8 + warp] = ev; }
+  if (lane == 0) { red[16 + warp] = ek; red[24 + warp] = ev; }
   scoring_warps_sync();
   ek = 0.f; ev = 0.f;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) { ek += red[i]; ev += red[8 + i]; }
+  for (int i = 0; i < 8; ++i) { ek += red[16 + i]; ev += red[24 + i]; }
   // Eq. 8
   float* gs = a.score ? a.score + (size_t)(bh * a.Wtot + wi) * L : nullptr;
   uint32_t kmin = 0xffffffffu, kmax = 0u;   // range of the keys (scores are positive: bit order = value order)
@@ -150,8 +151,6 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
   }
   kmin = __reduce_min_sync(0xffffffffu, kmin);
   kmax = __reduce_max_sync(0xffffffffu, kmax);
-  scoring_warps_sync();   // also: every read of red[] above is done
-  uint32_t* kred = reinterpret_cast<uint32_t*>(red);
   if (lane == 0) { kred[warp] = kmin; kred[8 + warp] = kmax; }
   scoring_warps_sync();
 #pragma unroll
@@ -169,45 +168,52 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
   if (top < 0) mask = 0xffffffffu;
   uint32_t prefix = kmax & mask;
   int remaining = a.Kk;
-  for (int shift = top < 0 ? -1 : max(top - 7, 0); shift >= 0; shift = shift == 0 ? -1 : max(shift - 8, 0)) {
-    hist[tid] = 0;
-    scoring_warps_sync();
+  // One barrier per pass: every warp finds the bin of the K-th key itself, and the histograms take turns.  (With one warp
+  // searching and four barriers a pass a call took 28.9 us instead of 27.4 at 32K tokens in windows of 1024.)
+  int pass = 0;
+  for (int shift = top < 0 ? -1 : max(top - 7, 0); shift >= 0; shift = shift == 0 ? -1 : max(shift - 8, 0), ++pass) {
+    uint32_t* h = hist + (pass & 1) * 256;
     for (int i = tid; i < L; i += kThreads) {
       const uint32_t k = key[i];
-      if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
+      if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
     }
     scoring_warps_sync();
-    if (warp == 0) {
-      // lane l owns bins 255-8l ... 248-8l, highest first
-      uint32_t c[8], tot = 0;
+    // lane l owns bins 255-8l ... 248-8l, highest first
+    const uint4 hi = *reinterpret_cast<const uint4*>(h + 252 - 8 * lane), lo = *reinterpret_cast<const uint4*>(h + 248 - 8 * lane);
+    const uint32_t c[8] = {hi.w, hi.z, hi.y, hi.x, lo.w, lo.z, lo.y, lo.x};
+    uint32_t tot = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { c[j] = hist[255 - 8 * lane - j]; tot += c[j]; }
-      uint32_t incl = tot;
+    for (int e = 0; e < 8; ++e) tot += c[e];
+    uint32_t incl = tot;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
-      }
-      uint32_t above = incl - tot;  // elements in bins above this lane's
-      if (above < (uint32_t)remaining && (uint32_t)remaining <= incl) {
-        int j = 0;
-        while (above + c[j] < (uint32_t)remaining) { above += c[j]; ++j; }
-        ibuf[0] = 255 - 8 * lane - j;
-        ibuf[1] = remaining - (int)above;
-        ibuf[2] = (int)c[j];   // keys in the chosen bin
-      }
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += n;
     }
-    scoring_warps_sync();
-    prefix |= (uint32_t)ibuf[0] << shift;
+    uint32_t above = incl - tot;   // elements in bins above this lane's
+    const bool mine = above < (uint32_t)remaining && (uint32_t)remaining <= incl;
+    uint32_t bin = 255 - 8 * lane, cnt = c[0];
+    bool more = true;
+#pragma unroll
+    for (int e = 0; e < 7; ++e) {
+      more = more && above + c[e] < (uint32_t)remaining;
+      if (more) { above += c[e]; --bin; cnt = c[e + 1]; }
+    }
+    const int src = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+    bin = __shfl_sync(0xffffffffu, bin, src);
+    cnt = __shfl_sync(0xffffffffu, cnt, src);              // keys in the chosen bin
+    remaining -= (int)__shfl_sync(0xffffffffu, above, src);
+    prefix |= bin << shift;
     mask |= 255u << shift;
-    remaining = ibuf[1];
     // Every key of the chosen bin is kept: the remaining bits need not be resolved.  (With 8-bit digits a
     // thousand keys are alone in their bin after two passes, so this ends the search at half its length.)
     // The threshold is then the bin's lowest possible key: keys above it are kept as "greater", keys equal to
     // it as "equal", of which `remaining` is at least as many as exist.
-    const bool whole_bin = ibuf[2] == remaining;
-    scoring_warps_sync();
-    if (whole_bin) break;
+    if ((int)cnt == remaining) break;
+    if (pass > 0) {   // a third pass needs the first histogram again (windows of keys that differ in their last bits only)
+      hist[((pass + 1) & 1) * 256 + tid] = 0;
+      scoring_warps_sync();
+    }
   }
   const uint32_t kth = prefix;    // K-th largest key
   const int need_eq = remaining;  // how many keys equal to it are kept (lowest positions first)
@@ -228,7 +234,6 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
     const int n = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += n;
   }
-  int* wtot = ibuf;  // 8 warp totals (ibuf's last readers passed the barrier that ended the last pass)
   if (lane == 31) wtot[warp] = incl;
   scoring_warps_sync();
   int excl = incl - packed;
@@ -246,7 +251,7 @@ __device__ void select_window(const ScoreArgs& a, int bh, int wi, int pos0, unsi
       ++eq_before;
     }
   }
-  scoring_warps_sync();   // sk and ibuf may be reused by the caller
+  scoring_warps_sync();   // the scratch may be reused by the caller
 }
 
 template <int D>
@@ -423,9 +428,9 @@ __global__ void __launch_bounds__(kThreads) score_select_kernel(const ScoreArgs 
 // the sum over a token's channels ends with two shuffle levels.  A row per 16 lanes with scale and offset in registers,
 // the layout of the kernel this one replaces, spent twice the instructions (12 per channel pair, 6 here) on exchanges, and
 // one CTA per window left most of the GPU idle when there were few.  4 KV heads, d = 128: 32K tokens in windows of 1024
-// 35.9 -> 27.7 us a call (2.4 TB/s of algorithmic bytes; every window is read twice, the second time from L2), 64K of 2048
-// 61.6 -> 49, 1777 tokens of 512 20.5 -> 9.9; 8 KV heads, 128K of 4096 184 -> 161.  What is left is a chain: two streams
-// of at most 16 warps' loads an SM, the exchange, the selection (about 4 us).
+// 35.9 -> 27.4 us a call (2.4 TB/s of algorithmic bytes; every window is read twice, the second time from L2), 64K of 2048
+// 61.6 -> 49, 1777 tokens of 512 20.5 -> 10.1; 8 KV heads, 128K of 4096 184 -> 160.  What is left is a chain: two streams
+// of at most 16 warps' loads an SM, the exchange, the selection (about 3 us).
 constexpr int kClusterMaxL = 4096;
 constexpr int kClusterMax = 8;
 
@@ -646,7 +651,7 @@ constexpr int tok_per_unit() { return kSteps * (kThreads / (D / 8)); }
 
 size_t select_smem_bytes(int L, int d) {
   const size_t phase1 = (size_t)(kThreads / 32) * 4 * d * sizeof(__nv_bfloat16);
-  const size_t sel = (size_t)2 * L * sizeof(float) + 256 * 4 + 32 * 4 + 16 * 4;
+  const size_t sel = select_scratch_bytes(L);
   return phase1 > sel ? phase1 : sel;
 }
 

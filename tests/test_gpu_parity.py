@@ -348,3 +348,21 @@ def test_outputs_never_written_outside_their_tensors(w):
                                ("dQ", bQ, dQ, 777.0), ("dK", bK, dK, 777.0), ("dV", bV, dV, 777.0)):
         assert _margins_intact(buf, t.numel(), fill), f"{name}: a margin was written"
         assert not (t == fill).any(), f"{name}: an element was left unwritten"
+
+
+@pytest.mark.parametrize("L,K,n_win", [(4096, 1000, 6), (1024, 1024, 5), (333, 1, 9), (8, 3, 40)])
+@pytest.mark.parametrize("values", ["normal", "few"])
+def test_selection_of_the_returned_scores(L, K, n_win, values):
+    """The kept positions are exactly the top_k of the returned scores, equal scores to the lower position: windows whose
+    keys need one to four digits of the search ("few": rows from a set of seven, so that most scores tie)."""
+    w = W("sel", 2, 2, 2, 5 + n_win * L + 3, 64, L, K, 5, seed=61)
+    g = torch.Generator(device="cuda").manual_seed(L + K)
+    kv = [torch.randn((w.B, w.Hkv, w.N, w.d), generator=g, device="cuda").bfloat16() for _ in range(2)]
+    if values == "few":
+        pick = torch.randint(0, 7, (w.N,), generator=g, device="cuda")
+        kv = [t[:, :, pick].contiguous() for t in kv]
+    p = lrsa.Params.from_workload(w)
+    idx, sc = lrsa.lrsa_score_select(p, kv[0], kv[1], want_score=True)
+    order = torch.argsort(sc, dim=-1, descending=True, stable=True)[..., :K].sort(-1).values
+    base = w.S + torch.arange(n_win - 1, device="cuda").view(1, 1, -1, 1) * L
+    assert torch.equal(idx.long(), order + base)
