@@ -4,10 +4,12 @@ from __future__ import annotations
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "liblrsa.so")
+CALL = os.path.join(_HERE, "_lrsa_call.so")   # Python module over two of the library's calls
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
 
@@ -17,9 +19,9 @@ def sources():
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + \
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.c")) + \
         glob.glob(os.path.join(_HERE, "..", "include", "*.h"))
     return any(os.path.getmtime(f) > os.path.getmtime(LIB) for f in deps)
 
@@ -29,6 +31,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
         subprocess.check_call(cmd)
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                               "-o", CALL, os.path.join(CSRC, "pycall.c"), "-L", _HERE, "-l:liblrsa.so",
+                               "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 

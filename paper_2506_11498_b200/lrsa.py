@@ -7,6 +7,7 @@ the import of any entry point raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -14,6 +15,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblrsa.so")
+CALL_PATH = os.path.join(_HERE, "_lrsa_call.so")
 
 STATUS = {0: "LRSA_OK", 1: "LRSA_ERR_INVALID_ARG", 2: "LRSA_ERR_UNSUPPORTED",
           3: "LRSA_ERR_WORKSPACE_TOO_SMALL", 4: "LRSA_ERR_CUDA", 5: "LRSA_ERR_TIMEOUT"}
@@ -75,8 +77,16 @@ class Params:
             object.__setattr__(self, "_ref", r)
         return r
 
+    def address(self) -> int:
+        """The same struct's address."""
+        a = self.__dict__.get("_address")
+        if a is None:
+            a = ctypes.cast(self.ref(), ctypes.c_void_p).value
+            object.__setattr__(self, "_address", a)
+        return a
+
     def __getstate__(self):
-        return {k: v for k, v in self.__dict__.items() if k != "_ref"}
+        return {k: v for k, v in self.__dict__.items() if k not in ("_ref", "_address")}
 
     @staticmethod
     def from_workload(w, **kw) -> "Params":
@@ -84,11 +94,12 @@ class Params:
 
 
 _lib = None
+_call = None   # the module of csrc/pycall.c: the two calls of a generated token without ctypes
 
 
 def lib() -> ctypes.CDLL:
     """Loads the CUDA library; raises if it has not been built."""
-    global _lib
+    global _lib, _call
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(f"{LIB_PATH} is missing: run `python -c 'import __graft_entry__ as g; g.build()'` "
@@ -122,6 +133,12 @@ def lib() -> ctypes.CDLL:
         for name in ("lrsa_num_sel_windows", "lrsa_workspace_bytes", "lrsa_score_select", "lrsa_attn_fwd",
                      "lrsa_attn_bwd", "lrsa_workspace_status", "lrsa_last_launch_count", "lrsa_debug_set_impl"):
             getattr(L, name).restype = ctypes.c_int
+        spec = importlib.util.spec_from_file_location("_lrsa_call", CALL_PATH)
+        if spec is None or not os.path.exists(CALL_PATH):
+            raise ImportError(f"{CALL_PATH} is missing: run `python -c 'import __graft_entry__ as g; g.build()'`")
+        call = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(call)
+        _call = call
         _lib = L
     return _lib
 
@@ -258,14 +275,17 @@ class KVCache:
         _check(lib().lrsa_cache_bytes(params.ref(), ctypes.byref(a), ctypes.byref(b)), "lrsa_cache_bytes")
         self.buf = torch.zeros(a.value, dtype=torch.uint8, device=device)
         self.ws = new_workspace(b.value, device)
+        self._lse = torch.empty((params.batch, params.n_q_heads), dtype=torch.float32, device=device)   # shape of an lse
         self.n_tokens = 0
 
     def append(self, k_new, v_new, stream=None):
         """k_new, v_new: bf16 [B, Hkv, n_new, d] (contiguous)."""
         n_new = k_new.shape[2]
-        _check(lib().lrsa_cache_append(self.params.ref(), _p(self.buf), self.buf.numel(), _p(k_new), _p(v_new),
-                                       self.n_tokens, n_new, _p(self.ws), self.ws.numel(), _stream(stream)),
-               "lrsa_cache_append")
+        buf, ws = self.buf, self.ws
+        status = _call.cache_append(self.params.address(), buf.data_ptr(), buf.numel(), _p(k_new), _p(v_new),
+                                    self.n_tokens, n_new, ws.data_ptr(), ws.numel(), _stream(stream))
+        if status:
+            _check(status, "lrsa_cache_append")
         self.n_tokens += n_new
 
     def decode(self, q, o=None, lse=None, stream=None):
@@ -273,9 +293,12 @@ class KVCache:
         if o is None:
             o = torch.empty_like(q)
         if lse is None:
-            lse = q.new_empty(q.shape[:2], dtype=torch.float32)
-        _check(lib().lrsa_attn_decode(self.params.ref(), _p(self.buf), self.buf.numel(), _p(q), self.n_tokens, _p(o),
-                                      _p(lse), _p(self.ws), self.ws.numel(), _stream(stream)), "lrsa_attn_decode")
+            lse = torch.empty_like(self._lse)
+        buf, ws = self.buf, self.ws
+        status = _call.attn_decode(self.params.address(), buf.data_ptr(), buf.numel(), _p(q), self.n_tokens,
+                                   o.data_ptr(), lse.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream))
+        if status:
+            _check(status, "lrsa_attn_decode")
         return o, lse
 
     def kept(self):
