@@ -227,22 +227,19 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     // ---------------- MMA issuer: dV(i), S^T(i+1), dK(i), dP^T(i+1), ... ----------------
     // One warp issues everything, so the products run in this order on the tensor core: S^T(i+1) may overwrite
     // P^T(i) and dP^T(i+1) may overwrite dS^T(i) without waiting for the products that read them.  The loop runs
-    // with all lanes (uniform control flow, descriptors computed once) and elects one lane per instruction.
+    // with all lanes (uniform control flow, descriptors computed once); one lane issues, by predicate.
     constexpr uint32_t idesc_s = make_idesc_bf16(kTile, kQRows, 0, 0);  // 128 keys x 128 queries
     constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);       // 128 keys x D
     const uint64_t descK = make_smem_desc_sw128(sK, 16, 1024), descV = make_smem_desc_sw128(sV, 16, 1024);
     const uint64_t descQ = make_smem_desc_sw128(sQ, 16, 1024), descO = make_smem_desc_sw128(sO, 16, 1024);   // K-major
     const uint64_t descQm = make_smem_desc_sw128(sQ, Cfg::kSubBytes, 1024);                                   // MN-major
     const uint64_t descOm = make_smem_desc_sw128(sO, Cfg::kSubBytes, 1024);
+    const uint32_t leader = elect_one();
     auto scores = [&](uint64_t dA, uint64_t dB, uint32_t d_tmem, uint64_t* bar) {
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t off = (kk >> 2) * Cfg::kSubBytes + (kk & 3) * 32;
-        const uint64_t ad = desc_advance(dA, off), bd = desc_advance(dB, off);
-        if (elect_one()) umma_ss(d_tmem, ad, bd, idesc_s, kk > 0 ? 1u : 0u);
-      }
-      if (elect_one()) umma_commit(smem_u32(bar));
-      __syncwarp();
+      for (int h = 0; h < Cfg::kSub; ++h)
+        umma_ss4(d_tmem, desc_advance(dA, h * Cfg::kSubBytes), desc_advance(dB, h * Cfg::kSubBytes), idesc_s, h > 0 ? 1u : 0u, leader);
+      umma_commit(smem_u32(bar), leader);
     };
     bool ok = mbar_wait_warp(smem_u32(&ctl.kv_full), 0, abort);
     if (ok) ok = mbar_wait_warp(smem_u32(&ctl.q_full[0]), 0, abort);
@@ -265,18 +262,11 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
           if (ok) ok = mbar_wait_warp(smem_u32(&ctl.p_full[half]), it & 1, abort);
           if (!ok) break;
           tc_fence_after_sync();
-#pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4) {
-            const int kk = 2 * k4 + half;
-            const uint64_t bd = desc_advance(dB, kk * 2048);
-            if (elect_one())
-              umma_ts(tmem + Cfg::kColV, tmem + Cfg::kColS + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a,
-                      kk > 0 ? 1u : acc0);
-          }
+          umma_ts4<32, 64, 96, 4096>(tmem + Cfg::kColV, tmem + Cfg::kColS + half * 8, desc_advance(dB, half * 2048), idesc_a,
+                                     half > 0 ? 1u : acc0, leader);
         }
         if (!ok) break;
-        if (elect_one()) umma_commit(smem_u32(&ctl.o_empty[slo]));
-        __syncwarp();
+        umma_commit(smem_u32(&ctl.o_empty[slo]), leader);
       }
       if (it + 1 < n) {
         ok = mbar_wait_warp(smem_u32(&ctl.q_full[nslq]), phq, abort);
@@ -289,13 +279,10 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
       {
         const uint64_t dB = desc_advance(descQm, slq * Cfg::kTileBytes);
 #pragma unroll
-        for (int kk = 0; kk < kQRows / 16; ++kk) {
-          const uint64_t bd = desc_advance(dB, kk * 2048);
-          if (elect_one())
-            umma_ts(tmem + Cfg::kColK, tmem + Cfg::kColP + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a, kk > 0 ? 1u : acc0);
-        }
-        if (elect_one()) umma_commit(smem_u32(&ctl.q_empty[slq]));
-        __syncwarp();
+        for (int h = 0; h < 2; ++h)
+          umma_ts4<8, 32, 40, 2048>(tmem + Cfg::kColK, tmem + Cfg::kColP + h * 64, desc_advance(dB, h * 4 * 2048), idesc_a,
+                                    h > 0 ? 1u : acc0, leader);
+        umma_commit(smem_u32(&ctl.q_empty[slq]), leader);
       }
       if (it + 1 < n) {
         ok = mbar_wait_warp(smem_u32(&ctl.o_full[nslo]), pho, abort);
@@ -304,8 +291,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
       }
       slq = nslq; slo = nslo;
     }
-    if (ok && elect_one()) umma_commit(smem_u32(&ctl.acc_done));
-    __syncwarp();
+    if (ok) umma_commit(smem_u32(&ctl.acc_done), leader);
   } else if (warp == 2) {
     // the mean key of head blockIdx.x from its partial sums, for the dQ kernel
     if (a.kpart && blockIdx.x < a.BHkv) {

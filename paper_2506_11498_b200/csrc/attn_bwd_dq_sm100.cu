@@ -154,7 +154,8 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
   } else if (warp == 1 || warp == 2) {
     // ---------------- S issuer (warp 1: Q K_j^T) and dP issuer (warp 2: dO V_j^T) ----------------
     // Each issuing warp runs its loop with all lanes (uniform control flow, descriptors computed once)
-    // and elects one lane per instruction.
+    // and issues through one lane, by predicate.
+    const uint32_t leader = elect_one();
     const int which = warp - 1;                                          // 0: K tiles, 1: V tiles
     constexpr uint32_t idesc_s = make_idesc_bf16(kTile, kKeys, 0, 0);   // 128 x 64
     const uint64_t descR = make_smem_desc_sw128(sRing, 16, 1024);       // K-major K_j / V_j
@@ -169,18 +170,14 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
       const uint32_t d_tmem = tmem + Cfg::kColBuf + b * 128 + which * Cfg::kColP;
       const uint64_t dT = desc_advance(descR, (it % NS) * Cfg::kKTileBytes);
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const uint64_t bd = desc_advance(dT, (kk >> 2) * Cfg::kKSubBytes + (kk & 3) * 32);
-        if (elect_one()) umma_ts(d_tmem, a_tmem + kk * 8, bd, idesc_s, kk > 0 ? 1u : 0u);
-      }
-      if (elect_one()) {
-        umma_commit(smem_u32(&bars.s_full[b]));
-        if (which == 1) umma_commit(smem_u32(&bars.kv_empty[it % NS]));   // V_j is used by dP only
-      }
-      __syncwarp();
+      for (int h = 0; h < Cfg::kSub; ++h)
+        umma_ts4<8, 16, 24, 32>(d_tmem, a_tmem + h * 32, desc_advance(dT, h * Cfg::kKSubBytes), idesc_s, h > 0 ? 1u : 0u, leader);
+      umma_commit(smem_u32(&bars.s_full[b]), leader);
+      if (which == 1) umma_commit(smem_u32(&bars.kv_empty[it % NS]), leader);   // V_j is used by dP only
     }
   } else if (warp == 3) {
     // ---------------- A issuer: A += dS K_j ----------------
+    const uint32_t leader = elect_one();
     constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);                  // 128 x D, B = K_j MN-major
     const uint64_t descRmn = make_smem_desc_sw128(sRing, Cfg::kKSubBytes, 1024);
     bool ok = true;
@@ -193,19 +190,11 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
       const uint64_t dKj = desc_advance(descRmn, (itK % NS) * Cfg::kKTileBytes);
       const uint32_t acc0 = j > 0 ? 1u : 0u;
       // packed dS: keys [0,32) in columns [0,16) of the S region, keys [32,64) in columns [32,48)
-#pragma unroll
-      for (int kk = 0; kk < kKeys / 16; ++kk) {
-        const uint64_t bd = desc_advance(dKj, kk * 2048);
-        if (elect_one()) umma_ts(tmem + Cfg::kColA, buf + (kk >> 1) * 32 + (kk & 1) * 8, bd, idesc_a, kk > 0 ? 1u : acc0);
-      }
-      if (elect_one()) {
-        umma_commit(smem_u32(&bars.kv_empty[itK % NS]));   // K_j: S (before the softmax) and A are done
-        umma_commit(smem_u32(&bars.buf_free[b]));          // tile j+2 may overwrite the buffer
-      }
-      __syncwarp();
+      umma_ts4<8, 32, 40, 2048>(tmem + Cfg::kColA, buf, dKj, idesc_a, acc0, leader);
+      umma_commit(smem_u32(&bars.kv_empty[itK % NS]), leader);   // K_j: S (before the softmax) and A are done
+      umma_commit(smem_u32(&bars.buf_free[b]), leader);          // tile j+2 may overwrite the buffer
     }
-    if (ok && elect_one()) umma_commit(smem_u32(&bars.acc_done));
-    __syncwarp();
+    if (ok) umma_commit(smem_u32(&bars.acc_done), leader);
   } else {
     // ---------------- softmax warps: warpgroup `half` takes key columns [32*half, 32*half+32) ----------------
     const int half = (warp - 4) >> 2, quad = warp & 3;

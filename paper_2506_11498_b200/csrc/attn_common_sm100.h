@@ -27,7 +27,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // The same wait executed by all 32 lanes of a converged warp, with one verdict for the warp.  The
 // warps that issue tcgen05.mma run in warp-uniform control flow with descriptors computed once
 // outside the loops (building a descriptor per instruction in a single-lane branch costs ~100
-// cycles per MMA, more than the MMA itself) and elect one lane per instruction.
+// cycles per MMA, more than the MMA itself) and issue through one lane, by predicate.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort) {
   const bool ok = mbar_wait(bar, parity, abort);
   return __all_sync(0xffffffffu, ok);

@@ -21,7 +21,7 @@
 // between a tile's products; scores were read twice; P was handed over in one piece.  Also measured: sixteen softmax
 // warps (16 rows x 128 columns each, 256-bit loads): 2.66 ms; exponentials started with the previous maximum, the tile
 // taken again when it was raised: 2.47 ms; a share of them on the FMA pipe: no gain at 1/8, 2.63 ms at 1/4.
-// The issuing warp runs its loop with all lanes and elects one lane per instruction.  All mbarrier waits are bounded;
+// The issuing warp runs its loop with all lanes; one lane issues, by predicate.  All mbarrier waits are bounded;
 // on expiry the CTA records LRSA_ERR_TIMEOUT in the workspace header and leaves.
 #include "attn_common_sm100.h"
 
@@ -167,6 +167,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     const uint64_t descK0 = make_smem_desc_sw128(sRing, 16, 1024);
     const uint64_t descV0 = make_smem_desc_sw128(sRing, Cfg::kSubBytes, 1024);   // V_j MN-major
     const uint64_t descQ0 = make_smem_desc_sw128(sQ, 16, 1024);
+    const uint32_t leader = elect_one();
     bool ok = mbar_wait_warp(smem_u32(&bars.q_full), 0, abort);
     int slot_v = 0, ph_v = 0, slot_k = 0, ph_k = 0;   // ring order: K_0, V_0, K_1, V_1, ...
     auto next = [](int& slot, int& ph) { if (++slot == NS) { slot = 0; ph ^= 1; } };
@@ -187,18 +188,11 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
             if (ok) ok = mbar_wait_warp(smem_u32(&bars.p_full[t][part]), j & 1, abort);
             if (!ok) break;
             tc_fence_after_sync();
-#pragma unroll
-            for (int k8 = 0; k8 < kTile / 16 / kPParts; ++k8) {
-              const int kk = part * (kTile / 16 / kPParts) + k8;
-              const uint64_t bd = desc_advance(dV, kk * 2048);
-              if (elect_one())
-                umma_ts(tmem + Cfg::kColO + t * kTile, tmem + Cfg::kColS + t * kTile + kk * 8, bd, idesc_pv,
-                        (kk > 0 || j > 0) ? 1u : 0u);
-            }
+            umma_ts4<8, 16, 24, 2048>(tmem + Cfg::kColO + t * kTile, tmem + Cfg::kColS + t * kTile + part * 32,
+                                      desc_advance(dV, part * 4 * 2048), idesc_pv, (part > 0 || j > 0) ? 1u : 0u, leader);
           }
           if (!ok) break;
-          if (elect_one()) umma_commit(smem_u32(&bars.pv_done[t]));     // phase j: O_t holds key tiles 0..j
-          __syncwarp();
+          umma_commit(smem_u32(&bars.pv_done[t]), leader);     // phase j: O_t holds key tiles 0..j
         }
         if (j + 1 < nt) {
           if (!k_here) {
@@ -210,21 +204,15 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
           tc_fence_after_sync();
           const uint64_t dQ = desc_advance(descQ0, t * Cfg::kQRegion);
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t off = (kk >> 2) * Cfg::kSubBytes + (kk & 3) * 32;
-            const uint64_t ad = desc_advance(dQ, off), bd = desc_advance(dK, off);
-            if (elect_one()) umma_ss(tmem + Cfg::kColS + t * kTile, ad, bd, idesc_qk, kk > 0 ? 1u : 0u);
-          }
-          if (elect_one()) umma_commit(smem_u32(&bars.s_full[t]));
-          __syncwarp();
+          for (int h = 0; h < Cfg::kSub; ++h)
+            umma_ss4(tmem + Cfg::kColS + t * kTile, desc_advance(dQ, h * Cfg::kSubBytes), desc_advance(dK, h * Cfg::kSubBytes),
+                     idesc_qk, h > 0 ? 1u : 0u, leader);
+          umma_commit(smem_u32(&bars.s_full[t]), leader);
         }
       }
       if (!ok) break;
-      if (elect_one()) {
-        if (j >= 0) umma_commit(smem_u32(&bars.kv_empty[slot_v]));
-        if (j + 1 < n) umma_commit(smem_u32(&bars.kv_empty[slot_k]));
-      }
-      __syncwarp();
+      if (j >= 0) umma_commit(smem_u32(&bars.kv_empty[slot_v]), leader);
+      if (j + 1 < n) umma_commit(smem_u32(&bars.kv_empty[slot_k]), leader);
       next(slot_v, ph_v);
       if (j >= 0) next(slot_v, ph_v);
       next(slot_k, ph_k);

@@ -95,31 +95,65 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// ---- tcgen05.mma, bf16 x bf16 -> fp32, issued by one thread ----
-// D[tmem] (+)= A[smem desc] * B[smem desc]
-__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                        uint32_t accumulate) {
+// ---- tcgen05.mma, bf16 x bf16 -> fp32: D[tmem] (+)= A * B ----
+// Issued by a converged warp through one lane: `leader` is 1 in the lane that elect_one() names (the same every time), the
+// instructions are predicated by it and a run of four k-steps of 16 is one block of straight code.  What a product costs in
+// the issuing warp counts.  With a branch around each product (if (elect_one()) ...) and with these, 28/4 heads, d = 128:
+// forward 98.3 -> 92.0 us at 4K tokens and 266 -> 250 at 8K, whole training step 394 -> 376 us at 4K, 10.36 -> 10.12 ms at 32K
+// (one predicated instruction at a time: 94.0 and 261 us).
+// SS: both operands K-major in a 128-byte-swizzled tile (32 bytes a step).
+__device__ __forceinline__ void umma_ss4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "add.s64 a, %1, 2;\n\tadd.s64 b, %2, 2;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, 1;\n\t"
+      "add.s64 a, %1, 4;\n\tadd.s64 b, %2, 4;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, 1;\n\t"
+      "add.s64 a, %1, 6;\n\tadd.s64 b, %2, 6;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, 1;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                        uint32_t accumulate) {
+// TS: A in tensor memory at a_tmem, + A1, + A2, + A3 columns; B advances by BStep bytes a step.
+template <int A1, int A2, int A3, int BStep>
+__device__ __forceinline__ void umma_ts4(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 b;\n\t.reg .b32 a;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t"
+      "add.s32 a, %1, %6;\n\tadd.s64 b, %2, %9;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, 1;\n\t"
+      "add.s32 a, %1, %7;\n\tadd.s64 b, %2, %10;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, 1;\n\t"
+      "add.s32 a, %1, %8;\n\tadd.s64 b, %2, %11;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, 1;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader), "n"(A1), "n"(A2), "n"(A3),
+        "n"(BStep / 16), "n"(BStep / 8), "n"(3 * BStep / 16)
       : "memory");
 }
-// mbarrier arrives once all MMAs issued so far by this thread have completed
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
+// One k-step, A in tensor memory.
+__device__ __forceinline__ void umma_ts1(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t accumulate, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
+      : "memory");
+}
+// mbarrier arrives once all MMAs issued so far by the leader have completed
+__device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader)
+      : "memory");
 }
 
 // Instruction descriptor, kind::f16: bf16 A and B, fp32 accumulator, M x N tile.
