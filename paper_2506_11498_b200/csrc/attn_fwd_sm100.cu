@@ -1,14 +1,16 @@
 // LRSA attention forward on tcgen05 tensor cores (Section 3.1 Eq. 3 under the chunked mask of
 // Section 3.2).
 //
-// A CTA owns up to 256 query rows of one (batch, query head) that share a key list (two 128-row tiles of
-// one query chunk) and walks the list (first n_front rows of the compact sinks+kept buffer, then a contiguous
-// range of original positions up to the diagonal) in 128-key tiles; every K_j / V_j tile in shared memory
-// serves both query tiles.  Roles:
+// A CTA owns one or two 128-row query tiles of one (batch, query head) and one query chunk, which share a key list, and
+// walks the list (first n_front rows of the compact sinks+kept buffer, then a contiguous range of original positions up to
+// the diagonal) in 128-key tiles.  Two tiles (TQ = 2, one CTA per SM): every K_j / V_j tile in shared memory serves both.
+// One tile (TQ = 1, two CTAs per SM): small grids and short lists, see one_tile().  The list's last tile often holds only as
+// many keys as there are sinks: with at most 16 it comes first, and its products and exponentials are 16 wide (1777 tokens
+// 45.8 -> 43.1 us, 4K 92.6 -> 88.0, 32K in eight sequences 870 -> 842, with few sinks and 28 heads).  Roles:
 //   warp 0      TMA producer: the Q tiles once, then K_j, V_j tiles through a ring of shared-memory slots
 //   warp 1      issues all products, per key tile and query tile  O_t += P_t V_j (P_t from tensor memory), then
 //               S_t = Q_t K_{j+1}^T (both operands in shared memory); owns the TMEM allocation
-//   warps 4-7   softmax of query tile 0, warps 8-11 of query tile 1: one thread per row, S from TMEM, online
+//   warps 4-7   softmax of query tile 0, warps 8-11 of query tile 1 (TQ = 2): one thread per row, S from TMEM, online
 //               softmax in fp32 with the maximum only raised when it grew by more than 2^8 (then O_t is
 //               rescaled in TMEM), P written back over S as packed bf16
 // The two tiles take turns on the tensor core: while one tile's scores are in its softmax warpgroup the
@@ -21,8 +23,10 @@
 // between a tile's products; scores were read twice; P was handed over in one piece.  Also measured: sixteen softmax
 // warps (16 rows x 128 columns each, 256-bit loads): 2.66 ms; exponentials started with the previous maximum, the tile
 // taken again when it was raised: 2.47 ms; a share of them on the FMA pipe: no gain at 1/8, 2.63 ms at 1/4.
-// The issuing warp runs its loop with all lanes; one lane issues, by predicate.  All mbarrier waits are bounded;
+// The issuing warp runs its loop with all lanes and elects one lane per instruction.  All mbarrier waits are bounded;
 // on expiry the CTA records LRSA_ERR_TIMEOUT in the workspace header and leaves.
+#include <algorithm>
+
 #include "attn_common_sm100.h"
 
 namespace lrsa {
@@ -30,7 +34,7 @@ namespace {
 
 using namespace ptx;
 
-template <int D>
+template <int D, int TQ>
 struct FwdCfg {
   static constexpr int kSub = D / 64;                 // 64-column (128-byte) sub-tiles per tile
   static constexpr int kSubBytes = kTile * 128;       // 16 KB
@@ -38,11 +42,12 @@ struct FwdCfg {
   // A Q tile is followed by 2 KB so that the output rows of the tile can be staged there with 16 bytes of
   // padding per row (128 rows x (2D + 16) bytes = tile + 2 KB); the next tile stays 1024-byte aligned.
   static constexpr int kQRegion = kTileBytes + 2048;
-  static constexpr int kStages = D == 128 ? 4 : 10;   // K/V ring slots
-  static constexpr int kSmem = 2 * kQRegion + kStages * kTileBytes + 1024;
-  static constexpr int kThreads = 384;
-  // TMEM columns: accumulator O of query tile t at 128t, its S (and, packed over it, P) at 256 + 128t
-  static constexpr uint32_t kColO = 0, kColS = 256;
+  static constexpr int kPerSm = 3 - TQ;                          // resident CTAs
+  static constexpr int kStages = (D == 128 ? 4 : 10) / kPerSm;   // K/V ring slots
+  static constexpr int kSmem = TQ * kQRegion + kStages * kTileBytes + 1024;
+  static constexpr int kThreads = 128 + 128 * TQ;
+  // TMEM columns: accumulator O of query tile t at 128t, its S (and, packed over it, P) behind the accumulators
+  static constexpr uint32_t kColO = 0, kColS = TQ * 128, kCols = 2 * TQ * 128;
 };
 
 template <int NSEQ>
@@ -62,6 +67,7 @@ struct FwdArgs {
   int* status;
 };
 
+constexpr int kShort = 16;    // keys of a tile of the short form
 constexpr int kPParts = 2;   // P_t is handed to the tensor core in two halves (64 keys each)
 
 struct FwdBars {
@@ -71,10 +77,10 @@ struct FwdBars {
   uint64_t p_full[2][kPParts];      // per query tile: the parts of P_t (128 / kPParts keys each) are stored
 };
 
-template <int D, int NSEQ>
-__global__ void __launch_bounds__(FwdCfg<D>::kThreads, 1)
+template <int D, int NSEQ, int TQ>
+__global__ void __launch_bounds__(FwdCfg<D, TQ>::kThreads, FwdCfg<D, TQ>::kPerSm)
 lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constant__ FwdArgs<NSEQ> a) {
-  using Cfg = FwdCfg<D>;
+  using Cfg = FwdCfg<D, TQ>;
   constexpr int NS = Cfg::kStages;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) FwdBars bars;
@@ -83,7 +89,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t sQ = smem0, sRing = smem0 + 2 * Cfg::kQRegion;
+  const uint32_t sQ = smem0, sRing = smem0 + TQ * Cfg::kQRegion;
 
   const int bh = blockIdx.x % a.BH;
   int blk = blockIdx.x / a.BH, sq = 0;
@@ -92,13 +98,14 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     blk -= a.block0[sq];
   }
   const RowBlock rb = decode_block(a.plan[sq], blk);
-  const size_t row0 = (size_t)bh * a.N + a.tok0[sq];   // the sequence's first row of O and LSE
   const int bh_kv = (bh / a.Hq) * a.Hkv + (bh % a.Hq) / a.G;
   const int n_ct = (rb.n_front + kTile - 1) / kTile;
   // key tiles of query tile t: the list, then the dense range up to the tile's last row (0: the tile is empty)
   const int n0 = n_ct + (min(rb.q_end, rb.q0 + kTile) - 1 - rb.dense_start) / kTile + 1;
-  const int n1 = rb.q0 + kTile < rb.q_end ? n_ct + (rb.q_end - 1 - rb.dense_start) / kTile + 1 : 0;
+  const int n1 = TQ == 2 && rb.q0 + kTile < rb.q_end ? n_ct + (rb.q_end - 1 - rb.dense_start) / kTile + 1 : 0;
   const int n = max(n0, n1);
+  // the list's last tile comes first when it holds no more than kShort keys: its products and exponentials are that wide
+  const int sh = n_ct > 0 && rb.n_front - (n_ct - 1) * kTile <= kShort ? 1 : 0;
 
   if (tid == 0) {
     abort_s = 0;
@@ -111,7 +118,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     }
     fence_barrier_init();
   }
-  if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), 512); tmem_relinquish(); }
+  if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), Cfg::kCols); tmem_relinquish(); }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -121,9 +128,10 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // The softmax threads hold a row of 128 scores: they take the registers the other warps do not need
-  // (128 x 72 + 256 x 216 = 384 x 168, what the CTA was launched with).
+  // (128 x 72 + 256 x 216 = 384 x 168, 128 x 48 + 128 x 208 = 256 x 128: what the CTA was launched with).
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    if constexpr (TQ == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    else asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
@@ -144,7 +152,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
           mbar_expect_tx(full, Cfg::kTileBytes);
           const bool compact = j < n_ct;
           const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
-          const int row = compact ? j * kTile : rb.dense_start + (j - n_ct) * kTile;
+          const int row = compact ? (j < sh ? n_ct - 1 : j - sh) * kTile : rb.dense_start + (j - n_ct) * kTile;
           for (int h = 0; h < Cfg::kSub; ++h)
             tma_load_3d(sRing + slot * Cfg::kTileBytes + h * Cfg::kSubBytes, map, h * 64, row, bh_kv, full);
         }
@@ -171,7 +179,50 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     bool ok = mbar_wait_warp(smem_u32(&bars.q_full), 0, abort);
     int slot_v = 0, ph_v = 0, slot_k = 0, ph_k = 0;   // ring order: K_0, V_0, K_1, V_1, ...
     auto next = [](int& slot, int& ph) { if (++slot == NS) { slot = 0; ph ^= 1; } };
-    for (int j = -1; j < n && ok; ++j) {
+    auto scores = [&](int t, uint64_t dK, uint32_t idesc) {
+      const uint64_t dQ = desc_advance(descQ0, t * Cfg::kQRegion);
+#pragma unroll
+      for (int h = 0; h < Cfg::kSub; ++h)
+        umma_ss4(tmem + Cfg::kColS + t * kTile, desc_advance(dQ, h * Cfg::kSubBytes), desc_advance(dK, h * Cfg::kSubBytes),
+                 idesc, h > 0 ? 1u : 0u, leader);
+      umma_commit(smem_u32(&bars.s_full[t]), leader);
+    };
+    if (sh) {
+      // the short tile (key tile 0), apart from the loop: with the choices inside it the two-tile form takes 253 instead of
+      // 244 us at 8K tokens (28 heads, d = 128)
+      constexpr uint32_t idesc_short = make_idesc_bf16(kTile, kShort, 0, 0);
+      if (ok) ok = mbar_wait_warp(smem_u32(&bars.kv_full[0]), 0, abort);
+      if (ok) {
+        tc_fence_after_sync();
+        scores(0, descK0, idesc_short);
+        if (n1 > 0) scores(1, descK0, idesc_short);
+        umma_commit(smem_u32(&bars.kv_empty[0]), leader);
+      }
+      next(slot_v, ph_v);                                   // V_0
+      next(slot_k, ph_k); next(slot_k, ph_k);               // K_1 (there is one: the dense range is never empty)
+      if (ok) ok = mbar_wait_warp(smem_u32(&bars.kv_full[slot_v]), ph_v, abort);
+      for (int t = 0; t < TQ && ok; ++t) {
+        if (t == 1 && n1 == 0) break;
+        for (int part = 0; part < kPParts; ++part)
+          if (ok) ok = mbar_wait_warp(smem_u32(&bars.p_full[t][part]), 0, abort);
+        if (!ok) break;
+        tc_fence_after_sync();
+        umma_ts1(tmem + Cfg::kColO + t * kTile, tmem + Cfg::kColS + t * kTile, desc_advance(descV0, slot_v * Cfg::kTileBytes),
+                  idesc_pv, 0u, leader);
+        umma_commit(smem_u32(&bars.pv_done[t]), leader);
+        if (t == 0) ok = mbar_wait_warp(smem_u32(&bars.kv_full[slot_k]), ph_k, abort);
+        if (!ok) break;
+        tc_fence_after_sync();
+        scores(t, desc_advance(descK0, slot_k * Cfg::kTileBytes), idesc_qk);
+      }
+      if (ok) {
+        umma_commit(smem_u32(&bars.kv_empty[slot_v]), leader);
+        umma_commit(smem_u32(&bars.kv_empty[slot_k]), leader);
+      }
+      next(slot_v, ph_v); next(slot_v, ph_v);
+      next(slot_k, ph_k); next(slot_k, ph_k);
+    }
+    for (int j = sh ? 1 : -1; j < n && ok; ++j) {
       uint64_t dV = 0, dK = 0;
       if (j >= 0) {
         ok = mbar_wait_warp(smem_u32(&bars.kv_full[slot_v]), ph_v, abort);
@@ -179,7 +230,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
         dV = desc_advance(descV0, slot_v * Cfg::kTileBytes);
       }
       bool k_here = false;
-      for (int t = 0; t < 2 && ok; ++t) {
+      for (int t = 0; t < TQ && ok; ++t) {
         const int nt = t == 0 ? n0 : n1;
         if (j >= 0 && j < nt) {
           // packed P_t: keys [16k, 16k+16) in columns [8k, 8k+8) of the tile's S region
@@ -189,10 +240,11 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
             if (!ok) break;
             tc_fence_after_sync();
             umma_ts4<8, 16, 24, 2048>(tmem + Cfg::kColO + t * kTile, tmem + Cfg::kColS + t * kTile + part * 32,
-                                      desc_advance(dV, part * 4 * 2048), idesc_pv, (part > 0 || j > 0) ? 1u : 0u, leader);
+                                     desc_advance(dV, part * 4 * 2048), idesc_pv, (part > 0 || j > 0) ? 1u : 0u, leader);
           }
           if (!ok) break;
           umma_commit(smem_u32(&bars.pv_done[t]), leader);     // phase j: O_t holds key tiles 0..j
+          if (TQ == 1) umma_commit(smem_u32(&bars.kv_empty[slot_v]), leader);
         }
         if (j + 1 < nt) {
           if (!k_here) {
@@ -202,16 +254,11 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
             k_here = true;
           }
           tc_fence_after_sync();
-          const uint64_t dQ = desc_advance(descQ0, t * Cfg::kQRegion);
-#pragma unroll
-          for (int h = 0; h < Cfg::kSub; ++h)
-            umma_ss4(tmem + Cfg::kColS + t * kTile, desc_advance(dQ, h * Cfg::kSubBytes), desc_advance(dK, h * Cfg::kSubBytes),
-                     idesc_qk, h > 0 ? 1u : 0u, leader);
-          umma_commit(smem_u32(&bars.s_full[t]), leader);
+          scores(t, dK, idesc_qk);
         }
       }
       if (!ok) break;
-      if (j >= 0) umma_commit(smem_u32(&bars.kv_empty[slot_v]), leader);
+      if (TQ == 2 && j >= 0) umma_commit(smem_u32(&bars.kv_empty[slot_v]), leader);
       if (j + 1 < n) umma_commit(smem_u32(&bars.kv_empty[slot_k]), leader);
       next(slot_v, ph_v);
       if (j >= 0) next(slot_v, ph_v);
@@ -220,7 +267,8 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     }
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+    if constexpr (TQ == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     // ---------------- softmax + epilogue: warpgroup t owns query tile t, one thread per row ----------------
     const int t = (warp - 4) >> 2, quad = warp & 3;
     const int row = quad * 32 + lane;
@@ -228,16 +276,43 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     const uint32_t S_addr = tmem + lane_addr + Cfg::kColS + t * kTile;
     const uint32_t O_addr = tmem + lane_addr + Cfg::kColO + t * kTile;
     const int nt = t == 0 ? n0 : n1;
-    const int qpos = rb.q0 + t * kTile + row;
+    // keys of tile j this row may see: the first list_end - 128 j of a list tile, dense_end - 128 j of a dense one
+    const int list_end = rb.n_front + sh * kTile, dense_end = rb.q0 + t * kTile + row + 1 - rb.dense_start + n_ct * kTile;
     const float c = a.scale_log2;
     float m = 0.f, l = 0.f;
     bool ok = true;
-    for (int j = 0; j < nt && ok; ++j) {
+    if (sh && nt > 0) {
+      ok = mbar_wait_warp(smem_u32(&bars.s_full[t]), 0, abort);
+      if (ok) {
+        tc_fence_after_sync();
+        const int limit = rb.n_front - (n_ct - 1) * kTile;
+        uint32_t s[32], pk[kShort / 2];   // only the first kShort columns hold scores
+        tmem_ld32(S_addr, s);
+        tmem_wait_ld();
+        m = __uint_as_float(s[0]);
+#pragma unroll
+        for (int i = 1; i < kShort; ++i) {
+          if (i >= limit) s[i] = 0xff800000u;
+          m = fmaxf(m, __uint_as_float(s[i]));
+        }
+#pragma unroll
+        for (int i = 0; i < kShort / 2; ++i) {
+          const float p0 = ex2(fmaf(__uint_as_float(s[2 * i]), c, -m * c)), p1 = ex2(fmaf(__uint_as_float(s[2 * i + 1]), c, -m * c));
+          l += p0 + p1;
+          pk[i] = pack_bf16(p0, p1);
+        }
+        tmem_st8(S_addr, pk);
+        tmem_wait_st();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane < kPParts) mbar_arrive(smem_u32(&bars.p_full[t][lane]));
+      }
+    }
+    for (int j = sh; j < nt && ok; ++j) {
       ok = mbar_wait_warp(smem_u32(&bars.s_full[t]), j & 1, abort);
       if (!ok) break;
       tc_fence_after_sync();
-      // keys of the tile this row may see: the first `limit`
-      const int limit = j < n_ct ? rb.n_front - j * kTile : qpos - (rb.dense_start + (j - n_ct) * kTile) + 1;
+      const int limit = (j < n_ct ? list_end : dense_end) - j * kTile;
       // the row's 128 scores and their maximum
       uint32_t s[kTile];
 #pragma unroll
@@ -333,6 +408,11 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     constexpr int kRowBytes = D * 2, kStageStride = kRowBytes + 16;
     static_assert(kTile * kStageStride <= Cfg::kQRegion, "staging fits the Q region");
     unsigned char* stage_out = smem_raw + (sQ - smem_u32(smem_raw)) + t * Cfg::kQRegion;
+    // (positions and pointers of the output are formed here, not kept in registers through the loop)
+    int blk_here = blockIdx.x;
+    asm volatile("" : "+r"(blk_here));
+    const size_t row0 = (size_t)(blk_here % a.BH) * a.N + a.tok0[sq];   // the sequence's first row of O and LSE
+    const int qpos = rb.q0 + t * kTile + row;
     const bool store = qpos < rb.q_end && nt > 0;
     if (ok && nt > 0) {
       tc_fence_after_sync();
@@ -379,7 +459,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
 
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 1) tmem_dealloc(tmem, Cfg::kCols);
   if (tid == 0 && abort_s) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
 }
 
@@ -449,11 +529,11 @@ int make_tmap_bf16_rows(CUtensorMap* map, const void* base, int d, long long row
 
 size_t attn_fwd_ws_bytes(const Geom& g) { return fwd_ws_layout(g).total; }
 
-template <int D, int NSEQ>
+template <int D, int NSEQ, int TQ>
 static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                         const __nv_bfloat16* V, const __nv_bfloat16* Kc, const __nv_bfloat16* Vc, __nv_bfloat16* O,
                         __nv_bfloat16* Olo, float* LSE, int* status, cudaStream_t st) {
-  using Cfg = FwdCfg<D>;
+  using Cfg = FwdCfg<D, TQ>;
   FwdMaps<NSEQ> m;
   FwdArgs<NSEQ> a;
   const long long BHq = (long long)whole.B * whole.Hq, BHkv = (long long)whole.B * whole.Hkv;
@@ -469,7 +549,7 @@ static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat1
     if (r == LRSA_OK) r = make_tmap_bf16(&m.kc[s], Kc + csh, D, rc, BHkv, kTile);
     if (r == LRSA_OK) r = make_tmap_bf16(&m.vc[s], Vc + csh, D, rc, BHkv, kTile);
     if (r != LRSA_OK) return r;
-    a.plan[s] = make_plan(g, 2 * kTile);
+    a.plan[s] = make_plan(g, TQ * kTile);
     a.tok0[s] = g.tok0;
     a.block0[s + 1] = a.block0[s] + a.plan[s].total;
   }
@@ -479,11 +559,30 @@ static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat1
   a.status = status;
   const long long grid = (long long)a.block0[b.n] * a.BH;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  auto kern = lrsa_fwd_kernel<D, NSEQ>;
+  auto kern = lrsa_fwd_kernel<D, NSEQ, TQ>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
   LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));
   launch_counter().n++;
   return LRSA_OK;
+}
+
+// One query tile per CTA and two CTAs per SM, or two tiles that share the K/V tiles in one CTA (d = 128)?  Two CTAs start and
+// end at different times and split a small grid more finely, but load K and V twice.  28 heads, us with one | two tiles:
+// few CTAs: 1777 tokens 41.4 | 43.1, 4K 86.1 | 88.0, 5K 114.0 | 119.1, 6K 184 | 181, 8K 246-257 | 244, 32K 2290 | 2143;
+// short lists: 16 x 600 tokens 115 | 145, 8 x 1300 160 | 181, 8 x 1777 211-218 | 220, 4 x 3000 (8 tiles) 225 | 220.
+// d = 64 (always one tile): 4K 37.1 | 41.1, 16K 166 | 178, 64K 1904 | 2084: its K/V tiles cost half as much to load.
+static bool one_tile(const Geom& whole, const SeqBatch& b) {
+  long long ctas = 0, keys = 0, tokens = 0;
+  for (int s = 0; s < b.n; ++s) {
+    const Geom& g = b.g[s];
+    ctas += (long long)make_plan(g, 2 * kTile).total * whole.B * whole.Hq;
+    // about the mean number of keys of a query: half of the history's kept tokens, the dense windows
+    const long long hist = g.C > 1 + g.ndp ? (long long)(g.C - 1 - g.ndp) * g.K / 2 : 0;
+    const long long dense = std::min<long long>(g.N / 2, g.L * g.ndp + g.L / 2);
+    keys += g.N * (g.S + hist + dense);
+    tokens += g.N;
+  }
+  return ctas <= 4 * 148 || 2 * keys <= 15 * kTile * tokens;   // 7.5 tiles
 }
 
 int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
@@ -504,8 +603,9 @@ int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
       LRSA_CUDA_CHECK(launch_dependent(compact_kv_kernel, dim3(blocks > 0 ? blocks : 1), dim3(256), 0, st, 1, c));
       launch_counter().n++;
     }
-    const auto fwd = g.d == 128 ? (b.n == 1 ? launch_fwd_t<128, 1> : launch_fwd_t<128, kMaxSeqs>)
-                                : (b.n == 1 ? launch_fwd_t<64, 1> : launch_fwd_t<64, kMaxSeqs>);
+    const auto fwd = g.d == 64         ? (b.n == 1 ? launch_fwd_t<64, 1, 1> : launch_fwd_t<64, kMaxSeqs, 1>)
+                     : one_tile(g, b) ? (b.n == 1 ? launch_fwd_t<128, 1, 1> : launch_fwd_t<128, kMaxSeqs, 1>)
+                                      : (b.n == 1 ? launch_fwd_t<128, 1, 2> : launch_fwd_t<128, kMaxSeqs, 2>);
     const int rc = fwd(g, b, Q, K, V, Kc, Vc, O, Olo, LSE, status, st);
     if (rc != LRSA_OK) return rc;
   }

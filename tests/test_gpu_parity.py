@@ -123,6 +123,42 @@ def test_attention_fwd_bwd(w, ndp):
         check_close("dV", f64(dV), odV)
 
 
+@pytest.mark.parametrize("S", [1, 16, 17, 80])
+@pytest.mark.parametrize("d", [64, 128])
+def test_last_list_tile_of_few_keys(d, S):
+    """K = 128 leaves S keys for the last tile of the sinks + kept list: the short form of the tile takes up to 16 (in the dQ
+    kernel, whose tiles hold 64 keys, S = 80 is 64 + 16)."""
+    w = W(f"a_tail{S}", 1, 2, 1, S + 900, d, 256, 128, S, seed=35)
+    host = workloads.generate(w)
+    bits = host_bits(host)
+    op = oparams(w, n_dense_prev=1)
+    oidx, _ = orc.score_select(op, bits["K"], bits["V"])
+    oO, oL = orc.attn_fwd(op, bits["Q"], bits["K"], bits["V"], oidx)
+    odQ, odK, odV = orc.attn_bwd(op, bits["Q"], bits["K"], bits["V"], bits["dO"], oidx)
+    O, LSE, dQ, dK, dV = _run_attention(w, 1, oidx, host)
+    check_close("O", f64(O), oO)
+    check_close("LSE", f64(LSE), oL, max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
+    check_close("dQ", f64(dQ), odQ)
+    check_close("dK", f64(dK), odK)
+    check_close("dV", f64(dV), odV)
+
+
+@pytest.mark.parametrize("S,N", [(1, 2949), (17, 3300)])
+def test_one_and_two_query_tiles_per_cta_agree(S, N):
+    """The forward of four sequences runs with two query tiles per CTA, that of one with one (fewer CTAs): every row does the
+    same arithmetic in the same order, so the results are the same bits."""
+    w = W(f"a_tiles{S}", 4, 28, 4, N, 128, 512, 128, S, seed=36)
+    dev = to_dev(workloads.generate(w))
+    p = lrsa.Params.from_workload(w, n_dense_prev=1)
+    idx = lrsa.lrsa_score_select(p, dev["K"], dev["V"])[0]
+    O, LSE = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx)
+    p1 = lrsa.Params.from_workload(W(f"a_tiles{S}", 1, 28, 4, N, 128, 512, 128, S, seed=36), n_dense_prev=1)
+    for b in range(4):
+        part = [t[b:b + 1].contiguous() for t in (dev["Q"], dev["K"], dev["V"], idx)]
+        o, lse = lrsa.lrsa_attn_fwd(p1, *part)
+        assert torch.equal(o, O[b:b + 1]) and torch.equal(lse, LSE[b:b + 1])
+
+
 @pytest.mark.parametrize("name", ["a_salient64", "a_offsets", "a_gqa7", "a_ndp0"])
 def test_cuda_core_validation_kernels_against_oracle(name):
     """The slow CUDA-core kernels (fp32 P and dS, no tensor cores) against the oracle at the same
