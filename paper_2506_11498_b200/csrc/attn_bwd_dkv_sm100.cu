@@ -88,9 +88,9 @@ struct DkvArgs {
 struct DkvCtl {
   uint64_t kv_full, acc_done;
   uint64_t q_full[4], q_empty[4], o_full[3], o_empty[3];
-  uint64_t s_full, dp_full;      // S^T / dP^T of the step are in tensor memory
+  uint64_t s_full[2];            // S^T of the step is in tensor memory and its statistics are staged (slot = step & 1)
+  uint64_t dp_full;              // dP^T of the step is in tensor memory
   uint64_t p_full[2];            // halves of P^T: the first / last 16 query columns of every warpgroup
-  uint64_t st_full[2];           // statistics of the step (slot = step & 1) are staged
   uint64_t ds_full[2];           // dS^T of the step is stored (slot = step & 1; also frees the statistics slot)
   uint32_t tmem_base;
   int abort;
@@ -144,12 +144,11 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     mbar_init(smem_u32(&ctl.acc_done), 1);
     for (int i = 0; i < NQ; ++i) { mbar_init(smem_u32(&ctl.q_full[i]), 1); mbar_init(smem_u32(&ctl.q_empty[i]), 1); }
     for (int i = 0; i < NO; ++i) { mbar_init(smem_u32(&ctl.o_full[i]), 1); mbar_init(smem_u32(&ctl.o_empty[i]), 1); }
-    mbar_init(smem_u32(&ctl.s_full), 1);
     mbar_init(smem_u32(&ctl.dp_full), 1);
     for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_u32(&ctl.p_full[b]), Cfg::kSoftWarps);   // one arrival per softmax warp
-      mbar_init(smem_u32(&ctl.st_full[b]), 1);
-      mbar_init(smem_u32(&ctl.ds_full[b]), Cfg::kSoftWarps);
+      mbar_init(smem_u32(&ctl.p_full[b]), 32 * Cfg::kSoftWarps);   // every softmax thread (a lane per warp: 0.6 % slower)
+      mbar_init(smem_u32(&ctl.s_full[b]), 2);   // the product and the statistics
+      mbar_init(smem_u32(&ctl.ds_full[b]), 32 * Cfg::kSoftWarps);
     }
     fence_barrier_init();
   }
@@ -244,7 +243,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     bool ok = mbar_wait_warp(smem_u32(&ctl.kv_full), 0, abort);
     if (ok) ok = mbar_wait_warp(smem_u32(&ctl.q_full[0]), 0, abort);
     if (ok) {
-      scores(descK, descQ, tmem + Cfg::kColS, &ctl.s_full);
+      scores(descK, descQ, tmem + Cfg::kColS, &ctl.s_full[0]);
       ok = mbar_wait_warp(smem_u32(&ctl.o_full[0]), 0, abort);
     }
     if (ok) scores(descV, descO, tmem + Cfg::kColP, &ctl.dp_full);
@@ -254,6 +253,8 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
       if (nslq == 0) phq ^= 1;
       if (nslo == 0) pho ^= 1;
       const uint32_t acc0 = it > 0 ? 1u : 0u;
+      // (the next Q and dO are long here: waited for ahead of the softmax warps, not between two products)
+      if (it + 1 < n) ok = mbar_wait_warp(smem_u32(&ctl.q_full[nslq]), phq, abort);
       // packed P^T / dS^T: the 32 query columns of warpgroup w in columns [32w, 32w+16) of the region
       {
         const uint64_t dB = desc_advance(descOm, slo * Cfg::kTileBytes);
@@ -266,14 +267,13 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
                                      half > 0 ? 1u : acc0, leader);
         }
         if (!ok) break;
-        umma_commit(smem_u32(&ctl.o_empty[slo]), leader);
       }
       if (it + 1 < n) {
-        ok = mbar_wait_warp(smem_u32(&ctl.q_full[nslq]), phq, abort);
-        if (!ok) break;
-        scores(descK, desc_advance(descQ, nslq * Cfg::kTileBytes), tmem + Cfg::kColS, &ctl.s_full);
+        scores(descK, desc_advance(descQ, nslq * Cfg::kTileBytes), tmem + Cfg::kColS, &ctl.s_full[(it + 1) & 1]);
       }
-      ok = mbar_wait_warp(smem_u32(&ctl.ds_full[it & 1]), (it >> 1) & 1, abort);
+      umma_commit(smem_u32(&ctl.o_empty[slo]), leader);
+      if (it + 1 < n) ok = mbar_wait_warp(smem_u32(&ctl.o_full[nslo]), pho, abort);
+      if (ok) ok = mbar_wait_warp(smem_u32(&ctl.ds_full[it & 1]), (it >> 1) & 1, abort);
       if (!ok) break;
       tc_fence_after_sync();
       {
@@ -282,13 +282,9 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
         for (int h = 0; h < 2; ++h)
           umma_ts4<8, 32, 40, 2048>(tmem + Cfg::kColK, tmem + Cfg::kColP + h * 64, desc_advance(dB, h * 4 * 2048), idesc_a,
                                     h > 0 ? 1u : acc0, leader);
-        umma_commit(smem_u32(&ctl.q_empty[slq]), leader);
       }
-      if (it + 1 < n) {
-        ok = mbar_wait_warp(smem_u32(&ctl.o_full[nslo]), pho, abort);
-        if (!ok) break;
-        scores(descV, desc_advance(descO, nslo * Cfg::kTileBytes), tmem + Cfg::kColP, &ctl.dp_full);
-      }
+      if (it + 1 < n) scores(descV, desc_advance(descO, nslo * Cfg::kTileBytes), tmem + Cfg::kColP, &ctl.dp_full);
+      umma_commit(smem_u32(&ctl.q_empty[slq]), leader);
       slq = nslq; slo = nslo;
     }
     if (ok) umma_commit(smem_u32(&ctl.acc_done), leader);
@@ -333,7 +329,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
         cur[k] = nxt[k];
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&ctl.st_full[b]));
+      if (lane == 0) mbar_arrive(smem_u32(&ctl.s_full[b]));
       qt = qt_n; hd = hd_n;
     }
   } else if (warp >= 4) {
@@ -357,11 +353,9 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     for (int it = 0; it < n; ++it) {
       const int b = it & 1;
       const int lo = q_first - q0 - wg * 32;     // columns below it do not see the key
-      ok = mbar_wait_warp(smem_u32(&ctl.st_full[b]), (it >> 1) & 1, abort);
-      if (!ok) break;
       const float4* nl2v = reinterpret_cast<const float4*>(st_nl2 + b * kQRows + wg * 32);
       const float4* Dv = reinterpret_cast<const float4*>(st_D + b * kQRows + wg * 32);
-      ok = mbar_wait_warp(smem_u32(&ctl.s_full), it & 1, abort);
+      ok = mbar_wait_warp(smem_u32(&ctl.s_full[b]), (it >> 1) & 1, abort);
       if (!ok) break;
       tc_fence_after_sync();
       // P^T in halves of 16 columns: the tensor core starts dV on the first halves while the second are formed
@@ -393,8 +387,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
           tmem_st8(S_addr + 8 * h, pp);   // over the first half of this warpgroup's own columns, already loaded
           tmem_wait_st();
           tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&ctl.p_full[h]));
+          mbar_arrive(smem_u32(&ctl.p_full[h]));
         }
       }
       ok = mbar_wait_warp(smem_u32(&ctl.dp_full), it & 1, abort);
@@ -434,8 +427,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
       tmem_st16(P_addr, ds);
       tmem_wait_st();
       tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&ctl.ds_full[b]));
+      mbar_arrive(smem_u32(&ctl.ds_full[b]));
       float c8[8];   // index 2j + e: column 8j + 2(lane%4) + e of the warpgroup's 32
 #pragma unroll
       for (int j = 0; j < 4; ++j)
