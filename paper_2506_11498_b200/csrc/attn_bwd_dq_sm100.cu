@@ -9,8 +9,8 @@
 //   S  = Q K_j^T          (TMEM x smem -> TMEM)      P  = exp2(S*c - LSE*log2e)
 //   dP = dO V_j^T         (TMEM x smem -> TMEM)      dS = P * (dP - D)          (bf16, back into TMEM)
 //   A += dS K_j           (TMEM x smem -> TMEM)      epilogue: dQ = scale * (A - r * kbar) -> bf16
-// S/dP are double-buffered in TMEM, so the tensor core computes tile j+1 while tile j is in the
-// softmax; both softmax warpgroups work on every tile (32 key columns each) to keep the latency
+// S/dP are double-buffered in TMEM (NB = 2; NB = 1, two CTAs per SM: see launch_bwd_dq_sm100), so the
+// tensor core computes tile j+1 while tile j is in the softmax; both softmax warpgroups work on every tile (32 key columns each) to keep the latency
 // between "S ready" and "dS ready" short.  One warp issues all products, A_j before S_{j+2} and dP_{j+2}, which may then
 // overwrite the buffer without a barrier round trip (with a warp for each product and a "buffer free" barrier: whole step
 // 372 against 366 us at 4K tokens, 28/4 heads, d = 128; 3.96 against 3.86 ms for 32K tokens in eight sequences).
@@ -32,19 +32,20 @@ using namespace ptx;
 constexpr int kKeys = 64;   // keys per tile in this kernel
 constexpr int kShort = 16;
 
-template <int D>
+template <int D, int NB>
 struct DqCfg {
   static constexpr int kSub = D / 64;
   static constexpr int kQSubBytes = kTile * 128;           // 128 query rows x 128 bytes
   static constexpr int kQTileBytes = kSub * kQSubBytes;    // the Q or the dO tile
   static constexpr int kKSubBytes = kKeys * 128;           // 64 key rows x 128 bytes
   static constexpr int kKTileBytes = kSub * kKSubBytes;    // one K or V tile
-  static constexpr int kStages = D == 128 ? 9 : 16;        // ring slots, K and V tiles alternate
+  static constexpr int kStages = D == 128 ? 9 : 8 * NB;    // ring slots, K and V tiles alternate
   static constexpr int kSmem = 2 * kQTileBytes + kStages * kKTileBytes + 1024;
   static constexpr int kThreads = 384;
+  static constexpr int kPerSm = 3 - NB, kCols = 256 * NB;   // resident CTAs, TMEM columns
   // TMEM columns: Q and dO as packed bf16 (D/2 columns each), accumulator A at D, then buffer b with
-  // S at 256 + 128b and dP 64 columns further
-  static constexpr uint32_t kColQ = 0, kColdO = D / 2, kColA = D, kColBuf = 256, kColP = 64;
+  // S at 128 NB + 128 b and dP 64 columns further
+  static constexpr uint32_t kColQ = 0, kColdO = D / 2, kColA = D, kColBuf = 128 * NB, kColP = 64;
 };
 
 template <int NSEQ>
@@ -71,10 +72,10 @@ struct DqBars {
   uint64_t s_full[2], p_full[2];
 };
 
-template <int D, int NSEQ>
-__global__ void __launch_bounds__(DqCfg<D>::kThreads, 1)
+template <int D, int NSEQ, int NB>
+__global__ void __launch_bounds__(DqCfg<D, NB>::kThreads, DqCfg<D, NB>::kPerSm)
 lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_constant__ DqArgs<NSEQ> a) {
-  using Cfg = DqCfg<D>;
+  using Cfg = DqCfg<D, NB>;
   constexpr int NS = Cfg::kStages;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) DqBars bars;
@@ -112,7 +113,7 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
     }
     fence_barrier_init();
   }
-  if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), 512); tmem_relinquish(); }
+  if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), Cfg::kCols); tmem_relinquish(); }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -157,9 +158,9 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
       }
     }
   } else if (warp == 1) {
-    // ---------------- issuer: S_j, dP_j two tiles ahead of A += dS_j K_j ----------------
-    // One warp issues everything, so the products run in this order on the tensor core: S_{j+2} may overwrite dS_j, and
-    // dP_{j+2} dP_j, without waiting for the product that reads dS_j.
+    // ---------------- issuer: S_j, dP_j NB tiles ahead of A += dS_j K_j ----------------
+    // One warp issues everything, so the products run in this order on the tensor core: S_{j+NB} may overwrite dS_j, and
+    // dP_{j+NB} dP_j, without waiting for the product that reads dS_j.
     constexpr uint32_t idesc_full = make_idesc_bf16(kTile, kKeys, 0, 0), idesc_short = make_idesc_bf16(kTile, kShort, 0, 0);
     constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);       // 128 x D, B = K_j MN-major
     const uint64_t descR = make_smem_desc_sw128(sRing, 16, 1024);       // K-major K_j / V_j
@@ -176,11 +177,11 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
     };
     bool ok = mbar_wait_warp(smem_u32(&bars.qt_ready), 0, abort);   // Q and dO are in tensor memory
     tc_fence_after_sync();
-    for (int j = -2; j < n && ok; ++j) {
-      const int b = j & 1;
+    for (int j = -NB; j < n && ok; ++j) {
+      const int b = j & (NB - 1);
       const uint32_t buf = tmem + Cfg::kColBuf + b * 128;
       if (j >= 0) {
-        ok = mbar_wait_warp(smem_u32(&bars.p_full[b]), (j >> 1) & 1, abort);
+        ok = mbar_wait_warp(smem_u32(&bars.p_full[b]), (j >> (NB - 1)) & 1, abort);
         if (!ok) break;
         tc_fence_after_sync();
         // packed dS: keys [0,32) in columns [0,16) of the S region, keys [32,64) in columns [32,48)
@@ -191,8 +192,8 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
         slot_a += 2;
         if (slot_a >= NS) slot_a -= NS;
       }
-      if (j + 2 < n) {
-        const uint32_t idesc_s = j + 2 < sh ? idesc_short : idesc_full;
+      if (j + NB < n) {
+        const uint32_t idesc_s = j + NB < sh ? idesc_short : idesc_full;
         ok = scores(buf, tmem + Cfg::kColQ, idesc_s);
         if (++slot == NS) { slot = 0; ph ^= 1; }
         if (ok) ok = scores(buf + Cfg::kColP, tmem + Cfg::kColdO, idesc_s);
@@ -260,8 +261,8 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
       if (ok) mbar_arrive(smem_u32(&bars.p_full[0]));
     }
     for (int j = sh; j < n && ok; ++j) {
-      const int b = j & 1;
-      ok = mbar_wait(smem_u32(&bars.s_full[b]), (j >> 1) & 1, abort);
+      const int b = j & (NB - 1);
+      ok = mbar_wait(smem_u32(&bars.s_full[b]), (j >> (NB - 1)) & 1, abort);
       if (!ok) break;
       tc_fence_after_sync();
       const uint32_t S_addr = tmem + lane_addr + Cfg::kColBuf + b * 128 + half * 32;
@@ -347,15 +348,15 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
 
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 1) tmem_dealloc(tmem, Cfg::kCols);
   if (tid == 0 && abort_s) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
 }
 
 }  // namespace
 
-template <int D, int NSEQ>
+template <int D, int NSEQ, int NB>
 static int launch_dq_t(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, cudaStream_t st) {
-  using Cfg = DqCfg<D>;
+  using Cfg = DqCfg<D, NB>;
   DqMaps<NSEQ> m;
   DqArgs<NSEQ> a;
   const long long BHq = (long long)whole.B * whole.Hq, BHkv = (long long)whole.B * whole.Hkv;
@@ -383,7 +384,7 @@ static int launch_dq_t(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, c
   a.status = p.status;
   const long long grid = (long long)a.block0[b.n] * a.BH;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  auto kern = lrsa_bwd_dq_kernel<D, NSEQ>;
+  auto kern = lrsa_bwd_dq_kernel<D, NSEQ, NB>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
   LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));
   launch_counter().n++;
@@ -391,8 +392,15 @@ static int launch_dq_t(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, c
 }
 
 int launch_bwd_dq_sm100(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, cudaStream_t st) {
-  if (whole.d == 128) return b.n == 1 ? launch_dq_t<128, 1>(whole, b, p, st) : launch_dq_t<128, kMaxSeqs>(whole, b, p, st);
-  return b.n == 1 ? launch_dq_t<64, 1>(whole, b, p, st) : launch_dq_t<64, kMaxSeqs>(whole, b, p, st);
+  // d = 64: one S/dP buffer per CTA and two CTAs per SM, which start and end at different times, once every SM has more than
+  // two CTAs to run (whole step, 8 heads: 8K tokens 266 -> 260 us, 8 x 2000 333 -> 320; 16/2 heads, 5K: 225 -> 218);
+  // otherwise two buffers, the shorter chain of a CTA alone (4K, 264 CTAs: 123.7 us, with one buffer 127.4).
+  long long ctas = 0;
+  for (int s = 0; s < b.n; ++s) ctas += (long long)make_plan(b.g[s], kTile).total * whole.B * whole.Hq;
+  const auto dq = whole.d == 128   ? (b.n == 1 ? launch_dq_t<128, 1, 2> : launch_dq_t<128, kMaxSeqs, 2>)
+                  : ctas > 2 * 148 ? (b.n == 1 ? launch_dq_t<64, 1, 1> : launch_dq_t<64, kMaxSeqs, 1>)
+                                   : (b.n == 1 ? launch_dq_t<64, 1, 2> : launch_dq_t<64, kMaxSeqs, 2>);
+  return dq(whole, b, p, st);
 }
 
 }  // namespace lrsa

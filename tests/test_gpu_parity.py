@@ -124,11 +124,11 @@ def test_attention_fwd_bwd(w, ndp):
 
 
 @pytest.mark.parametrize("S", [1, 16, 17, 80])
-@pytest.mark.parametrize("d", [64, 128])
-def test_last_list_tile_of_few_keys(d, S):
+@pytest.mark.parametrize("d,B", [(64, 1), (128, 1), (64, 20)])
+def test_last_list_tile_of_few_keys(d, B, S):
     """K = 128 leaves S keys for the last tile of the sinks + kept list: the short form of the tile takes up to 16 (in the dQ
-    kernel, whose tiles hold 64 keys, S = 80 is 64 + 16)."""
-    w = W(f"a_tail{S}", 1, 2, 1, S + 900, d, 256, 128, S, seed=35)
+    kernel, whose tiles hold 64 keys, S = 80 is 64 + 16).  Batch 20: the dQ kernel's form for many CTAs at d = 64."""
+    w = W(f"a_tail{S}", B, 2, 1, S + 900, d, 256, 128, S, seed=35)
     host = workloads.generate(w)
     bits = host_bits(host)
     op = oparams(w, n_dense_prev=1)
