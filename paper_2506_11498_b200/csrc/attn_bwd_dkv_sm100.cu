@@ -116,24 +116,6 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
   const uint32_t sK = smem0, sV = smem0 + Cfg::kTileBytes;
   const uint32_t sQ = smem0 + Cfg::kOffRingQ, sO = smem0 + Cfg::kOffRingO;
 
-  // ---- which tile, which segment ----
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int bh_kv = blockIdx.x % a.BHkv;
-  int seg = blockIdx.x / a.BHkv, sq = 0;
-  if constexpr (NSEQ > 1) {
-    while (sq + 1 < a.n_seqs && seg >= a.seg0[sq + 1]) ++sq;
-    seg -= a.seg0[sq];
-  }
-  const DkvPlan& p = a.plan[sq];
-  const int tok0 = a.tok0[sq];
-  const int32_t* kept = a.idx + (size_t)bh_kv * a.kept_stride + a.kept_off[sq];   // this head's, this sequence's windows
-  const int2 ts = a.seg_map[a.map0[sq] + seg];
-  const KvTile kt = describe_tile(p, ts.x);
-  const int it_begin = ts.y * p.seg;
-  const int n = min(p.seg, p.G * kt.nq - it_begin);
-  const int hq0 = (bh_kv / a.Hkv) * a.Hq + (bh_kv % a.Hkv) * p.G;   // first query head of the group
-
   if (smem0 & 1023u) {   // the swizzled tiles need it; dynamic shared memory starts there when nothing is static
     if (tid == 0) atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
     return;
@@ -158,6 +140,25 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
   tc_fence_after_sync();
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort = &ctl.abort;
+
+  // ---- which tile, which segment ----
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int bh_kv = blockIdx.x % a.BHkv;
+  int seg = blockIdx.x / a.BHkv, sq = 0;
+  if constexpr (NSEQ > 1) {
+    while (sq + 1 < a.n_seqs && seg >= a.seg0[sq + 1]) ++sq;
+    seg -= a.seg0[sq];
+  }
+  const DkvPlan& p = a.plan[sq];
+  const int tok0 = a.tok0[sq];
+  const int32_t* kept = a.idx + (size_t)bh_kv * a.kept_stride + a.kept_off[sq];   // this head's, this sequence's windows
+  const int2 ts = a.seg_map[a.map0[sq] + seg];
+  const KvTile kt = describe_tile(p, ts.x);
+  const int it_begin = ts.y * p.seg;
+  const int n = min(p.seg, p.G * kt.nq - it_begin);
+  const int hq0 = (bh_kv / a.Hkv) * a.Hq + (bh_kv % a.Hkv) * p.G;   // first query head of the group
+
   // iteration gi of the tile: query tile nq-1 - gi/G (from the last query backwards) of head gi % G
   const int qt0 = kt.nq - 1 - it_begin / p.G, hd0 = it_begin % p.G;
 
