@@ -19,7 +19,8 @@
 // What bounds it: the chain of a tile from S_t over its exponentials (one MUFU result per two clocks and thread, 1024
 // cycles a tile) to O_t and the next S_t, and the 1000 W power limit, under which the clock settles near 1.65 GHz.
 // At 32K tokens, 28/4 heads, d = 128, one kept token in four: 2.75 -> 2.44 ms (of 1.50 at the measured bf16 rate); at
-// 64K 9.5 -> 8.5 ms, 15.1 -> 13.3 M cycles.  Before, two warps issued (S, and O += P V), with a barrier round trip
+// 64K 9.5 -> 8.5 ms, 15.1 -> 13.3 M cycles; with the products issued by predicate 2.14 and 8.52 ms for
+// whole prefill calls, selection included (2.02 the kernel alone and uncapped, tensor pipe 62 %, was 51).  Before, two warps issued (S, and O += P V), with a barrier round trip
 // between a tile's products; scores were read twice; P was handed over in one piece.  Also measured: sixteen softmax
 // warps (16 rows x 128 columns each, 256-bit loads): 2.66 ms; exponentials started with the previous maximum, the tile
 // taken again when it was raised: 2.47 ms; a share of them on the FMA pipe: no gain at 1/8, 2.63 ms at 1/4.
