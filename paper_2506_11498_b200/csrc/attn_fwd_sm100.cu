@@ -296,6 +296,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
           if (i >= limit) s[i] = 0xff800000u;
           m = fmaxf(m, __uint_as_float(s[i]));
         }
+        if (m == -INFINITY) m = 0.f;   // no key of the tile counts: P = 0, as in the full tiles below
 #pragma unroll
         for (int i = 0; i < kShort / 2; ++i) {
           const float p0 = ex2(fmaf(__uint_as_float(s[2 * i]), c, -m * c)), p1 = ex2(fmaf(__uint_as_float(s[2 * i + 1]), c, -m * c));

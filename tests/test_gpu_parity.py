@@ -143,6 +143,29 @@ def test_last_list_tile_of_few_keys(d, B, S):
     check_close("dV", f64(dV), odV)
 
 
+@pytest.mark.parametrize("S", [1, 4, 16, 40])
+@pytest.mark.parametrize("d,B,L,n", [(64, 1, 256, 700), (128, 1, 256, 700), (128, 30, 1024, 2100)])
+def test_sinks_with_scores_of_minus_infinity(d, B, L, n, S):
+    """A score that overflows to -inf has probability zero, also where the sinks are all that a query's first list tile
+    holds (up to 16 of them: the short tile; batch 30: two query tiles per CTA).  The queries at the sinks see nothing else
+    and have no defined output."""
+    w = W(f"a_inf{S}", B, 2, 1, S + n, d, L, 64, S, seed=37)
+    host = workloads.generate(w, ("Q", "K", "V"))
+    host["Q"][..., 0] = 4.0
+    host["K"][:, :, :S] = 0.0
+    host["K"][:, :, :S, 0] = -3e38
+    dev = to_dev(host)
+    p = lrsa.Params.from_workload(w)
+    idx, _ = lrsa.lrsa_score_select(p, dev["K"], dev["V"])
+    O, LSE = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx)
+    one = w.with_(B=1)
+    bits = host_bits({k: v[:1] for k, v in host.items()})
+    oO, oL = orc.attn_fwd(oparams(one), bits["Q"], bits["K"], bits["V"], idx[:1].cpu().numpy())
+    check_close("O", f64(O[:1, :, S:]), oO[:, :, S:])
+    check_close("LSE", f64(LSE[:1, :, S:]), oL[:, :, S:], max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
+    assert torch.isfinite(O[:, :, S:].float()).all() and torch.isfinite(LSE[:, :, S:]).all()
+
+
 @pytest.mark.parametrize("S,N", [(1, 2949), (17, 3300)])
 def test_one_and_two_query_tiles_per_cta_agree(S, N):
     """The forward of four sequences runs with two query tiles per CTA, that of one with one (fewer CTAs): every row does the
