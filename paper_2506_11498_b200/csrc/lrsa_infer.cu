@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
           for (int e = 0; e < 2; ++e) {
 #pragma unroll
             for (int x = 4; x < 32; x <<= 1) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], x));
-            const float mn = fmaxf(m[h][e], mx[e]);   // finite: a block holds at least one key
+            const float mn = fmaxf(m[h][e], mx[e]);   // -inf while every score has been (f = 0 then)
             const float f = m[h][e] == -INFINITY ? 0.f : exp2f(m[h][e] - mn);
             m[h][e] = mn;
             l[h][e] *= f;
@@ -276,12 +276,13 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
             for (int i = 0; i < MT; ++i) { o[h][i][e] *= f; o[h][i][e + 2] *= f; }
           }
         }
+        const float ref[2] = {m[h][0] == -INFINITY ? 0.f : m[h][0], m[h][1] == -INFINITY ? 0.f : m[h][1]};
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           float p[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            p[e] = exp2f(s[u][e] - m[h][e & 1]);
+            p[e] = exp2f(s[u][e] - ref[e & 1]);
             l[h][e & 1] += p[e];
           }
           const uint32_t b0 = transpose_8x8(ptx::pack_bf16(p[0], p[1])), b1 = transpose_8x8(ptx::pack_bf16(p[2], p[3]));
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
         float ov = 0.f, ls = 0.f;
 #pragma unroll 4
         for (int r = 0; r < a.n_split; ++r) {
-          const float f = exp2f(ld_cluster(&fin_m[hd], r) - M);   // every split holds at least one key: finite
+          const float f = M == -INFINITY ? 0.f : exp2f(ld_cluster(&fin_m[hd], r) - M);   // -inf: no score of the head was finite
           ov = fmaf(ld_cluster(&fin_o[hd][c], r), f, ov);
           ls = fmaf(ld_cluster(&fin_l[hd], r), f, ls);
         }
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* part, __nv
   float ov = 0.f, ls = 0.f;
 #pragma unroll 4
   for (int r = 0; r < n_group; ++r) {
-    const float f = exp2f(__ldcg(base + r * stride + D) - M);
+    const float f = M == -INFINITY ? 0.f : exp2f(__ldcg(base + r * stride + D) - M);
     ov = fmaf(__ldcg(base + r * stride + c), f, ov);
     ls = fmaf(__ldcg(base + r * stride + D + 1), f, ls);
   }

@@ -156,3 +156,34 @@ def test_decode_against_fp64(G, d, B, N):
     want = torch.einsum("bhgk,bhkd->bhgd", s.softmax(-1), vv).reshape(B, 2 * G, d)
     check_close("o", f64(o), want.cpu().numpy())
     check_close("lse", f64(lse), s.logsumexp(-1).reshape(B, 2 * G).cpu().numpy(), max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("G", [7, 12])
+@pytest.mark.parametrize("S,N", [(32, 33), (32, 700), (1024, 9000), (40000, 70000), (500, 500)])
+def test_decode_scores_of_minus_infinity(d, G, S, N):
+    """Keys whose scores overflow to -inf have probability zero, also where a warp's block, a CTA or a whole cluster (long
+    caches: several for a head) has no other key: the output is that of attention over the remaining keys.  With no other key at all
+    (S = N) it is not defined, and lse is -inf."""
+    L, K = 256, 256 if N > 2500 else 64
+    g = torch.Generator(device="cuda").manual_seed(8)
+    k, v = (torch.randn((1, 2, N, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    q = torch.randn((1, 2 * G, d), generator=g, device="cuda").bfloat16()
+    q[..., 0] = 4.0
+    k[:, :, :S] = 0.0
+    k[:, :, :S, 0] = -3e38
+    cache = lrsa.KVCache(lrsa.Params(1, 2 * G, 2, N, d, L, K, S))
+    cache.append(k, v)
+    o, lse = cache.decode(q)
+    assert cache.status() == 0
+    if S == N:
+        assert (lse == -float("inf")).all()
+        return
+    nc = cache.windows_compressed()
+    pos = torch.cat([cache.kept()[0, :, :nc].reshape(2, -1).long(), torch.arange(S + nc * L, N, device="cuda").expand(2, -1)], -1)
+    ix = pos[..., None].expand(-1, -1, d)
+    kk, vv = k[0].gather(1, ix).double(), v[0].gather(1, ix).double()
+    s = torch.einsum("hgd,hkd->hgk", q.double().view(2, G, d), kk) / d ** 0.5
+    want = torch.einsum("hgk,hkd->hgd", s.softmax(-1), vv).reshape(1, 2 * G, d)
+    check_close("o", f64(o), want.cpu().numpy())
+    check_close("lse", f64(lse), s.logsumexp(-1).reshape(1, 2 * G).cpu().numpy(), max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
