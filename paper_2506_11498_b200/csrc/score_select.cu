@@ -646,6 +646,9 @@ score_select_cluster_kernel(const __grid_constant__ ScoreArgs a, const __grid_co
   }
 }
 
+// Longest window the one-slice-per-CTA kernel takes: 25 448 tokens, 201 KB of selection scratch.
+constexpr int kUnitMaxL = 25448;
+
 template <int D>
 constexpr int tok_per_unit() { return kSteps * (kThreads / (D / 8)); }
 
@@ -763,6 +766,7 @@ static int launch_cluster(const Geom* gs, int n_seqs, const __nv_bfloat16* K, co
 static int launch_unit(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat16* V, int32_t* idx, float* score, void* ws,
                        cudaStream_t st) {
   if (g.Wsel == 0) return LRSA_OK;  // nothing is scored
+  if (g.L > kUnitMaxL) return LRSA_ERR_UNSUPPORTED;
   const ScoreWs lay = score_ws_layout(g);
   unsigned char* base = static_cast<unsigned char*>(ws);
   // The status word (the header) is cleared once per call by the caller; the ticket, the counters and the statistics here.
@@ -777,7 +781,6 @@ static int launch_unit(const Geom& g, const __nv_bfloat16* K, const __nv_bfloat1
   const int tok = g.d == 128 ? tok_per_unit<128>() : tok_per_unit<64>();
   a.n_slices = (g.L + tok - 1) / tok;
   const size_t smem = select_smem_bytes(g.L, g.d);
-  if (smem > 200 * 1024) return LRSA_ERR_UNSUPPORTED;
   const long long units = (long long)a.BH * g.W * a.n_slices;
   if (units > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
   auto kern = g.d == 128 ? score_select_kernel<128> : score_select_kernel<64>;

@@ -51,6 +51,25 @@ def test_score_select(w, ddof):
     assert torch.equal(idx, idx2)
 
 
+def test_longest_window_that_is_scored():
+    """25 448 tokens is the longest lag window of the selection (its scores lie in shared memory); one more is refused."""
+    w = W("s_longest", 1, 1, 1, 2 * 25448 + 1, 64, 25448, 700, 1, seed=44)
+    host = workloads.generate(w, ("K", "V"))
+    bits = host_bits(host)
+    oidx, osc = orc.score_select(oparams(w), bits["K"], bits["V"])
+    dev = to_dev(host)
+    p = lrsa.Params.from_workload(w)
+    ws = lrsa.new_workspace(lrsa.lrsa_workspace_bytes(p)[0])
+    idx, sc = lrsa.lrsa_score_select(p, dev["K"], dev["V"], workspace=ws, want_score=True)
+    assert lrsa.lrsa_workspace_status(ws) == 0
+    np.testing.assert_allclose(f64(sc), osc, rtol=2e-5, atol=0)
+    compare_idx(idx.cpu().numpy(), oidx, osc, w.S, w.L)
+    longer = lrsa.Params(1, 1, 1, 2 * 25449, 64, 25449, 700, 0)
+    with pytest.raises(lrsa.LrsaError) as e:
+        lrsa.lrsa_score_select(longer, dev["K"], dev["V"])
+    assert e.value.status == 2
+
+
 def test_score_zero_range_channel():
     w = W("s_const", 1, 2, 2, 2 + 4 * 128, 128, 128, 32, 2, seed=20)
     host = workloads.generate(w, ("K", "V"))
