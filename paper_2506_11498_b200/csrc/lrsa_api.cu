@@ -1,6 +1,8 @@
 // C ABI entry points: argument validation on the host, workspace layout, kernel dispatch.
 #include <math.h>
 
+#include <mutex>
+
 #include "attn_common_sm100.h"
 
 namespace lrsa {
@@ -8,6 +10,44 @@ namespace lrsa {
 LaunchCounter& launch_counter() {
   static thread_local LaunchCounter c;
   return c;
+}
+
+// Never launched: stands for a kernel of one CTA per 1 / per_sm of an SM's shared memory.
+static __global__ void room_kernel() {}
+
+// The groups of SMs that a cluster has to fit into differ in size and between devices, so the device is asked.  (With eight groups
+// of 18 SMs assumed, eight clusters of 16 large CTAs were planned for where seven run: one sequence of 8/8 heads, d = 64,
+// 8.7K keys 17.9 us instead of 10.7 with clusters of eight, 32/8 heads, d = 128, 9.5K keys 26.1 instead of 16.6.)
+static void ask_room(ClusterRoom* room) {
+  const bool ok = cudaFuncSetAttribute(room_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10) == cudaSuccess &&
+                  cudaFuncSetAttribute(room_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  for (int p = 0; p < 3; ++p)
+    for (int c = 0; c < 5; ++c) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(1 << c);
+      cfg.blockDim = dim3(128);
+      cfg.dynamicSmemBytes = (200 << 10) >> p;
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = 1 << c;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      // (none, or no answer: such clusters take turns in every plan)
+      room->n[p][c] = ok && cudaOccupancyMaxActiveClusters(&n, room_kernel, &cfg) == cudaSuccess && n > 0 ? n : 1;
+    }
+  (void)cudaGetLastError();
+}
+
+const ClusterRoom& cluster_room() {
+  constexpr int kDevices = 64;
+  static ClusterRoom room[kDevices];
+  static std::once_flag asked[kDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) dev = 0;
+  std::call_once(asked[dev], ask_room, &room[dev]);
+  return room[dev];
 }
 
 static int g_impl = 0;  // 0: tensor-core kernels, 1: CUDA-core validation kernels

@@ -422,17 +422,18 @@ DecodePlan decode_plan(const Geom& g, int n_keys, int max_splits = kDecMaxSplits
   // 16 warps (8 with two groups of heads) are resident per SM, as one large CTA or several small ones.  Large ones
   // have fewer partial results to merge; small ones fill the SMs more evenly when every SM has several blocks per warp
   // to do.  A round of blocks takes about 1.3 us, a CTA's start and merge as long as two, the second kernel as three; a
-  // cluster lies in one of the eight groups of 18 SMs.  (One sequence, 4 heads, d = 128: 9471 keys, one cluster for a
+  // cluster lies in one group of SMs (ClusterRoom).  (One sequence, 4 heads, d = 128: 9471 keys, one cluster for a
   // head 17.7 us a token with 8 CTAs, 15.8 with 16; 66 000 keys 107 us with one cluster of 16, 34.5 with two.)
   const int max_warps = dec_max_warps(p.nh);
   p.warps = BH * p.blocks > 2LL * 148 * max_warps ? 4 : max_warps;
   const int per_sm = max_warps / p.warps;
+  const ClusterRoom& room = cluster_room();
   long long best = -1;
   for (int s = 1; s <= max_splits; s *= 2)
     for (int grp = 1; grp <= kDecMaxGroups; grp *= 2) {
       const int n = s * grp;
       if (n > 1 && ((n - 1) * p.warps >= p.blocks || BH * n > 148LL * per_sm * 4)) break;
-      const long long at_once = s == 1 ? 148 * per_sm : 8 * (18 * per_sm / s);
+      const long long at_once = room.at_once(per_sm, s);
       const long long waves = (BH * grp + at_once - 1) / at_once;
       const int per_cta = (p.blocks + n - 1) / n;
       const long long cost = waves * ((per_cta + p.warps - 1) / p.warps + 2) + (grp > 1 ? 3 : 0);

@@ -141,6 +141,18 @@ cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// lrsa_api.cu : clusters of 2^c CTAs that the current device runs at a time with 2^p CTAs on an SM, n[p][c].
+struct ClusterRoom {
+  int n[3][5];
+  int at_once(int per_sm, int cluster) const {
+    int p = 0, c = 0;
+    while ((1 << p) < per_sm) ++p;
+    while ((1 << c) < cluster) ++c;
+    return n[p][c];
+  }
+};
+const ClusterRoom& cluster_room();
+
 #define LRSA_CUDA_CHECK(expr)                                 \
   do {                                                        \
     cudaError_t _e = (expr);                                  \
