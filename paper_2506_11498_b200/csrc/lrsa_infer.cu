@@ -12,8 +12,9 @@
 // chunk c arrives: not earlier, because the queries of chunk c-1 still see it whole.
 //
 // Decode attention reads the list prefix and the ring once per KV head for (up to 16) query heads of the group
-// (HBM-bound: 4*d bytes per key, a few FMAs per byte): the keys are split over CTAs and warps, every warp keeps an
-// online softmax of its keys, and the CTAs of a head form a cluster that merges the partial results.
+// (HBM-bound: 4*d bytes per key, a few FMAs per byte).  Two kernels: in decode_kernel the keys are split over CTAs and
+// warps, every warp keeps an online softmax of its keys, and the CTAs of a head form a cluster that merges the partial
+// results; decode_split_kernel (groups of more than eight heads, use_split_kernel) takes 128 keys a CTA and a merge kernel.
 #include "lrsa_internal.h"
 #include "sm100_ptx.h"
 
@@ -103,22 +104,38 @@ int launch_cache_rows(CacheRows a, int BH, cudaStream_t st) {
 
 // ---- decode attention ----
 constexpr int kDecMaxWarps = 16;
+constexpr int kDecThreads = 128;  // of the split kernel
+constexpr int kDecHeads = 16;     // its query heads of a group per pass over the keys (the M of the tensor-core product)
+constexpr int kDecKeys = 128;     // its keys per CTA (32 per warp), staged in shared memory
 // Warps of the largest CTA: 128 registers hold the operands of one group of 8 heads; two groups take more.
 __host__ __device__ constexpr int dec_max_warps(int nh) { return nh == 1 ? kDecMaxWarps : kDecMaxWarps / 2; }
 
 struct DecodeArgs {
   const __nv_bfloat16 *q, *k_list, *k_ring;
   long long v_of_list, v_of_ring;   // bytes from a K row to its V row
-  float* part;          // [BHkv][n_group][G][D + 2]: unnormalised output, maximum (log2 domain), sum
+  float* part;          // [BHkv][n_group, or splits][G][D + 2]: unnormalised output, maximum (log2 domain), sum
   __nv_bfloat16* o;     // [B][Hq][D]
   float* lse;           // [B][Hq], optional
   int* status;          // workspace status word
   int Hq, Hkv, G, rows_list, ring_rows;
   int n_list, n_keys, ring0;   // keys: list rows [0, n_list), then ring rows from ring row ring0 on (wrapping)
   int n_split, n_group, blocks;   // key blocks per (batch, KV head), dealt out evenly to n_group clusters of n_split CTAs
+                                  // (split kernel: n_split CTAs of kDecKeys keys)
   float scale_log2;
 };
 
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
 // D (16x8, fp32) += A (16x16, bf16, row) * B (16x8, bf16, col)
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                           uint32_t b1) {
@@ -387,27 +404,265 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
   }
 }
 
-// Merges the clusters of one (batch, query head): one thread per channel.
+// Decode of groups of more than eight query heads where the whole work is a wave or so of small CTAs (use_split_kernel).
+// Grid (n_split, BHkv), one CTA of four warps per kDecKeys keys.  The query heads of the group are the rows of the products
+// (16 a pass; the unused ones zero), so a 16-head group costs what one head does, where decode_kernel above repeats its products
+// for every eight heads and, with the second group's operands, has half as many warps an SM.  Every key row of the CTA is
+// fetched at once (a bulk copy each of K and of V per thread) into rows padded by 16 bytes, and everything after
+// that is short: a warp takes 32 keys, Q, K and V fragments through ldmatrix, the softmax of its keys in registers, P as the A operand
+// of the second product.  The four warps are merged through shared memory, the splits by decode_merge_kernel.
+// A layer of a model (caches in turn, larger together than L2; CUDA graph), decode_kernel | this one, us: 20/1 heads, d = 64,
+// 9471 keys 22.7 | 10.6; 24/2, d = 128 17.0 | 11.4; 40/2 24.7 | 14.1, 38 000 keys 39.0 | 42.5; 320/8 62.7 | 47.4.
 template <int D>
-__global__ void __launch_bounds__(D) decode_merge_kernel(const float* part, __nv_bfloat16* o, float* lse, int Hq, int Hkv, int G,
-                                                         int n_group) {
-  const int bhq = blockIdx.x, b = bhq / Hq, hq = bhq % Hq, c = threadIdx.x;
-  const float* base = part + (((size_t)(b * Hkv + hq / G) * n_group) * G + hq % G) * (D + 2);
-  const size_t stride = (size_t)G * (D + 2);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+__global__ void __launch_bounds__(kDecThreads) decode_split_kernel(const DecodeArgs a) {
+  constexpr int CPR = D / 8;                 // 16-byte chunks per row
+  constexpr int KS = D / 16;                 // k-steps of Q K^T
+  constexpr int NT = D / 8;                  // 8-channel tiles of the output
+  constexpr int kRowBytes = D * 2, kStride = kRowBytes + 16;
+  extern __shared__ __align__(128) unsigned char dec_smem[];   // K rows [kDecKeys], V rows [kDecKeys], Q rows [16]
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ int s_fail;
+  const int bh = blockIdx.y, split = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_keys = a.n_keys;
+  const int k_lo = split * kDecKeys, k_hi = min(n_keys, k_lo + kDecKeys), nk = k_hi - k_lo;
+  const int b = bh / a.Hkv, hkv = bh % a.Hkv;
+  const uint32_t sK = ptx::smem_u32(dec_smem), sV = sK + kDecKeys * kStride, sQ = sV + kDecKeys * kStride;
+  unsigned char* gQ = dec_smem + 2 * kDecKeys * kStride;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the cache rows of the kernel in front of this one
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  float M = -INFINITY;
-#pragma unroll 4
-  for (int r = 0; r < n_group; ++r) M = fmaxf(M, __ldcg(base + r * stride + D));
-  float ov = 0.f, ls = 0.f;
-#pragma unroll 4
-  for (int r = 0; r < n_group; ++r) {
-    const float f = M == -INFINITY ? 0.f : exp2f(__ldcg(base + r * stride + D) - M);
-    ov = fmaf(__ldcg(base + r * stride + c), f, ov);
-    ls = fmaf(__ldcg(base + r * stride + D + 1), f, ls);
+  if (tid == 0) {
+    s_fail = 0;
+    ptx::mbar_init(ptx::smem_u32(&bar), 1);
+    ptx::fence_barrier_init();
+    ptx::mbar_expect_tx(ptx::smem_u32(&bar), (uint32_t)nk * kRowBytes * 2);   // every row copy below reports here
+    // the only writer of the status word before a wait below can expire (seconds later)
+    if (split == 0 && bh == 0) *a.status = 0;
   }
-  o[(size_t)bhq * D + c] = __float2bfloat16(ov / ls);
-  if (c == 0 && lse) lse[bhq] = (M + log2f(ls)) * 0.6931471805599453f;
+  __syncthreads();
+  {
+    // this thread's row of K and of V
+    const int r = tid;
+    if (r < nk) {
+      const int k = k_lo + r;
+      const bool in_list = k < a.n_list;
+      const size_t row = in_list ? (size_t)bh * a.rows_list + k
+                                 : (size_t)bh * a.ring_rows + (a.ring0 + (k - a.n_list)) % a.ring_rows;
+      const unsigned char* ks = reinterpret_cast<const unsigned char*>(in_list ? a.k_list : a.k_ring) + row * kRowBytes;
+      bulk_load(sK + r * kStride, ks, kRowBytes, ptx::smem_u32(&bar));
+      bulk_load(sV + r * kStride, ks + (in_list ? a.v_of_list : a.v_of_ring), kRowBytes, ptx::smem_u32(&bar));
+    } else {
+      // rows beyond the split's keys: their probabilities are zero, their V must not be NaN
+#pragma unroll
+      for (int c = 0; c < CPR; ++c) {
+        *reinterpret_cast<uint4*>(dec_smem + r * kStride + c * 16) = make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(dec_smem + (kDecKeys + r) * kStride + c * 16) = make_uint4(0, 0, 0, 0);
+      }
+    }
+  }
+
+  const int row = lane >> 2, cpair = (lane & 3) * 2;   // fragment coordinates of this lane
+  for (int g0 = 0; g0 < a.G; g0 += kDecHeads) {
+    const int ng = min(kDecHeads, a.G - g0);
+    // Q of this pass: 16 rows (heads g0 ..., zero beyond the group) into shared memory, 16 bytes per thread and step
+    for (int i = tid; i < kDecHeads * CPR; i += kDecThreads) {
+      const int g = i / CPR, cch = i % CPR;
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (g < ng) v = *reinterpret_cast<const uint4*>(a.q + ((size_t)(b * a.Hq + hkv * a.G + g0 + g)) * D + cch * 8);
+      *reinterpret_cast<uint4*>(gQ + g * kStride + cch * 16) = v;
+    }
+    if (g0 == 0) {
+      // bounded wait for the copies; a CTA that gives up records it, waits once more for its copies (they write
+      // this CTA's shared memory) and leaves its partial result empty
+      bool got = ptx::mbar_try_wait(ptx::smem_u32(&bar), 0);
+      const long long t0 = clock64();
+      while (!got) {
+        got = ptx::mbar_try_wait(ptx::smem_u32(&bar), 0);
+        if (!got && clock64() - t0 > 4000000000LL) { s_fail = 1; break; }
+      }
+    }
+    __syncthreads();
+    if (s_fail) {
+      if (tid == 0) {
+        atomicExch(a.status, (int)LRSA_ERR_TIMEOUT);
+        const long long t0 = clock64();
+        while (!ptx::mbar_try_wait(ptx::smem_u32(&bar), 0) && clock64() - t0 < 4000000000LL) {}
+      }
+      __syncthreads();
+      // empty partial results: maximum -inf, the merge kernel skips them
+      for (int i = tid; i < ng; i += kDecThreads) {
+        float* dst = a.part + (((size_t)bh * a.n_split + split) * a.G + g0 + i) * (D + 2);
+        dst[D] = -INFINITY; dst[D + 1] = 0.f;
+      }
+      continue;
+    }
+    // Q as A fragments: matrices (heads 0-7, channels k..k+7), (heads 8-15, same), then channels k+8..k+15
+    uint32_t qa[KS][4];
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+      ldmatrix_x4(sQ + ((lane & 7) + 8 * ((lane >> 3) & 1)) * kStride + (2 * ks + (lane >> 4)) * 16, qa[ks]);
+    // S = Q K^T for this warp's 32 keys: four tiles of 8 keys
+    float s[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
+      const int key = warp * 32 + 8 * j + (lane & 7);
+#pragma unroll
+      for (int q4 = 0; q4 < CPR / 4; ++q4) {
+        uint32_t kb[4];
+        ldmatrix_x4(sK + key * kStride + (4 * q4 + (lane >> 3)) * 16, kb);
+        const uint32_t (&q0)[4] = qa[2 * q4], (&q1)[4] = qa[2 * q4 + 1];
+        mma_16816(s[j], q0[0], q0[1], q0[2], q0[3], kb[0], kb[1]);
+        mma_16816(s[j], q1[0], q1[1], q1[2], q1[3], kb[2], kb[3]);
+      }
+    }
+    // scale, mask the keys beyond the split, row maxima and sums (rows: head `row` -> index 0, `row + 8` -> 1)
+    float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int key = warp * 32 + 8 * j + cpair + (e & 1);
+        s[j][e] = key < nk ? s[j][e] * a.scale_log2 : -INFINITY;
+        mx[e >> 1] = fmaxf(mx[e >> 1], s[j][e]);
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+    }
+    float sum[2] = {0.f, 0.f};
+    uint32_t pa[2][4];   // P as A fragments of the two 16-key steps
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float pr[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        pr[e] = mx[e >> 1] == -INFINITY ? 0.f : exp2f(s[j][e] - mx[e >> 1]);
+        sum[e >> 1] += pr[e];
+      }
+      pa[j >> 1][(j & 1) * 2 + 0] = ptx::pack_bf16(pr[0], pr[1]);
+      pa[j >> 1][(j & 1) * 2 + 1] = ptx::pack_bf16(pr[2], pr[3]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      sum[h] += __shfl_xor_sync(0xffffffffu, sum[h], 1);
+      sum[h] += __shfl_xor_sync(0xffffffffu, sum[h], 2);
+    }
+    // O = P V: V fragments transposed on the way out of shared memory (keys are the contraction index)
+    float o[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
+      uint32_t vb[4];
+      ldmatrix_x4_trans(sV + (warp * 32 + lane) * kStride + nt * 16, vb);
+      mma_16816(o[nt], pa[0][0], pa[0][1], pa[0][2], pa[0][3], vb[0], vb[1]);
+      mma_16816(o[nt], pa[1][0], pa[1][1], pa[1][2], pa[1][3], vb[2], vb[3]);
+    }
+    // merge the four warps through shared memory (the K rows are no longer needed once every warp is here;
+    // with more than one pass over the heads they are needed again, so the merge buffer then follows V)
+    __syncthreads();
+    float* mrg = reinterpret_cast<float*>(dec_smem + (a.G > kDecHeads ? (2 * kDecKeys + kDecHeads) * kStride : 0));
+    float* mo = mrg;                                   // [4 warps][16 heads][D]
+    float* mm_ = mrg + 4 * kDecHeads * D;              // [4][16] maxima
+    float* ml = mm_ + 4 * kDecHeads;                   // [4][16] sums
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      *reinterpret_cast<float2*>(mo + ((warp * kDecHeads + row) * D + nt * 8 + cpair)) = make_float2(o[nt][0], o[nt][1]);
+      *reinterpret_cast<float2*>(mo + ((warp * kDecHeads + row + 8) * D + nt * 8 + cpair)) = make_float2(o[nt][2], o[nt][3]);
+    }
+    if ((lane & 3) == 0) {
+      mm_[warp * kDecHeads + row] = mx[0]; mm_[warp * kDecHeads + row + 8] = mx[1];
+      ml[warp * kDecHeads + row] = sum[0]; ml[warp * kDecHeads + row + 8] = sum[1];
+    }
+    __syncthreads();
+    for (int i = tid; i < ng * D; i += kDecThreads) {
+      const int g = i / D, c = i % D;
+      float M = -INFINITY;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) M = fmaxf(M, mm_[w * kDecHeads + g]);
+      float ov = 0.f, lsum = 0.f;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const float mw = mm_[w * kDecHeads + g];
+        const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
+        ov = fmaf(mo[(w * kDecHeads + g) * D + c], f, ov);
+        lsum = fmaf(ml[w * kDecHeads + g], f, lsum);
+      }
+      float* dst = a.part + (((size_t)bh * a.n_split + split) * a.G + g0 + g) * (D + 2);
+      dst[c] = ov;
+      if (c == 0) { dst[D] = M; dst[D + 1] = lsum; }
+    }
+    __syncthreads();   // the merge buffer is reused by the next pass
+  }
+}
+
+// One CTA per (batch, query head): merges the partial results of its splits, or of its clusters.  kRows thread rows (one
+// for clusters, of which there are at most kDecMaxGroups) take alternate results, four at a time with all their loads issued before the
+// arithmetic (the kernel is a chain of L2 round trips otherwise), then the rows are merged through shared memory.
+constexpr int kMergeRows = 8;
+template <int D, int kRows>
+__global__ void __launch_bounds__(kRows * D) decode_merge_kernel(const float* part, __nv_bfloat16* o, float* lse, int Hq,
+                                                                  int Hkv, int G, int n_split) {
+  __shared__ float sm_m[kRows], sm_l[kRows], sm_o[kRows][D];
+  const int bhq = blockIdx.x, b = bhq / Hq, hq = bhq % Hq, hkv = hq / G, g = hq % G;
+  const int c = threadIdx.x % D, row = threadIdx.x / D;
+  const float* base = part + (((size_t)(b * Hkv + hkv) * n_split) * G + g) * (D + 2);
+  const size_t stride = (size_t)G * (D + 2);
+  float M = -INFINITY, acc = 0.f, l = 0.f;
+  constexpr int kBatch = 4;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the partial results of the kernel in front of this one
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int s0 = row; s0 < n_split; s0 += kRows * kBatch) {
+    float ms[kBatch], vs[kBatch], ls[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int s = s0 + u * kRows;
+      const bool in = s < n_split;
+      ms[u] = in ? __ldcg(base + s * stride + D) : -INFINITY;
+      vs[u] = in ? __ldcg(base + s * stride + c) : 0.f;
+      ls[u] = in ? __ldcg(base + s * stride + D + 1) : 0.f;
+    }
+    float mn = M;
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) mn = fmaxf(mn, ms[u]);
+    if (mn == -INFINITY) continue;
+    const float f0 = exp2f(M - mn);   // exp2f(-inf) = 0 while nothing has been merged
+    acc *= f0; l *= f0;
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const float f = exp2f(ms[u] - mn);
+      acc = fmaf(vs[u], f, acc);
+      l = fmaf(ls[u], f, l);
+    }
+    M = mn;
+  }
+  sm_o[row][c] = acc;
+  if (c == 0) { sm_m[row] = M; sm_l[row] = l; }
+  __syncthreads();
+  if (row == 0) {
+    float Mt = -INFINITY;
+    for (int r = 0; r < kRows; ++r) Mt = fmaxf(Mt, sm_m[r]);
+    float at = 0.f, lt = 0.f;
+    for (int r = 0; r < kRows; ++r) {
+      const float f = sm_m[r] == -INFINITY ? 0.f : exp2f(sm_m[r] - Mt);
+      at = fmaf(sm_o[r][c], f, at);
+      lt = fmaf(sm_l[r], f, lt);
+    }
+    o[(size_t)bhq * D + c] = __float2bfloat16(at / lt);
+    if (c == 0 && lse) lse[bhq] = (Mt + log2f(lt)) * 0.6931471805599453f;
+  }
+}
+
+// Groups of more than eight query heads: the split kernel up to three of its CTAs an SM (what is resident), four when
+// decode_kernel goes over the keys more than once (more than 16 heads); beyond, decode_kernel's transfers are the better ones.  Its merge
+// has a CTA per query head: not for hundreds of them.  us, decode_kernel | split kernel (data as in that kernel's head):
+// 18/2 heads, 148 CTAs 16.4 | 11.0, 600 23.6 | 28.1; 72/8, 112 CTAs 12.1 | 9.2, 592 24.1 | 23.8; batch 16 of 18/2, 448 16.5 | 21.5;
+// 160/8, 592 CTAs 40.4 | 32.6; batch 16 of 40/2, 448 CTAs 29.3 | 33.9.
+constexpr int kSplitSms = 148;
+int decode_splits(int n_keys) { return n_keys > 0 ? (n_keys + kDecKeys - 1) / kDecKeys : 1; }
+long long split_ctas_limit(const Geom& g) { return kSplitSms * (g.G > kDecHeads ? 4LL : 3LL); }
+bool use_split_kernel(const Geom& g, int n_keys) {
+  return g.G > 8 && (long long)g.B * g.Hq <= 512 && (long long)g.B * g.Hkv * decode_splits(n_keys) <= split_ctas_limit(g);
 }
 
 // How the keys of the (batch, KV head) pairs are dealt out: to `groups` clusters of `splits` CTAs of `warps` warps each.
@@ -453,6 +708,24 @@ cudaError_t launch_decode_t(DecodeArgs& a, const DecodePlan& pl, int BHkv, cudaS
   return launch_dependent(kern, dim3(pl.splits * pl.groups, BHkv), dim3(pl.warps * 32), 0, st, pl.splits, a);
 }
 
+template <int D>
+cudaError_t launch_split_t(const Geom& g, DecodeArgs& a, cudaStream_t st) {
+  // K and V rows; the merge buffer (4 warps x 16 heads x (d + 2) floats) lies over them, or behind them when the
+  // group has more than 16 query heads and the rows are read again
+  const size_t rows_bytes = (size_t)(2 * kDecKeys + kDecHeads) * (D * sizeof(__nv_bfloat16) + 16);   // K, V and Q rows, padded
+  const size_t merge_bytes = (size_t)4 * kDecHeads * (D + 2) * sizeof(float);
+  const size_t smem = g.G > kDecHeads ? rows_bytes + merge_bytes : (rows_bytes > merge_bytes ? rows_bytes : merge_bytes);
+  const cudaError_t e = cudaFuncSetAttribute(decode_split_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(decode_split_kernel<D>, dim3(a.n_split, g.B * g.Hkv), dim3(kDecThreads), smem, st, 1, a);
+}
+
+template <int kRows>
+cudaError_t launch_merge(const Geom& g, const DecodeArgs& a, int n, cudaStream_t st) {
+  return launch_dependent(g.d == 128 ? decode_merge_kernel<128, kRows> : decode_merge_kernel<64, kRows>, dim3(g.B * g.Hq),
+                          dim3(kRows * g.d), 0, st, 1, (const float*)a.part, a.o, a.lse, g.Hq, g.Hkv, g.G, n);
+}
+
 cudaError_t launch_decode(const Geom& g, DecodeArgs& a, const DecodePlan& pl, cudaStream_t st) {
   const int BHkv = g.B * g.Hkv;
   if (g.d == 128) return pl.nh == 1 ? launch_decode_t<128, 1>(a, pl, BHkv, st) : launch_decode_t<128, 2>(a, pl, BHkv, st);
@@ -480,8 +753,12 @@ int lrsa_cache_bytes(const lrsa_params_t* params, size_t* cache_bytes, size_t* w
     const size_t a = score_select_ws_bytes(all);
     // or the partial results of decode (see decode_plan: several clusters for a head only below 592 CTAs of 16 warps)
     const long long BH = (long long)g.B * g.Hkv;
-    const size_t b = sizeof(WsHeader) +
-                     (BH <= 4 * 592 ? (size_t)BH * kDecMaxGroups * g.G * (g.d + 2) * sizeof(float) : 0);
+    size_t parts = BH <= 4 * 592 ? (size_t)BH * kDecMaxGroups : 0;
+    // (or those of the split kernel; a query never sees more than S + Wcap*K + 2L keys)
+    const size_t splits = (size_t)BH * decode_splits(cache_layout(g).rows_list + 2 * g.L);
+    const size_t most = splits < (size_t)split_ctas_limit(g) ? splits : (size_t)split_ctas_limit(g);
+    if (g.G > 8 && most > parts) parts = most;
+    const size_t b = sizeof(WsHeader) + parts * g.G * (g.d + 2) * sizeof(float);
     *workspace_bytes = a > b ? a : b;
   }
   return LRSA_OK;
@@ -635,6 +912,13 @@ int lrsa_attn_decode(const lrsa_params_t* params, const void* cache, size_t cach
   }
   a.scale_log2 = g.scale * 1.4426950408889634f;
   a.status = &reinterpret_cast<WsHeader*>(workspace)->status;
+  if (use_split_kernel(g, a.n_keys)) {
+    a.n_split = decode_splits(a.n_keys);
+    LRSA_CUDA_CHECK(g.d == 128 ? launch_split_t<128>(g, a, st) : launch_split_t<64>(g, a, st));
+    LRSA_CUDA_CHECK(launch_merge<kMergeRows>(g, a, a.n_split, st));
+    launch_counter().n += 2;
+    return LRSA_OK;
+  }
   DecodePlan pl = decode_plan(g, a.n_keys);
   cudaError_t e = launch_decode(g, a, pl, st);
   if (e != cudaSuccess && pl.splits > 8) {   // clusters of 16 are not portable: a part of a GPU may not have room for them
@@ -645,9 +929,7 @@ int lrsa_attn_decode(const lrsa_params_t* params, const void* cache, size_t cach
   LRSA_CUDA_CHECK(e);
   launch_counter().n++;
   if (pl.groups > 1) {
-    const float* part = a.part;
-    LRSA_CUDA_CHECK(launch_dependent(g.d == 128 ? decode_merge_kernel<128> : decode_merge_kernel<64>, dim3(g.B * g.Hq),
-                                     dim3(g.d), 0, st, 1, part, a.o, lse, g.Hq, g.Hkv, g.G, pl.groups));
+    LRSA_CUDA_CHECK(launch_merge<1>(g, a, pl.groups, st));
     launch_counter().n++;
   }
   return LRSA_OK;

@@ -187,3 +187,29 @@ def test_decode_scores_of_minus_infinity(d, G, S, N):
     want = torch.einsum("hgk,hkd->hgd", s.softmax(-1), vv).reshape(1, 2 * G, d)
     check_close("o", f64(o), want.cpu().numpy())
     check_close("lse", f64(lse), s.logsumexp(-1).reshape(1, 2 * G).cpu().numpy(), max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
+
+
+@pytest.mark.parametrize("G", [17, 24, 40])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,N,launches", [(1, 1, 2), (1, 129, 2), (2, 700, 2), (3, 5000, 2), (40, 2500, 1), (1, 70000, 2)])
+def test_decode_of_wide_groups(G, d, B, N, launches):
+    """Groups that take two or three passes of 16 query heads, against fp64 attention: the split kernel (one CTA per 128 keys, two launches with
+    its merge) on one key, ragged last splits and full ones; clusters of CTAs for large batches (one launch) and long caches
+    (several clusters and the merge)."""
+    w = W("i_wide", B, 2 * G, 2, N, d, 256, 256 if N > 5000 else 64, min(4, N), seed=92)
+    g = torch.Generator(device="cuda").manual_seed(9)
+    k, v = (torch.randn((B, 2, N, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    q = torch.randn((B, 2 * G, d), generator=g, device="cuda").bfloat16()
+    cache = lrsa.KVCache(lrsa.Params.from_workload(w))
+    cache.append(k, v)
+    o, lse = cache.decode(q)
+    assert lrsa.lrsa_last_launch_count() == launches
+    assert cache.status() == 0
+    nc = cache.windows_compressed()
+    pos = torch.cat([torch.arange(w.S, device="cuda").expand(B, 2, -1), cache.kept()[:, :, :nc].reshape(B, 2, -1).long(),
+                     torch.arange(w.S + nc * w.L, N, device="cuda").expand(B, 2, -1)], -1)
+    ix = pos[..., None].expand(-1, -1, -1, d)
+    s = torch.einsum("bhgd,bhkd->bhgk", q.double().view(B, 2, G, d), k.gather(2, ix).double()) / d ** 0.5
+    want = torch.einsum("bhgk,bhkd->bhgd", s.softmax(-1), v.gather(2, ix).double()).reshape(B, 2 * G, d)
+    check_close("o", f64(o), want.cpu().numpy())
+    check_close("lse", f64(lse), s.logsumexp(-1).reshape(B, 2 * G).cpu().numpy(), max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
