@@ -679,18 +679,26 @@ ScoreWs score_ws_layout(const Geom& g) {
   return w;
 }
 
-// Run length and cluster size by the measured cost of a CTA, in tokens streamed (21 ns each with two CTAs an SM): (run + 1)
-// windows' parts, 290 for launch, exchange and selection of the first scored window, 550 for every further one (a chain of
-// barriers, and half as many loads in flight beside the folded statistics).  At d = 128, 4 KV heads, run x C: 32K tokens in
-// windows of 1024: 1x1 30.4 us, 1x2 27.6, 1x4 33.3, 2x4 32.5, 4x8 45.7; 64K in windows of 2048: 1x2 49.1, 2x4 53.8;
-// 8 heads, 128K in windows of 4096: 1x1 171, 2x2 161, 4x4 175, 2x1 219.
+// Run length and cluster size by the measured cost of a CTA, in tokens streamed (21 ns each at d = 128 with two CTAs an SM):
+// (run + 1) windows' parts, 290 for launch, exchange and selection of the first scored window, 550 for every further one (a chain
+// of barriers, and half as many loads in flight beside the folded statistics).  At d = 64 a row is half as long and the folded
+// form, with two rows of it in flight, streams at two thirds of the other's rate: from windows between 512 and 1000 tokens on that is
+// more than it saves, and a CTA takes one window.
+// us, run x C: d = 128, 4 heads: 32K tokens in windows of 1024 1x1 23.4, 1x2 22.8, 1x4 30.5, 2x4 28.1; of 256 1x1 26.9, 2x1 25.4; 64K of
+// 2048 1x1 56.5, 1x2 48.6, 2x4 49.9; 8 heads: 32K of 512 1x1 48.4, 2x1 43.3; 64K of 512 1x1 88.0, 2x1 90.4, 4x1 79.3; 128K of 512
+// 1x1 150.7, 4x1 159.6, 7x1 133.0, 8x1 148.6; 128K of 4096 1x1 167.8, 2x2 160.1, 4x4 171.0; batch 2 of it 2x1 289.9, 4x2 288.9.
+// d = 64, 8 heads: 64K of 512 1x1 56.7, 4x1 57.1; of 1000 1x1 55.3, 2x1 61.4; of 2048 1x1 51.4, 2x2 60.5; of 4096 1x2 55.4, 2x4 71.2;
+// 128K of 512 1x1 104.4, 7x1 100.7; of 1000 1x1 102.0, 4x1 105.5; of 4096 1x1 97.5, 2x2 117.9; 16K of 333 1x1 32.8, 2x1 25.6.
+// (Calls back to back on one set of tensors.)
+constexpr int kFoldMaxL64 = 768;
 struct ClusterPlan { int run, C; };
-ClusterPlan cluster_plan(int BH, int Wsel, int L) {
+ClusterPlan cluster_plan(int BH, int Wsel, int L, int d) {
   ClusterPlan best = {1, 1};
+  const ClusterRoom& room = cluster_room();
   double cost = -1;
   for (int C = 1; C <= kClusterMax; C *= 2) {
-    const long long slots = C == 1 ? 2 * 148 : 8 * (2 * 18 / C);   // clusters at a time (eight groups of 18 SMs)
-    for (int r = 1; r <= Wsel; r = r < 8 ? r + 1 : r * 2) {
+    const long long slots = room.at_once(2, C);
+    for (int r = 1; r <= (d == 64 && L > kFoldMaxL64 ? 1 : Wsel); r = r < 8 ? r + 1 : r * 2) {
       const long long clusters = (long long)BH * ((Wsel + r - 1) / r), waves = (clusters + slots - 1) / slots;
       const double c = waves * ((r + 1.0) * ((L + C - 1) / C) + 290.0 + (r - 1) * 550.0);
       if (cost < 0 || c < cost) { cost = c; best.run = r; best.C = C; }
@@ -734,7 +742,7 @@ static int launch_cluster(const Geom* gs, int n_seqs, const __nv_bfloat16* K, co
     const Geom& g = gs[s0];
     ScoreArgs a = score_args(g, K, V, idx, score, ws);
     a.clear_status = clear_status ? 1 : 0;
-    const ClusterPlan pl = cluster_plan(a.BH, windows, g.L);
+    const ClusterPlan pl = cluster_plan(a.BH, windows, g.L, g.d);
     q.n = 0;
     q.item0[0] = 0;
     for (int s = s0; s < s1; ++s) {

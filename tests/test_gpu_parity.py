@@ -51,6 +51,33 @@ def test_score_select(w, ddof):
     assert torch.equal(idx, idx2)
 
 
+@pytest.mark.parametrize("B,Hkv,N,d,L,cuts", [
+    (1, 8, 16384, 64, 333, ()),              # d = 64, two windows a CTA
+    (2, 8, 33000, 64, 500, ()),              # four
+    (1, 8, 16384, 64, 333, (5000, 5001, 11000)),   # the same over the sequences of a packed row
+    (1, 8, 33000, 128, 512, ()),
+    (1, 8, 33000, 128, 512, (700, 9000, 25000)),
+    (1, 4, 2100 * 9, 64, 2100, ()),          # long windows at d = 64: one window a CTA, or a cluster's
+])
+def test_selection_with_several_windows_per_cta(B, Hkv, N, d, L, cuts):
+    """Enough windows that a CTA walks a run of them and folds the statistics of each while it is scored, against the oracle."""
+    w = W("s_runs", B, Hkv, Hkv, N, d, L, L // 4, 4, seed=45, values="channel_offset")
+    host = workloads.generate(w, ("K", "V"))
+    bits = host_bits(host)
+    op = oparams(w)
+    cu = (0, *cuts, N)
+    oidx, osc = orc.score_select_packed(op, bits["K"], bits["V"], cu)
+    dev = to_dev(host)
+    p = lrsa.Params.from_workload(w, cu_seqlens=cu if cuts else ())
+    idx, sc = lrsa.lrsa_score_select(p, dev["K"], dev["V"], want_score=True)
+    np.testing.assert_allclose(f64(sc), osc, rtol=2e-5, atol=0)
+    got = idx.cpu().numpy()
+    for t0, n, wsel, woff in orc.packed_windows(op, cu):
+        if wsel:
+            compare_idx(got[:, :, woff:woff + wsel] - t0, oidx[:, :, woff:woff + wsel] - t0, osc[:, :, woff:woff + wsel],
+                        min(w.S, n), w.L)
+
+
 def test_longest_window_that_is_scored():
     """25 448 tokens is the longest lag window of the selection (its scores lie in shared memory); one more is refused."""
     w = W("s_longest", 1, 1, 1, 2 * 25448 + 1, 64, 25448, 700, 1, seed=44)
