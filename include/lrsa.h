@@ -86,7 +86,8 @@ typedef struct lrsa_params {
 /* Number of scored windows W_sel (see Geometry).  idx has W_sel * top_k entries per KV head. */
 int lrsa_num_sel_windows(const lrsa_params_t* params, int32_t* w_sel);
 
-/* Workspace sizes in bytes for the three calls (any output pointer may be NULL). */
+/* Workspace sizes in bytes for the three calls (any output pointer may be NULL).  They follow the shape alone, not
+ * cu_seqlens: a workspace of the row serves every packing of it. */
 int lrsa_workspace_bytes(const lrsa_params_t* params, size_t* score_select, size_t* attn_fwd,
                          size_t* attn_bwd);
 

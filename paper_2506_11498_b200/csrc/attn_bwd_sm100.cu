@@ -1,6 +1,8 @@
 // LRSA attention backward: workspace layout, the kernels in front of and behind the tensor-core kernels, the sequence of
 // launches: prep (statistics, zeroed accumulators, compact K/V, launch order, partial mean key), dK/dV (also the accurate
 // D of every query row and the mean key), dQ, conversion of dK, dV to bf16.
+#include <algorithm>
+
 #include "attn_bwd_sm100.h"
 
 namespace lrsa {
@@ -144,38 +146,57 @@ __global__ void __launch_bounds__(256) convert_dkv_kernel(const float* __restric
   *reinterpret_cast<uint2*>(dV + e) = vo;
 }
 
-// Launch order tables of all sequences: inner iterations per CTA, sizes.
-struct DkvSizes {
+// What a call needs per batch of sequences: inner iterations per CTA; compact rows, and entries of the launch order tables.
+struct BwdSizes {
   int seg;
-  long long tiles, segs;
+  long long rows, tiles, segs;
 };
-DkvSizes dkv_sizes(const Geom& g) {
-  DkvSizes z = {kSegMax, 0, 0};
+BwdSizes bwd_sizes(const Geom& g) {
+  BwdSizes z = {kSegMax, compact_rows_used(g), 0, 0};
   SeqBatch b;
   long long iters = 0;
-  for (SeqBatches it(g); it.next(&b);)
+  for (SeqBatches it(g); it.next(&b);) {
+    long long tiles = 0;
     for (int s = 0; s < b.n; ++s) {
       const DkvPlan p = make_dkv_plan(b.g[s], kSegMax);
-      z.tiles += p.n_tiles;
+      tiles += p.n_tiles;
       for (int i = 0; i < p.n_tiles; ++i) iters += (long long)p.G * describe_tile(p, i).nq;
     }
+    z.tiles = std::max(z.tiles, tiles);
+  }
   iters *= (long long)g.B * g.Hkv;
   z.seg = dkv_segment(iters);
-  for (SeqBatches it(g); it.next(&b);)
+  for (SeqBatches it(g); it.next(&b);) {
+    long long segs = 0;
     for (int s = 0; s < b.n; ++s) {
       const DkvPlan p = make_dkv_plan(b.g[s], z.seg);
-      for (int i = 0; i < p.n_tiles; ++i) z.segs += tile_segments(p, describe_tile(p, i));
+      for (int i = 0; i < p.n_tiles; ++i) segs += tile_segments(p, describe_tile(p, i));
     }
+    z.segs = std::max(z.segs, segs);
+  }
+  return z;
+}
+
+// The same for any packing of rows of this shape, from above.  Tiles: every sequence rounds its list, its sinks and its last window
+// up.  Query tiles of a tile: all of the row for a list tile; a window is seen whole for at most two windows' length (from its own tokens on), a
+// sink by the sinks.  Segments: one more per tile than iterations / seg, and seg is 128 or keeps iterations / seg below 592 * 17 / 16.
+BwdSizes bwd_sizes_bound(const Geom& g) {
+  auto up = [](long long x, long long y) { return (x + y - 1) / y; };
+  const long long seqs = std::min(kMaxSeqs, g.N), rows = compact_rows_bound(g);
+  const long long list = rows / kTile + seqs, sinks = seqs * up(g.S, kTile), dense = (g.N / g.L + seqs) * up(g.L, kTile);
+  const long long iters = list * up(g.N, kQRows) + sinks * up(g.S, kQRows) + dense * up(2LL * g.L, kQRows);
+  BwdSizes z = {kSegMax, rows, list + sinks + dense, 0};
+  z.segs = z.tiles + 630 + g.G * iters / kSegMax;
   return z;
 }
 
 struct BwdWs {
   size_t kbar, kpart, dacc, kc, vc, stats, cnt, map, dkf, acc, total;
 };
-BwdWs bwd_ws_layout(const Geom& g, const DkvSizes& z) {
+BwdWs bwd_ws_layout(const Geom& g, const BwdSizes& z) {
   BwdWs w;
-  const size_t BHkv = (size_t)g.B * g.Hkv, rc = g.Rtot > 0 ? g.Rtot : 1;
-  const size_t cbytes = align_up(BHkv * rc * g.d * sizeof(__nv_bfloat16), 1024);
+  const size_t BHkv = (size_t)g.B * g.Hkv;
+  const size_t cbytes = align_up(BHkv * z.rows * g.d * sizeof(__nv_bfloat16), 1024);
   size_t off = 1024;
   w.kbar = off; off += align_up(BHkv * g.d * sizeof(float), 1024);
   w.kpart = off; off += align_up(kMeanSplits * BHkv * g.d * sizeof(float), 1024);
@@ -193,13 +214,14 @@ BwdWs bwd_ws_layout(const Geom& g, const DkvSizes& z) {
 
 }  // namespace
 
-size_t attn_bwd_ws_bytes(const Geom& g) { return bwd_ws_layout(g, dkv_sizes(g)).total; }
+size_t attn_bwd_ws_bytes(const Geom& g) { return bwd_ws_layout(g, bwd_sizes(g)).total; }
+size_t attn_bwd_ws_bound(const Geom& g) { return bwd_ws_layout(g, bwd_sizes_bound(g)).total; }
 
 int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                           const __nv_bfloat16* V, const __nv_bfloat16* O, const __nv_bfloat16* dO,
                           const float* LSE, const int32_t* idx, __nv_bfloat16* dQ, __nv_bfloat16* dK,
                           __nv_bfloat16* dV, void* ws, cudaStream_t st) {
-  const DkvSizes z = dkv_sizes(g);
+  const BwdSizes z = bwd_sizes(g);
   const BwdWs lay = bwd_ws_layout(g, z);
   unsigned char* base = static_cast<unsigned char*>(ws);
   auto at = [&](size_t off) { return base + off; };
@@ -221,9 +243,9 @@ int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
   const int BHkv = g.B * g.Hkv;
   SeqBatches batches(g);
   SeqBatch b;
-  int cnt = 0, map = 0;
   for (bool first = true; batches.next(&b); first = false) {
     PrepArgs a;
+    int cnt = 0, map = 0;
     for (int s = 0; s < b.n; ++s) {
       const DkvPlan dp = make_dkv_plan(b.g[s], z.seg);
       a.db.plan[s] = dp;

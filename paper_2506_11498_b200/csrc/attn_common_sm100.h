@@ -109,10 +109,27 @@ struct SeqBatch {
 struct SeqBatches {
   const Geom& whole;
   int s = 0, woff = 0;
-  long long row0 = 0;
   explicit SeqBatches(const Geom& w) : whole(w) {}
   bool next(SeqBatch* b);   // false: none left
 };
+
+// Rows of the compact buffers per KV head: what the largest batch of a call takes, and what a batch takes at most in any
+// packing of rows of this shape (k sequences have k - 1 times the sinks more than the row unpacked, and never more kept rows).
+inline long long compact_rows_used(const Geom& g) {
+  if (g.n_seqs == 0) return g.Rc > 0 ? g.Rc : 1;
+  long long most = 1, sum = 0;
+  for (int s = 0; s < g.n_seqs; ++s) {
+    if (s % kMaxSeqs == 0) sum = 0;
+    const int n = g.cu[s + 1] - g.cu[s], S = g.S < n ? g.S : n, w = (n - S) / g.L;
+    sum += S + (long long)(w > 1 ? w - 1 : 0) * g.K;
+    if (sum > most) most = sum;
+  }
+  return most;
+}
+inline long long compact_rows_bound(const Geom& g) {
+  const long long rows = g.Rc + (kMaxSeqs - 1LL) * g.S;
+  return rows < 1 ? 1 : rows < g.N ? rows : g.N;
+}
 
 // Gather of the sink rows and the kept rows of K and V into the compact buffers: per sequence Kc, Vc [B*Hkv][Rc][d] (the
 // condensed KV cache of Section 3.2) for the query-outer kernels, which stream the list once per query tile (a TMA row

@@ -489,10 +489,9 @@ EncodeFn encode_fn() {
 struct FwdWs {
   size_t kc, vc, total;
 };
-FwdWs fwd_ws_layout(const Geom& g) {
+FwdWs fwd_ws_layout(const Geom& g, long long rows) {
   FwdWs w;
-  const size_t rc = g.Rtot > 0 ? g.Rtot : 1;
-  const size_t bytes = align_up((size_t)g.B * g.Hkv * rc * g.d * sizeof(__nv_bfloat16), 1024);
+  const size_t bytes = align_up((size_t)g.B * g.Hkv * rows * g.d * sizeof(__nv_bfloat16), 1024);
   w.kc = 1024;
   w.vc = w.kc + bytes;
   w.total = w.vc + bytes;
@@ -529,7 +528,8 @@ int make_tmap_bf16_rows(CUtensorMap* map, const void* base, int d, long long row
   return r == CUDA_SUCCESS ? LRSA_OK : LRSA_ERR_CUDA;
 }
 
-size_t attn_fwd_ws_bytes(const Geom& g) { return fwd_ws_layout(g).total; }
+size_t attn_fwd_ws_bytes(const Geom& g) { return fwd_ws_layout(g, compact_rows_used(g)).total; }
+size_t attn_fwd_ws_bound(const Geom& g) { return fwd_ws_layout(g, compact_rows_bound(g)).total; }
 
 template <int D, int NSEQ, int TQ>
 static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat16* Q, const __nv_bfloat16* K,
@@ -590,7 +590,7 @@ static bool one_tile(const Geom& whole, const SeqBatch& b) {
 int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                           const __nv_bfloat16* V, const int32_t* idx, __nv_bfloat16* O, float* LSE, void* ws,
                           cudaStream_t st) {
-  const FwdWs lay = fwd_ws_layout(g);
+  const FwdWs lay = fwd_ws_layout(g, compact_rows_used(g));
   unsigned char* base = static_cast<unsigned char*>(ws);
   __nv_bfloat16* Kc = reinterpret_cast<__nv_bfloat16*>(base + lay.kc);
   __nv_bfloat16* Vc = reinterpret_cast<__nv_bfloat16*>(base + lay.vc);

@@ -1,6 +1,7 @@
 // C ABI entry points: argument validation on the host, workspace layout, kernel dispatch.
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "attn_common_sm100.h"
@@ -82,19 +83,17 @@ int make_geom(const lrsa_params_t* p, Geom* g) {
   if (reinterpret_cast<uintptr_t>(p->o_residual) & 15u) return LRSA_ERR_INVALID_ARG;
   g->has_o_res = p->o_residual != nullptr;
   if (p->n_seqs < 0) return LRSA_ERR_INVALID_ARG;
-  g->cu = nullptr; g->n_seqs = 0; g->Rtot = g->Rc;
+  g->cu = nullptr; g->n_seqs = 0;
   if (p->n_seqs > 0) {
     if (!p->cu_seqlens || p->cu_seqlens[0] != 0 || p->cu_seqlens[p->n_seqs] != p->seq_len) return LRSA_ERR_INVALID_ARG;
-    int wtot = 0, rtot = 0;
+    int wtot = 0;
     for (int s = 0; s < p->n_seqs; ++s) {
       const int n = p->cu_seqlens[s + 1] - p->cu_seqlens[s];
       if (n < 1) return LRSA_ERR_INVALID_ARG;
       const int w = n > g->S ? (n - g->S) / g->L : 0;
       wtot += w > 1 ? w - 1 : 0;
-      rtot += (n < g->S ? n : g->S) + (w > 1 ? w - 1 : 0) * g->K;
     }
     g->Wtot = wtot;
-    g->Rtot = rtot;
     g->cu = p->cu_seqlens; g->n_seqs = p->n_seqs;
   }
   return LRSA_OK;
@@ -114,12 +113,13 @@ void seq_geom(const Geom& whole, const int32_t* cu, int n_seqs, int s, int woff,
   g.Wsel = g.W > 1 ? g.W - 1 : 0;
   g.Rc = g.S + g.Wsel * g.K;
   g.woff = woff;
-  g.cu = nullptr; g.n_seqs = 0; g.Rtot = g.Rc;
+  g.cu = nullptr; g.n_seqs = 0;
 }
 
 bool SeqBatches::next(SeqBatch* b) {
   const int total = whole.n_seqs > 0 ? whole.n_seqs : 1;
   b->n = 0;
+  long long row0 = 0;   // the compact buffers are used again by every batch of sequences
   for (; s < total && b->n < kMaxSeqs; ++s) {
     Geom g;
     seq_geom(whole, whole.cu, whole.n_seqs, s, woff, &g);
@@ -156,14 +156,8 @@ int run_score_select(const lrsa_params_t* p, const Geom& whole, const __nv_bfloa
 
 static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-static size_t fwd_ws_bytes(const Geom& g) {
-  const size_t a = attn_ref_fwd_ws_bytes(g), b = attn_fwd_ws_bytes(g);
-  return a > b ? a : b;
-}
-static size_t bwd_ws_bytes(const Geom& g) {
-  const size_t a = attn_ref_bwd_ws_bytes(g), b = attn_bwd_ws_bytes(g);
-  return a > b ? a : b;
-}
+static size_t fwd_ws_bytes(const Geom& g) { return std::max(attn_ref_fwd_ws_bytes(g), attn_fwd_ws_bytes(g)); }
+static size_t bwd_ws_bytes(const Geom& g) { return std::max(attn_ref_bwd_ws_bytes(g), attn_bwd_ws_bytes(g)); }
 
 }  // namespace lrsa
 
@@ -186,8 +180,9 @@ int lrsa_workspace_bytes(const lrsa_params_t* params, size_t* score_select, size
   const int rc = make_geom(params, &g);
   if (rc != LRSA_OK) return rc;
   if (score_select) *score_select = score_select_ws_bytes(g);
-  if (attn_fwd) *attn_fwd = fwd_ws_bytes(g);
-  if (attn_bwd) *attn_bwd = bwd_ws_bytes(g);
+  // the same for every packing of the row: a workspace made for one batch serves the next
+  if (attn_fwd) *attn_fwd = std::max(attn_ref_fwd_ws_bytes(g), attn_fwd_ws_bound(g));
+  if (attn_bwd) *attn_bwd = std::max(attn_ref_bwd_ws_bytes(g), attn_bwd_ws_bound(g));
   return LRSA_OK;
 }
 

@@ -33,7 +33,6 @@ struct Geom {
   // Packed batches, host only: the boundaries (valid during the call) and number of sequences (0: one sequence).
   const int32_t* cu;
   int n_seqs;
-  int Rtot;        // rows of the compact buffers per KV head over all sequences (<= N)
   int has_o_res;   // the caller gave a buffer for the rounding remainder of O (lrsa_params_t::o_residual)
 };
 
@@ -105,7 +104,9 @@ int launch_attn_ref_bwd(const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat
                         __nv_bfloat16* dV, void* ws, cudaStream_t st);
 
 // attn_fwd_sm100.cu : tcgen05 / TMEM forward (workspace: header + compact K/V).
+// (*_ws_bytes: what a call of this geometry uses; *_ws_bound: enough for every packing of rows of this shape)
 size_t attn_fwd_ws_bytes(const Geom& g);
+size_t attn_fwd_ws_bound(const Geom& g);
 int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                           const __nv_bfloat16* V, const int32_t* idx, __nv_bfloat16* O, float* LSE,
                           void* ws, cudaStream_t st);
@@ -117,6 +118,7 @@ int launch_attn_ref_bwd_dkv(const Geom& g, const __nv_bfloat16* Q, const __nv_bf
 
 // attn_bwd_*_sm100.cu : tcgen05 / TMEM backward.
 size_t attn_bwd_ws_bytes(const Geom& g);
+size_t attn_bwd_ws_bound(const Geom& g);
 int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                           const __nv_bfloat16* V, const __nv_bfloat16* O, const __nv_bfloat16* dO,
                           const float* LSE, const int32_t* idx, __nv_bfloat16* dQ, __nv_bfloat16* dK,

@@ -100,3 +100,15 @@ def test_o_residual_must_be_16_byte_aligned():
     assert lrsa.lib().lrsa_num_sel_windows(ctypes.byref(cp), ctypes.byref(out)) == 0
     cp.o_residual = 4096 + 8
     assert lrsa.lib().lrsa_num_sel_windows(ctypes.byref(cp), ctypes.byref(out)) == 1
+
+
+@pytest.mark.parametrize("shape", [dict(), dict(seq_len=32768, n_q_heads=28, n_kv_heads=4, lag=1024, top_k=256),
+                                   dict(seq_len=32768, head_dim=64, lag=256, top_k=64, n_sink=16), dict(seq_len=700, lag=500, n_sink=40)])
+def test_workspace_sizes_do_not_depend_on_the_packing(shape):
+    """A workspace sized for one batch of a data loader serves the next: the sizes follow the row's shape alone."""
+    import random
+    args = {**GOOD, **shape}
+    want = lrsa.lrsa_workspace_bytes(lrsa.Params(**args))
+    n, r = args["seq_len"], random.Random(5)
+    for cuts in ([], [n // 2], range(16, n, 16), range(1, 18), sorted(r.sample(range(1, n), 15)), sorted(r.sample(range(1, n), 40))):
+        assert lrsa.lrsa_workspace_bytes(lrsa.Params(**args, cu_seqlens=(0, *cuts, n))) == want

@@ -350,6 +350,39 @@ def test_packed_sequences(w, cu, ndp):
     check_close("dV", f64(dV), odV)
 
 
+@pytest.mark.parametrize("N,d,L,K,S", [(700, 64, 40, 13, 5), (2048, 128, 64, 64, 16), (1500, 128, 600, 100, 40), (333, 64, 8, 3, 0)])
+def test_one_workspace_for_every_packing_of_a_row(N, d, L, K, S):
+    """The workspace of the unpacked row, between margins that must stay untouched, through packings of a few sequences to
+    very many (several batches of sequences, the compact buffers and launch tables used again by each), the shortest ones all sinks.  O is
+    bit-equal to that of each sequence on its own."""
+    w = W("p_ws", 1, 4, 2, N, d, L, K, S, seed=57)
+    dev = to_dev(workloads.generate(w))
+    sizes = lrsa.lrsa_workspace_bytes(lrsa.Params.from_workload(w))
+    bufs = [torch.full((n + 8192,), 0xA5, dtype=torch.uint8, device="cuda") for n in sizes]
+    ws = [b[4096:4096 + n] for b, n in zip(bufs, sizes)]
+    rng = np.random.default_rng(N)
+    packings = [[], range(max(S, 1), N, max(S, 1)), range(S + 2 * L, N, S + 2 * L)]
+    packings += [sorted(rng.choice(np.arange(1, N), int(k), replace=False).tolist()) for k in (1, 5, 14, 15, 16, 40)]
+    for cuts in packings:
+        cu = (0, *[c for c in cuts][:300], N)
+        p = lrsa.Params.from_workload(w, cu_seqlens=cu)
+        idx, _ = lrsa.lrsa_score_select(p, dev["K"], dev["V"], workspace=ws[0])
+        O, LSE = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx, workspace=ws[1])
+        grads = lrsa.lrsa_attn_bwd(p, dev["Q"], dev["K"], dev["V"], O, dev["dO"], LSE, idx, workspace=ws[2])
+        assert all(lrsa.lrsa_workspace_status(x) == 0 for x in ws)
+        assert all(torch.isfinite(t.float()).all() for t in (O, LSE, *grads))
+        for b, n in zip(bufs, sizes):
+            assert (b[:4096] == 0xA5).all() and (b[4096 + n:] == 0xA5).all()
+        for i in rng.choice(len(cu) - 1, min(4, len(cu) - 1), replace=False):
+            lo, hi = cu[i], cu[i + 1]
+            one = W("p_ws1", 1, 4, 2, hi - lo, d, L, K, min(S, hi - lo))
+            q, k, v = (dev[x][:, :, lo:hi].contiguous() for x in "QKV")
+            p1 = lrsa.Params.from_workload(one)
+            i1, _ = lrsa.lrsa_score_select(p1, k, v)
+            o1, l1 = lrsa.lrsa_attn_fwd(p1, q, k, v, i1)
+            assert torch.equal(o1, O[:, :, lo:hi]) and torch.equal(l1, LSE[:, :, lo:hi])
+
+
 def test_packed_single_sequence_equals_unpacked():
     w = W("p_one", 1, 4, 2, 4 + 5 * 256 + 77, 128, 256, 64, 4, seed=55)
     dev = to_dev(workloads.generate(w))
