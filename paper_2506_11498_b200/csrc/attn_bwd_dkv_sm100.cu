@@ -311,7 +311,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
 #pragma unroll
       for (int k = 0; k < kQRows / 32; ++k) {
         const int q = q0 + lane + 32 * k;
-        v[k] = q < kt.qend ? __ldg(a.stats + (size_t)hq * a.Nrow + tok0 + q) : make_float2(-INFINITY, 0.f);
+        v[k] = q < kt.qend ? a.stats[(size_t)hq * a.Nrow + tok0 + q] : make_float2(-INFINITY, 0.f);
       }
     };
     float2 cur[kQRows / 32], nxt[kQRows / 32];

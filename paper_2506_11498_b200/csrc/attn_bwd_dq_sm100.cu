@@ -326,7 +326,7 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
           float f[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e)
-            f[e] = fmaf(-r, __ldg(kb + q * 32 + 8 * v + e), __uint_as_float(o[8 * v + e])) * a.scale;
+            f[e] = fmaf(-r, kb[q * 32 + 8 * v + e], __uint_as_float(o[8 * v + e])) * a.scale;
           uint4 w;
           w.x = pack_bf16(f[0], f[1]); w.y = pack_bf16(f[2], f[3]);
           w.z = pack_bf16(f[4], f[5]); w.w = pack_bf16(f[6], f[7]);

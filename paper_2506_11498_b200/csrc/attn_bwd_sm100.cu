@@ -129,9 +129,8 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __grid_constant__ P
 }
 
 // bf16 outputs from the fp32 accumulators [BHkv][N][d]; n4 = number of float4 groups
-__global__ void __launch_bounds__(256) convert_dkv_kernel(const float* __restrict__ dKf, const float* __restrict__ dVf,
-                                                          __nv_bfloat16* __restrict__ dK, __nv_bfloat16* __restrict__ dV,
-                                                          long long n4) {
+__global__ void __launch_bounds__(256) convert_dkv_kernel(const float* dKf, const float* dVf, __nv_bfloat16* dK,
+                                                          __nv_bfloat16* dV, long long n4) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;

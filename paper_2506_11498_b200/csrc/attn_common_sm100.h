@@ -165,10 +165,11 @@ __device__ __forceinline__ void compact_rows(const CompactArgs& c, int block) {
   int s = 0;
   while (item >= c.item0[s + 1]) ++s;
   const int i = item - c.item0[s], bh = i / c.Rc[s], r = i - bh * c.Rc[s];
-  const int pos = r < c.S[s] ? r + c.tok0[s] : __ldg(c.idx + (size_t)bh * c.kept_stride + c.kept_off[s] + (r - c.S[s]));
+  const int pos = r < c.S[s] ? r + c.tok0[s] : c.idx[(size_t)bh * c.kept_stride + c.kept_off[s] + (r - c.S[s])];
   const size_t src = ((size_t)bh * c.Nrow + pos) * c.cpr + ch, dst = (size_t)(c.row0[s] + i) * c.cpr + ch;
-  reinterpret_cast<uint4*>(c.Kc)[dst] = __ldg(reinterpret_cast<const uint4*>(c.K) + src);
-  reinterpret_cast<uint4*>(c.Vc)[dst] = __ldg(reinterpret_cast<const uint4*>(c.V) + src);
+  const uint4 k = reinterpret_cast<const uint4*>(c.K)[src], v = reinterpret_cast<const uint4*>(c.V)[src];
+  reinterpret_cast<uint4*>(c.Kc)[dst] = k;
+  reinterpret_cast<uint4*>(c.Vc)[dst] = v;
 }
 
 // 2-D bf16 tensor map over [rows][d] with a (64 x 1) box and 128-byte swizzle, for row gathers
@@ -180,9 +181,9 @@ int make_tmap_bf16_rows(CUtensorMap* map, const void* base, int d, long long row
 // points at that head's idx entries.  Rows at or beyond n_rows are never used by a product (their scores
 // are masked); they map to position 0 so that the row fetched for them is valid, finite data.
 // Positions are local to the sequence (kept entries are positions in the whole row, tok0 + local).
-__device__ __forceinline__ int compact_row_pos(const int32_t* __restrict__ kept, int S, int n_rows, int r, int tok0) {
+__device__ __forceinline__ int compact_row_pos(const int32_t* kept, int S, int n_rows, int r, int tok0) {
   if (r >= n_rows) return 0;
-  return r < S ? r : __ldg(kept + (r - S)) - tok0;
+  return r < S ? r : kept[r - S] - tok0;
 }
 
 }  // namespace lrsa

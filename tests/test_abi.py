@@ -112,3 +112,15 @@ def test_workspace_sizes_do_not_depend_on_the_packing(shape):
     n, r = args["seq_len"], random.Random(5)
     for cuts in ([], [n // 2], range(16, n, 16), range(1, 18), sorted(r.sample(range(1, n), 15)), sorted(r.sample(range(1, n), 40))):
         assert lrsa.lrsa_workspace_bytes(lrsa.Params(**args, cu_seqlens=(0, *cuts, n))) == want
+
+
+def test_dependent_launches_read_through_plain_loads():
+    """A kernel that may start while the one in front of it still writes must not read that data through the read-only path
+    (__ldg, ld.global.nc, which const __restrict__ pointers invite too): such loads are not ordered by griddepcontrol.wait."""
+    csrc = os.path.join(ROOT, "paper_2506_11498_b200", "csrc")
+    files = [f for f in os.listdir(csrc) if f.endswith(".cu") and "griddepcontrol.wait" in open(os.path.join(csrc, f)).read()]
+    assert len(files) >= 6
+    for f in files + ["attn_common_sm100.h", "attn_bwd_sm100.h", "sm100_ptx.h"]:
+        code = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, f)).read())
+        for word in ("__ldg", "ld.global.nc", "__restrict__"):
+            assert word not in code, (f, word)
