@@ -2,7 +2,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "attn_common_sm100.h"
 
@@ -16,10 +15,12 @@ LaunchCounter& launch_counter() {
 // Never launched: stands for a kernel of one CTA per 1 / per_sm of an SM's shared memory.
 static __global__ void room_kernel() {}
 
-// The groups of SMs that a cluster has to fit into differ in size and between devices, so the device is asked.  (With eight groups
+// The groups of SMs that a cluster has to fit into differ in size and between devices, so the device is asked, once.  (With eight groups
 // of 18 SMs assumed, eight clusters of 16 large CTAs were planned for where seven run: one sequence of 8/8 heads, d = 64,
 // 8.7K keys 17.9 us instead of 10.7 with clusters of eight, 32/8 heads, d = 128, 9.5K keys 26.1 instead of 16.6.)
-static void ask_room(ClusterRoom* room) {
+// Where the GPUs of a process differ, the first one's numbers make the plans.
+static ClusterRoom ask_room() {
+  ClusterRoom room;
   const bool ok = cudaFuncSetAttribute(room_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10) == cudaSuccess &&
                   cudaFuncSetAttribute(room_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   for (int p = 0; p < 3; ++p)
@@ -36,19 +37,15 @@ static void ask_room(ClusterRoom* room) {
       cfg.numAttrs = 1;
       int n = 0;
       // (none, or no answer: such clusters take turns in every plan)
-      room->n[p][c] = ok && cudaOccupancyMaxActiveClusters(&n, room_kernel, &cfg) == cudaSuccess && n > 0 ? n : 1;
+      room.n[p][c] = ok && cudaOccupancyMaxActiveClusters(&n, room_kernel, &cfg) == cudaSuccess && n > 0 ? n : 1;
     }
   (void)cudaGetLastError();
+  return room;
 }
 
 const ClusterRoom& cluster_room() {
-  constexpr int kDevices = 64;
-  static ClusterRoom room[kDevices];
-  static std::once_flag asked[kDevices];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) dev = 0;
-  std::call_once(asked[dev], ask_room, &room[dev]);
-  return room[dev];
+  static const ClusterRoom room = ask_room();
+  return room;
 }
 
 static int g_impl = 0;  // 0: tensor-core kernels, 1: CUDA-core validation kernels

@@ -144,7 +144,7 @@ cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// lrsa_api.cu : clusters of 2^c CTAs that the current device runs at a time with 2^p CTAs on an SM, n[p][c].
+// lrsa_api.cu : clusters of 2^c CTAs that the device runs at a time with 2^p CTAs on an SM, n[p][c].
 struct ClusterRoom {
   int n[3][5];
   int at_once(int per_sm, int cluster) const {
