@@ -53,6 +53,8 @@ class Params:
     softmax_scale: float = 0.0
     cu_seqlens: tuple = ()    # packed batch: boundaries (0, ..., seq_len) of the sequences on the token axis
 
+    __slots__ = ("_struct", "__dict__", "__weakref__")   # the C struct lies beside the fields, not among them
+
     def c(self, o_residual=None) -> lrsa_params_t:
         """The C struct; `o_residual`: a bf16 tensor shaped like O (or None), see lrsa_attn_fwd."""
         cp = lrsa_params_t(self.batch, self.n_q_heads, self.n_kv_heads, self.seq_len, self.head_dim,
@@ -66,27 +68,25 @@ class Params:
             cp._keepalive = arr          # the host array lives as long as the struct
         return cp
 
-    def ref(self, o_residual=None):
-        """The C struct by reference, for a call.  Without a residual it is built once per object, whose fields cannot
-        change (the library only reads it): building it on every call took a third of a decode step's host time."""
-        if o_residual is not None:
-            return ctypes.byref(self.c(o_residual))
-        r = self.__dict__.get("_ref")
-        if r is None:
-            r = ctypes.byref(self.c())
-            object.__setattr__(self, "_ref", r)
-        return r
+    def struct(self) -> lrsa_params_t:
+        """The C struct of a call without a residual (the library only reads it), built once per object: building it on every
+        call took a third of a decode step's host time.  Boundaries in a list may change and are read each time.  The
+        caller holds on to the struct while it uses its address."""
+        if type(self.cu_seqlens) is not tuple:
+            return self.c()
+        try:
+            return self._struct
+        except AttributeError:
+            cp = self.c()
+            object.__setattr__(self, "_struct", cp)
+            return cp
 
-    def address(self) -> int:
-        """The same struct's address."""
-        a = self.__dict__.get("_address")
-        if a is None:
-            a = ctypes.cast(self.ref(), ctypes.c_void_p).value
-            object.__setattr__(self, "_address", a)
-        return a
+    def ref(self, o_residual=None):
+        """The C struct by reference, for a call (the reference keeps it alive)."""
+        return ctypes.byref(self.struct() if o_residual is None else self.c(o_residual))
 
     def __getstate__(self):
-        return {k: v for k, v in self.__dict__.items() if k not in ("_ref", "_address")}
+        return dict(self.__dict__)   # without the struct, which holds addresses of this process
 
     @staticmethod
     def from_workload(w, **kw) -> "Params":
@@ -282,7 +282,8 @@ class KVCache:
         """k_new, v_new: bf16 [B, Hkv, n_new, d] (contiguous)."""
         n_new = k_new.shape[2]
         buf, ws = self.buf, self.ws
-        status = _call.cache_append(self.params.address(), buf.data_ptr(), buf.numel(), _p(k_new), _p(v_new),
+        cp = self.params.struct()
+        status = _call.cache_append(ctypes.addressof(cp), buf.data_ptr(), buf.numel(), _p(k_new), _p(v_new),
                                     self.n_tokens, n_new, ws.data_ptr(), ws.numel(), _stream(stream))
         if status:
             _check(status, "lrsa_cache_append")
@@ -295,7 +296,8 @@ class KVCache:
         if lse is None:
             lse = torch.empty_like(self._lse)
         buf, ws = self.buf, self.ws
-        status = _call.attn_decode(self.params.address(), buf.data_ptr(), buf.numel(), _p(q), self.n_tokens,
+        cp = self.params.struct()
+        status = _call.attn_decode(ctypes.addressof(cp), buf.data_ptr(), buf.numel(), _p(q), self.n_tokens,
                                    o.data_ptr(), lse.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream))
         if status:
             _check(status, "lrsa_attn_decode")

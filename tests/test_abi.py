@@ -124,3 +124,65 @@ def test_dependent_launches_read_through_plain_loads():
         code = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, f)).read())
         for word in ("__ldg", "ld.global.nc", "__restrict__"):
             assert word not in code, (f, word)
+
+
+def test_params_keep_their_value_semantics_after_a_call():
+    """The struct that calls reuse is no part of the parameters: fields, equality, copies and pickles stay those of the fields."""
+    import copy, dataclasses, pickle
+    p = lrsa.Params(**GOOD, cu_seqlens=(0, 300, 1000))
+    fields = dict(vars(p))
+    n = lrsa.lrsa_num_sel_windows(p)
+    assert vars(p) == fields and lrsa.Params(**vars(p)) == p
+    for q in (copy.copy(p), copy.deepcopy(p), pickle.loads(pickle.dumps(p)), dataclasses.replace(p)):
+        assert q == p and hash(q) == hash(p) and lrsa.lrsa_num_sel_windows(q) == n
+    assert lrsa.lrsa_num_sel_windows(dataclasses.replace(p, n_sink=44)) == (300 - 44) // 128 - 1 + (700 - 44) // 128 - 1
+
+
+def test_boundaries_in_a_list_are_read_at_each_call():
+    p = lrsa.Params(**GOOD, cu_seqlens=[0, 300, 1000])
+    for cut in (300, 500, 262):
+        p.cu_seqlens[1] = cut
+        assert lrsa.lrsa_num_sel_windows(p) == lrsa.lrsa_num_sel_windows(lrsa.Params(**GOOD, cu_seqlens=(0, cut, 1000)))
+
+
+def test_threads_that_build_the_struct_together_hold_live_ones(monkeypatch):
+    """Two threads find no struct yet and both build one: every address handed to the library is that of a live struct,
+    in these calls and in later ones (the structs made in between take the place of one that was let go)."""
+    import sys
+    import threading
+    import torch
+    lrsa.lib()
+    build, seen = lrsa.Params.c, []
+
+    class Calls:                   # stands for the helper module: what the struct holds when the library reads it
+        @staticmethod
+        def cache_append(address, *rest):
+            seen.append(lrsa.lrsa_params_t.from_address(address).seq_len)
+            return 0
+
+    t = torch.zeros(1, 2, 1, 128)
+    stream = type("S", (), {"cuda_stream": 0})
+    monkeypatch.setattr(lrsa, "_call", Calls)
+    interval = sys.getswitchinterval()
+    sys.setswitchinterval(1e-6)
+    try:
+        for _ in range(200):
+            together = threading.Barrier(2)
+
+            def slow(self, *a):
+                cp = build(self, *a)
+                together.wait(10)
+                return cp
+
+            monkeypatch.setattr(lrsa.Params, "c", slow)
+            cache = lrsa.KVCache.__new__(lrsa.KVCache)
+            cache.params, cache.buf, cache.ws, cache.n_tokens = lrsa.Params(**GOOD), t, t, 0
+            threads = [threading.Thread(target=cache.append, args=(t, t, stream)) for _ in range(2)]
+            [x.start() for x in threads]
+            [x.join() for x in threads]
+            others = [lrsa.lrsa_params_t() for _ in range(64)]
+            cache.append(t, t, stream)
+            del others
+    finally:
+        sys.setswitchinterval(interval)
+    assert seen == [1000] * 600
