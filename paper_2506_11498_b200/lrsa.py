@@ -275,7 +275,6 @@ class KVCache:
         _check(lib().lrsa_cache_bytes(params.ref(), ctypes.byref(a), ctypes.byref(b)), "lrsa_cache_bytes")
         self.buf = torch.zeros(a.value, dtype=torch.uint8, device=device)
         self.ws = new_workspace(b.value, device)
-        self._lse = torch.empty((params.batch, params.n_q_heads), dtype=torch.float32, device=device)   # shape of an lse
         self.n_tokens = 0
 
     def append(self, k_new, v_new, stream=None):
@@ -283,6 +282,8 @@ class KVCache:
         n_new = k_new.shape[2]
         buf, ws = self.buf, self.ws
         cp = self.params.struct()
+        if _call is None:      # a cache that came from another process
+            lib()
         status = _call.cache_append(ctypes.addressof(cp), buf.data_ptr(), buf.numel(), _p(k_new), _p(v_new),
                                     self.n_tokens, n_new, ws.data_ptr(), ws.numel(), _stream(stream))
         if status:
@@ -294,9 +295,11 @@ class KVCache:
         if o is None:
             o = torch.empty_like(q)
         if lse is None:
-            lse = torch.empty_like(self._lse)
+            lse = q.new_empty(q.shape[:2], dtype=torch.float32)
         buf, ws = self.buf, self.ws
         cp = self.params.struct()
+        if _call is None:
+            lib()
         status = _call.attn_decode(ctypes.addressof(cp), buf.data_ptr(), buf.numel(), _p(q), self.n_tokens,
                                    o.data_ptr(), lse.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream))
         if status:

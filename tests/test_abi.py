@@ -186,3 +186,22 @@ def test_threads_that_build_the_struct_together_hold_live_ones(monkeypatch):
     finally:
         sys.setswitchinterval(interval)
     assert seen == [1000] * 600
+
+
+def test_a_cache_works_in_a_process_that_has_made_no_call(monkeypatch):
+    """As after unpickling: the library is loaded by the first append or decode.  A cache saved before a field was added
+    works too.  (Calls that the library refuses before it touches the GPU.)"""
+    import torch
+    cache = lrsa.KVCache(lrsa.Params(**GOOD), device="cpu")
+    assert set(vars(cache)) == {"params", "buf", "ws", "n_tokens"}
+    stream = type("S", (), {"cuda_stream": 0})
+    k = torch.zeros((1, 2, 1, 128), dtype=torch.bfloat16)
+    q = torch.zeros((1, 4, 128), dtype=torch.bfloat16)
+    cache.n_tokens = 1000                     # full: one more token is an invalid argument
+    for call in (lambda: cache.append(k, k, stream), lambda: cache.decode(q, stream=stream)):
+        monkeypatch.setattr(lrsa, "_call", None)
+        monkeypatch.setattr(lrsa, "_lib", None)
+        with pytest.raises(lrsa.LrsaError) as e:
+            call()
+        assert e.value.status == 1
+        cache.n_tokens = 0                    # nothing to decode
