@@ -684,16 +684,17 @@ DecodePlan decode_plan(const Geom& g, int n_keys, int max_splits = kDecMaxSplits
   const int per_sm = max_warps / p.warps;
   const ClusterRoom& room = cluster_room();
   long long best = -1;
-  for (int s = 1; s <= max_splits; s *= 2)
+  for (int s = 1; s <= max_splits; s *= 2) {
+    const long long at_once = room.at_once(per_sm, s);
     for (int grp = 1; grp <= kDecMaxGroups; grp *= 2) {
       const int n = s * grp;
       if (n > 1 && ((n - 1) * p.warps >= p.blocks || BH * n > 148LL * per_sm * 4)) break;
-      const long long at_once = room.at_once(per_sm, s);
       const long long waves = (BH * grp + at_once - 1) / at_once;
       const int per_cta = (p.blocks + n - 1) / n;
       const long long cost = waves * ((per_cta + p.warps - 1) / p.warps + 2) + (grp > 1 ? 3 : 0);
       if (best < 0 || cost < best) { best = cost; p.splits = s; p.groups = grp; }
     }
+  }
   return p;
 }
 

