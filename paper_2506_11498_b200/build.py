@@ -2,14 +2,17 @@
 from __future__ import annotations
 
 import glob
+import importlib.machinery
 import os
 import subprocess
+import sys
 import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "liblrsa.so")
-CALL = os.path.join(_HERE, "_lrsa_call.so")   # Python module over two of the library's calls
+# Python module over two of the library's calls, for the interpreter that builds it.  The binding works without it.
+CALL = os.path.join(_HERE, "_lrsa_call" + importlib.machinery.EXTENSION_SUFFIXES[0])
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
 
@@ -18,12 +21,35 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _older(target, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(f) > os.path.getmtime(target) for f in deps)
+
+
+def _abi():
+    return glob.glob(os.path.join(_HERE, "..", "include", "*.h"))
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALL):
-        return True
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.c")) + \
-        glob.glob(os.path.join(_HERE, "..", "include", "*.h"))
-    return any(os.path.getmtime(f) > os.path.getmtime(LIB) for f in deps)
+    return _older(LIB, sources() + glob.glob(os.path.join(CSRC, "*.h")) + _abi())
+
+
+def call_is_stale() -> bool:
+    return _older(CALL, [os.path.join(CSRC, "pycall.c")] + _abi())
+
+
+def build_call() -> bool:
+    """Compiles the helper module.  Where that is not possible (no compiler, no Python.h) none is left behind: an older one
+    would call the library with the interface it was built for."""
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", CALL,
+           os.path.join(CSRC, "pycall.c"), "-L", _HERE, "-l:liblrsa.so", "-Wl,-rpath,$ORIGIN"]
+    if os.path.exists(CALL):
+        os.remove(CALL)
+    try:
+        subprocess.check_call(cmd)
+    except (OSError, subprocess.CalledProcessError) as e:
+        print(f"{os.path.basename(CALL)} was not built ({e}): its calls go through ctypes", file=sys.stderr)
+        return False
+    return True
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -31,9 +57,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
         subprocess.check_call(cmd)
-        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
-                               "-o", CALL, os.path.join(CSRC, "pycall.c"), "-L", _HERE, "-l:liblrsa.so",
-                               "-Wl,-rpath,$ORIGIN"])
+    if force or call_is_stale():
+        build_call()
     return LIB
 
 

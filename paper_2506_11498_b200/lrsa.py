@@ -7,6 +7,7 @@ the import of any entry point raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
 import importlib.util
 import os
 from dataclasses import dataclass
@@ -15,7 +16,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblrsa.so")
-CALL_PATH = os.path.join(_HERE, "_lrsa_call.so")
+CALL_PATH = os.path.join(_HERE, "_lrsa_call" + importlib.machinery.EXTENSION_SUFFIXES[0])
 
 STATUS = {0: "LRSA_OK", 1: "LRSA_ERR_INVALID_ARG", 2: "LRSA_ERR_UNSUPPORTED",
           3: "LRSA_ERR_WORKSPACE_TOO_SMALL", 4: "LRSA_ERR_CUDA", 5: "LRSA_ERR_TIMEOUT"}
@@ -93,7 +94,7 @@ class Params:
 
 
 _lib = None
-_call = None   # the module of csrc/pycall.c: the two calls of a generated token without ctypes
+_call = None   # the module of csrc/pycall.c, the two calls of a generated token without ctypes, or what stands for it
 
 
 def lib() -> ctypes.CDLL:
@@ -132,14 +133,30 @@ def lib() -> ctypes.CDLL:
         for name in ("lrsa_num_sel_windows", "lrsa_workspace_bytes", "lrsa_score_select", "lrsa_attn_fwd",
                      "lrsa_attn_bwd", "lrsa_workspace_status", "lrsa_last_launch_count", "lrsa_debug_set_impl"):
             getattr(L, name).restype = ctypes.c_int
-        spec = importlib.util.spec_from_file_location("_lrsa_call", CALL_PATH)
-        if spec is None or not os.path.exists(CALL_PATH):
-            raise ImportError(f"{CALL_PATH} is missing: run `python -c 'import __graft_entry__ as g; g.build()'`")
-        call = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(call)
-        _call = call
+        _call = _token_calls(L)
         _lib = L
     return _lib
+
+
+class _CtypesCalls:
+    """The helper module's two calls where there is none for this interpreter (about 1 us a call more)."""
+
+    def __init__(self, L):
+        at = ctypes.POINTER(lrsa_params_t)
+        self.cache_append = lambda params, *args: L.lrsa_cache_append(ctypes.cast(params, at), *args)
+        self.attn_decode = lambda params, *args: L.lrsa_attn_decode(ctypes.cast(params, at), *args)
+
+
+def _token_calls(L):
+    spec = importlib.util.spec_from_file_location("_lrsa_call", CALL_PATH)
+    try:
+        if spec is None:
+            raise ImportError(CALL_PATH)
+        call = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(call)
+        return call
+    except (ImportError, OSError):
+        return _CtypesCalls(L)
 
 
 def status_string(status: int) -> str:

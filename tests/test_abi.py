@@ -206,3 +206,43 @@ def test_a_cache_works_in_a_process_that_has_made_no_call(monkeypatch):
             call()
         assert e.value.status == 1
         cache.n_tokens = 0                    # nothing to decode
+
+
+@pytest.mark.parametrize("name,content", [("_lrsa_call.so", None), ("_lrsa_call.so", "no module"), ("none", None)])
+def test_the_library_works_without_its_helper_module(monkeypatch, tmp_path, name, content):
+    """The module is built for one interpreter and only saves time: without it, or with one that does not load, every call is there."""
+    import torch
+    path = tmp_path / name
+    if content:
+        path.write_text(content)
+    monkeypatch.setattr(lrsa, "CALL_PATH", str(path))
+    monkeypatch.setattr(lrsa, "_lib", None)
+    monkeypatch.setattr(lrsa, "_call", None)
+    p = lrsa.Params(**GOOD)
+    assert lrsa.lrsa_num_sel_windows(p) == (1000 - 4) // 128 - 1
+    cache = lrsa.KVCache(p, device="cpu")
+    cache.n_tokens = 1000
+    k, q = torch.zeros((1, 2, 1, 128), dtype=torch.bfloat16), torch.zeros((1, 4, 128), dtype=torch.bfloat16)
+    stream = type("S", (), {"cuda_stream": 0})
+    with pytest.raises(lrsa.LrsaError) as e:      # refused by the library: the arguments arrived in their places
+        cache.append(k, k, stream)
+    assert e.value.status == 1
+    cache.n_tokens = 0
+    with pytest.raises(lrsa.LrsaError) as e:
+        cache.decode(q, stream=stream)
+    assert e.value.status == 1
+
+
+def test_the_helper_module_is_rebuilt_when_it_is_the_older_one(monkeypatch, tmp_path):
+    """Whatever the age of the library; and a build that fails leaves no older module behind."""
+    path = tmp_path / "_lrsa_call.so"
+    path.write_bytes(b"old")
+    os.utime(path, (1, 1))
+    monkeypatch.setattr(lib_build, "CALL", str(path))
+    assert lib_build.call_is_stale()
+    monkeypatch.setenv("CC", "false")
+    lib_build.build()
+    assert not path.exists()
+    monkeypatch.delenv("CC")
+    lib_build.build()
+    assert path.exists() and not lib_build.call_is_stale()
