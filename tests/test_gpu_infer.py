@@ -213,3 +213,13 @@ def test_decode_of_wide_groups(G, d, B, N, launches):
     want = torch.einsum("bhgk,bhkd->bhgd", s.softmax(-1), v.gather(2, ix).double()).reshape(B, 2 * G, d)
     check_close("o", f64(o), want.cpu().numpy())
     check_close("lse", f64(lse), s.logsumexp(-1).reshape(B, 2 * G).cpu().numpy(), max_abs=2e-3, rel_l2=1e-4, ulp=0.0)
+
+
+@pytest.mark.parametrize("G", [1, 8])
+@pytest.mark.parametrize("d", [64, 128])
+def test_decode_on_small_ctas(G, d):
+    """Enough blocks of keys for the plan of four-warp CTAs (more than two per warp of the whole GPU) with one group of heads."""
+    B, N = 100, 2500
+    keys = 4 + (N - 1 - 4) // 256 * 64 - 64 + N - 4 - ((N - 1 - 4) // 256 - 1) * 256
+    assert 2 * B * -(-keys // (2048 // d)) > 2 * 148 * 16
+    test_decode_against_fp64(G, d, B, N)

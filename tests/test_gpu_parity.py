@@ -383,6 +383,59 @@ def test_one_workspace_for_every_packing_of_a_row(N, d, L, K, S):
             assert torch.equal(o1, O[:, :, lo:hi]) and torch.equal(l1, LSE[:, :, lo:hi])
 
 
+@pytest.mark.parametrize("heads,d,L,K,S,lens", [
+    ((28, 4), 128, 512, 128, 4, (3000, 3100, 2901)),           # forward of two query tiles per CTA, packed
+    ((8, 8), 64, 256, 64, 16, (1800, 2100, 77, 2500, 2523)),   # dQ with one score buffer per CTA, packed
+])
+def test_packed_forms_for_many_ctas(heads, d, L, K, S, lens):
+    """Packed rows large enough for the forms that only large grids take, against each sequence on its own (the forms for small
+    grids, which the oracle cases cover): O and LSE bit-equal, gradients within the bound of two bf16 results."""
+    N, cu = sum(lens), (0, *np.cumsum(lens).tolist())
+    w = W("p_many", 1, *heads, N, d, L, K, S, seed=58, values="channel_offset")
+
+    def blocks(n, rows):       # query blocks of a sequence: sinks, full windows, tail
+        wins, tail = (n - S) // L, (n - S) % L
+        return -(-S // rows) + wins * -(-L // rows) + -(-tail // rows)
+    if d == 128:
+        keys = sum(n * (S + max(-(-(n - S) // L) - 2, 0) * K // 2 + min(n // 2, L + L // 2)) for n in lens)
+        assert sum(blocks(n, 256) for n in lens) * heads[0] > 4 * 148 and 2 * keys > 15 * 128 * N
+    else:
+        assert sum(blocks(n, 128) for n in lens) * heads[0] > 2 * 148
+    dev = to_dev(workloads.generate(w))
+    p = lrsa.Params.from_workload(w, cu_seqlens=cu)
+    ws = [lrsa.new_workspace(n) for n in lrsa.lrsa_workspace_bytes(p)]
+    idx, _ = lrsa.lrsa_score_select(p, dev["K"], dev["V"], workspace=ws[0])
+    O, LSE = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx, workspace=ws[1])
+    grads = lrsa.lrsa_attn_bwd(p, dev["Q"], dev["K"], dev["V"], O, dev["dO"], LSE, idx, workspace=ws[2])
+    assert all(lrsa.lrsa_workspace_status(x) == 0 for x in ws)
+    woff = 0
+    for lo, hi in zip(cu[:-1], cu[1:]):
+        one = w.with_(N=hi - lo)
+        q, k, v, do = (dev[x][:, :, lo:hi].contiguous() for x in ("Q", "K", "V", "dO"))
+        p1 = lrsa.Params.from_workload(one)
+        i1, _ = lrsa.lrsa_score_select(p1, k, v)
+        assert torch.equal(i1 + lo, idx[:, :, woff:woff + i1.shape[2]])
+        woff += i1.shape[2]
+        o1, l1 = lrsa.lrsa_attn_fwd(p1, q, k, v, i1)
+        assert torch.equal(o1, O[:, :, lo:hi]) and torch.equal(l1, LSE[:, :, lo:hi])
+        for name, a, b in zip(("dQ", "dK", "dV"), grads, lrsa.lrsa_attn_bwd(p1, q, k, v, o1, do, l1, i1)):
+            check_close(name, f64(a[:, :, lo:hi]), f64(b))
+
+
+@pytest.mark.parametrize("B,heads,N,d,L,S", [(1, (28, 4), 6000, 128, 512, 4), (4, (28, 4), 3000, 128, 512, 17), (2, (8, 8), 8000, 64, 256, 16)])
+def test_forward_gives_the_same_bits_every_time(B, heads, N, d, L, S):
+    """P is overwritten by the next scores as soon as the product that reads it has been issued, on the order in which the tensor
+    core runs one thread's products.  An overlap of the two would depend on timing and show between repeats."""
+    w = W("a_repeat", B, *heads, N, d, L, L // 4, S, seed=59)
+    dev = to_dev(workloads.generate(w, ("Q", "K", "V")))
+    p = lrsa.Params.from_workload(w)
+    idx, _ = lrsa.lrsa_score_select(p, dev["K"], dev["V"])
+    O, LSE = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx)
+    for _ in range(20):
+        o, lse = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx)
+        assert torch.equal(o, O) and torch.equal(lse, LSE)
+
+
 def test_packed_single_sequence_equals_unpacked():
     w = W("p_one", 1, 4, 2, 4 + 5 * 256 + 77, 128, 256, 64, 4, seed=55)
     dev = to_dev(workloads.generate(w))
