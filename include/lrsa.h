@@ -23,8 +23,8 @@
  *            (Section 3.2 applied to it alone): its sinks and windows are counted from its first token
  *            (a sequence shorter than S is all sinks) and no query sees another sequence.  Scored
  *            windows are numbered sequence after sequence, W_sel is their total, and kept positions
- *            are positions on the packed token axis.  The sequences are processed one after the
- *            other on the stream.
+ *            are positions on the packed token axis.  Up to 16 sequences share a launch of each
+ *            kernel.
  * Stream   : `cuda_stream` is a cudaStream_t passed as void* (NULL = default stream).  Calls
  *            enqueue work and return without synchronising.  Two calls that use the same
  *            workspace must be ordered (same stream, or otherwise serialised).

@@ -17,9 +17,9 @@
 // memory has left beside the two D-wide accumulators) suffice, and the exponentials of step i+1 run while dK(i) and
 // dP^T(i+1) are computed, the rest of the softmax while dV and S^T are.  128 x 128 steps instead of 128 x 64 read
 // K_j and V_j half as often from shared memory (the tensor core's operands, 192 KB a step, are what bounds the
-// kernel together with the exponentials) and pay for half as many hand-offs: 5.23 -> 4.58 ms at 32K tokens, 28/4
-// heads, d = 128, one kept token in four (4.02 alone and uncapped with the products issued by predicate and the waits for
-// Q and dO out of the way: tensor pipe 73 %, was 55).  Warps: 0 TMA producer, 1 issuer, 3 row statistics, 4-19 softmax and
+// kernel together with the exponentials) and pay for half as many hand-offs.  At 32K tokens, 28/4 heads, d = 128, one kept
+// token in four: 4.02 ms alone and uncapped, tensor pipe 73 % active (128 x 64 steps: 5.23; these with a branch around each
+// product and the waits for Q and dO between two products: 4.58).  Warps: 0 TMA producer, 1 issuer, 3 row statistics, 4-19 softmax and
 // epilogue.  A softmax warpgroup takes 32 query columns of every step: four warps per scheduler hide the latency
 // of one another's exponentials and tensor-memory accesses (two warps with 64 columns each: 4.71 ms), and P^T is
 // handed over in two halves so that dV starts on the first (in one piece: 4.90 ms).  The softmax warps also sum
@@ -226,8 +226,8 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: dV(i), S^T(i+1), dK(i), dP^T(i+1), ... ----------------
-    // One warp issues everything, so the products run in this order on the tensor core: S^T(i+1) may overwrite
-    // P^T(i) and dP^T(i+1) may overwrite dS^T(i) without waiting for the products that read them.  The loop runs
+    // One thread issues everything, and the tensor core runs its products in this order (sm100_ptx.h): S^T(i+1) may
+    // overwrite P^T(i) and dP^T(i+1) may overwrite dS^T(i) without waiting for the products that read them.  The loop runs
     // with all lanes (uniform control flow, descriptors computed once); one lane issues, by predicate.
     constexpr uint32_t idesc_s = make_idesc_bf16(kTile, kQRows, 0, 0);  // 128 keys x 128 queries
     constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);       // 128 keys x D

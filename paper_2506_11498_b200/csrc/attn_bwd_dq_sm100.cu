@@ -159,8 +159,8 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
     }
   } else if (warp == 1) {
     // ---------------- issuer: S_j, dP_j NB tiles ahead of A += dS_j K_j ----------------
-    // One warp issues everything, so the products run in this order on the tensor core: S_{j+NB} may overwrite dS_j, and
-    // dP_{j+NB} dP_j, without waiting for the product that reads dS_j.
+    // One thread issues everything, and the tensor core runs its products in this order (sm100_ptx.h): S_{j+NB} may
+    // overwrite dS_j, and dP_{j+NB} dP_j, without waiting for the product that reads dS_j.
     constexpr uint32_t idesc_full = make_idesc_bf16(kTile, kKeys, 0, 0), idesc_short = make_idesc_bf16(kTile, kShort, 0, 0);
     constexpr uint32_t idesc_a = make_idesc_bf16(kTile, D, 0, 1);       // 128 x D, B = K_j MN-major
     const uint64_t descR = make_smem_desc_sw128(sRing, 16, 1024);       // K-major K_j / V_j
@@ -398,7 +398,7 @@ int launch_bwd_dq_sm100(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, 
   long long ctas = 0;
   for (int s = 0; s < b.n; ++s) ctas += (long long)make_plan(b.g[s], kTile).total * whole.B * whole.Hq;
   const auto dq = whole.d == 128   ? (b.n == 1 ? launch_dq_t<128, 1, 2> : launch_dq_t<128, kMaxSeqs, 2>)
-                  : ctas > 2 * 148 ? (b.n == 1 ? launch_dq_t<64, 1, 1> : launch_dq_t<64, kMaxSeqs, 1>)
+                  : ctas > 2 * kSms ? (b.n == 1 ? launch_dq_t<64, 1, 1> : launch_dq_t<64, kMaxSeqs, 1>)
                                    : (b.n == 1 ? launch_dq_t<64, 1, 2> : launch_dq_t<64, kMaxSeqs, 2>);
   return dq(whole, b, p, st);
 }

@@ -8,10 +8,13 @@ namespace lrsa {
 constexpr int kQRows = 128;   // query rows per inner tile
 // Inner iterations per CTA of the dK/dV kernel, from their number in the whole call: at most 128 (a CTA's start and its
 // additions to the accumulators are then lost in the rest), fewer in small problems, so that the longest list does not
-// outlast an even share by much.
+// outlast an even share (iterations / 148) by much, and never below 16.  Whole backward, us, at 8 | 16 | 32 | 64 | 128 iterations a CTA (the
+// rule's): 8/8 heads, d = 64: 4K tokens 88 | 85 | 94 | 94 | 94 (16), 8K 203 | 190 | 183 | 181 | 181 (16), 16K 685 | 601 | 578 | 566 | 561 (45);
+// 28/4, d = 128: 1777 tokens 110 | 112 | 114 | 159 | 216 (16), 4K 299 | 284 | 283 | 297 | 334 (16), 8K 878 | 785 | 754 | 731 | 725 (41),
+// 16K 2909 | 2671 | 2620 | 2471 | 2487 (128), 32K 9793 | 8645 | 8089 | 7809 | 7675 (128; 256: 7679); 32/8, 2K 170 | 122 | 125 | 173 | 173 (16).
 constexpr int kSegMax = 128;
 inline int dkv_segment(long long iters) {
-  const long long s = iters / (148 * 4);
+  const long long s = iters / (kSms * 4);
   return s < 16 ? 16 : s > kSegMax ? kSegMax : (int)s;
 }
 

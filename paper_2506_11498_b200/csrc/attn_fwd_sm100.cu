@@ -18,14 +18,12 @@
 // threads exchange nothing, and its 128 scores are held in registers at once (setmaxnreg: 216 for these threads).
 // What bounds it: the chain of a tile from S_t over its exponentials (one MUFU result per two clocks and thread, 1024
 // cycles a tile) to O_t and the next S_t, and the 1000 W power limit, under which the clock settles near 1.65 GHz.
-// At 32K tokens, 28/4 heads, d = 128, one kept token in four: 2.75 -> 2.44 ms (of 1.50 at the measured bf16 rate); at
-// 64K 9.5 -> 8.5 ms, 15.1 -> 13.3 M cycles; with the products issued by predicate 2.14 and 8.52 ms for
-// whole prefill calls, selection included (2.02 the kernel alone and uncapped, tensor pipe 62 %, was 51).  Before, two warps issued (S, and O += P V), with a barrier round trip
-// between a tile's products; scores were read twice; P was handed over in one piece.  Also measured: sixteen softmax
-// warps (16 rows x 128 columns each, 256-bit loads): 2.66 ms; exponentials started with the previous maximum, the tile
-// taken again when it was raised: 2.47 ms; a share of them on the FMA pipe: no gain at 1/8, 2.63 ms at 1/4.
-// The issuing warp runs its loop with all lanes and elects one lane per instruction.  All mbarrier waits are bounded;
-// on expiry the CTA records LRSA_ERR_TIMEOUT in the workspace header and leaves.
+// At 32K tokens, 28/4 heads, d = 128, one kept token in four: 2.02 ms alone and uncapped (1.50 at the measured bf16 rate;
+// tensor pipe 62 % active); 2.14 ms as a prefill call with its selection, 8.5 at 64K.  With an issuing warp for S and one for O += P V,
+// a barrier round trip between a tile's products and P handed over in one piece it takes 2.75 and 9.5 ms.  Measured on the way
+// (2.44 ms then) and not taken: sixteen softmax warps (16 rows x 128 columns each, 256-bit loads) 2.66; exponentials started with the
+// previous maximum, the tile taken again when it was raised, 2.47; a share of them on the FMA pipe, no gain at 1/8, 2.63 at 1/4.
+// All mbarrier waits are bounded; on expiry the CTA records LRSA_ERR_TIMEOUT in the workspace header and leaves.
 #include <algorithm>
 
 #include "attn_common_sm100.h"
@@ -44,7 +42,8 @@ struct FwdCfg {
   // padding per row (128 rows x (2D + 16) bytes = tile + 2 KB); the next tile stays 1024-byte aligned.
   static constexpr int kQRegion = kTileBytes + 2048;
   static constexpr int kPerSm = 3 - TQ;                          // resident CTAs
-  static constexpr int kStages = (D == 128 ? 4 : 10) / kPerSm;   // K/V ring slots
+  static constexpr int kStages = D == 64 ? 5 : 4 / kPerSm;       // K/V ring slots
+  static_assert(D == 128 || TQ == 1, "d = 64 runs with one tile per CTA");
   static constexpr int kSmem = TQ * kQRegion + kStages * kTileBytes + 1024;
   static constexpr int kThreads = 128 + 128 * TQ;
   // TMEM columns: accumulator O of query tile t at 128t, its S (and, packed over it, P) behind the accumulators
@@ -73,7 +72,7 @@ constexpr int kPParts = 2;   // P_t is handed to the tensor core in two halves (
 
 struct FwdBars {
   uint64_t q_full;
-  uint64_t kv_full[12], kv_empty[12];
+  uint64_t kv_full[5], kv_empty[5];
   uint64_t s_full[2], pv_done[2];   // per query tile
   uint64_t p_full[2][kPParts];      // per query tile: the parts of P_t (128 / kPParts keys each) are stored
 };
@@ -169,8 +168,8 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     }
   } else if (warp == 1) {
     // ---------------- issuer: per key tile j and query tile t  O_t += P_t V_j, then S_t = Q_t K_{j+1}^T ----------------
-    // One warp issues everything, so the products run in this order on the tensor core: S_t of the next key tile may
-    // overwrite P_t without waiting for the product that reads it.
+    // One thread issues everything, and the tensor core runs its products in this order (sm100_ptx.h): S_t of the next
+    // key tile may overwrite P_t without waiting for the product that reads it.
     constexpr uint32_t idesc_qk = make_idesc_bf16(kTile, kTile, 0, 0);
     constexpr uint32_t idesc_pv = make_idesc_bf16(kTile, D, 0, 1);
     const uint64_t descK0 = make_smem_desc_sw128(sRing, 16, 1024);
@@ -584,7 +583,7 @@ static bool one_tile(const Geom& whole, const SeqBatch& b) {
     keys += g.N * (g.S + hist + dense);
     tokens += g.N;
   }
-  return ctas <= 4 * 148 || 2 * keys <= 15 * kTile * tokens;   // 7.5 tiles
+  return ctas <= 4 * kSms || 2 * keys <= 15 * kTile * tokens;   // 7.5 tiles
 }
 
 int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,

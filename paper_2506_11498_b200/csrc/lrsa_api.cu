@@ -130,7 +130,7 @@ bool SeqBatches::next(SeqBatch* b) {
   return b->n > 0;
 }
 
-int run_score_select(const lrsa_params_t* p, const Geom& whole, const __nv_bfloat16* K, const __nv_bfloat16* V,
+int run_score_select(const Geom& whole, const __nv_bfloat16* K, const __nv_bfloat16* V,
                      int32_t* idx, float* score, void* ws, cudaStream_t st) {
   // the first launch clears the status word when it can: a single launch then, but for very many sequences
   const bool in_kernel = score_select_clears_status(whole);
@@ -195,7 +195,7 @@ int lrsa_score_select(const lrsa_params_t* params, const void* K, const void* V,
   if (!aligned(K, 16) || !aligned(V, 16) || !aligned(idx, 4) || !aligned(score, 4) || !aligned(workspace, 256))
     return LRSA_ERR_INVALID_ARG;
   if (workspace_bytes < score_select_ws_bytes(g)) return LRSA_ERR_WORKSPACE_TOO_SMALL;
-  return run_score_select(params, g, static_cast<const __nv_bfloat16*>(K), static_cast<const __nv_bfloat16*>(V),
+  return run_score_select(g, static_cast<const __nv_bfloat16*>(K), static_cast<const __nv_bfloat16*>(V),
                           idx, score, workspace, static_cast<cudaStream_t>(cuda_stream));
 }
 

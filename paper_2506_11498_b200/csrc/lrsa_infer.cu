@@ -658,9 +658,8 @@ __global__ void __launch_bounds__(kRows * D) decode_merge_kernel(const float* pa
 // has a CTA per query head: not for hundreds of them.  us, decode_kernel | split kernel (data as in that kernel's head):
 // 18/2 heads, 148 CTAs 16.4 | 11.0, 600 23.6 | 28.1; 72/8, 112 CTAs 12.1 | 9.2, 592 24.1 | 23.8; batch 16 of 18/2, 448 16.5 | 21.5;
 // 160/8, 592 CTAs 40.4 | 32.6; batch 16 of 40/2, 448 CTAs 29.3 | 33.9.
-constexpr int kSplitSms = 148;
 int decode_splits(int n_keys) { return n_keys > 0 ? (n_keys + kDecKeys - 1) / kDecKeys : 1; }
-long long split_ctas_limit(const Geom& g) { return kSplitSms * (g.G > kDecHeads ? 4LL : 3LL); }
+long long split_ctas_limit(const Geom& g) { return kSms * (g.G > kDecHeads ? 4LL : 3LL); }
 bool use_split_kernel(const Geom& g, int n_keys) {
   return g.G > 8 && (long long)g.B * g.Hq <= 512 && (long long)g.B * g.Hkv * decode_splits(n_keys) <= split_ctas_limit(g);
 }
@@ -680,7 +679,7 @@ DecodePlan decode_plan(const Geom& g, int n_keys, int max_splits = kDecMaxSplits
   // cluster lies in one group of SMs (ClusterRoom).  (One sequence, 4 heads, d = 128: 9471 keys, one cluster for a
   // head 17.7 us a token with 8 CTAs, 15.8 with 16; 66 000 keys 107 us with one cluster of 16, 34.5 with two.)
   const int max_warps = dec_max_warps(p.nh);
-  p.warps = BH * p.blocks > 2LL * 148 * max_warps ? 4 : max_warps;
+  p.warps = BH * p.blocks > 2LL * kSms * max_warps ? 4 : max_warps;
   const int per_sm = max_warps / p.warps;
   const ClusterRoom& room = cluster_room();
   long long best = -1;
@@ -688,7 +687,7 @@ DecodePlan decode_plan(const Geom& g, int n_keys, int max_splits = kDecMaxSplits
     const long long at_once = room.at_once(per_sm, s);
     for (int grp = 1; grp <= kDecMaxGroups; grp *= 2) {
       const int n = s * grp;
-      if (n > 1 && ((n - 1) * p.warps >= p.blocks || BH * n > 148LL * per_sm * 4)) break;
+      if (n > 1 && ((n - 1) * p.warps >= p.blocks || BH * n > (long long)kSms * per_sm * 4)) break;
       const long long waves = (BH * grp + at_once - 1) / at_once;
       const int per_cta = (p.blocks + n - 1) / n;
       const long long cost = waves * ((per_cta + p.warps - 1) / p.warps + 2) + (grp > 1 ? 3 : 0);

@@ -42,6 +42,8 @@ void seq_geom(const Geom& whole, const int32_t* cu, int n_seqs, int s, int woff,
 // Validates `p` and fills `g`. Returns an lrsa_status.
 int make_geom(const lrsa_params_t* p, Geom* g);
 
+constexpr int kSms = 148;   // of a B200; used in the rules that choose between forms (what a cluster finds room in is asked: ClusterRoom)
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Workspace header (first 256 bytes of every workspace).
@@ -79,8 +81,8 @@ struct LaunchCounter {
 };
 LaunchCounter& launch_counter();
 
-// lrsa_api.cu : clears the status header of `ws`, then scores and selects sequence after sequence.
-int run_score_select(const lrsa_params_t* p, const Geom& whole, const __nv_bfloat16* K, const __nv_bfloat16* V,
+// lrsa_api.cu : scores and selects every sequence of the row; the status word of `ws` is cleared by the first launch.
+int run_score_select(const Geom& whole, const __nv_bfloat16* K, const __nv_bfloat16* V,
                      int32_t* idx, float* score, void* ws, cudaStream_t st);
 
 // score_select.cu : scores and selects the windows of n sequences of a packed row (or one sequence).  The status header of
@@ -110,11 +112,6 @@ size_t attn_fwd_ws_bound(const Geom& g);
 int launch_attn_fwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                           const __nv_bfloat16* V, const int32_t* idx, __nv_bfloat16* O, float* LSE,
                           void* ws, cudaStream_t st);
-
-int launch_attn_ref_bwd_dkv(const Geom& g, const __nv_bfloat16* Q, const __nv_bfloat16* K,
-                            const __nv_bfloat16* V, const __nv_bfloat16* dO, const float* LSE,
-                            const int32_t* idx, const float* Dsum, __nv_bfloat16* dK, __nv_bfloat16* dV,
-                            cudaStream_t st);
 
 // attn_bwd_*_sm100.cu : tcgen05 / TMEM backward.
 size_t attn_bwd_ws_bytes(const Geom& g);

@@ -60,7 +60,7 @@ extern "C" int lrsa_score_select_static(const lrsa_params_t* params, const void*
   if (sc != LRSA_OK) return sc;
   // The status word, counters and statistics that must start at zero are cleared on the stream before the
   // kernel; whatever else the previous call left in the array is overwritten before it is read.
-  return run_score_select(params, g, static_cast<const __nv_bfloat16*>(K), static_cast<const __nv_bfloat16*>(V),
+  return run_score_select(g, static_cast<const __nv_bfloat16*>(K), static_cast<const __nv_bfloat16*>(V),
                           idx, score, scratch, static_cast<cudaStream_t>(cuda_stream));
 }
 

@@ -51,9 +51,6 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ---- proxies / fences ----
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void tc_fence_before_sync() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -101,6 +98,10 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 // the issuing warp counts.  With a branch around each product (if (elect_one()) ...) and with these, 28/4 heads, d = 128:
 // forward 98.3 -> 92.0 us at 4K tokens and 266 -> 250 at 8K, whole training step 394 -> 376 us at 4K, 10.36 -> 10.12 ms at 32K
 // (one predicated instruction at a time: 94.0 and 261 us).
+// Order: the kernels let a product overwrite columns of tensor memory that an earlier product of the same thread reads (S over P,
+// dP over dS) without waiting in between.  PTX states that pipelining for products on one accumulator in one shape only.  That all
+// products of a thread run in the order of issue, whatever their accumulators and shapes, is what sm_100a does here, not a documented
+// guarantee; an overlap would show as outputs that change between repeats (tests/test_gpu_parity.py repeats the forward).
 // SS: both operands K-major in a 128-byte-swizzled tile (32 bytes a step).
 __device__ __forceinline__ void umma_ss4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate, uint32_t leader) {
@@ -176,17 +177,6 @@ __device__ __forceinline__ uint64_t make_smem_desc_sw128(uint32_t saddr, uint32_
   d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
   d |= (uint64_t)1 << 46;   // descriptor version for sm_100
   d |= (uint64_t)2 << 61;   // SWIZZLE_128B
-  return d;
-}
-
-// The same for an operand without swizzle, K-major: core matrices of 8 rows x 16 bytes (128 contiguous bytes),
-// lbo bytes from one 8-element k-group to the next, sbo bytes from one group of eight rows to the next.
-__device__ __forceinline__ uint64_t make_smem_desc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
   return d;
 }
 
@@ -290,14 +280,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
-}
-
-// x as the sum of three bf16 numbers (24 bits): x = lo half, hi half of .x, lo half of .y.
-__device__ __forceinline__ uint2 split_bf16x3(float x) {
-  const uint32_t h = pack_bf16(x, 0.f) & 0xffffu;
-  const float r = x - __uint_as_float(h << 16);
-  const uint32_t m = pack_bf16(r, 0.f) & 0xffffu;
-  return make_uint2(h | (m << 16), pack_bf16(r - __uint_as_float(m << 16), 0.f));
 }
 
 }  // namespace ptx
