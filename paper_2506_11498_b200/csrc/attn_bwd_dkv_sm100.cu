@@ -74,7 +74,8 @@ struct DkvArgs {
   const int32_t* idx;    // kept positions: head bh at idx + bh * kept_stride
   int kept_stride;       // Wtot * K entries per (batch, KV head)
   int Nrow;              // tokens per (batch, head) row (the stride of every tensor)
-  const float* kpart;    // when not null: partial sums of the mean key, to be finished
+  const float* kpart;    // when not null: partial sums of the mean key (splits of them), to be finished
+  int splits;
   float* kbar;
   const float2* stats;   // per query row: (-LSE * log2(e), D~ = rowsum(dO * O) from the bf16 O)
   float* Dacc;           // [B*Hq][N], zeroed: receives sum_j P_tj dP_tj, the accurate D for the dQ kernel
@@ -136,15 +137,8 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     fence_barrier_init();
   }
   if (warp == 1) { tmem_alloc(smem_u32(&ctl.tmem_base), 512); tmem_relinquish(); }
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = ctl.tmem_base;
-  volatile int* abort = &ctl.abort;
 
   // ---- which tile, which segment ----
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int bh_kv = blockIdx.x % a.BHkv;
   int seg = blockIdx.x / a.BHkv, sq = 0;
   if constexpr (NSEQ > 1) {
@@ -152,23 +146,38 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
     seg -= a.seg0[sq];
   }
   const DkvPlan& p = a.plan[sq];
+  if (tid == 0) {
+    prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.dO[sq]); prefetch_tensormap(&maps.k[sq]);
+    prefetch_tensormap(&maps.v[sq]); prefetch_tensormap(&maps.kg[sq]); prefetch_tensormap(&maps.vg[sq]);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
   const int tok0 = a.tok0[sq];
   const int32_t* kept = a.idx + (size_t)bh_kv * a.kept_stride + a.kept_off[sq];   // this head's, this sequence's windows
   const int2 ts = a.seg_map[a.map0[sq] + seg];
   const KvTile kt = describe_tile(p, ts.x);
-  const int it_begin = ts.y * p.seg;
-  const int n = min(p.seg, p.G * kt.nq - it_begin);
+  const int seg_len = segment_length(p, p.G * kt.nq), it_begin = ts.y * seg_len;
+  const int n = min(seg_len, p.G * kt.nq - it_begin);
   const int hq0 = (bh_kv / a.Hkv) * a.Hq + (bh_kv % a.Hkv) * p.G;   // first query head of the group
 
   // iteration gi of the tile: query tile nq-1 - gi/G (from the last query backwards) of head gi % G
   const int qt0 = kt.nq - 1 - it_begin / p.G, hd0 = it_begin % p.G;
 
+  // TMA producer's loads of the step with query tile qt of head hd (of the group)
+  auto load_q = [&](int slot, int qt, int hd) {
+    const uint32_t full = smem_u32(&ctl.q_full[slot]);
+    mbar_expect_tx(full, Cfg::kTileBytes);
+    for (int h = 0; h < Cfg::kSub; ++h)
+      tma_load_3d(sQ + slot * Cfg::kTileBytes + h * Cfg::kSubBytes, &maps.q[sq], h * 64, kt.qb + qt * kQRows, hq0 + hd, full);
+  };
+  auto load_o = [&](int slot, int qt, int hd) {
+    const uint32_t full = smem_u32(&ctl.o_full[slot]);
+    mbar_expect_tx(full, Cfg::kTileBytes);
+    for (int h = 0; h < Cfg::kSub; ++h)
+      tma_load_3d(sO + slot * Cfg::kTileBytes + h * Cfg::kSubBytes, &maps.dO[sq], h * 64, kt.qb + qt * kQRows, hq0 + hd, full);
+  };
   if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.dO[sq]);
-      mbar_expect_tx(smem_u32(&ctl.kv_full), 2 * Cfg::kTileBytes);
-    }
+    // K_j, V_j and the first Q and dO are fetched while the other warps get their tensor memory
+    if (lane == 0) mbar_expect_tx(smem_u32(&ctl.kv_full), 2 * Cfg::kTileBytes);
     __syncwarp();
     if (kt.kind == 0) {
       // every lane gathers four rows of the list tile from their positions in K and V
@@ -186,29 +195,33 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
         tma_load_3d(sV + h * Cfg::kSubBytes, &maps.v[sq], h * 64, kt.row0, bh_kv, smem_u32(&ctl.kv_full));
       }
     }
+    if (lane == 0) { load_q(0, qt0, hd0); load_o(0, qt0, hd0); }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = ctl.tmem_base;
+  volatile int* abort = &ctl.abort;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  if (warp == 0) {
+    // ---------------- TMA producer: the other steps ----------------
     if (lane == 0) {
-      int qt = qt0, hd = hd0, slq = 0, slo = 0, phq = 0, pho = 0;
-      int nq_issued = 0, no_issued = 0;
+      int qt = qt0, hd = hd0, slq = 1, slo = 1, phq = 0, pho = 0;
+      int nq_issued = 1, no_issued = 1;
       bool ok = true;
-      for (int it = 0; it < n; ++it) {
-        const int hq = hq0 + hd, q0 = kt.qb + qt * kQRows;
+      for (int it = 1; it < n; ++it) {
+        if (++hd == p.G) { hd = 0; --qt; }
         if (it >= NQ) ok = mbar_wait(smem_u32(&ctl.q_empty[slq]), phq ^ 1, abort);
         if (!ok) break;
-        const uint32_t qf = smem_u32(&ctl.q_full[slq]);
-        mbar_expect_tx(qf, Cfg::kTileBytes);
-        for (int h = 0; h < Cfg::kSub; ++h)
-          tma_load_3d(sQ + slq * Cfg::kTileBytes + h * Cfg::kSubBytes, &maps.q[sq], h * 64, q0, hq, qf);
+        load_q(slq, qt, hd);
         ++nq_issued;
         if (it >= NO) ok = mbar_wait(smem_u32(&ctl.o_empty[slo]), pho ^ 1, abort);
         if (!ok) break;
-        const uint32_t of = smem_u32(&ctl.o_full[slo]);
-        mbar_expect_tx(of, Cfg::kTileBytes);
-        for (int h = 0; h < Cfg::kSub; ++h)
-          tma_load_3d(sO + slo * Cfg::kTileBytes + h * Cfg::kSubBytes, &maps.dO[sq], h * 64, q0, hq, of);
+        load_o(slo, qt, hd);
         ++no_issued;
         if (++slq == NQ) { slq = 0; phq ^= 1; }
         if (++slo == NO) { slo = 0; pho ^= 1; }
-        if (++hd == p.G) { hd = 0; --qt; }
       }
       if (!ok) {
         // give loads already in flight a bounded chance to land before the CTA's smem is released
@@ -296,7 +309,7 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
       for (int ch = lane * 4; ch < D; ch += 128) {
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
-        for (int i = 0; i < kMeanSplits; ++i) {
+        for (int i = 0; i < a.splits; ++i) {
           const float4 x = *reinterpret_cast<const float4*>(a.kpart + ((size_t)i * a.BHkv + blockIdx.x) * D + ch);
           sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
         }
@@ -458,22 +471,32 @@ lrsa_bwd_dkv_kernel(const __grid_constant__ DkvMaps<NSEQ> maps, const __grid_con
       const bool is_k = wg < 2;
       const uint32_t acc = tmem + lane_addr + (is_k ? Cfg::kColK : Cfg::kColV) + (wg & 1) * CH;
       const float mul = is_k ? a.scale : 1.0f;
-      // a row of a compact tile lands on the position it was gathered from
-      const int out_row = kt.kind == 0
-                              ? compact_row_pos(kept, p.S, p.Rc, kt.row0 + r, tok0)
-                              : kt.row0 + r;
-      float* dst = (is_k ? a.dKf : a.dVf) + ((size_t)bh_kv * a.Nrow + tok0 + out_row) * D + (wg & 1) * CH;
+      // A row of a compact tile lands on the position it was gathered from.  The rows go through shared memory (the rings are
+      // idle: every product is done), so that a warp adds to whole lines: every lane a row of its own, the epilogue is bound by
+      // the 32 lines that each instruction touches.  Rows are padded by 16 bytes so that a warp's stores spread over the banks.
+      const int out_row = !key_ok ? -1 : kt.kind == 0 ? compact_row_pos(kept, p.S, p.Rc, kt.row0 + r, tok0) : kt.row0 + r;
+      constexpr int kStride = CH + 4;
+      static_assert(Cfg::kSoftWarps * 32 * kStride * 4 <= Cfg::kOffStats - Cfg::kOffRingQ, "the rows of every warp fit the rings");
+      float* stage = reinterpret_cast<float*>(smem_raw + Cfg::kOffRingQ) + (warp - 4) * 32 * kStride;
 #pragma unroll
       for (int q = 0; q < CH / 32; ++q) {
         uint32_t o[32];
         tmem_ld32(acc + q * 32, o);
         tmem_wait_ld();
-        if (key_ok) {
 #pragma unroll
-          for (int v = 0; v < 8; ++v)
-            red_add_v4(dst + q * 32 + v * 4, __uint_as_float(o[4 * v]) * mul, __uint_as_float(o[4 * v + 1]) * mul,
-                       __uint_as_float(o[4 * v + 2]) * mul, __uint_as_float(o[4 * v + 3]) * mul);
-        }
+        for (int v = 0; v < 8; ++v)
+          *reinterpret_cast<float4*>(stage + lane * kStride + q * 32 + v * 4) =
+              make_float4(__uint_as_float(o[4 * v]) * mul, __uint_as_float(o[4 * v + 1]) * mul,
+                          __uint_as_float(o[4 * v + 2]) * mul, __uint_as_float(o[4 * v + 3]) * mul);
+      }
+      __syncwarp();
+      constexpr int kLanes = CH / 4, kRows = 32 / kLanes;   // lanes per row, rows per instruction
+      float* dst = (is_k ? a.dKf : a.dVf) + ((size_t)bh_kv * a.Nrow + tok0) * D + (wg & 1) * CH + lane % kLanes * 4;
+#pragma unroll 4
+      for (int i = 0; i < 32; i += kRows) {
+        const int row = i + lane / kLanes, to = __shfl_sync(0xffffffffu, out_row, row);
+        const float4 x = *reinterpret_cast<const float4*>(stage + row * kStride + lane % kLanes * 4);
+        if (to >= 0) red_add_v4(dst + (size_t)to * D, x.x, x.y, x.z, x.w);
       }
     }
   }
@@ -512,7 +535,7 @@ static int launch_dkv_t(const Geom& whole, const SeqBatch& b, const DkvBatch& db
   a.n_seqs = b.n;
   a.BHkv = (int)BHkv; a.Hq = whole.Hq; a.Hkv = whole.Hkv;
   a.idx = p.idx; a.kept_stride = whole.Wtot * whole.K; a.Nrow = whole.Nrow;
-  a.kpart = mean ? p.kpart : nullptr; a.kbar = p.kbar;
+  a.kpart = mean ? p.kpart : nullptr; a.kbar = p.kbar; a.splits = mean_splits(whole.Nrow);
   a.stats = p.stats; a.Dacc = p.Dacc; a.seg_map = p.seg_map; a.dKf = p.dKf; a.dVf = p.dVf;
   a.scale = whole.scale; a.scale_log2 = whole.scale * 1.4426950408889634f; a.status = p.status;
   auto kern = lrsa_bwd_dkv_kernel<D, NSEQ>;

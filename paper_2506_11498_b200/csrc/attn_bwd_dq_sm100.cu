@@ -101,7 +101,20 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
   // the list's last tile comes first when it holds no more than kShort keys: its products are that wide only
   const int sh = n_ct > 0 && rb.n_front - (n_ct - 1) * kKeys <= kShort ? 1 : 0;
 
+  // K or V tile `it` of the order K_0, V_0, K_1, ... into its ring slot
+  auto load_tile = [&](int it) {
+    const int j = it >> 1, which = it & 1, slot = it % NS;
+    const uint32_t full = smem_u32(&bars.kv_full[slot]);
+    mbar_expect_tx(full, Cfg::kKTileBytes);
+    const bool compact = j < n_ct;
+    const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
+    const int row = compact ? (j < sh ? n_ct - 1 : j - sh) * kKeys : rb.dense_start + (j - n_ct) * kKeys;
+    for (int h = 0; h < Cfg::kSub; ++h)
+      tma_load_3d(sRing + slot * Cfg::kKTileBytes + h * Cfg::kKSubBytes, map, h * 64, row, bh_kv, full);
+  };
   if (tid == 0) {
+    prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.dO[sq]); prefetch_tensormap(&maps.k[sq]);
+    prefetch_tensormap(&maps.v[sq]); prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
     abort_s = 0;
     mbar_init(smem_u32(&bars.q_full), 1);
     mbar_init(smem_u32(&bars.qt_ready), 256);
@@ -112,6 +125,14 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
       mbar_init(smem_u32(&bars.p_full[b]), 256);    // every softmax thread
     }
     fence_barrier_init();
+    // the first loads, while the other warps get their tensor memory
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+    mbar_expect_tx(smem_u32(&bars.q_full), 2 * Cfg::kQTileBytes);
+    for (int h = 0; h < Cfg::kSub; ++h) {
+      tma_load_3d(sQ + h * Cfg::kQSubBytes, &maps.q[sq], h * 64, rb.q0, bh, smem_u32(&bars.q_full));
+      tma_load_3d(sdO + h * Cfg::kQSubBytes, &maps.dO[sq], h * 64, rb.q0, bh, smem_u32(&bars.q_full));
+    }
+    for (int it = 0; it < min(NS, 2 * n); ++it) load_tile(it);
   }
   if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), Cfg::kCols); tmem_relinquish(); }
   tc_fence_before_sync();
@@ -119,38 +140,22 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
   volatile int* abort = &abort_s;
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.dO[sq]); prefetch_tensormap(&maps.k[sq]);
-      prefetch_tensormap(&maps.v[sq]); prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
-      mbar_expect_tx(smem_u32(&bars.q_full), 2 * Cfg::kQTileBytes);
-      for (int h = 0; h < Cfg::kSub; ++h) {
-        tma_load_3d(sQ + h * Cfg::kQSubBytes, &maps.q[sq], h * 64, rb.q0, bh, smem_u32(&bars.q_full));
-        tma_load_3d(sdO + h * Cfg::kQSubBytes, &maps.dO[sq], h * 64, rb.q0, bh, smem_u32(&bars.q_full));
-      }
-      int it = 0;
+      int it = NS;   // the first NS tiles are on their way
       bool ok = true;
-      for (int j = 0; j < n && ok; ++j) {
-        for (int which = 0; which < 2 && ok; ++which, ++it) {
-          const int slot = it % NS, use = it / NS;
-          if (use > 0) ok = mbar_wait(smem_u32(&bars.kv_empty[slot]), (use - 1) & 1, abort);
-          if (!ok) break;
-          const uint32_t full = smem_u32(&bars.kv_full[slot]);
-          mbar_expect_tx(full, Cfg::kKTileBytes);
-          const bool compact = j < n_ct;
-          const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
-          const int row = compact ? (j < sh ? n_ct - 1 : j - sh) * kKeys : rb.dense_start + (j - n_ct) * kKeys;
-          for (int h = 0; h < Cfg::kSub; ++h)
-            tma_load_3d(sRing + slot * Cfg::kKTileBytes + h * Cfg::kKSubBytes, map, h * 64, row, bh_kv, full);
-        }
+      for (; it < 2 * n; ++it) {
+        ok = mbar_wait(smem_u32(&bars.kv_empty[it % NS]), (it / NS - 1) & 1, abort);
+        if (!ok) break;
+        load_tile(it);
       }
       if (!ok) {
         // give loads already in flight a bounded chance to land before the CTA's smem is released
-        for (int back = 1; back <= NS && back <= it; ++back) {
+        for (int back = 1; back <= NS; ++back) {
           const int i2 = it - back;
           const long long t0 = clock64();
           while (!mbar_try_wait(smem_u32(&bars.kv_full[i2 % NS]), (i2 / NS) & 1) && clock64() - t0 < 2000000) {}
@@ -305,8 +310,9 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
     asm volatile("bar.sync 1, 256;" ::: "memory");   // the eight softmax warps, whether or not a wait gave up
     if (ok) ok = mbar_wait(smem_u32(&bars.acc_done), 0, abort);
     // The dQ rows go through shared memory (the Q and dO tiles are idle since their copy into tensor
-    // memory) and leave as one bulk copy per row: per-thread 16-byte stores to rows 256 bytes apart cost
+    // memory), so that a warp writes whole half rows: per-thread 16-byte stores to rows 256 bytes apart cost
     // a transaction each.  Rows are padded by 16 bytes so that a warp's stores spread over the banks.
+    // (With a bulk copy per row a CTA waits for the copies to have read them before it may end.)
     constexpr int kRowBytes = D * 2, kStageStride = kRowBytes + 16;
     unsigned char* stage_out = smem_raw + (sQ - smem_u32(smem_raw));
     if (ok) {
@@ -333,16 +339,12 @@ lrsa_bwd_dq_kernel(const __grid_constant__ DqMaps<NSEQ> maps, const __grid_const
           *reinterpret_cast<uint4*>(srow + (q * 4 + v) * 16) = w;
         }
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy reads these stores
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");   // both halves of every row are staged (or a wait gave up)
-    if (half == 0 && live && !*abort) {
-      __nv_bfloat16* orow = a.dQ + (row0 + qpos) * D;
-      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(orow),
-                   "r"(smem_u32(stage_out + row * kStageStride)), "r"((uint32_t)kRowBytes)
-                   : "memory");
-      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory is released at exit
+      __syncwarp();
+      if (!*abort) {
+        const int q = rb.q0 + quad * 32;   // the warp's first row
+        store_rows<D>(stage_out + quad * 32 * kStageStride + half * D, kStageStride,
+                      reinterpret_cast<unsigned char*>(a.dQ + (row0 + q) * D) + half * D, kRowBytes, rb.q_end - q, lane);
+      }
     }
   }
 

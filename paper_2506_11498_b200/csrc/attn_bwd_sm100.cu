@@ -21,7 +21,7 @@ struct PrepArgs {
   float* kpart;
   float4* zero;          // the fp32 accumulators
   long long zero_n, rows;
-  int N, d, BHkv;
+  int N, d, BHkv, splits;
   int* status;           // cleared when not null
   int* seg_cnt;
   int2* seg_map;
@@ -73,12 +73,12 @@ __device__ __forceinline__ void prep_stats(const PrepArgs& a, long long block) {
   }
 }
 
-// kpart[split][bh][c] = (1/N) * sum of K[bh][t][c] over the split's rows.
+// kpart[split][bh][c] = (1/N) * sum of K[bh][t][c] over the split's rows (a.splits of them).
 __device__ __forceinline__ void prep_mean(const PrepArgs& a, int block) {
   __shared__ float red[256 * 8];
-  const int bh = block / kMeanSplits, split = block % kMeanSplits, tid = threadIdx.x, d = a.d;
+  const int bh = block / a.splits, split = block % a.splits, tid = threadIdx.x, d = a.d;
   const int lpr = d / 8, rps = 256 / lpr;          // lanes per row (16 bytes each), rows per step
-  const int chunk = tid % lpr, r_in = tid / lpr, per = (a.N + kMeanSplits - 1) / kMeanSplits;
+  const int chunk = tid % lpr, r_in = tid / lpr, per = (a.N + a.splits - 1) / a.splits;
   const int r0 = split * per, r1 = min(a.N, r0 + per);
   float acc[8];
 #pragma unroll
@@ -106,7 +106,9 @@ __device__ __forceinline__ void prep_mean(const PrepArgs& a, int block) {
 
 // Everything that has to be in place before the dK/dV kernel, in one launch: its parts are bound by memory (O, dO and K
 // read once, the accumulators written) or by one block's serial work (launch order) and overlap.  As four kernels and two
-// memsets they took 206 us of a 32K step (28/4 heads, d = 128) and 33 us with the gaps of a 4K one (8 heads, d = 64).
+// memsets they took 206 us of a 32K step (28/4 heads, d = 128) and 33 us with the gaps of a 4K one (8 heads, d = 64).  In
+// small problems the block of the launch order and the number of blocks bound it: with one thread adding up the order's table and 64 parts
+// of the mean key per head whatever its length 7.8 us at 4K (8 heads, d = 64), now 5.7.
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const __grid_constant__ PrepArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -255,9 +257,11 @@ int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
       cnt += dp.n_tiles;
       map += a.db.segs[s];
     }
+    const bool by_length = order_by_length((long long)map * BHkv);
+    for (int s = 0; s < b.n; ++s) a.db.plan[s].by_length = by_length;
     a.O = O; a.Olo = p.Olo; a.dO = dO; a.K = K; a.LSE = LSE; a.stats = p.stats; a.Dacc = p.Dacc; a.kpart = p.kpart;
     a.seg_cnt = p.seg_cnt; a.seg_map = p.seg_map;
-    a.N = g.Nrow; a.d = g.d; a.BHkv = BHkv;
+    a.N = g.Nrow; a.d = g.d; a.BHkv = BHkv; a.splits = mean_splits(g.Nrow);
     a.c = compact_args(g, b, K, V, idx, p.Kc, p.Vc, nullptr);
     a.status = first ? p.status : nullptr;
     a.zero = reinterpret_cast<float4*>(p.dKf);
@@ -266,7 +270,7 @@ int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
     a.rows = first ? (long long)g.B * g.Hq * g.Nrow : 0;
     const long long rows_per_block = 8LL * kPrepUnroll * (32 / (g.d >> 3));
     long long nb = b.n;
-    a.b_setup = (int)nb; nb += first ? kMeanSplits * BHkv : 0;
+    a.b_setup = (int)nb; nb += first ? a.splits * BHkv : 0;
     a.b_mean = (int)nb; nb += a.c.blocks();
     a.b_compact = (int)nb; nb += (a.rows + rows_per_block - 1) / rows_per_block;
     a.b_stats = (int)nb; nb += (a.zero_n + 256 * kZeroPerThread - 1) / (256 * kZeroPerThread);

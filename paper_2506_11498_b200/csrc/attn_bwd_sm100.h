@@ -18,6 +18,14 @@ inline int dkv_segment(long long iters) {
   return s < 16 ? 16 : s > kSegMax ? kSegMax : (int)s;
 }
 
+// Launch order of the dK/dV kernel: by length (see dkv_setup), with segments of a tile made about equally long?  Up to four CTAs per SM what
+// the last ones leave idle is what counts, beyond that the query tiles that neighbours share in L2.  Whole backward, us, by
+// length up to 0 | 4 | 6 | 8 CTAs per SM: 1777 tokens (28/4 heads, d = 128) 107 | 99 | 99 | 99, 5K (16/2, d = 64) 155 | 153 | 153 | 153;
+// 4K (28/4) 278 | 279 | 285 | 285, 8K 875 | 874 | 904 | 914, 8K (8/8, d = 64) 181 | 181 | 187 | 187, 16K (28/4) 2430 | 2440 | 2446 | 2509.
+inline bool order_by_length(long long ctas) {
+  return ctas <= 4 * kSms;
+}
+
 struct DkvPlan {
   int S, L, K, N, W, T, C, Wsel, ndp, Rc, G;
   int n_cmp;       // compact tiles
@@ -26,6 +34,7 @@ struct DkvPlan {
   int per_tail;    // dense tiles of the tail
   int n_tiles;
   int seg;         // inner iterations per CTA at most
+  int by_length;   // launch order
 };
 
 struct KvTile {
@@ -46,6 +55,7 @@ inline DkvPlan make_dkv_plan(const Geom& g, int seg) {
   p.per_tail = (g.T + kTile - 1) / kTile;
   p.n_tiles = p.n_cmp + p.n_sink + g.W * p.per_win + p.per_tail;
   p.seg = seg;
+  p.by_length = 0;
   return p;
 }
 
@@ -89,64 +99,107 @@ __host__ __device__ inline int tile_segments(const DkvPlan& p, const KvTile& t) 
   return (p.G * t.nq + p.seg - 1) / p.seg;
 }
 
+// Iterations per segment of a tile with `iters` of them (the last segment may have fewer).
+__host__ __device__ inline int segment_length(const DkvPlan& p, int iters) {
+  if (!p.by_length) return p.seg;
+  const int k = (iters + p.seg - 1) / p.seg;   // as many segments, of about the same length
+  return (iters + k - 1) / k;
+}
+
+// Exclusive prefix sums over a block of 256 threads; *total: the sum.  Ends with a barrier.
+__device__ inline int block_prefix(int v, int* total) {
+  __shared__ int warp_sum[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += n;
+  }
+  if (lane == 31) warp_sum[warp] = incl;
+  __syncthreads();
+  int before = incl - v, sum = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w < warp) before += warp_sum[w];
+    sum += warp_sum[w];
+  }
+  *total = sum;
+  __syncthreads();
+  return before;
+}
+
 // Launch order of the (tile, segment) pairs (one block of 256 threads).  Iteration i of a tile is query tile
 // nq-1 - i/G (counted from the last query) of head i%G, so segment s of every compact tile covers the
-// same queries of the same heads.  Compact tiles are therefore issued segment-major: the CTAs that run at
-// the same time then stream the same Q_i / dO_i tiles and share them through L2 instead of fetching
-// them from DRAM once per key tile.  Dense tiles (short lists, neighbours already overlap) follow in
-// position order.  seg_cnt: scratch of n_tiles + 1 ints; seg_map[x] = (tile, segment of the tile).
+// same queries of the same heads.
+//   by length  (small grids): the longest segments first, so that the last ones to start are short.
+//   otherwise  compact tiles are issued segment-major: the CTAs that run at the same time then stream the same Q_i / dO_i
+//              tiles and share them through L2 instead of fetching them from DRAM once per key tile.  Dense tiles (short
+//              lists, neighbours already overlap) follow in position order.
+// seg_cnt: scratch of n_tiles + 1 ints; seg_map[x] = (tile, segment of the tile).
 constexpr int kMaxSegsPerTile = 2048;
 __device__ inline void dkv_setup(const DkvPlan& p, int* seg_cnt, int2* seg_map) {
-  __shared__ int off[kMaxSegsPerTile + 1];   // off[s] = pairs of compact tiles with a segment index below s
-  __shared__ int s_mode, s_cmp_total;
-  __shared__ int run_sum[256];   // blockDim.x = 256
-  for (int i = threadIdx.x; i < p.n_tiles; i += blockDim.x) seg_cnt[i] = tile_segments(p, describe_tile(p, i));
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // segment-major order needs the compact tiles' segment counts to be non-increasing (later rows are
-    // seen by later chunks only) and few enough for the table; otherwise keep tile-major order
-    bool mono = p.n_cmp > 0 && seg_cnt[0] <= kMaxSegsPerTile;
-    for (int c = 1; c < p.n_cmp && mono; ++c) mono = seg_cnt[c] <= seg_cnt[c - 1];
-    int total = 0;
-    if (mono) {
-      int c = p.n_cmp;   // tiles [0, c) have more than s segments
-      const int maxs = seg_cnt[0];
-      for (int sgm = 0; sgm < maxs; ++sgm) {
-        while (c > 0 && seg_cnt[c - 1] <= sgm) --c;
-        off[sgm] = total;
-        total += c;
-      }
-    } else {
-      for (int c = 0; c < p.n_cmp; ++c) {
-        for (int sgm = 0; sgm < seg_cnt[c]; ++sgm) seg_map[total + sgm] = make_int2(c, sgm);
-        total += seg_cnt[c];
-      }
+  __shared__ int off[kMaxSegsPerTile];   // off[s] = pairs of compact tiles with a segment index below s; by length: see below
+  const int tid = threadIdx.x, nt = blockDim.x;   // 256
+  int total;
+  if (p.by_length) {
+    // off[k]: where the next segment of p.seg - k iterations goes
+    for (int k = tid; k < p.seg; k += nt) off[k] = 0;
+    __syncthreads();
+    for (int i = tid; i < p.n_tiles; i += nt) {
+      const int iters = p.G * describe_tile(p, i).nq;
+      if (iters == 0) continue;
+      const int len = segment_length(p, iters), full = (iters - 1) / len;
+      if (full) atomicAdd(&off[p.seg - len], full);
+      atomicAdd(&off[p.seg - (iters - full * len)], 1);
     }
-    s_mode = mono ? 1 : 0;
-    s_cmp_total = total;
+    __syncthreads();
+    const int at = block_prefix(tid < p.seg ? off[tid] : 0, &total);   // p.seg <= kSegMax < 256
+    if (tid < p.seg) off[tid] = at;
+    __syncthreads();
+    for (int i = tid; i < p.n_tiles; i += nt) {
+      const int iters = p.G * describe_tile(p, i).nq;
+      if (iters == 0) continue;
+      const int len = segment_length(p, iters), full = (iters - 1) / len;
+      const int pos = full ? atomicAdd(&off[p.seg - len], full) : 0;
+      for (int k = 0; k < full; ++k) seg_map[pos + k] = make_int2(i, k);
+      seg_map[atomicAdd(&off[p.seg - (iters - full * len)], 1)] = make_int2(i, full);
+    }
+    return;
   }
-  // dense tiles, position order: every thread takes a run of consecutive tiles
-  const int nd = p.n_tiles - p.n_cmp, per = (nd + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int d_lo = min(p.n_tiles, p.n_cmp + (int)threadIdx.x * per), d_hi = min(p.n_tiles, d_lo + per);
+  for (int i = tid; i < p.n_tiles; i += nt) seg_cnt[i] = tile_segments(p, describe_tile(p, i));
+  __syncthreads();
+  // segment-major order needs the compact tiles' segment counts to be non-increasing (later rows are
+  // seen by later chunks only) and few enough for the table; otherwise every tile is taken in position order
+  bool mono = p.n_cmp > 0 && seg_cnt[0] <= kMaxSegsPerTile;
+  for (int c = 1 + tid; c < p.n_cmp; c += nt) mono = mono && seg_cnt[c] <= seg_cnt[c - 1];
+  mono = __syncthreads_and(mono);
+  int base = 0;
+  if (mono) {
+    const int maxs = seg_cnt[0], per = (maxs + nt - 1) / nt;
+    const int lo = min(maxs, tid * per), hi = min(maxs, lo + per);
+    int c = p.n_cmp, mine = 0;   // tiles [0, c) have more than s segments
+    auto more_than = [&](int sgm, int c1) {
+      int a = 0, b = c1;
+      while (a < b) { const int m = (a + b) >> 1; if (seg_cnt[m] > sgm) a = m + 1; else b = m; }
+      return a;
+    };
+    for (int sgm = lo; sgm < hi; ++sgm) { c = more_than(sgm, c); off[sgm] = mine; mine += c; }
+    const int at = block_prefix(mine, &base);
+    for (int sgm = lo; sgm < hi; ++sgm) off[sgm] += at;
+    __syncthreads();
+    for (int t = tid; t < p.n_cmp; t += nt)
+      for (int sgm = 0; sgm < seg_cnt[t]; ++sgm) seg_map[off[sgm] + t] = make_int2(t, sgm);
+  }
+  // position order: every thread takes a run of consecutive tiles
+  const int first = mono ? p.n_cmp : 0, nd = p.n_tiles - first, per = (nd + nt - 1) / nt;
+  const int d_lo = min(p.n_tiles, first + tid * per), d_hi = min(p.n_tiles, d_lo + per);
   int mine = 0;
   for (int t = d_lo; t < d_hi; ++t) mine += seg_cnt[t];
-  run_sum[threadIdx.x] = mine;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = s_cmp_total;
-    for (int i = 0; i < (int)blockDim.x; ++i) { const int v = run_sum[i]; run_sum[i] = acc; acc += v; }
-  }
-  __syncthreads();
-  {
-    int pos = run_sum[threadIdx.x];
-    for (int t = d_lo; t < d_hi; ++t) {
-      for (int sgm = 0; sgm < seg_cnt[t]; ++sgm) seg_map[pos + sgm] = make_int2(t, sgm);
-      pos += seg_cnt[t];
-    }
-  }
-  if (s_mode) {
-    for (int c = threadIdx.x; c < p.n_cmp; c += blockDim.x)
-      for (int sgm = 0; sgm < seg_cnt[c]; ++sgm) seg_map[off[sgm] + c] = make_int2(c, sgm);
+  int pos = base + block_prefix(mine, &total);
+  for (int t = d_lo; t < d_hi; ++t) {
+    for (int sgm = 0; sgm < seg_cnt[t]; ++sgm) seg_map[pos + sgm] = make_int2(t, sgm);
+    pos += seg_cnt[t];
   }
 }
 
@@ -165,7 +218,9 @@ struct BwdPtrs {
   float *dKf, *dVf;         // fp32 accumulators [B*Hkv][N][d], zeroed
   int* status;
 };
+// Parts of the sum for the mean key: at most kMeanSplits, of 256 rows or more.
 constexpr int kMeanSplits = 64;
+inline int mean_splits(int rows) { return rows >= 256 * kMeanSplits ? kMeanSplits : rows > 256 ? rows / 256 : 1; }
 
 // Per sequence of the batch: its plan, where its parts of seg_cnt and seg_map start, its number of (tile, segment) pairs.
 struct DkvBatch {

@@ -172,6 +172,18 @@ __device__ __forceinline__ void compact_rows(const CompactArgs& c, int block) {
   reinterpret_cast<uint4*>(c.Vc)[dst] = v;
 }
 
+// Writes `BYTES` bytes (whole 16-byte chunks) of each of a warp's 32 rows from shared memory, `stride` bytes apart, to rows
+// `row_bytes` apart in global memory: neighbouring lanes take neighbouring chunks of a row.  Rows at or beyond n_rows are skipped.
+template <int BYTES>
+__device__ __forceinline__ void store_rows(const unsigned char* src, int stride, unsigned char* dst, int row_bytes, int n_rows, int lane) {
+  constexpr int kLanes = BYTES / 16, kRows = 32 / kLanes;   // lanes per row, rows per instruction
+  const int chunk = lane % kLanes * 16;
+#pragma unroll
+  for (int r = lane / kLanes; r < 32; r += kRows)
+    if (r < n_rows)
+      *reinterpret_cast<uint4*>(dst + (size_t)r * row_bytes + chunk) = *reinterpret_cast<const uint4*>(src + r * stride + chunk);
+}
+
 // 2-D bf16 tensor map over [rows][d] with a (64 x 1) box and 128-byte swizzle, for row gathers
 // (tile::gather4).  The key-outer dK/dV kernel loads its one list tile per CTA this way, four rows per
 // copy, straight from K and V into the swizzled operand tile.

@@ -59,6 +59,7 @@ struct FwdArgs {
   int tok0[NSEQ];          // first token of the sequence
   int block0[NSEQ + 1];    // blocks of the sequences before, per (batch, head)
   int n_seqs;
+  int fold;                // see block_rank
   int BH, Hq, Hkv, G, N;   // N: tokens per (batch, head) row of O and LSE (the row stride)
   __nv_bfloat16* O;
   __nv_bfloat16* Olo;        // optional: receives bf16(O_fp32 - O), the part of the output the bf16 O cannot hold
@@ -77,6 +78,15 @@ struct FwdBars {
   uint64_t p_full[2][kPParts];      // per query tile: the parts of P_t (128 / kPParts keys each) are stored
 };
 
+// Place of this CTA among the blocks of all heads, which are numbered heaviest first.  The CTAs of a grid of between one and
+// two per SM (`fold`: how many more than one) all start at once, the second ones on the first SMs again: the heaviest blocks get an SM of
+// their own, the others are paired heavy with light.
+__device__ __forceinline__ int block_rank(int fold) {
+  const int x = blockIdx.x;
+  if (fold == 0) return x;
+  return x >= kSms ? kSms + fold - 1 - (x - kSms) : x < fold ? kSms - fold + x : x - fold;
+}
+
 template <int D, int NSEQ, int TQ>
 __global__ void __launch_bounds__(FwdCfg<D, TQ>::kThreads, FwdCfg<D, TQ>::kPerSm)
 lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constant__ FwdArgs<NSEQ> a) {
@@ -91,8 +101,8 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = smem0, sRing = smem0 + TQ * Cfg::kQRegion;
 
-  const int bh = blockIdx.x % a.BH;
-  int blk = blockIdx.x / a.BH, sq = 0;
+  const int bh = block_rank(a.fold) % a.BH;
+  int blk = block_rank(a.fold) / a.BH, sq = 0;
   if constexpr (NSEQ > 1) {
     while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
     blk -= a.block0[sq];
@@ -108,6 +118,8 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   const int sh = n_ct > 0 && rb.n_front - (n_ct - 1) * kTile <= kShort ? 1 : 0;
 
   if (tid == 0) {
+    prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.k[sq]); prefetch_tensormap(&maps.v[sq]);
+    prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
     abort_s = 0;
     mbar_init(smem_u32(&bars.q_full), 1);
     for (int i = 0; i < NS; ++i) { mbar_init(smem_u32(&bars.kv_full[i]), 1); mbar_init(smem_u32(&bars.kv_empty[i]), 1); }
@@ -117,6 +129,19 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
       mbar_init(smem_u32(&bars.pv_done[t]), 1);
     }
     fence_barrier_init();
+    // Q, K_0 and V_0 are fetched while the other warps get their tensor memory
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+    mbar_expect_tx(smem_u32(&bars.q_full), (n1 > 0 ? 2 : 1) * Cfg::kTileBytes);
+    for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)
+      for (int h = 0; h < Cfg::kSub; ++h)
+        tma_load_3d(sQ + t * Cfg::kQRegion + h * Cfg::kSubBytes, &maps.q[sq], h * 64, rb.q0 + t * kTile, bh, smem_u32(&bars.q_full));
+    const int row = n_ct > 0 ? (sh ? n_ct - 1 : 0) * kTile : rb.dense_start;
+    for (int which = 0; which < 2; ++which) {
+      const CUtensorMap* map = n_ct > 0 ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
+      mbar_expect_tx(smem_u32(&bars.kv_full[which]), Cfg::kTileBytes);
+      for (int h = 0; h < Cfg::kSub; ++h)
+        tma_load_3d(sRing + which * Cfg::kTileBytes + h * Cfg::kSubBytes, map, h * 64, row, bh_kv, smem_u32(&bars.kv_full[which]));
+    }
   }
   if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), Cfg::kCols); tmem_relinquish(); }
   tc_fence_before_sync();
@@ -124,7 +149,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
   volatile int* abort = &abort_s;
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // The softmax threads hold a row of 128 scores: they take the registers the other warps do not need
@@ -135,15 +160,9 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.k[sq]); prefetch_tensormap(&maps.v[sq]);
-      prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
-      mbar_expect_tx(smem_u32(&bars.q_full), (n1 > 0 ? 2 : 1) * Cfg::kTileBytes);
-      for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)
-        for (int h = 0; h < Cfg::kSub; ++h)
-          tma_load_3d(sQ + t * Cfg::kQRegion + h * Cfg::kSubBytes, &maps.q[sq], h * 64, rb.q0 + t * kTile, bh, smem_u32(&bars.q_full));
-      int it = 0;
+      int it = 2;
       bool ok = true;
-      for (int j = 0; j < n && ok; ++j) {
+      for (int j = 1; j < n && ok; ++j) {
         for (int which = 0; which < 2 && ok; ++which, ++it) {
           const int slot = it % NS, use = it / NS;
           if (use > 0) ok = mbar_wait(smem_u32(&bars.kv_empty[slot]), (use - 1) & 1, abort);
@@ -404,23 +423,32 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     }
     if (ok && nt > 0) ok = mbar_wait_warp(smem_u32(&bars.pv_done[t]), (nt - 1) & 1, abort);
     // The output rows go through shared memory (the tile's Q region, idle once its last S product is done,
-    // which pv_done implies) and leave as one bulk copy per row: per-thread 16-byte stores to rows 256 bytes
+    // which pv_done implies), so that a warp writes whole rows: per-thread 16-byte stores to rows 256 bytes
     // apart cost a transaction each.  Rows are padded by 16 bytes so that a warp's stores spread over the banks.
+    // (With a bulk copy per row a CTA waits for the copies to have read them before it may end.)
     constexpr int kRowBytes = D * 2, kStageStride = kRowBytes + 16;
     static_assert(kTile * kStageStride <= Cfg::kQRegion, "staging fits the Q region");
-    unsigned char* stage_out = smem_raw + (sQ - smem_u32(smem_raw)) + t * Cfg::kQRegion;
-    // (positions and pointers of the output are formed here, not kept in registers through the loop)
-    int blk_here = blockIdx.x;
-    asm volatile("" : "+r"(blk_here));
-    const size_t row0 = (size_t)(blk_here % a.BH) * a.N + a.tok0[sq];   // the sequence's first row of O and LSE
-    const int qpos = rb.q0 + t * kTile + row;
-    const bool store = qpos < rb.q_end && nt > 0;
     if (ok && nt > 0) {
+    // (where the rows lie is formed here again, from the thread and block numbers: kept through the loop it costs registers
+    // that the scores need)
+    int blk = block_rank(a.fold), thread = threadIdx.x;
+    asm volatile("" : "+r"(blk), "+r"(thread));
+    const int bh = blk % a.BH, w = thread >> 5, t = (w - 4) >> 2, row0_w = (w & 3) * 32, lane = thread & 31;   // row0_w: the warp's first row
+    blk /= a.BH;
+    int sq = 0;
+    if constexpr (NSEQ > 1) {
+      while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
+      blk -= a.block0[sq];
+    }
+    const RowBlock rb = decode_block(a.plan[sq], blk);
+    const int q = rb.q0 + t * kTile + row0_w, left = rb.q_end - q;   // first query of the warp, rows from there on
+    const size_t row0 = (size_t)bh * a.N + a.tok0[sq] + q;           // its row of O and LSE
+    unsigned char* stage = smem_raw + (smem0 - smem_u32(smem_raw)) + t * Cfg::kQRegion + row0_w * kStageStride;
       tc_fence_after_sync();
       const float inv = 1.0f / l;
-      unsigned char* srow = stage_out + row * kStageStride;
+      unsigned char* srow = stage + lane * kStageStride;
       // the remainder goes straight to global memory (contiguous bytes per thread, written once)
-      __nv_bfloat16* lo_row = a.Olo && store ? a.Olo + (row0 + qpos) * D : nullptr;
+      __nv_bfloat16* lo_row = a.Olo && lane < left ? a.Olo + (row0 + lane) * D : nullptr;
 #pragma unroll
       for (int q = 0; q < D / 32; ++q) {
         uint32_t o[32];
@@ -445,16 +473,9 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
           }
         }
       }
-      if (store) a.LSE[row0 + qpos] = m * a.scale + logf(l);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy reads this thread's stores
-      if (store && !*abort) {
-        __nv_bfloat16* orow = a.O + (row0 + qpos) * D;
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(orow),
-                     "r"(smem_u32(srow)), "r"((uint32_t)kRowBytes)
-                     : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory is released at exit
-      }
+      if (lane < left) a.LSE[row0 + lane] = m * a.scale + logf(l);
+      __syncwarp();
+      if (!*abort) store_rows<kRowBytes>(stage, kStageStride, reinterpret_cast<unsigned char*>(a.O + row0 * D), kRowBytes, left, lane);
     }
   }
 
@@ -560,6 +581,7 @@ static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat1
   a.status = status;
   const long long grid = (long long)a.block0[b.n] * a.BH;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
+  a.fold = Cfg::kPerSm == 2 && grid > kSms && grid <= 2 * kSms ? (int)grid - kSms : 0;
   auto kern = lrsa_fwd_kernel<D, NSEQ, TQ>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
   LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));

@@ -422,6 +422,33 @@ def test_packed_forms_for_many_ctas(heads, d, L, K, S, lens):
             check_close(name, f64(a[:, :, lo:hi]), f64(b))
 
 
+@pytest.mark.parametrize("B,heads,N,d,L,K,S", [
+    (37, (1, 1), 304, 64, 128, 32, 4), (149, (1, 1), 100, 64, 128, 32, 0), (74, (1, 1), 304, 64, 128, 32, 4),   # 148, 149, 296 blocks
+    (75, (1, 1), 304, 64, 128, 32, 4), (150, (1, 1), 304, 128, 128, 32, 4),   # 300; dK/dV of more than 592 CTAs
+    (2, (14, 2), 2500, 128, 256, 64, 4), (9, (14, 2), 2500, 128, 256, 64, 4),   # tiles of several segments, in both orders
+])
+def test_launch_orders_of_small_and_large_grids(B, heads, N, d, L, K, S):
+    """The order of a grid's blocks (which of them share an SM, longest segments first) follows its size: every sequence of a batch
+    as on its own.  O and LSE bit-equal, gradients (sums in another order) within the bound of two bf16 results."""
+    w = W("a_order", B, *heads, N, d, L, K, S, seed=61, values="channel_offset")
+    dev = to_dev(workloads.generate(w))
+
+    def run(p, t):
+        ws = [lrsa.new_workspace(n) for n in lrsa.lrsa_workspace_bytes(p)]
+        idx, _ = lrsa.lrsa_score_select(p, t["K"], t["V"], workspace=ws[0])
+        O, LSE = lrsa.lrsa_attn_fwd(p, t["Q"], t["K"], t["V"], idx, workspace=ws[1])
+        grads = lrsa.lrsa_attn_bwd(p, t["Q"], t["K"], t["V"], O, t["dO"], LSE, idx, workspace=ws[2])
+        assert all(lrsa.lrsa_workspace_status(x) == 0 for x in ws)
+        return idx, O, LSE, *grads
+    whole = run(lrsa.Params.from_workload(w), dev)
+    for b in (0, B // 2, B - 1):
+        one = run(lrsa.Params.from_workload(w.with_(B=1)), {x: dev[x][b:b + 1].contiguous() for x in dev})
+        for t, o in zip(whole[:3], one[:3]):
+            assert torch.equal(t[b:b + 1], o)
+        for name, t, o in zip(("dQ", "dK", "dV"), whole[3:], one[3:]):
+            check_close(name, f64(t[b:b + 1]), f64(o))
+
+
 @pytest.mark.parametrize("B,heads,N,d,L,S", [(1, (28, 4), 6000, 128, 512, 4), (4, (28, 4), 3000, 128, 512, 17), (2, (8, 8), 8000, 64, 256, 16)])
 def test_forward_gives_the_same_bits_every_time(B, heads, N, d, L, S):
     """P is overwritten by the next scores as soon as the product that reads it has been issued, on the order in which the tensor
