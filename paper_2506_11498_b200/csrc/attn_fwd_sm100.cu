@@ -421,7 +421,6 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
       f2_unpack(sum2, sum0, sum1);
       l += sum0 + sum1;
     }
-    if (ok && nt > 0) ok = mbar_wait_warp(smem_u32(&bars.pv_done[t]), (nt - 1) & 1, abort);
     // The output rows go through shared memory (the tile's Q region, idle once its last S product is done,
     // which pv_done implies), so that a warp writes whole rows: per-thread 16-byte stores to rows 256 bytes
     // apart cost a transaction each.  Rows are padded by 16 bytes so that a warp's stores spread over the banks.
@@ -429,53 +428,55 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     constexpr int kRowBytes = D * 2, kStageStride = kRowBytes + 16;
     static_assert(kTile * kStageStride <= Cfg::kQRegion, "staging fits the Q region");
     if (ok && nt > 0) {
-    // (where the rows lie is formed here again, from the thread and block numbers: kept through the loop it costs registers
-    // that the scores need)
-    int blk = block_rank(a.fold), thread = threadIdx.x;
-    asm volatile("" : "+r"(blk), "+r"(thread));
-    const int bh = blk % a.BH, w = thread >> 5, t = (w - 4) >> 2, row0_w = (w & 3) * 32, lane = thread & 31;   // row0_w: the warp's first row
-    blk /= a.BH;
-    int sq = 0;
-    if constexpr (NSEQ > 1) {
-      while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
-      blk -= a.block0[sq];
-    }
-    const RowBlock rb = decode_block(a.plan[sq], blk);
-    const int q = rb.q0 + t * kTile + row0_w, left = rb.q_end - q;   // first query of the warp, rows from there on
-    const size_t row0 = (size_t)bh * a.N + a.tok0[sq] + q;           // its row of O and LSE
-    unsigned char* stage = smem_raw + (smem0 - smem_u32(smem_raw)) + t * Cfg::kQRegion + row0_w * kStageStride;
-      tc_fence_after_sync();
-      const float inv = 1.0f / l;
-      unsigned char* srow = stage + lane * kStageStride;
-      // the remainder goes straight to global memory (contiguous bytes per thread, written once)
-      __nv_bfloat16* lo_row = a.Olo && lane < left ? a.Olo + (row0 + lane) * D : nullptr;
+      // (where the rows lie is formed here again, from the thread and block numbers: kept through the loop it costs registers
+      // that the scores need)
+      int blk = block_rank(a.fold), thread = threadIdx.x;
+      asm volatile("" : "+r"(blk), "+r"(thread));
+      const int bh = blk % a.BH, w = thread >> 5, t = (w - 4) >> 2, row0_w = (w & 3) * 32, lane = thread & 31;   // row0_w: the warp's first row
+      blk /= a.BH;
+      int sq = 0;
+      if constexpr (NSEQ > 1) {
+        while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
+        blk -= a.block0[sq];
+      }
+      const RowBlock rb = decode_block(a.plan[sq], blk);
+      const int q = rb.q0 + t * kTile + row0_w, left = rb.q_end - q;   // first query of the warp, rows from there on
+      const size_t row0 = (size_t)bh * a.N + a.tok0[sq] + q;           // its row of O and LSE
+      unsigned char* stage = smem_raw + (smem0 - smem_u32(smem_raw)) + t * Cfg::kQRegion + row0_w * kStageStride;
+      if (mbar_wait_warp(smem_u32(&bars.pv_done[t]), (nt - 1) & 1, abort)) {
+        tc_fence_after_sync();
+        const float inv = 1.0f / l;
+        unsigned char* srow = stage + lane * kStageStride;
+        // the remainder goes straight to global memory (contiguous bytes per thread, written once)
+        __nv_bfloat16* lo_row = a.Olo && lane < left ? a.Olo + (row0 + lane) * D : nullptr;
 #pragma unroll
-      for (int q = 0; q < D / 32; ++q) {
-        uint32_t o[32];
-        tmem_ld32(O_addr + q * 32, o);
-        tmem_wait_ld();
+        for (int q = 0; q < D / 32; ++q) {
+          uint32_t o[32];
+          tmem_ld32(O_addr + q * 32, o);
+          tmem_wait_ld();
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          float f[8];
+          for (int v = 0; v < 4; ++v) {
+            float f[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(o[8 * v + e]) * inv;
-          uint4 w;
-          w.x = pack_bf16(f[0], f[1]); w.y = pack_bf16(f[2], f[3]);
-          w.z = pack_bf16(f[4], f[5]); w.w = pack_bf16(f[6], f[7]);
-          *reinterpret_cast<uint4*>(srow + (q * 4 + v) * 16) = w;
-          if (lo_row) {
-            const uint32_t hw[4] = {w.x, w.y, w.z, w.w};
-            uint32_t lw[4];
+            for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(o[8 * v + e]) * inv;
+            uint4 w;
+            w.x = pack_bf16(f[0], f[1]); w.y = pack_bf16(f[2], f[3]);
+            w.z = pack_bf16(f[4], f[5]); w.w = pack_bf16(f[6], f[7]);
+            *reinterpret_cast<uint4*>(srow + (q * 4 + v) * 16) = w;
+            if (lo_row) {
+              const uint32_t hw[4] = {w.x, w.y, w.z, w.w};
+              uint32_t lw[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-              lw[e] = pack_bf16(f[2 * e] - __uint_as_float(hw[e] << 16), f[2 * e + 1] - __uint_as_float(hw[e] & 0xffff0000u));
-            *reinterpret_cast<uint4*>(lo_row + q * 32 + v * 8) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+              for (int e = 0; e < 4; ++e)
+                lw[e] = pack_bf16(f[2 * e] - __uint_as_float(hw[e] << 16), f[2 * e + 1] - __uint_as_float(hw[e] & 0xffff0000u));
+              *reinterpret_cast<uint4*>(lo_row + q * 32 + v * 8) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+            }
           }
         }
+        if (lane < left) a.LSE[row0 + lane] = m * a.scale + logf(l);
+        __syncwarp();
+        if (!*abort) store_rows<kRowBytes>(stage, kStageStride, reinterpret_cast<unsigned char*>(a.O + row0 * D), kRowBytes, left, lane);
       }
-      if (lane < left) a.LSE[row0 + lane] = m * a.scale + logf(l);
-      __syncwarp();
-      if (!*abort) store_rows<kRowBytes>(stage, kStageStride, reinterpret_cast<unsigned char*>(a.O + row0 * D), kRowBytes, left, lane);
     }
   }
 
