@@ -110,6 +110,12 @@ constexpr int kDecKeys = 128;     // its keys per CTA (32 per warp), staged in s
 // Warps of the largest CTA: 128 registers hold the operands of one group of 8 heads; two groups take more.
 __host__ __device__ constexpr int dec_max_warps(int nh) { return nh == 1 ? kDecMaxWarps : kDecMaxWarps / 2; }
 
+// Blocks of keys that a warp brings into L2 while the kernel in front ends, where every warp has at least kDecPrefetchMin to do: the
+// transfers then start about 2 us earlier.  us a token, without | with 2 | 4 | 16 blocks: 16 sequences of 28/4 heads at 32K (16 blocks a
+// warp) 56.1 | 53.9 | 54.6 | 72, four of 32/8 (8 blocks) 32.2 | 30.7 | 32.8 | 38, eight at 8K (3 blocks) 19.9 | 20.1 | 21 | 21, one at 32K (2.3
+// blocks, in L2 already) 12.9 | 13.7 | 13.9 | 13.9.
+constexpr int kDecPrefetch = 2, kDecPrefetchMin = 4;
+
 struct DecodeArgs {
   const __nv_bfloat16 *q, *k_list, *k_ring;
   long long v_of_list, v_of_ring;   // bytes from a K row to its V row
@@ -199,9 +205,6 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
   const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nw = blockDim.x >> 5, g = lane >> 2, t = lane & 3;
   const int b = bh / a.Hkv, hkv = bh % a.Hkv;
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the cache rows of the kernel in front of this one
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (blockIdx.x == 0 && bh == 0 && tid == 0) *a.status = 0;
   const unsigned char* kl = reinterpret_cast<const unsigned char*>(a.k_list) + (size_t)bh * a.rows_list * (D * 2);
   const unsigned char* kr = reinterpret_cast<const unsigned char*>(a.k_ring) + (size_t)bh * a.ring_rows * (D * 2);
   // K row of key `key`, and what leads from there to its V row
@@ -215,6 +218,16 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
   };
   const int nx = a.n_split * a.n_group;
   const int blk0 = (int)((long long)a.blocks * blockIdx.x / nx), blk1 = (int)((long long)a.blocks * (blockIdx.x + 1) / nx);
+  // While the kernel in front of this one ends, the warp's first blocks of the list are brought into L2 (a hint: what that kernel
+  // writes is read from L2 all the same, after the wait).
+  if (lane < 2 && blk1 - blk0 >= kDecPrefetchMin * nw) {
+    for (int blk = blk0 + warp, i = 0; blk < blk1 && i < kDecPrefetch && (blk + 1) * 16 * U <= a.n_list; blk += nw, ++i)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kl + (size_t)blk * (16 * U * D * 2) + (lane ? a.v_of_list : 0)),
+                   "r"(16 * U * D * 2) : "memory");
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the cache rows of the kernel in front of this one
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blockIdx.x == 0 && bh == 0 && tid == 0) *a.status = 0;
 
   for (int g0 = 0; g0 < a.G; g0 += 8 * NH) {
     // Q of head g0 + 8h + g as the B operand: the chunks this lane also takes of every key row.  The same for every warp;
