@@ -129,7 +129,9 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
       mbar_init(smem_u32(&bars.pv_done[t]), 1);
     }
     fence_barrier_init();
-    // Q, K_0 and V_0 are fetched while the other warps get their tensor memory
+    // Q, K_0 and V_0 are fetched while the other warps get their tensor memory, Q into L2 while the kernel in front ends
+    for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)
+      for (int h = 0; h < Cfg::kSub; ++h) tma_prefetch_3d(&maps.q[sq], h * 64, rb.q0 + t * kTile, bh);
     asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
     mbar_expect_tx(smem_u32(&bars.q_full), (n1 > 0 ? 2 : 1) * Cfg::kTileBytes);
     for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)

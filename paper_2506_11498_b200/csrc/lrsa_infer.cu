@@ -66,22 +66,23 @@ struct CacheRows {
 // A 32K prompt (windows of 1024 tokens, 4 KV heads, d = 128): window after window, three launches each, 1.25 ms;
 // scoring all windows in one launch and this kernel behind it 42 us.
 __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
   const int rpb = 256 / a.cpr;   // rows per block
   const int bh = blockIdx.x / a.blocks, item = (blockIdx.x % a.blocks) * rpb + threadIdx.x / a.cpr, ch = threadIdx.x % a.cpr;
   const int n_tok = a.n_sink + a.n_ins;
-  if (item >= n_tok + a.n_keep) return;
   const size_t list0 = (size_t)bh * a.rows_list, ring0 = (size_t)bh * 2 * a.L;
-  size_t src, dst;
+  size_t src = 0, dst = 0;
   bool from_ring = false, to_list = true;
   if (item < n_tok) {
     const int p = item < a.n_sink ? a.p_first + item : a.p0 + (item - a.n_sink);
     src = (size_t)bh * a.n_new + (p - a.p_first);
     to_list = p < a.S;
     dst = to_list ? list0 + p : ring0 + (p - a.S) % (2 * a.L);
-  } else {
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
+  if (item >= n_tok + a.n_keep) return;
+  if (item >= n_tok) {
     const int r = item - n_tok;
     const int pos = a.idx[((size_t)bh * a.Wcap + a.w0) * a.K + r];
     from_ring = a.keep_from_ring != 0;
@@ -222,8 +223,7 @@ __global__ void __launch_bounds__(dec_max_warps(NH) * 32, 1) decode_kernel(const
   // writes is read from L2 all the same, after the wait).
   if (lane < 2 && blk1 - blk0 >= kDecPrefetchMin * nw) {
     for (int blk = blk0 + warp, i = 0; blk < blk1 && i < kDecPrefetch && (blk + 1) * 16 * U <= a.n_list; blk += nw, ++i)
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kl + (size_t)blk * (16 * U * D * 2) + (lane ? a.v_of_list : 0)),
-                   "r"(16 * U * D * 2) : "memory");
+      ptx::prefetch_l2(kl + (size_t)blk * (16 * U * D * 2) + (lane ? a.v_of_list : 0), 16 * U * D * 2);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the cache rows of the kernel in front of this one
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
