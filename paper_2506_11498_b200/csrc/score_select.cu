@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kThreads) score_select_kernel(const ScoreArgs 
 // the sum over a token's channels ends with two shuffle levels.  A row per 16 lanes with scale and offset in registers,
 // the layout of the kernel this one replaces, spent twice the instructions (12 per channel pair, 6 here) on exchanges, and
 // one CTA per window left most of the GPU idle when there were few.  Calls back to back on one set of tensors, that kernel | this one, us:
-// 4 KV heads, d = 128: 32K tokens in windows of 1024 32.8 | 22.5 (with inputs that change from call to call 35.9 | 27.5, 2.4 TB/s of
+// 4 KV heads, d = 128: 32K tokens in windows of 1024 32.8 | 22.5 (with inputs that change from call to call 35.9 | 25.5, 2.6 TB/s of
 // algorithmic bytes; every window is read twice, the second time from L2), 64K of 2048 61.2 | 48.4, 32K of 256 41.0 | 26.7, 1777 tokens
 // of 512 20.5 | 9.0; 8 KV heads, 128K of 4096 184 | 160.  What is left is a chain: two streams
 // of at most 16 warps' loads an SM, the exchange, the selection (about 3 us).
