@@ -80,7 +80,8 @@ struct FwdBars {
 
 // Place of this CTA among the blocks of all heads, which are numbered heaviest first.  The CTAs of a grid of between one and
 // two per SM (`fold`: how many more than one) all start at once, the second ones on the first SMs again: the heaviest blocks get an SM of
-// their own, the others are paired heavy with light.
+// their own, the others are paired heavy with light (4K tokens, 8 heads, d = 64, 264
+// blocks: 27.8 -> 26.5 us).
 __device__ __forceinline__ int block_rank(int fold) {
   const int x = blockIdx.x;
   if (fold == 0) return x;
@@ -426,7 +427,8 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     // The output rows go through shared memory (the tile's Q region, idle once its last S product is done,
     // which pv_done implies), so that a warp writes whole rows: per-thread 16-byte stores to rows 256 bytes
     // apart cost a transaction each.  Rows are padded by 16 bytes so that a warp's stores spread over the banks.
-    // (With a bulk copy per row a CTA waits for the copies to have read them before it may end.)
+    // (With a bulk copy per row a CTA waits for the copies to have read them before it may end: 1777 tokens, 28 heads, 31.0 -> 30.5 us, and
+    // 30.2 with the first loads ahead of tensor memory.)
     constexpr int kRowBytes = D * 2, kStageStride = kRowBytes + 16;
     static_assert(kTile * kStageStride <= Cfg::kQRegion, "staging fits the Q region");
     if (ok && nt > 0) {
