@@ -11,7 +11,8 @@ constexpr int kTile = 128;                 // rows of a query tile, keys of a ke
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz: no wait in a correct run gets close
 
 // Waits for the phase with the given parity; gives up (returns false, raises *abort) when another
-// thread of the CTA has given up or after kWaitCycles.
+// thread of the CTA has given up or after kWaitCycles.  For a branch of one thread: every lane reads the clock and *abort
+// by itself, so the lanes of a warp may give up apart from one another.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
   if (ptx::mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
@@ -24,13 +25,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-// The same wait executed by all 32 lanes of a converged warp, with one verdict for the warp.  The
+// The same wait executed by all 32 lanes of a converged warp, with one verdict for the warp: what follows is
+// warp-wide (tensor-memory accesses, __syncwarp) and must be reached by all lanes or by none.  The
 // warps that issue tcgen05.mma run in warp-uniform control flow with descriptors computed once
 // outside the loops (building a descriptor per instruction in a single-lane branch costs ~100
 // cycles per MMA, more than the MMA itself) and issue through one lane, by predicate.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort) {
   const bool ok = mbar_wait(bar, parity, abort);
   return __all_sync(0xffffffffu, ok);
+}
+
+// The same wait executed by all 32 lanes, with a verdict for each: the caller must not branch on them before it has voted
+// (__all_sync), so that the lanes stay together.
+__device__ __forceinline__ bool mbar_wait_lanes(uint32_t bar, uint32_t parity, volatile int* abort) {
+  return mbar_wait(bar, parity, abort);
 }
 
 // A block of query rows that share one key list: rows [q0, q_end) (at most `rows_per_block`), all in
