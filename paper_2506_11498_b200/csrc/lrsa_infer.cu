@@ -64,25 +64,29 @@ struct CacheRows {
 // the list (items: tokens first, then kept rows; a thread moves 16 bytes of K and of V).  Bound by the rows it moves
 // (one read and one write each); one launch for a whole prompt, whose tokens go to the ring only if they stay there.
 // A 32K prompt (windows of 1024 tokens, 4 KV heads, d = 128): window after window, three launches each, 1.25 ms;
-// scoring all windows in one launch and this kernel behind it 42 us.
+// scoring all windows in one launch and this kernel behind it 34 us.
+// The wait comes first, not behind the index work.  The decode kernel behind this one starts when every block here has passed the wait,
+// and its clusters take the SMs that are free then: with shorter blocks most tokens take 0.2 us less, but where the clusters
+// about fill the GPU some find room a round later.  Index work behind | ahead of the wait, us a token: 28/4 heads, d = 128, at 33K
+// 14.7 | 14.4, eight sequences at 16K 28.3 | 25.6, two at 120K 30.2 | 32.1; two of 32/8 at 120K 47.6 | 50.1; 8/8 heads, d = 64, four at 33K
+// 18.8 | 22.0; 16/2, sixteen at 16K 18.2 | 20.0 (the wait first, and prefetch in neither kernel: 15.0, 28.6, 30.9, 48.4, 20.0, 18.5).
 __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
   const int rpb = 256 / a.cpr;   // rows per block
   const int bh = blockIdx.x / a.blocks, item = (blockIdx.x % a.blocks) * rpb + threadIdx.x / a.cpr, ch = threadIdx.x % a.cpr;
   const int n_tok = a.n_sink + a.n_ins;
+  if (item >= n_tok + a.n_keep) return;
   const size_t list0 = (size_t)bh * a.rows_list, ring0 = (size_t)bh * 2 * a.L;
-  size_t src = 0, dst = 0;
+  size_t src, dst;
   bool from_ring = false, to_list = true;
   if (item < n_tok) {
     const int p = item < a.n_sink ? a.p_first + item : a.p0 + (item - a.n_sink);
     src = (size_t)bh * a.n_new + (p - a.p_first);
     to_list = p < a.S;
     dst = to_list ? list0 + p : ring0 + (p - a.S) % (2 * a.L);
-  }
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
-  if (item >= n_tok + a.n_keep) return;
-  if (item >= n_tok) {
+  } else {
     const int r = item - n_tok;
     const int pos = a.idx[((size_t)bh * a.Wcap + a.w0) * a.K + r];
     from_ring = a.keep_from_ring != 0;
