@@ -59,7 +59,6 @@ struct FwdArgs {
   int tok0[NSEQ];          // first token of the sequence
   int block0[NSEQ + 1];    // blocks of the sequences before, per (batch, head)
   int n_seqs;
-  int fold;                // see block_rank
   int BH, Hq, Hkv, G, N;   // N: tokens per (batch, head) row of O and LSE (the row stride)
   __nv_bfloat16* O;
   __nv_bfloat16* Olo;        // optional: receives bf16(O_fp32 - O), the part of the output the bf16 O cannot hold
@@ -78,16 +77,6 @@ struct FwdBars {
   uint64_t p_full[2][kPParts];      // per query tile: the parts of P_t (128 / kPParts keys each) are stored
 };
 
-// Place of this CTA among the blocks of all heads, which are numbered heaviest first.  The CTAs of a grid of between one and
-// two per SM (`fold`: how many more than one) all start at once, the second ones on the first SMs again: the heaviest blocks get an SM of
-// their own, the others are paired heavy with light (4K tokens, 8 heads, d = 64, 264
-// blocks: 27.8 -> 26.5 us).
-__device__ __forceinline__ int block_rank(int fold) {
-  const int x = blockIdx.x;
-  if (fold == 0) return x;
-  return x >= kSms ? kSms + fold - 1 - (x - kSms) : x < fold ? kSms - fold + x : x - fold;
-}
-
 template <int D, int NSEQ, int TQ>
 __global__ void __launch_bounds__(FwdCfg<D, TQ>::kThreads, FwdCfg<D, TQ>::kPerSm)
 lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constant__ FwdArgs<NSEQ> a) {
@@ -102,8 +91,8 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = smem0, sRing = smem0 + TQ * Cfg::kQRegion;
 
-  const int bh = block_rank(a.fold) % a.BH;
-  int blk = block_rank(a.fold) / a.BH, sq = 0;
+  const int bh = blockIdx.x % a.BH;
+  int blk = blockIdx.x / a.BH, sq = 0;
   if constexpr (NSEQ > 1) {
     while (sq + 1 < a.n_seqs && blk >= a.block0[sq + 1]) ++sq;
     blk -= a.block0[sq];
@@ -434,7 +423,7 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
     if (ok && nt > 0) {
       // (where the rows lie is formed here again, from the thread and block numbers: kept through the loop it costs registers
       // that the scores need)
-      int blk = block_rank(a.fold), thread = threadIdx.x;
+      int blk = blockIdx.x, thread = threadIdx.x;
       asm volatile("" : "+r"(blk), "+r"(thread));
       const int bh = blk % a.BH, w = thread >> 5, t = (w - 4) >> 2, row0_w = (w & 3) * 32, lane = thread & 31;   // row0_w: the warp's first row
       blk /= a.BH;
@@ -586,7 +575,6 @@ static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat1
   a.status = status;
   const long long grid = (long long)a.block0[b.n] * a.BH;
   if (grid > 0x7fffffffLL) return LRSA_ERR_UNSUPPORTED;
-  a.fold = Cfg::kPerSm == 2 && grid > kSms && grid <= 2 * kSms ? (int)grid - kSms : 0;
   auto kern = lrsa_fwd_kernel<D, NSEQ, TQ>;
   LRSA_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
   LRSA_CUDA_CHECK(launch_dependent(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmem, st, 1, m, a));
