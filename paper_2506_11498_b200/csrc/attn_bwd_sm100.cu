@@ -12,6 +12,7 @@ using namespace ptx;
 
 constexpr int kPrepUnroll = 4;
 constexpr int kZeroPerThread = 16;   // float4 per thread of a zeroing block
+constexpr int kMeanPrefetch = 256;   // rows of K that a block of the mean key brings into L2 ahead
 
 struct PrepArgs {
   const __nv_bfloat16 *O, *Olo, *dO, *K;
@@ -111,8 +112,10 @@ __device__ __forceinline__ void prep_mean(const PrepArgs& a, int block) {
 // of the mean key per head whatever its length 7.8 us at 4K (8 heads, d = 64), now 5.7.
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const __grid_constant__ PrepArgs a) {
   const int b = blockIdx.x;
-  // while the kernel in front ends: the rows of dO or K that the block reads, into L2 (a hint; with the forward's Q 119.6 -> 119.0 us
-  // for a 4K training step of 8 heads, d = 64)
+  // While the kernel in front ends: the rows of dO or the first rows of K that the block reads, into L2 (a hint).  Whole backward with
+  // neither | dO | both, us: 1000 tokens (28/4 heads, d = 128) 62.3 | 62.0 | 61.5, 1777 102.0 | 101.2 | 101.0, 4K (8/8, d = 64) 83.6 | 83.1 | 82.7; with
+  // a kernel in front that writes dO and lets nothing start early 67.5 | 67.5 | 65.9, 110.6 | 110.6 | 110.3, 87.4 | 87.5 | 86.3 (1777 tokens of 8/8
+  // 55.4 | 55.5 | 56.0).  Bounded, because at 128K tokens the parts of K are together several times as large as L2.
   if (threadIdx.x == 0) {
     if (b >= a.b_compact && b < a.b_stats) {
       const long long per = 8LL * kPrepUnroll * (32 / (a.d >> 3)), row = (b - a.b_compact) * per;
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __grid_constant__ P
     } else if (b >= a.b_setup && b < a.b_mean) {
       const int bh = (b - a.b_setup) / a.splits, split = (b - a.b_setup) % a.splits, per = (a.N + a.splits - 1) / a.splits;
       const int r0 = split * per, r1 = min(a.N, r0 + per);
-      if (r1 > r0) prefetch_l2(a.K + ((size_t)bh * a.N + r0) * a.d, (uint32_t)((r1 - r0) * a.d * 2));
+      if (r1 > r0) prefetch_l2(a.K + ((size_t)bh * a.N + r0) * a.d, (uint32_t)(min(r1 - r0, kMeanPrefetch) * a.d * 2));
     }
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
