@@ -46,6 +46,10 @@ struct FwdCfg {
   static_assert(D == 128 || TQ == 1, "d = 64 runs with one tile per CTA");
   static constexpr int kSmem = TQ * kQRegion + kStages * kTileBytes + 1024;
   static constexpr int kThreads = 128 + 128 * TQ;
+  // Loaded ahead of the block's barrier: Q, at d = 64 (half as many copies) also K_0 and V_0, with Q into L2 before that.  Every warp waits for the
+  // thread that issues them.  us, Q only | all of them: d = 128, 28/4 heads: 32K tokens in eight sequences (kernel alone) 782 | 811, 1777 29.6 | 29.8,
+  // 32K 2136 | 2155; 32/8, sixteen sequences of 2048 (kernel alone) 518 | 530; d = 64: 1777 tokens (8/8) 18.4 | 18.1, 4K 27.3 | 27.0, (16/2) 41.0 | 40.8.
+  static constexpr bool kFirstTiles = D == 64;
   // TMEM columns: accumulator O of query tile t at 128t, its S (and, packed over it, P) behind the accumulators
   static constexpr uint32_t kColO = 0, kColS = TQ * 128, kCols = 2 * TQ * 128;
 };
@@ -107,6 +111,17 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   // the list's last tile comes first when it holds no more than kShort keys: its products and exponentials are that wide
   const int sh = n_ct > 0 && rb.n_front - (n_ct - 1) * kTile <= kShort ? 1 : 0;
 
+  // K or V tile `it` of the order K_0, V_0, K_1, ... into its ring slot
+  auto load_tile = [&](int it) {
+    const int j = it >> 1, which = it & 1, slot = it % NS;
+    const uint32_t full = smem_u32(&bars.kv_full[slot]);
+    mbar_expect_tx(full, Cfg::kTileBytes);
+    const bool compact = j < n_ct;
+    const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
+    const int row = compact ? (j < sh ? n_ct - 1 : j - sh) * kTile : rb.dense_start + (j - n_ct) * kTile;
+    for (int h = 0; h < Cfg::kSub; ++h)
+      tma_load_3d(sRing + slot * Cfg::kTileBytes + h * Cfg::kSubBytes, map, h * 64, row, bh_kv, full);
+  };
   if (tid == 0) {
     prefetch_tensormap(&maps.q[sq]); prefetch_tensormap(&maps.k[sq]); prefetch_tensormap(&maps.v[sq]);
     prefetch_tensormap(&maps.kc[sq]); prefetch_tensormap(&maps.vc[sq]);
@@ -119,21 +134,14 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
       mbar_init(smem_u32(&bars.pv_done[t]), 1);
     }
     fence_barrier_init();
-    // Q, K_0 and V_0 are fetched while the other warps get their tensor memory, Q into L2 while the kernel in front ends
-    for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)
-      for (int h = 0; h < Cfg::kSub; ++h) tma_prefetch_3d(&maps.q[sq], h * 64, rb.q0 + t * kTile, bh);
+    // the first loads, while the other warps get their tensor memory
+    if constexpr (Cfg::kFirstTiles) tma_prefetch_3d(&maps.q[sq], 0, rb.q0, bh);   // while the kernel in front ends
     asm volatile("griddepcontrol.wait;" ::: "memory");   // started before the kernel in front of it has ended
     mbar_expect_tx(smem_u32(&bars.q_full), (n1 > 0 ? 2 : 1) * Cfg::kTileBytes);
     for (int t = 0; t < (n1 > 0 ? 2 : 1); ++t)
       for (int h = 0; h < Cfg::kSub; ++h)
         tma_load_3d(sQ + t * Cfg::kQRegion + h * Cfg::kSubBytes, &maps.q[sq], h * 64, rb.q0 + t * kTile, bh, smem_u32(&bars.q_full));
-    const int row = n_ct > 0 ? (sh ? n_ct - 1 : 0) * kTile : rb.dense_start;
-    for (int which = 0; which < 2; ++which) {
-      const CUtensorMap* map = n_ct > 0 ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
-      mbar_expect_tx(smem_u32(&bars.kv_full[which]), Cfg::kTileBytes);
-      for (int h = 0; h < Cfg::kSub; ++h)
-        tma_load_3d(sRing + which * Cfg::kTileBytes + h * Cfg::kSubBytes, map, h * 64, row, bh_kv, smem_u32(&bars.kv_full[which]));
-    }
+    if constexpr (Cfg::kFirstTiles) { load_tile(0); load_tile(1); }
   }
   if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_s), Cfg::kCols); tmem_relinquish(); }
   tc_fence_before_sync();
@@ -152,21 +160,12 @@ lrsa_fwd_kernel(const __grid_constant__ FwdMaps<NSEQ> maps, const __grid_constan
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      int it = 2;
+      int it = Cfg::kFirstTiles ? 2 : 0;
       bool ok = true;
-      for (int j = 1; j < n && ok; ++j) {
-        for (int which = 0; which < 2 && ok; ++which, ++it) {
-          const int slot = it % NS, use = it / NS;
-          if (use > 0) ok = mbar_wait(smem_u32(&bars.kv_empty[slot]), (use - 1) & 1, abort);
-          if (!ok) break;
-          const uint32_t full = smem_u32(&bars.kv_full[slot]);
-          mbar_expect_tx(full, Cfg::kTileBytes);
-          const bool compact = j < n_ct;
-          const CUtensorMap* map = compact ? (which ? &maps.vc[sq] : &maps.kc[sq]) : (which ? &maps.v[sq] : &maps.k[sq]);
-          const int row = compact ? (j < sh ? n_ct - 1 : j - sh) * kTile : rb.dense_start + (j - n_ct) * kTile;
-          for (int h = 0; h < Cfg::kSub; ++h)
-            tma_load_3d(sRing + slot * Cfg::kTileBytes + h * Cfg::kSubBytes, map, h * 64, row, bh_kv, full);
-        }
+      for (; it < 2 * n; ++it) {
+        if (it >= NS) ok = mbar_wait(smem_u32(&bars.kv_empty[it % NS]), (it / NS - 1) & 1, abort);
+        if (!ok) break;
+        load_tile(it);
       }
       if (!ok) {
         // give loads already in flight a bounded chance to land before the CTA's smem is released
