@@ -423,12 +423,12 @@ def test_packed_forms_for_many_ctas(heads, d, L, K, S, lens):
 
 
 @pytest.mark.parametrize("B,heads,N,d,L,K,S", [
-    (37, (1, 1), 304, 64, 128, 32, 4), (149, (1, 1), 100, 64, 128, 32, 0), (74, (1, 1), 304, 64, 128, 32, 4),   # 148, 149, 296 blocks
+    (37, (1, 1), 304, 64, 128, 32, 4), (149, (1, 1), 100, 64, 128, 32, 0), (74, (1, 1), 304, 64, 128, 32, 4),   # forward and dQ: 148, 149, 296 blocks
     (75, (1, 1), 304, 64, 128, 32, 4), (150, (1, 1), 304, 128, 128, 32, 4),   # 300; dK/dV of more than 592 CTAs
     (2, (14, 2), 2500, 128, 256, 64, 4), (9, (14, 2), 2500, 128, 256, 64, 4),   # tiles of several segments, in both orders
 ])
 def test_launch_orders_of_small_and_large_grids(B, heads, N, d, L, K, S):
-    """The order of a grid's blocks (which of them share an SM, longest segments first) follows its size: every sequence of a batch
+    """The launch order of dK/dV (longest segments first, or segment-major) follows the size of the grid: every sequence of a batch
     as on its own.  O and LSE bit-equal, gradients (sums in another order) within the bound of two bf16 results."""
     w = W("a_order", B, *heads, N, d, L, K, S, seed=61, values="channel_offset")
     dev = to_dev(workloads.generate(w))
@@ -461,6 +461,40 @@ def test_forward_gives_the_same_bits_every_time(B, heads, N, d, L, S):
     for _ in range(20):
         o, lse = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx)
         assert torch.equal(o, O) and torch.equal(lse, LSE)
+
+
+def _backward(w):
+    """Inputs of a backward call, and the call."""
+    dev = to_dev(workloads.generate(w))
+    p = lrsa.Params.from_workload(w)
+    idx, _ = lrsa.lrsa_score_select(p, dev["K"], dev["V"])
+    O, LSE = lrsa.lrsa_attn_fwd(p, dev["Q"], dev["K"], dev["V"], idx)
+    return lambda: lrsa.lrsa_attn_bwd(p, dev["Q"], dev["K"], dev["V"], O, dev["dO"], LSE, idx)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_dk_and_dv_have_the_same_bits_every_time(d):
+    """The same order of products, S^T over P^T and dP^T over dS^T.  No window is compressed here and a key tile is one CTA's (16 pairs
+    of head and query tile at most), so that every row of dK and dV is one sum of one thread block, added to zero."""
+    call = _backward(W("a_repeat_kv", 4, 16, 8, 1024, d, 512, 128, 0, seed=67))
+    _, dK, dV = call()
+    for _ in range(20):
+        _, dk, dv = call()
+        assert torch.equal(dk, dK) and torch.equal(dv, dV)
+
+
+@pytest.mark.parametrize("B,heads,N,d,L,S", [(1, (28, 4), 6000, 128, 512, 4), (2, (8, 8), 8000, 64, 256, 16)])
+def test_dq_is_the_same_every_time_but_for_roundings(B, heads, N, d, L, S):
+    """dS overwritten by the next scores, as above.  The rows' D is added up in any order, which moves it by fp32 roundings and with it
+    some bf16 roundings of dS and dQ: by 2^-7 of an element each, so by no more than that of a block's norm.  A product that
+    read a tile's next scores instead would move a whole block by a part of its own size."""
+    call = _backward(W("a_repeat_q", B, *heads, N, d, L, L // 4, S, seed=71))
+    blocks = lambda t: t.float().view(-1, 100 * d)   # 100 rows of one head
+    dQ = blocks(call()[0])
+    worst = 0.0
+    for _ in range(20):
+        worst = max(worst, float(((blocks(call()[0]) - dQ).norm(dim=1) / dQ.norm(dim=1)).max()))
+    assert worst <= 2.0 ** -7, worst
 
 
 def test_packed_single_sequence_equals_unpacked():
