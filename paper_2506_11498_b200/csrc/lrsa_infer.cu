@@ -57,6 +57,7 @@ struct CacheRows {
   int p0, n_ins;        // tokens [p0, p0 + n_ins) go to the sink rows of the list or to the ring
   int w0, n_keep;       // kept rows: n_keep = windows * K rows of windows w0 ...
   int blocks;           // thread blocks per (batch, KV head)
+  int wait_first;       // see below
   int keep_from_ring;   // their source: the ring (a window that had entered the cache before) or the new tokens
 };
 
@@ -65,28 +66,28 @@ struct CacheRows {
 // (one read and one write each); one launch for a whole prompt, whose tokens go to the ring only if they stay there.
 // A 32K prompt (windows of 1024 tokens, 4 KV heads, d = 128): window after window, three launches each, 1.25 ms;
 // scoring all windows in one launch and this kernel behind it 34 us.
-// The wait comes first, not behind the index work.  The decode kernel behind this one starts when every block here has passed the wait,
-// and its clusters take the SMs that are free then: with shorter blocks most tokens take 0.2 us less, but where the clusters
-// about fill the GPU some find room a round later.  Index work behind | ahead of the wait, us a token: 28/4 heads, d = 128, at 33K
-// 14.7 | 14.4, eight sequences at 16K 28.3 | 25.6, two at 120K 30.2 | 32.1; two of 32/8 at 120K 47.6 | 50.1; 8/8 heads, d = 64, four at 33K
-// 18.8 | 22.0; 16/2, sixteen at 16K 18.2 | 20.0 (the wait first, and prefetch in neither kernel: 15.0, 28.6, 30.9, 48.4, 20.0, 18.5).
-__global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
+__device__ __forceinline__ void wait_for_front() {
   asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
+}
+__global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
+  if (a.wait_first) wait_for_front();
   const int rpb = 256 / a.cpr;   // rows per block
   const int bh = blockIdx.x / a.blocks, item = (blockIdx.x % a.blocks) * rpb + threadIdx.x / a.cpr, ch = threadIdx.x % a.cpr;
   const int n_tok = a.n_sink + a.n_ins;
-  if (item >= n_tok + a.n_keep) return;
   const size_t list0 = (size_t)bh * a.rows_list, ring0 = (size_t)bh * 2 * a.L;
-  size_t src, dst;
+  size_t src = 0, dst = 0;
   bool from_ring = false, to_list = true;
   if (item < n_tok) {
     const int p = item < a.n_sink ? a.p_first + item : a.p0 + (item - a.n_sink);
     src = (size_t)bh * a.n_new + (p - a.p_first);
     to_list = p < a.S;
     dst = to_list ? list0 + p : ring0 + (p - a.S) % (2 * a.L);
-  } else {
+  }
+  if (!a.wait_first) wait_for_front();
+  if (a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
+  if (item >= n_tok + a.n_keep) return;
+  if (item >= n_tok) {
     const int r = item - n_tok;
     const int pos = a.idx[((size_t)bh * a.Wcap + a.w0) * a.K + r];
     from_ring = a.keep_from_ring != 0;
@@ -99,9 +100,18 @@ __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
   reinterpret_cast<uint4*>(to_list ? a.v_list : a.v_ring)[dst * a.cpr + ch] = v;
 }
 
+// Wait for the kernel in front before the index work, not behind it?  Behind it most tokens take 0.1 to 0.4 us less.  But the decode kernel that
+// follows starts when every block here has passed the wait, and its clusters, whose CTAs take an SM each, go where there is room then: where they about
+// fill the GPU, shorter blocks here leave some of them a round late.  us a token, before | behind, 16 to 32 (batch, KV head) pairs: 8/8 heads,
+// d = 64, four sequences at 33K 18.8 | 21.9, at 16K 14.6 | 16.5; 16/2, sixteen at 33K 22.6 | 24.4; 32/8, d = 128, two at 120K 47.2 | 49.7, four at
+// 66K 52.2 | 55.1; 28/4 eight at 33K 37.3 | 38.3 (at 16K 28.6 | 25.6).  Others: 28/4, one at 33K 14.7 | 14.4, two at 120K 30.1 | 32.0 (in a CUDA
+// graph 29.3 | 29.8); 8/8, d = 64, one at 33K 12.3 | 11.9, eight at 16K 19.1 | 18.8; 16/2, four at 16K 11.1 | 10.7, thirty-two 16.3 | 15.9.
+inline int wait_first(int BH) { return BH >= 16 && BH <= 32; }
+
 int launch_cache_rows(CacheRows a, int BH, cudaStream_t st) {
   const int rows = a.n_sink + a.n_ins + a.n_keep, rpb = 256 / a.cpr;
   a.blocks = (rows + rpb - 1) / rpb;
+  a.wait_first = wait_first(BH);
   LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), 0, st, 1, a));
   launch_counter().n++;
   return LRSA_OK;
