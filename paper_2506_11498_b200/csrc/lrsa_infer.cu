@@ -61,15 +61,16 @@ struct CacheRows {
   int keep_from_ring;   // their source: the ring (a window that had entered the cache before) or the new tokens
 };
 
+__device__ __forceinline__ void wait_for_front() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // New tokens into the sink rows of the list or into the ring, and the kept rows of newly compressed windows into
 // the list (items: tokens first, then kept rows; a thread moves 16 bytes of K and of V).  Bound by the rows it moves
 // (one read and one write each); one launch for a whole prompt, whose tokens go to the ring only if they stay there.
 // A 32K prompt (windows of 1024 tokens, 4 KV heads, d = 128): window after window, three launches each, 1.25 ms;
 // scoring all windows in one launch and this kernel behind it 34 us.
-__device__ __forceinline__ void wait_for_front() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // may be launched before the kernel in front of it has ended
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
   if (a.wait_first) wait_for_front();
   const int rpb = 256 / a.cpr;   // rows per block
@@ -100,18 +101,20 @@ __global__ void __launch_bounds__(256) cache_rows_kernel(const CacheRows a) {
   reinterpret_cast<uint4*>(to_list ? a.v_list : a.v_ring)[dst * a.cpr + ch] = v;
 }
 
-// Wait for the kernel in front before the index work, not behind it?  Behind it most tokens take 0.1 to 0.4 us less.  But the decode kernel that
-// follows starts when every block here has passed the wait, and its clusters, whose CTAs take an SM each, go where there is room then: where they about
-// fill the GPU, shorter blocks here leave some of them a round late.  us a token, before | behind, 16 to 32 (batch, KV head) pairs: 8/8 heads,
-// d = 64, four sequences at 33K 18.8 | 21.9, at 16K 14.6 | 16.5; 16/2, sixteen at 33K 22.6 | 24.4; 32/8, d = 128, two at 120K 47.2 | 49.7, four at
-// 66K 52.2 | 55.1; 28/4 eight at 33K 37.3 | 38.3 (at 16K 28.6 | 25.6).  Others: 28/4, one at 33K 14.7 | 14.4, two at 120K 30.1 | 32.0 (in a CUDA
-// graph 29.3 | 29.8); 8/8, d = 64, one at 33K 12.3 | 11.9, eight at 16K 19.1 | 18.8; 16/2, four at 16K 11.1 | 10.7, thirty-two 16.3 | 15.9.
-inline int wait_first(int BH) { return BH >= 16 && BH <= 32; }
+// Does the wait for the kernel in front come ahead of the index work?  With the index work first most tokens take 0.1 to 0.4 us less.  But the
+// decode kernel that follows starts when every block here has passed the wait, and its clusters, whose CTAs take an SM each, go where there is room
+// then: where they about fill the GPU, shorter blocks here leave some of them a round late.  us a token, wait first | index work first, 16 to 32
+// (batch, KV head) pairs: 8/8 heads, d = 64, four sequences at 33K 18.8 | 21.9, at 16K 14.6 | 16.5; 16/2, sixteen at 33K 22.6 | 24.4; 32/8, d = 128,
+// two at 120K 47.2 | 49.7, four at 66K 52.2 | 55.1; 28/4, eight at 33K 37.3 | 38.3 (at 16K 28.6 | 25.6).  Others: 28/4, one at 33K 14.7 | 14.4, two at
+// 120K 30.1 | 32.0 (in a CUDA graph 29.3 | 29.8); 8/8, d = 64, one at 33K 12.3 | 11.9, eight at 16K 19.1 | 18.8; 16/2, four at 16K 11.1 | 10.7,
+// thirty-two 16.3 | 15.9.  What finds room differs between GPUs: a second one gave 18.9 | 19.0 for four of 8/8,
+// 22.7 | 21.2 for sixteen of 16/2 and 47.6 | 50.1 for two of 32/8.  (Only for a token: behind the rows of a prompt comes its next piece, or nothing.)
+inline int wait_first(int n_new, int BH) { return n_new == 1 && BH >= 16 && BH <= 32; }
 
 int launch_cache_rows(CacheRows a, int BH, cudaStream_t st) {
   const int rows = a.n_sink + a.n_ins + a.n_keep, rpb = 256 / a.cpr;
   a.blocks = (rows + rpb - 1) / rpb;
-  a.wait_first = wait_first(BH);
+  a.wait_first = wait_first(a.n_new, BH);
   LRSA_CUDA_CHECK(launch_dependent(cache_rows_kernel, dim3((unsigned)a.blocks * BH), dim3(256), 0, st, 1, a));
   launch_counter().n++;
   return LRSA_OK;
@@ -126,9 +129,10 @@ constexpr int kDecKeys = 128;     // its keys per CTA (32 per warp), staged in s
 __host__ __device__ constexpr int dec_max_warps(int nh) { return nh == 1 ? kDecMaxWarps : kDecMaxWarps / 2; }
 
 // Blocks of keys that a warp brings into L2 while the kernel in front ends, where every warp has at least kDecPrefetchMin to do: the
-// transfers then start about 2 us earlier.  us a token, without | with 2 | 4 | 16 blocks: 16 sequences of 28/4 heads at 32K (16 blocks a
-// warp) 56.1 | 53.9 | 54.6 | 72, four of 32/8 (8 blocks) 32.2 | 30.7 | 32.8 | 38, eight at 8K (3 blocks) 19.9 | 20.1 | 21 | 21, one at 32K (2.3
-// blocks, in L2 already) 12.9 | 13.7 | 13.9 | 13.9.
+// transfers then start about 2 us earlier.  us a token, without | with 2 blocks: 16 sequences of 28/4 heads at 33K (16 blocks a warp) 53.1 |
+// 52.4, four of 32/8 34.3 | 33.7, eight of 8/8, d = 64, 30.1 | 28.3, one of 28/4 at 120K 22.0 | 21.5.  More is slower (16 sequences of 28/4 with 2 | 4 | 16
+// blocks 53.9 | 54.6 | 72, four of 32/8 30.7 | 32.8 | 38), and so it is for warps of fewer blocks (eight sequences at 8K, 3 blocks, without | with 2
+// 19.9 | 20.1, one at 32K, 2.3 blocks, in L2 already 12.9 | 13.7).
 constexpr int kDecPrefetch = 2, kDecPrefetchMin = 4;
 
 struct DecodeArgs {

@@ -73,6 +73,12 @@ def test_cache_growth_and_decode(w, steps):
         print(f"{w.name}: {checked} decode steps checked, {ties} windows differ only at oracle ties")
 
 
+@pytest.mark.parametrize("B,Hkv,d", [(15, 1, 64), (8, 2, 128), (16, 2, 64), (33, 1, 128)])   # 15, 16, 32, 33 pairs
+def test_growth_on_both_sides_of_the_row_copies_rule(B, Hkv, d):
+    """For one token of 16 to 32 (batch, KV head) pairs the row copies wait for the kernel in front before they form their indexes."""
+    test_cache_growth_and_decode(W("i_wait", B, 2 * Hkv, Hkv, 4 + 4 * 64 + 9, d, 64, 16, 4, seed=97), (1, 2, 70, 1, 64, 90))
+
+
 def test_decode_equals_forward_row():
     """The decode kernel and the training forward agree on the last row (same mask, different kernels)."""
     w = W("i_vs_fwd", 1, 8, 2, 4 + 6 * 256 + 100, 128, 256, 64, 4, seed=87)
