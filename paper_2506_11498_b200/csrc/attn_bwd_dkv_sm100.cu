@@ -18,7 +18,7 @@
 // dP^T(i+1) are computed, the rest of the softmax while dV and S^T are.  128 x 128 steps instead of 128 x 64 read
 // K_j and V_j half as often from shared memory (the tensor core's operands, 192 KB a step, are what bounds the
 // kernel together with the exponentials) and pay for half as many hand-offs.  At 32K tokens, 28/4 heads, d = 128, one kept
-// token in four: 4.02 ms alone and uncapped, tensor pipe 73 % active (128 x 64 steps: 5.23; these with a branch around each
+// token in four: 3.84 ms alone and uncapped, tensor pipe 74 % active (when it was 4.02: 128 x 64 steps 5.23; these with a branch around each
 // product and the waits for Q and dO between two products: 4.58).  Warps: 0 TMA producer, 1 issuer, 3 row statistics, 4-19 softmax and
 // epilogue.  A softmax warpgroup takes 32 query columns of every step: four warps per scheduler hide the latency
 // of one another's exponentials and tensor-memory accesses (two warps with 64 columns each: 4.71 ms), and P^T is

@@ -401,8 +401,9 @@ static int launch_dq_t(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, c
 
 int launch_bwd_dq_sm100(const Geom& whole, const SeqBatch& b, const BwdPtrs& p, cudaStream_t st) {
   // d = 64: one S/dP buffer per CTA and two CTAs per SM, which start and end at different times, once every SM has more than
-  // two CTAs to run (whole step, 8 heads: 8K tokens 266 -> 260 us, 8 x 2000 333 -> 320; 16/2 heads, 5K: 225 -> 218);
-  // otherwise two buffers, the shorter chain of a CTA alone (4K, 264 CTAs: 123.7 us, with one buffer 127.4).
+  // two CTAs to run; otherwise two buffers, the shorter chain of a CTA alone.  Whole backward, us, with one | two buffers (windows of 512): 8/8
+  // heads: 2K tokens (136 CTAs) 62.3 | 52.5, 3K (200) 65.7 | 60.2, 4K (264) 85.6 | 81.1, 5K (328) 100.8 | 100.7, 8K (520) 181.0 | 186.8,
+  // 8 x 2000 221.5 | 229.6; 16/2 heads: 2K (272) 62.9 | 60.3, 3K (400) 91.6 | 93.4, 5K (656) 168.0 | 172.5.
   long long ctas = 0;
   for (int s = 0; s < b.n; ++s) ctas += (long long)make_plan(b.g[s], kTile).total * whole.B * whole.Hq;
   const auto dq = whole.d == 128   ? (b.n == 1 ? launch_dq_t<128, 1, 2> : launch_dq_t<128, kMaxSeqs, 2>)

@@ -9,9 +9,14 @@ constexpr int kQRows = 128;   // query rows per inner tile
 // Inner iterations per CTA of the dK/dV kernel, from their number in the whole call: at most 128 (a CTA's start and its
 // additions to the accumulators are then lost in the rest), fewer in small problems, so that the longest list does not
 // outlast an even share (iterations / 148) by much, and never below 16.  Whole backward, us, at 8 | 16 | 32 | 64 | 128 iterations a CTA (the
-// rule's): 8/8 heads, d = 64: 4K tokens 88 | 85 | 94 | 94 | 94 (16), 8K 203 | 190 | 183 | 181 | 181 (16), 16K 685 | 601 | 578 | 566 | 561 (45);
-// 28/4, d = 128: 1777 tokens 110 | 112 | 114 | 159 | 216 (16), 4K 299 | 284 | 283 | 297 | 334 (16), 8K 878 | 785 | 754 | 731 | 725 (41),
-// 16K 2909 | 2671 | 2620 | 2471 | 2487 (128), 32K 9793 | 8645 | 8089 | 7809 | 7675 (128; 256: 7679); 32/8, 2K 170 | 122 | 125 | 173 | 173 (16).
+// rule's), windows of 512 and a quarter kept where nothing else stands:
+// 8/8 heads, d = 64: 2K tokens 42 | 52 | 52 | 52 | 52 (16), 4K 83 | 81 | 90 | 90 | 90 (16), 8K 192 | 181 | 175 | 174 | 173 (16), windows of 1024
+// 240 | 216 | 212 | 212 | 212 (16), 16K 555 | 509 | 496 | 488 | 484 (37: 489), of 1024 649 | 579 | 570 | 563 | 562 (45: 560);
+// 16/2, d = 64: 4K 138 | 132 | 126 | 157 | 240 (16), 8K 334 | 310 | 297 | 297 | 314 (23: 307);
+// 28/4, d = 128: 1777 105 | 98 | 99 | 139 | 213 (16), 4K 298 | 278 | 276 | 268 | 306 (16), 8K 819 | 750 | 734 | 739 | 715 (41: 725), windows of
+// 1024 995 | 922 | 892 | 886 | 915 (53: 878), 16K 2910 | 2628 | 2508 | 2414 | 2420 (128), 32K 9197 | 8269 | 7771 | 7555 | 7480 (128);
+// 32/8: 2K 141 | 129 | 133 | 180 | 179 (16), 4K 348 | 326 | 321 | 312 | 362 (16), 20K of 256 3785 | 3416 | 3264 | 3113 | 3093 (128).
+// At d = 64 the rule is 4 % off around 8K tokens and a fifth at 2K, where 8 would fill the SMs better.
 constexpr int kSegMax = 128;
 inline int dkv_segment(long long iters) {
   const long long s = iters / (kSms * 4);
@@ -19,9 +24,10 @@ inline int dkv_segment(long long iters) {
 }
 
 // Launch order of the dK/dV kernel: by length (see dkv_setup), with segments of a tile made about equally long?  Up to four CTAs per SM what
-// the last ones leave idle is what counts, beyond that the query tiles that neighbours share in L2.  Whole backward, us, by
-// length up to 0 | 4 | 6 | 8 CTAs per SM: 1777 tokens (28/4 heads, d = 128) 107 | 99 | 99 | 99, 5K (16/2, d = 64) 155 | 153 | 153 | 153;
-// 4K (28/4) 278 | 279 | 285 | 285, 8K 875 | 874 | 904 | 914, 8K (8/8, d = 64) 181 | 181 | 187 | 187, 16K (28/4) 2430 | 2440 | 2446 | 2509.
+// the last ones leave idle is what counts, beyond that the query tiles that neighbours share in L2.  Whole backward, us, by length
+// up to 0 | 4 | 6 | 8 CTAs per SM (windows of 512, a quarter kept): 1777 tokens (28/4 heads, d = 128) 107 | 99 | 99 | 99, 5K (16/2, d = 64)
+// 155 | 153 | 153 | 153; 4K (28/4) 278 | 279 | 285 | 285, 8K (8/8, d = 64) 181 | 181 | 187 | 187; windows of 1024 (28/4): 8K 875 | 874 | 904 | 914,
+// 16K 2430 | 2440 | 2446 | 2509.
 inline bool order_by_length(long long ctas) {
   return ctas <= 4 * kSms;
 }
@@ -132,7 +138,8 @@ __device__ inline int block_prefix(int v, int* total) {
 // Launch order of the (tile, segment) pairs (one block of 256 threads).  Iteration i of a tile is query tile
 // nq-1 - i/G (counted from the last query) of head i%G, so segment s of every compact tile covers the
 // same queries of the same heads.
-//   by length  (small grids): the longest segments first, so that the last ones to start are short.
+//   by length  (small grids): the longest segments of the sequence first, so that its last ones to start are short (the sequences of
+//              a packed row come one after another).
 //   otherwise  compact tiles are issued segment-major: the CTAs that run at the same time then stream the same Q_i / dO_i
 //              tiles and share them through L2 instead of fetching them from DRAM once per key tile.  Dense tiles (short
 //              lists, neighbours already overlap) follow in position order.
@@ -218,7 +225,7 @@ struct BwdPtrs {
   float *dKf, *dVf;         // fp32 accumulators [B*Hkv][N][d], zeroed
   int* status;
 };
-// Parts of the sum for the mean key: at most kMeanSplits, of 256 rows or more.
+// Parts of the sum for the mean key: at most kMeanSplits, of about 256 rows or more (a row of fewer is one part; the last may be shorter).
 constexpr int kMeanSplits = 64;
 inline int mean_splits(int rows) { return rows >= 256 * kMeanSplits ? kMeanSplits : rows > 256 ? rows / 256 : 1; }
 

@@ -70,8 +70,9 @@ inline BlockPlan make_plan(const Geom& g, int rows) {
   return p;
 }
 
-// Blocks are numbered heaviest first: tail chunk, then full chunks from the last to the first (inside
-// a chunk from the last rows to the first), then the sink region.
+// Blocks are numbered from the end of the sequence: tail chunk, then full chunks from the last to the first (inside a chunk
+// from the last rows to the first), then the sink region.  That is roughly heaviest first: the list grows from chunk to chunk, but with
+// L > K the first rows of a chunk have fewer keys than the last rows of the chunk in front of it.
 __device__ __forceinline__ RowBlock decode_block(const BlockPlan& p, int blk) {
   RowBlock r;
   int c, i;

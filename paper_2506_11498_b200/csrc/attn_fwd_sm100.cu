@@ -18,8 +18,8 @@
 // threads exchange nothing, and its 128 scores are held in registers at once (setmaxnreg: 216 for these threads).
 // What bounds it: the chain of a tile from S_t over its exponentials (one MUFU result per two clocks and thread, 1024
 // cycles a tile) to O_t and the next S_t, and the 1000 W power limit, under which the clock settles near 1.65 GHz.
-// At 32K tokens, 28/4 heads, d = 128, one kept token in four: 2.02 ms alone and uncapped (1.50 at the measured bf16 rate;
-// tensor pipe 62 % active); 2.14 ms as a prefill call with its selection, 8.5 at 64K.  With an issuing warp for S and one for O += P V,
+// At 32K tokens, 28/4 heads, d = 128, one kept token in four: 1.97 ms alone and uncapped (1.50 at the measured bf16 rate;
+// tensor pipe 63 % active); 2.14 ms under the power limit, 8.6 at 64K with its selection.  With an issuing warp for S and one for O += P V,
 // a barrier round trip between a tile's products and P handed over in one piece it takes 2.75 and 9.5 ms.  Measured on the way
 // (2.44 ms then) and not taken: sixteen softmax warps (16 rows x 128 columns each, 256-bit loads) 2.66; exponentials started with the
 // previous maximum, the tile taken again when it was raised, 2.47; a share of them on the FMA pipe, no gain at 1/8, 2.63 at 1/4.
@@ -583,8 +583,8 @@ static int launch_fwd_t(const Geom& whole, const SeqBatch& b, const __nv_bfloat1
 
 // One query tile per CTA and two CTAs per SM, or two tiles that share the K/V tiles in one CTA (d = 128)?  Two CTAs start and
 // end at different times and split a small grid more finely, but load K and V twice.  28 heads, us with one | two tiles:
-// few CTAs: 1777 tokens 41.4 | 43.1, 4K 86.1 | 88.0, 5K 114.0 | 119.1, 6K 184 | 181, 8K 246-257 | 244, 32K 2290 | 2143;
-// short lists: 16 x 600 tokens 115 | 145, 8 x 1300 160 | 181, 8 x 1777 211-218 | 220, 4 x 3000 (8 tiles) 225 | 220.
+// few CTAs (windows of 512): 1777 tokens 29.9 | 31.8, 3K 53.6 | 56.7, 4K 77.3 | 76.4, 5K 107.0 | 103.7, 6K 138 | 136, 8K 214 | 205, of 1024
+// 265 | 251, 32K of 1024 2329 | 2190; short lists: 16 x 600 tokens (of 256) 100 | 128, 8 x 1300 149 | 158, 8 x 1777 207 | 204, 4 x 3000 (8 tiles) 209 | 206.
 // d = 64 (always one tile): 4K 37.1 | 41.1, 16K 166 | 178, 64K 1904 | 2084: its K/V tiles cost half as much to load.
 static bool one_tile(const Geom& whole, const SeqBatch& b) {
   long long ctas = 0, keys = 0, tokens = 0;

@@ -121,7 +121,8 @@ int launch_attn_bwd_sm100(const lrsa_params_t* params, const Geom& g, const __nv
                           const float* LSE, const int32_t* idx, __nv_bfloat16* dQ, __nv_bfloat16* dK,
                           __nv_bfloat16* dV, void* ws, cudaStream_t st);
 // Launch (in clusters of `cluster` CTAs) that may start before the kernel in front of it has ended: the kernel itself waits
-// for that (griddepcontrol.wait) before it touches memory.  Memory that the kernel in front may have written is not read-only for
+// for that (griddepcontrol.wait) before it reads or writes memory; in front of that it may at most bring lines that it will read into
+// L2 (a hint: they are read behind the wait, from L2 where all writes meet).  Memory that the kernel in front may have written is not read-only for
 // such a kernel's lifetime: plain loads (or __ldcg), no __ldg and no __restrict__, which the compiler may also move ahead of the wait.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, A... args) {

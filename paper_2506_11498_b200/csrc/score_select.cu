@@ -484,7 +484,9 @@ score_select_cluster_kernel(const __grid_constant__ ScoreArgs a, const __grid_co
 
   const int first = i0 + wz * 8 * T;   // this warp's first token
   // While the kernel in front of this one ends: the warps' first two rounds of loads, into L2 (a hint: what that kernel writes is read from
-  // L2 all the same, after the wait).  Calls back to back with inputs that change, us, without | with one | two | all rounds:
+  // L2 all the same, after the wait).  It pays behind a kernel that lets this one start early and has not just written K and V, such as this library's.
+  // Behind one that has written them without | with two rounds, us, both kernels: 32K tokens (28/4 heads, d = 128, windows of 1024) 49.4 | 49.9,
+  // of 256 53.6 | 54.8, 128K of 4096 184.4 | 183.5, 32K (8/8, d = 64) 51.1 | 50.2, of 256 62.9 | 61.1.  Calls back to back with inputs that change, us, without | with one | two | all rounds:
   // 32K tokens (4 heads, d = 128, windows of 1024) 27.0 | 26.3 | 25.5 | 25.9, as part of a prompt's append 34.0 | 33.0 | 33.2 | 33.4, of a 4K training
   // step 120.6 | 119.4 | 119.5 | 119.4; a call for which the GPU is waited 42.2 | 42.2 | 42.4 | 45.
   if (lane == 0 && wz == 0 && i1 > i0)

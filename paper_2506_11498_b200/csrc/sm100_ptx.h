@@ -109,7 +109,7 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 // Order: the kernels let a product overwrite columns of tensor memory that an earlier product of the same thread reads (S over P,
 // dP over dS) without waiting in between.  PTX states that pipelining for products on one accumulator in one shape only.  That all
 // products of a thread run in the order of issue, whatever their accumulators and shapes, is what sm_100a does here, not a documented
-// guarantee; an overlap would show as outputs that change between repeats (tests/test_gpu_parity.py repeats the forward).
+// guarantee; an overlap would show as outputs that change between repeats (tests/test_gpu_parity.py repeats the forward and the backward).
 // SS: both operands K-major in a 128-byte-swizzled tile (32 bytes a step).
 __device__ __forceinline__ void umma_ss4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate, uint32_t leader) {
