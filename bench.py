@@ -194,7 +194,7 @@ def run_reference(args, w):
 # DRAM bytes per backward call (dK/dV + dQ kernels: dram__bytes_read.sum + dram__bytes_write.sum of one launch
 # each) from the ncu summary under profiles/, per workload; a workload without a capture of the current
 # kernels carries null
-BWD_DRAM_BYTES = {"cfg2_32k_gqa7_d128": 3.130e9}
+BWD_DRAM_BYTES = {"cfg2_32k_gqa7_d128": 3.094e9}
 
 
 def spawn_ranks(n: int) -> int:
